@@ -31,6 +31,8 @@ struct SpeciesState {
     double q_over_e = 0, m_over_me = 1, alpha = 0, h = 0;
     int64_t cap = 0, n = 0;
     Species64 s64{};            // FP64 path
+    int32_t *id64 = nullptr;    // FP64 path: id of every storage slot while sorted64
+    bool sorted64 = false;      // FP64 path: storage order is that of a sort (else it is id order)
     SpeciesMixed mb[2]{};       // mixed path: current and sort target
     int cur = 0;
     int *tile_start = nullptr;  // ntiles + 1, offsets of the current layout
@@ -60,6 +62,12 @@ struct Run {
     SpeciesState sp[PIC_MAX_SPECIES];
     int *offsets = nullptr, *block_sums = nullptr;
     int *perm = nullptr;        // sort scratch, max species capacity
+    // FP64 path: node averages, and the sort's scratch (null when the allocator had no room: no sort then)
+    double2 *nf64 = nullptr;
+    double *M64 = nullptr;      // moment planes of the current
+    int *counts64 = nullptr;
+    double *spare64 = nullptr;  // one particle array of the largest capacity
+    bool rotate64 = false;      // equal capacities: a gathered array trades places with the spare one
     double *rho_s = nullptr, *rho_tot = nullptr, *divb = nullptr;
     int smooth = 0;             // current smoothing passes per step (App. A.3.4)
     void *sbuf[2] = {nullptr, nullptr};     // compact smoothing buffers, 3 planes of 8-byte values each
@@ -140,6 +148,14 @@ struct pic_ctx {
 namespace {
 
 constexpr int64_t kHistCap = 1 << 16;
+// The FP64 path sorts its particles where the arrays they gather from and add to (48 B
+// of node fields and 64 or 96 B of moments per cell) exceed what L2 holds besides the
+// particle stream.  Measured per step, sorted every 16 steps against never: 128^3 with 32
+// particles per cell and species 56.2 against 94.1 ms, 4096^2 with 2 17.9 against 35.3,
+// 1024^2 with 50 (117 MB) 22.3 against 22.5; below, the sort only costs: 64^3 (45 MB) 7.50
+// against 7.45, 300 x 211 0.83 against 0.82.  An interval of 4 costs 58.7 ms at 128^3.
+constexpr int kSort64Interval = 16;
+constexpr size_t kSort64Bytes = 100u << 20;
 
 pic_status fail(pic_ctx *c, pic_status st, const char *fmt, ...) {
     char buf[512];
@@ -196,6 +212,23 @@ void *dev_alloc(pic_ctx *ctx, size_t bytes) {
     else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
     if (p) ctx->allocs.push_back({p, bytes});
     return p;
+}
+
+// As dev_alloc for memory the context can do without; clears the error of a failed cudaMalloc.
+void *dev_try_alloc(pic_ctx *ctx, size_t bytes) {
+    void *p = dev_alloc(ctx, bytes);
+    if (!p) cudaGetLastError();
+    return p;
+}
+
+void dev_release(pic_ctx *ctx, void *p) {
+    for (size_t q = 0; q < ctx->allocs.size(); ++q)
+        if (p && ctx->allocs[q].first == p) {
+            if (ctx->have_alloc) ctx->alloc.free(p, ctx->allocs[q].second, ctx->alloc.user);
+            else cudaFree(p);
+            ctx->allocs.erase(ctx->allocs.begin() + q);
+            return;
+        }
 }
 
 size_t real_size(const pic_ctx *ctx) { return ctx->precision == PIC_FP64 ? sizeof(double) : sizeof(float); }
@@ -327,9 +360,10 @@ __global__ void k_pick_mixed(Geom g, SpeciesMixed s, const int *inv, const long 
     }
 }
 
-__global__ void k_pick64(Species64 s, const long long *ids, long long m, int ndim, double *st) {
+// inv (nullable): storage slot of every id
+__global__ void k_pick64(Species64 s, const int *inv, const long long *ids, long long m, int ndim, double *st) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
-        const long long p = ids[q];
+        const long long p = inv ? inv[ids[q]] : ids[q];
         for (int c = 0; c < 3; ++c) {
             st[c * m + q] = (c < ndim) ? s.x[c][p] : 0.0;
             st[(3 + c) * m + q] = s.u[c][p];
@@ -352,6 +386,18 @@ __global__ void k_download_by_id(Geom g, SpeciesMixed s, const int *inv, long lo
         st[3 * stride + q] = s.u[0][p];
         st[4 * stride + q] = s.u[1][p];
         st[5 * stride + q] = s.u[2][p];
+    }
+}
+
+// The same of the FP64 path.
+__global__ void k_download64_by_id(Species64 s, const int *inv, int ndim, long long a, long long m, double *st,
+                                   long long stride) {
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
+        const int p = inv[a + q];
+        for (int c = 0; c < 3; ++c) {
+            st[c * stride + q] = c < ndim ? s.x[c][p] : 0.0;
+            st[(3 + c) * stride + q] = s.u[c][p];
+        }
     }
 }
 
@@ -562,7 +608,8 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
             return fail(ctx, PIC_EINVAL, "tile %dx%dx%d needs more shared memory than a CTA has", r.t.T[0], r.t.T[1],
                         r.t.T[2]);
     }
-    const int G = mixed ? r.t.H : 0;
+    // FP64: the cells around the box that a path or its faces reach (one below, two above)
+    const int G = mixed ? r.t.H : 2;
     Geom &g = r.g;
     g.ndim = d.ndim; g.nx = d.nx; g.ny = d.ny; g.nz = d.ndim == 2 ? 1 : d.nz;
     g.G = G; g.Gz = d.ndim == 3 ? G : 0;
@@ -593,6 +640,11 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         r.perm = (int *)dev_alloc(ctx, sizeof(int) * capmax);
         if (!r.nfA || !r.nfB || !r.offsets || !r.block_sums || !r.perm)
             return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
+    }
+    if (!mixed) {
+        r.nf64 = (double2 *)dev_alloc(ctx, 3 * sizeof(double2) * g.pcells);
+        r.M64 = (double *)dev_alloc(ctx, moment_planes64(d.ndim) * sizeof(double) * g.pcells);
+        if (!r.nf64 || !r.M64) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the node fields");
     }
     r.rho_s = (double *)dev_alloc(ctx, sizeof(double) * ncell);
     r.rho_tot = (double *)dev_alloc(ctx, sizeof(double) * ncell);
@@ -649,6 +701,70 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         }
     }
     return PIC_OK;
+}
+
+// Scratch of the FP64 sort: an id per particle, and for the largest species one
+// spare array and the permutation.  Allocated after everything a context needs; a
+// context that gets none of it steps unsorted (slower, the same result).
+void setup_sort64(pic_ctx *ctx, Run &r) {
+    const long long ncell = (long long)r.g.nx * r.g.ny * r.g.nz;
+    if ((size_t)r.g.pcells * (48 + 8 * moment_planes64(r.d.ndim)) <= kSort64Bytes || ncell > INT32_MAX) return;
+    int64_t cap = 0;
+    bool equal = true;
+    for (int s = 0; s < r.d.nspecies; ++s) {
+        if (s > 0 && r.sp[s].cap != r.sp[0].cap) equal = false;
+        cap = std::max(cap, r.sp[s].cap);
+    }
+    if (cap == 0) return;
+    std::vector<void *> got;
+    bool ok = true;
+    auto take = [&](size_t bytes) {
+        void *p = ok ? dev_try_alloc(ctx, bytes) : nullptr;
+        if (p) got.push_back(p);
+        else ok = false;
+        return p;
+    };
+    for (int s = 0; s < r.d.nspecies; ++s)
+        r.sp[s].id64 = (int32_t *)take(sizeof(int32_t) * (size_t)std::max<int64_t>(r.sp[s].cap, 1));
+    r.perm = (int *)take(sizeof(int) * cap);
+    r.counts64 = (int *)take(sizeof(int) * ncell);
+    r.offsets = (int *)take(sizeof(int) * ncell);
+    r.block_sums = (int *)take(sizeof(int) * sort_scan_scratch(ncell));
+    r.spare64 = (double *)take(sizeof(double) * cap);
+    r.rotate64 = equal;
+    if (ok) return;
+    for (void *p : got) dev_release(ctx, p);
+    for (int s = 0; s < r.d.nspecies; ++s) r.sp[s].id64 = nullptr;
+    r.perm = r.counts64 = r.offsets = r.block_sums = nullptr;
+    r.spare64 = nullptr;
+}
+
+// Reorder one species by r.perm (slot -> present slot), one array at a time.
+pic_status permute64(pic_ctx *ctx, Run &r, SpeciesState &S, bool keep_ids) {
+    cudaStream_t s = ctx->stream;
+    auto pass = [&](double *&a) -> pic_status {
+        launch_gather64(r.spare64, a, r.perm, S.n, s);
+        if (r.rotate64) std::swap(a, r.spare64);
+        else CK(cudaMemcpyAsync(a, r.spare64, sizeof(double) * S.n, cudaMemcpyDeviceToDevice, s));
+        return PIC_OK;
+    };
+    for (int a = 0; a < 3; ++a) {
+        if (a < r.d.ndim)
+            if (pic_status st = pass(S.s64.x[a])) return st;
+        if (pic_status st = pass(S.s64.u[a])) return st;
+    }
+    if (keep_ids) {
+        launch_gather_ids((int32_t *)r.spare64, S.sorted64 ? S.id64 : nullptr, r.perm, S.n, s);
+        CK(cudaMemcpyAsync(S.id64, r.spare64, sizeof(int32_t) * S.n, cudaMemcpyDeviceToDevice, s));
+    }
+    CK(cudaGetLastError());
+    S.sorted64 = keep_ids;
+    return PIC_OK;
+}
+
+pic_status sort_species64(pic_ctx *ctx, Run &r, SpeciesState &S) {
+    launch_perm64(r.g, S.s64, S.n, r.counts64, r.offsets, r.block_sums, (int *)r.spare64, r.perm, ctx->stream);
+    return permute64(ctx, r, S, true);
 }
 
 pic_status check_run(pic_ctx *ctx, int run) {
@@ -1067,23 +1183,41 @@ const typename SmoothValue<JT>::type *smooth_current(pic_ctx *ctx, Run &r, JT *c
     return launch_smooth_current<JT>(r.g, J, r.smooth, buf, ctx->stream);
 }
 
-void step_run(pic_ctx *ctx, Run &r) {
+pic_status step_run(pic_ctx *ctx, Run &r) {
     cudaStream_t s = ctx->stream;
     double *hslot = (r.hist_n < r.hist_cap) ? r.hist + 8 * r.hist_n : nullptr;
     const int nsp = r.d.nspecies;
     if (ctx->precision == PIC_FP64) {
         FieldPtrs<double> f = fields_of<double>(r);
+        int launches = 0;
+        if (r.spare64 && (!r.sorted || r.since_sort >= kSort64Interval)) {
+            KTimer t(ctx, PIC_KERNEL_SORT);
+            for (int q = 0; q < nsp; ++q)
+                if (r.sp[q].n > 0) {
+                    if (pic_status st = sort_species64(ctx, r, r.sp[q])) return st;
+                    launches += 5 + 2 * r.d.ndim;
+                }
+            r.sorted = true;
+            r.since_sort = 0;
+        }
+        r.since_sort++;
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{hslot, nullptr, 0}, s);
+            // after the first step the energy at u^{t-1/2} is what the step before recorded
+            launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{hslot, nullptr, 0},
+                                     hslot && r.hist_n > 0 ? hslot - 7 : nullptr, s);
+            launch_node_fields64(r.g, f, r.nf64, s);
         }
         double *J[3] = {jplane<double>(r, r.jcur, 0), jplane<double>(r, r.jcur, 1), jplane<double>(r, r.jcur, 2)};
         {
             KTimer t(ctx, PIC_KERNEL_PUSH);
+            CK(cudaMemsetAsync(r.M64, 0, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells, s));
             for (int q = 0; q < nsp; ++q) {
                 SpeciesState &S = r.sp[q];
-                launch_push_fp64(r.g, f, J, S.s64, S.n, S.h, S.alpha, r.d.dt, 0, S.m_over_me, hslot, ctx->d_err, s);
+                launch_push_fp64(r.g, r.nf64, r.M64, S.s64, S.n, S.sorted64, S.h, S.q_over_e < 0, r.d.dt,
+                                 S.m_over_me, hslot, r.hist_n == 0, ctx->d_err, s);
             }
+            launch_current64(r.g, r.M64, J, std::fabs(r.sp[0].alpha), s);
         }
         double *Z[3] = {jplane<double>(r, 1 - r.jcur, 0), jplane<double>(r, 1 - r.jcur, 1),
                         jplane<double>(r, 1 - r.jcur, 2)};
@@ -1091,12 +1225,12 @@ void step_run(pic_ctx *ctx, Run &r) {
         const double *Js = smooth_current<double>(ctx, r, J);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{nullptr, nullptr, 0}, s);
+            launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{nullptr, nullptr, 0}, nullptr, s);
             if (Js) launch_e_advance_smoothed<double, double, double>(r.g, f, Js, 1.0, Z, r.d.dt, nullptr, s);
             else launch_e_advance<double>(r.g, f, Jc, Z, r.d.dt, s);
         }
         ctx->bytes_per_ps = r.d.ndim == 2 ? 80.0 : 96.0;
-        ctx->launch_total += 3 + nsp + (Js ? r.smooth : 0);
+        ctx->launch_total += launches + 5 + nsp + (Js ? 1 + r.smooth : 0);   // shell fold + passes
     } else {
         int launches = 0;
         if (!r.sorted || r.since_sort >= r.sort_interval) {
@@ -1111,7 +1245,7 @@ void step_run(pic_ctx *ctx, Run &r) {
         FieldPtrs<float> f = fields_of<float>(r);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, hist_ref(r), s);
+            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, hist_ref(r), nullptr, s);
             launch_node_fields(r.g, f, r.nfA, r.nfB, s);
         }
         typedef unsigned long long u64;
@@ -1154,7 +1288,7 @@ void step_run(pic_ctx *ctx, Run &r) {
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
             const double alpha_abs = 2.0 / (r.d.n_x * r.d.n_x * r.d.rho_sp0);
-            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, HistRef{nullptr, nullptr, 0}, s);
+            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, HistRef{nullptr, nullptr, 0}, nullptr, s);
             if (Js)
                 launch_e_advance_smoothed<float, u64, long long>(r.g, f, Js, alpha_abs * 0x1p-36, Z, (float)r.d.dt,
                                                                  r.hist_idx, s);
@@ -1168,6 +1302,7 @@ void step_run(pic_ctx *ctx, Run &r) {
     r.jcur = 1 - r.jcur;
     r.step++;
     if (r.hist_n < r.hist_cap) r.hist_n++;
+    return PIC_OK;
 }
 
 }  // namespace
@@ -1179,7 +1314,8 @@ namespace {
 
 pic_status one_step(pic_ctx *ctx, int slot) {
     if (ctx->multi) return step_multi(ctx, slot);
-    for (auto &r : ctx->runs) step_run(ctx, r);
+    for (auto &r : ctx->runs)
+        if (pic_status st = step_run(ctx, r)) return st;
     return PIC_OK;
 }
 
@@ -1398,6 +1534,8 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
     ctx->mlpLoss = (double *)dev_alloc(ctx, sizeof(double));
     ctx->mlpF = (double *)dev_alloc(ctx, sizeof(double) * (size_t)ncombo * (kMjTable + 1));
     ctx->mlpPar = (double *)dev_alloc(ctx, sizeof(double) * 8 * ncombo);
+    if (precision == PIC_FP64)
+        for (auto &r : ctx->runs) setup_sort64(ctx, r);
     if (!ctx->staging || !ctx->mj_table || !ctx->mlpW || !ctx->mlpG || !ctx->mlpM || !ctx->mlpV || !ctx->mlpWh ||
         !ctx->mlpX || !ctx->mlpT || !ctx->mlpLoss || !ctx->mlpF || !ctx->mlpPar) {
         pic_destroy(ctx);
@@ -1473,6 +1611,7 @@ pic_status pic_set_state(pic_ctx *ctx, int run, const pic_state_view *in) {
         SpeciesState &S = r.sp[s];
         const int64_t n = in->count[s];
         S.n = n;
+        S.sorted64 = false;
         const double *P = in->particles[s];
         if (ctx->precision == PIC_FP64) {
             for (int a = 0; a < 3; ++a) {
@@ -1560,7 +1699,19 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
         out->count[s] = n;
         double *P = out->particles[s];
         if (n == 0 || !P) continue;
-        if (ctx->precision == PIC_FP64) {
+        if (ctx->precision == PIC_FP64 && S.sorted64) {
+            // as the mixed path below: by id, straight into page-locked buffers or through the staging buffer
+            k_id_index<<<nblk(n), 256, 0, sm>>>(S.id64, n, r.perm);
+            double *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n);
+            const int64_t chunk = Pm ? n : (int64_t)(ctx->staging_bytes / (6 * sizeof(double)));
+            for (int64_t a0 = 0; a0 < n; a0 += chunk) {
+                const int64_t m = std::min(chunk, n - a0);
+                k_download64_by_id<<<nblk(m), 256, 0, sm>>>(S.s64, r.perm, g.ndim, a0, m, Pm ? Pm : stg, m);
+                CK(cudaGetLastError());
+                for (int a = 0; !Pm && a < 6; ++a)
+                    CK(cudaMemcpyAsync(P + a * n + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
+            }
+        } else if (ctx->precision == PIC_FP64) {
             for (int a = 0; a < 3; ++a) {
                 if (a < g.ndim) CK(cudaMemcpyAsync(P + a * n, S.s64.x[a], sizeof(double) * n, cudaMemcpyDeviceToHost, sm));
                 CK(cudaMemcpyAsync(P + (3 + a) * n, S.s64.u[a], sizeof(double) * n, cudaMemcpyDeviceToHost, sm));
@@ -1605,14 +1756,14 @@ pic_status pic_get_particles(pic_ctx *ctx, int run, int species, const int64_t *
     // chunk are copied behind them
     const int64_t chunk = (int64_t)(ctx->staging_bytes / (7 * sizeof(double)));
     double *stg = (double *)ctx->staging;
-    if (ctx->precision == PIC_MIXED && S.n > 0)
-        k_id_index<<<nblk(S.n), 256, 0, sm>>>(S.mb[S.cur].id, S.n, r.perm);
+    if (S.n > 0 && (ctx->precision == PIC_MIXED || S.sorted64))
+        k_id_index<<<nblk(S.n), 256, 0, sm>>>(ctx->precision == PIC_MIXED ? S.mb[S.cur].id : S.id64, S.n, r.perm);
     for (int64_t a0 = 0; a0 < nids; a0 += chunk) {
         const int64_t m = std::min(chunk, nids - a0);
         long long *dids = reinterpret_cast<long long *>(stg + 6 * m);
         CK(cudaMemcpyAsync(dids, ids + a0, sizeof(long long) * m, cudaMemcpyHostToDevice, sm));
         if (ctx->precision == PIC_MIXED) k_pick_mixed<<<nblk(m), 256, 0, sm>>>(r.g, S.mb[S.cur], r.perm, dids, m, stg);
-        else k_pick64<<<nblk(m), 256, 0, sm>>>(S.s64, dids, m, r.d.ndim, stg);
+        else k_pick64<<<nblk(m), 256, 0, sm>>>(S.s64, S.sorted64 ? r.perm : nullptr, dids, m, r.d.ndim, stg);
         CK(cudaGetLastError());
         for (int a = 0; a < 6; ++a)
             CK(cudaMemcpyAsync(out + a * nids + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
@@ -1971,6 +2122,11 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
                                    (long long)C->n, n);
         colocate = 1;
     }
+    // a partner's positions are taken by id: bring it back to id order
+    if (C && C->sorted64) {
+        k_id_index<<<nblk(C->n), 256, 0, ctx->stream>>>(C->id64, C->n, r.perm);
+        if ((st = permute64(ctx, r, *C, false))) return st;
+    }
     if (method == PIC_MJ_MLP) return mlp_load(ctx, run, species, n, theta, beta, profile, L, x0, colocate_with, seed);
     const int naive = method == PIC_MJ_NAIVE_BOOST;
     const double b0 = std::sqrt(b2);
@@ -1992,6 +2148,7 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
     S.n = n;
     S.tiled = false;
     S.counted = false;
+    S.sorted64 = false;
     r.sorted = false;
     r.since_sort = 0;
     // initial staggering of the momenta: one Boris step of -dt/2 (App. A.3.1)
@@ -2000,9 +2157,8 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
         launch_node_fields(g, f, r.nfA, r.nfB, sm);
         launch_half_back_mixed(g, r.nfA, r.nfB, S.mb[S.cur], n, (float)S.h, (float)r.d.dt, sm);
     } else {
-        double *J[3] = {jplane<double>(r, r.jcur, 0), jplane<double>(r, r.jcur, 1), jplane<double>(r, r.jcur, 2)};
-        launch_push_fp64(g, fields_of<double>(r), J, S.s64, n, S.h, S.alpha, r.d.dt, 1, S.m_over_me, nullptr,
-                         ctx->d_err, sm);
+        launch_node_fields64(g, fields_of<double>(r), r.nf64, sm);
+        launch_half_back64(g, r.nf64, S.s64, n, S.h, r.d.dt, sm);
     }
     CK(cudaGetLastError());
     r.step = 0;
@@ -2093,6 +2249,7 @@ pic_status mlp_load(pic_ctx *ctx, int run, int species, long long n, double thet
     S.n = n;
     S.tiled = false;
     S.counted = false;
+    S.sorted64 = false;
     r.sorted = false;
     r.since_sort = 0;
     if (mixed) {
@@ -2100,9 +2257,8 @@ pic_status mlp_load(pic_ctx *ctx, int run, int species, long long n, double thet
         launch_node_fields(r.g, f, r.nfA, r.nfB, sm);
         launch_half_back_mixed(r.g, r.nfA, r.nfB, S.mb[S.cur], n, (float)S.h, (float)r.d.dt, sm);
     } else {
-        double *J[3] = {jplane<double>(r, r.jcur, 0), jplane<double>(r, r.jcur, 1), jplane<double>(r, r.jcur, 2)};
-        launch_push_fp64(r.g, fields_of<double>(r), J, S.s64, n, S.h, S.alpha, r.d.dt, 1, S.m_over_me, nullptr,
-                         ctx->d_err, sm);
+        launch_node_fields64(r.g, fields_of<double>(r), r.nf64, sm);
+        launch_half_back64(r.g, r.nf64, S.s64, n, S.h, r.d.dt, sm);
     }
     CK(cudaGetLastError());
     r.step = 0;

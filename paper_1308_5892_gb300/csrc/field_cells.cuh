@@ -246,38 +246,53 @@ __device__ __forceinline__ void e_smoothed_cell(const Geom &g, const FieldPtrs<R
 
 // Staggered value read by the gather; with conductor walls a value located
 // inside the conductor, or a tangential e / normal b on the wall, reads zero.
-__device__ inline float sval(const Geom &g, const float *a, bool xstag, int i, int j, int k) {
+template <typename R>
+__device__ inline R sval(const Geom &g, const R *a, bool xstag, int i, int j, int k) {
     if (g.bcx == 1) {
-        if (xstag) { if (i < 0 || i > g.nx - 1) return 0.f; }
-        else { if (i <= 0 || i >= g.nx) return 0.f; }
+        if (xstag) { if (i < 0 || i > g.nx - 1) return R(0); }
+        else { if (i <= 0 || i >= g.nx) return R(0); }
     }
     return ldro(a + g.widx(i, j, k));
 }
 
-// Node-averaged fields (App. A.3.3) at every padded node: e over its two edge
-// neighbours, b over its four face neighbours.  Stored as {E_x,E_y,E_z,B_x} and {B_y,B_z}.
+// Node-averaged fields (App. A.3.3) at padded node p: e over its two edge
+// neighbours, b over its four face neighbours.
+template <typename R>
+__device__ __forceinline__ void node_average(const Geom &g, const FieldPtrs<R> &f, long long p, R (&E)[3],
+                                             R (&B)[3]) {
+    int pi, pj, pk;
+    padded_coords(g, p, pi, pj, pk);
+    // node coordinate (not wrapped: the conductor masking needs the true x)
+    int i = pi - g.G;
+    const int j = pj - g.G, k = pk - g.Gz;
+    if (g.bcx == 0) i = g.wx(i);
+    E[0] = R(0.5) * (sval(g, f.e[0], true, i - 1, j, k) + sval(g, f.e[0], true, i, j, k));
+    E[1] = R(0.5) * (sval(g, f.e[1], false, i, j - 1, k) + sval(g, f.e[1], false, i, j, k));
+    E[2] = R(0.5) * (sval(g, f.e[2], false, i, j, k - 1) + sval(g, f.e[2], false, i, j, k));
+    B[0] = R(0.25) * (sval(g, f.b[0], false, i, j, k) + sval(g, f.b[0], false, i, j - 1, k) +
+                      sval(g, f.b[0], false, i, j, k - 1) + sval(g, f.b[0], false, i, j - 1, k - 1));
+    B[1] = R(0.25) * (sval(g, f.b[1], true, i, j, k) + sval(g, f.b[1], true, i - 1, j, k) +
+                      sval(g, f.b[1], true, i, j, k - 1) + sval(g, f.b[1], true, i - 1, j, k - 1));
+    B[2] = R(0.25) * (sval(g, f.b[2], true, i, j, k) + sval(g, f.b[2], true, i - 1, j, k) +
+                      sval(g, f.b[2], true, i - 1, j - 1, k) + sval(g, f.b[2], true, i, j - 1, k));
+}
+
+// Mixed path: stored as {E_x,E_y,E_z,B_x} and {B_y,B_z}.
 __device__ __forceinline__ void node_cell(const Geom &g, const FieldPtrs<float> &f, float4 *nfA, float2 *nfB,
                                           long long p) {
-    {
-        int pi, pj, pk;
-        padded_coords(g, p, pi, pj, pk);
-        // node coordinate (not wrapped: the conductor masking needs the true x)
-        int i = pi - g.G;
-        const int j = pj - g.G, k = pk - g.Gz;
-        if (g.bcx == 0) i = g.wx(i);
-        float E[3], B[3];
-        E[0] = 0.5f * (sval(g, f.e[0], true, i - 1, j, k) + sval(g, f.e[0], true, i, j, k));
-        E[1] = 0.5f * (sval(g, f.e[1], false, i, j - 1, k) + sval(g, f.e[1], false, i, j, k));
-        E[2] = 0.5f * (sval(g, f.e[2], false, i, j, k - 1) + sval(g, f.e[2], false, i, j, k));
-        B[0] = 0.25f * (sval(g, f.b[0], false, i, j, k) + sval(g, f.b[0], false, i, j - 1, k) +
-                        sval(g, f.b[0], false, i, j, k - 1) + sval(g, f.b[0], false, i, j - 1, k - 1));
-        B[1] = 0.25f * (sval(g, f.b[1], true, i, j, k) + sval(g, f.b[1], true, i - 1, j, k) +
-                        sval(g, f.b[1], true, i, j, k - 1) + sval(g, f.b[1], true, i - 1, j, k - 1));
-        B[2] = 0.25f * (sval(g, f.b[2], true, i, j, k) + sval(g, f.b[2], true, i - 1, j, k) +
-                        sval(g, f.b[2], true, i - 1, j - 1, k) + sval(g, f.b[2], true, i, j - 1, k));
-        nfA[p] = make_float4(E[0], E[1], E[2], B[0]);
-        nfB[p] = make_float2(B[1], B[2]);
-    }
+    float E[3], B[3];
+    node_average<float>(g, f, p, E, B);
+    nfA[p] = make_float4(E[0], E[1], E[2], B[0]);
+    nfB[p] = make_float2(B[1], B[2]);
+}
+
+// FP64 path: three planes of double2, {E_x,E_y} {E_z,B_x} {B_y,B_z}.
+__device__ __forceinline__ void node_cell64(const Geom &g, const FieldPtrs<double> &f, double2 *nf, long long p) {
+    double E[3], B[3];
+    node_average<double>(g, f, p, E, B);
+    nf[p] = make_double2(E[0], E[1]);
+    nf[g.pcells + p] = make_double2(E[2], B[0]);
+    nf[2 * g.pcells + p] = make_double2(B[1], B[2]);
 }
 
 }  // namespace

@@ -22,11 +22,13 @@ namespace pic {
 namespace {
 
 // b <- b - h curl e over every padded cell; with a history slot, the interior
-// sums of e^2 and b^2 are added to it.
+// sums of e^2 and b^2 are added to it.  kin_prev (nullable): the kinetic energy the
+// previous step recorded at u^{t-1/2}, which is this step's first entry.
 template <typename R>
-__global__ void k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist) {
+__global__ void k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, const double *kin_prev) {
     const long long stride = (long long)gridDim.x * blockDim.x;
     double *slot = hist.slot();
+    if (slot && kin_prev && blockIdx.x == 0 && threadIdx.x == 0) slot[0] = *kin_prev;
     double *energy_acc = slot ? slot + 2 : nullptr;
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
@@ -86,6 +88,12 @@ __global__ void k_node_fields(Geom g, FieldPtrs<float> f, float4 *nfA, float2 *n
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
         node_cell(g, f, nfA, nfB, p);
+}
+
+__global__ void k_node_fields64(Geom g, FieldPtrs<double> f, double2 *nf) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
+        node_cell64(g, f, nf, p);
 }
 
 // Batched over runs: block b belongs to the run r with block_prefix[r] <= b <
@@ -166,8 +174,8 @@ inline int grid_for(long long n, int threads) {
 }  // namespace
 
 template <typename R>
-void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, cudaStream_t s) {
-    k_b_advance<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, h, energy);
+void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s) {
+    k_b_advance<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, h, energy, kin_prev);
 }
 
 template <typename R>
@@ -179,6 +187,10 @@ void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *con
 
 void launch_node_fields(const Geom &g, FieldPtrs<float> f, float4 *nfA, float2 *nfB, cudaStream_t s) {
     k_node_fields<<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, nfA, nfB);
+}
+
+void launch_node_fields64(const Geom &g, FieldPtrs<double> f, double2 *nf, cudaStream_t s) {
+    k_node_fields64<<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, nf);
 }
 
 void launch_fields_multi(int phase, const FieldRunF *runs_dev, const int *block_prefix_dev, int nblocks, int nruns,
@@ -209,8 +221,9 @@ void launch_add_uniform(const Geom &g, FieldPtrs<R> f, const double e0[3], const
     k_add_uniform<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, e0[0], e0[1], e0[2], b0[0], b0[1], b0[2]);
 }
 
-template void launch_b_advance<float>(const Geom &, FieldPtrs<float>, float, HistRef, cudaStream_t);
-template void launch_b_advance<double>(const Geom &, FieldPtrs<double>, double, HistRef, cudaStream_t);
+template void launch_b_advance<float>(const Geom &, FieldPtrs<float>, float, HistRef, const double *, cudaStream_t);
+template void launch_b_advance<double>(const Geom &, FieldPtrs<double>, double, HistRef, const double *,
+                                       cudaStream_t);
 template void launch_e_advance<float>(const Geom &, FieldPtrs<float>, const float *const[3], float *const[3], float,
                                       cudaStream_t);
 template void launch_e_advance<double>(const Geom &, FieldPtrs<double>, const double *const[3], double *const[3],

@@ -14,8 +14,10 @@
 //    accumulated while the other is zeroed); node fields (mixed path): one
 //    float4 pair per padded cell, {E_x,E_y,E_z,B_x} {B_y,B_z,0,0}, the node
 //    averages of App. A.3.3 at time t.
+//  - FP64 path: node fields, three planes of double2, and the moment planes of the
+//    current (push_fp64.cu).
 //  - particles, FP64 path: SoA planes x,y,z,u_x,u_y,u_z of double (absolute
-//    positions); mixed path: packed cell coordinates (uint32), FP32 offsets
+//    positions), sorted by cell every few steps (then with an int32 id); mixed path: packed cell coordinates (uint32), FP32 offsets
 //    (SoA), FP32 momenta (SoA) and an int32 id, kept sorted by tile.
 #pragma once
 #include <cstdint>
@@ -206,12 +208,14 @@ struct HistRef {
 // ---- kernel launchers (implemented in the .cu files) ----
 
 // fields.cu
+// kin_prev (nullable): copied to slot[0] of the energy record
 template <typename R>
-void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, cudaStream_t s);
+void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s);
 template <typename R>
 void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *const Jzero[3], R dt,
                       cudaStream_t s);
 void launch_node_fields(const Geom &g, FieldPtrs<float> f, float4 *nfA, float2 *nfB, cudaStream_t s);
+void launch_node_fields64(const Geom &g, FieldPtrs<double> f, double2 *nf, cudaStream_t s);
 // e += dt curl b + |alpha| * J for the fixed-point current of the mixed path
 // hist_inc (nullable): the step counter of the energy history, incremented once
 void launch_e_advance_fx(const Geom &g, FieldPtrs<float> f, const unsigned long long *const J[3],
@@ -243,10 +247,27 @@ const typename SmoothValue<JT>::type *launch_smooth_current(const Geom &g, JT *c
 // one smoothing pass of one compact plane, in -> out (distinct arrays)
 void launch_smooth(const Geom &g, const double *in, double *out, cudaStream_t s);
 
-// push_fp64.cu
-void launch_push_fp64(const Geom &g, FieldPtrs<double> f, double *const J[3], Species64 sp, long long n,
-                      double h, double alpha, double dt, int mode, double m_over_me, double *kin_acc, int *err,
-                      cudaStream_t s);
+// push_fp64.cu: nf holds the node averages (three planes of double2); M the moment planes
+// of the current (moment_planes64 of them, zero before the first species), to which a
+// species adds with the sign of its charge; kin_acc (nullable): kinetic energy at
+// u^{t-1/2} (only with kin0) and at u^{t+1/2}
+int moment_planes64(int ndim);
+void launch_push_fp64(const Geom &g, const double2 *nf, double *M, Species64 sp, long long n, bool sorted, double h,
+                      bool negative, double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s);
+// the interior of the padded current planes J from the moments
+void launch_current64(const Geom &g, const double *M, double *const J[3], double alpha_abs, cudaStream_t s);
+// initial staggering of the momenta by -dt/2
+void launch_half_back64(const Geom &g, const double2 *nf, Species64 sp, long long n, double h, double dt,
+                        cudaStream_t s);
+// log2 of the particles a lane of the push walks in a sorted block of 32 << lg particles
+int walk_lg64(long long n);
+
+// sort_fp64.cu: counting sort by cell.  counts and offsets hold an int per interior
+// cell, block_sums sort_scan_scratch(cells) ints, rank and perm n ints
+void launch_perm64(const Geom &g, const Species64 &s, long long n, int *counts, int *offsets, int *block_sums,
+                   int *rank, int *perm, cudaStream_t st);
+void launch_gather64(double *dst, const double *src, const int *perm, long long n, cudaStream_t st);
+void launch_gather_ids(int32_t *dst, const int32_t *src, const int *perm, long long n, cudaStream_t st);
 
 // push_mixed.cu
 struct MixedStepArgs {
