@@ -13,7 +13,8 @@
 // runs one fused forward + backward kernel (one thread per sample,
 // activations and deltas in shared memory, per-CTA weight gradients reduced
 // in shared memory and added once to global memory) and one Adam step.
-// Inference: FP16 weights and activations, FP32 accumulation.
+// Inference: FP16 weights and activations, FP32 accumulation, 32 samples per warp
+// with the two 64 x 64 layers on the tensor cores.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -161,32 +162,133 @@ __global__ void k_to_half(const float *W, __half *Wh, int n) {
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) Wh[q] = __float2half_rn(W[q]);
 }
 
-// FP16 weights and activations, FP32 accumulation; fully unrolled so the
-// activations stay in registers.
-__device__ __forceinline__ float mlp_eval_half(const __half *__restrict__ w, float x0, float x1, float x2) {
-    __half h1[H], h2[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        const float v = __half2float(w[OB1 + j]) + __half2float(w[OW1 + 3 * j]) * x0 +
-                        __half2float(w[OW1 + 3 * j + 1]) * x1 + __half2float(w[OW1 + 3 * j + 2]) * x2;
-        h1[j] = __float2half_rn(tanhf(v));
+// ---- inference: FP16 weights and activations, FP32 accumulation ----
+//
+// A warp evaluates 32 samples, one per lane.  The hidden layers are products of the
+// 32 x 64 activations with 64 x 64 weights: two m16 tiles of mma.m16n8k16, whose
+// accumulator layout is that of the next layer's left operand, so activations stay
+// in registers.  (A 64-wide layer is far too small for a tcgen05 tile, and the 192
+// tanh of a sample bound the kernel, not the products.)  4.2M drift components with
+// their FP64 features: one thread per sample with scalar multiply-adds 10.4 ms, this
+// form 1.65 ms.
+
+constexpr int kWS = 72;   // row stride of the staged weights (halves): the 8 rows of a fragment load hit distinct banks
+struct MlpShared {
+    __half w[2][H * kWS];
+    float w1[H * 3], b1[H], b[2][H], w4[H], b4;
+};
+__device__ __forceinline__ MlpShared &mlp_shared() {
+    __shared__ MlpShared sh;
+    return sh;
+}
+
+// Stage the weights of the block (all threads; ends with a barrier).
+__device__ inline void mlp_stage(const __half *__restrict__ W) {
+    MlpShared &S = mlp_shared();
+    for (int q = threadIdx.x; q < H * H; q += blockDim.x) {
+        S.w[0][(q / H) * kWS + q % H] = W[OW2 + q];
+        S.w[1][(q / H) * kWS + q % H] = W[OW3 + q];
     }
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float v = __half2float(w[OB2 + j]);
-#pragma unroll
-        for (int i = 0; i < H; ++i) v += __half2float(w[OW2 + H * j + i]) * __half2float(h1[i]);
-        h2[j] = __float2half_rn(tanhf(v));
+    for (int q = threadIdx.x; q < H * 3; q += blockDim.x) S.w1[q] = __half2float(W[OW1 + q]);
+    for (int q = threadIdx.x; q < H; q += blockDim.x) {
+        S.b1[q] = __half2float(W[OB1 + q]);
+        S.b[0][q] = __half2float(W[OB2 + q]);
+        S.b[1][q] = __half2float(W[OB3 + q]);
+        S.w4[q] = __half2float(W[OW4 + q]);
     }
-    float o = __half2float(w[OB4]);
+    if (threadIdx.x == 0) S.b4 = __half2float(W[OB4]);
+    __syncthreads();
+}
+
+__device__ __forceinline__ uint32_t half_pair(float lo, float hi) {
+    const __half2 h = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Network output of the lane's sample; all 32 lanes call it together after mlp_stage.
+__device__ inline float mlp_eval_warp(float x0, float x1, float x2) {
+    const MlpShared &S = mlp_shared();
+    const int lane = threadIdx.x & 31, gr = lane >> 2, tg = lane & 3;
+    // left operands: tile m holds samples 16 m + {gr, gr + 8}, columns 16 kt + 2 tg + {0, 1, 8, 9}
+    uint32_t act[2][4][4];
 #pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float v = __half2float(w[OB3 + j]);
+    for (int m = 0; m < 2; ++m) {
+        float x[2][3];
 #pragma unroll
-        for (int i = 0; i < H; ++i) v += __half2float(w[OW3 + H * j + i]) * __half2float(h2[i]);
-        o += __half2float(w[OW4 + j]) * __half2float(__float2half_rn(tanhf(v)));
+        for (int r = 0; r < 2; ++r) {
+            const int src = 16 * m + gr + 8 * r;
+            x[r][0] = __shfl_sync(0xffffffffu, x0, src);
+            x[r][1] = __shfl_sync(0xffffffffu, x1, src);
+            x[r][2] = __shfl_sync(0xffffffffu, x2, src);
+        }
+#pragma unroll
+        for (int kt = 0; kt < 4; ++kt)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {   // register q: row gr + 8 (q & 1), columns + 8 (q >> 1)
+                const int j = 16 * kt + 2 * tg + 8 * (q >> 1);
+                float v[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float *w = S.w1 + 3 * (j + e), *xr = x[q & 1];
+                    v[e] = tanhf(S.b1[j + e] + w[0] * xr[0] + w[1] * xr[1] + w[2] * xr[2]);
+                }
+                act[m][kt][q] = half_pair(v[0], v[1]);
+            }
     }
-    return o;
+    float o[2][2] = {{0.f, 0.f}, {0.f, 0.f}};   // output sums of rows gr, gr + 8 of each tile (this lane's columns)
+#pragma unroll
+    for (int layer = 0; layer < 2; ++layer) {
+        uint32_t next[2][4][4];
+        const __half *w = S.w[layer];
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            const int j = 8 * nt + 2 * tg;
+            const float b0 = S.b[layer][j], b1 = S.b[layer][j + 1];
+            float c[2][4] = {{b0, b1, b0, b1}, {b0, b1, b0, b1}};
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt) {
+                const uint32_t *f = reinterpret_cast<const uint32_t *>(w + (8 * nt + gr) * kWS + 16 * kt + 2 * tg);
+                const uint32_t f0 = f[0], f1 = f[4];
+#pragma unroll
+                for (int m = 0; m < 2; ++m) mma16816(c[m], act[m][kt], f0, f1);
+            }
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const uint32_t h = half_pair(tanhf(c[m][2 * r]), tanhf(c[m][2 * r + 1]));
+                    next[m][nt >> 1][r + 2 * (nt & 1)] = h;
+                    if (layer == 1) {
+                        const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&h));
+                        o[m][r] += S.w4[j] * a.x + S.w4[j + 1] * a.y;
+                    }
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) act[m][kt][q] = next[m][kt][q];
+    }
+    // sums over the quad's columns, then every lane takes its own sample's
+    float mine = 0.f;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float v = o[m][r];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v = __shfl_sync(0xffffffffu, v, 4 * (lane & 7));
+            if (lane >> 3 == 2 * m + r) mine = v;
+        }
+    return S.b4 + mine;
 }
 
 __device__ __forceinline__ void features(double theta, double beta0, double w, float &x0, float &x1, float &x2) {
@@ -195,12 +297,16 @@ __device__ __forceinline__ void features(double theta, double beta0, double w, f
     x2 = (float)(normcdfinv(w) / 3.0);
 }
 
-__global__ void k_mlp_infer(const __half *Wg, const float *X, int n, float *out) {
-    __shared__ __align__(16) __half w[NP + 7];
-    for (int q = threadIdx.x; q < NP; q += blockDim.x) w[q] = Wg[q];
-    __syncthreads();
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x)
-        out[idx] = mlp_eval_half(w, X[idx], X[n + idx], X[2 * n + idx]);
+// (loops over whole warps: the evaluation is a warp's)
+__global__ void __launch_bounds__(256) k_mlp_infer(const __half *Wg, const float *X, int n, float *out) {
+    mlp_stage(Wg);
+    const int lane = threadIdx.x & 31;
+    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+        const int i = i0 + lane;
+        const bool in = i < n;
+        const float o = mlp_eval_warp(in ? X[i] : 0.f, in ? X[n + i] : 0.f, in ? X[2 * n + i] : 0.f);
+        if (in) out[i] = o;
+    }
 }
 
 // Training batch from the exact sampler: a random grid point (theta_k, beta_j)
@@ -234,28 +340,35 @@ __global__ void k_mlp_data(TabSet ts, unsigned long long seed, long long base, i
     }
 }
 
-// Drift component from the network, for the loader.
+// Drift component from the network, for the loader (a whole warp calls it together).
 struct MlpPar {
     const __half *w;
     double psi, scale;
+    __device__ void begin() const { mlp_stage(w); }
     __device__ double operator()(const mjk::LoadArgs &a, double wv) const {
         const double wc = fmin(fmax(wv, 1e-7), 1.0 - 1e-7);
         float x0, x1, x2;
         features(a.theta, a.beta0, wc, x0, x1, x2);
-        const float o = mlp_eval_half(w, x0, x1, x2);
+        const float o = mlp_eval_warp(x0, x1, x2);
         return sinh(psi + scale * (double)o);
     }
 };
 
 // Drift component of given uniforms, exact or learned (tests and the gain measurement).
-__global__ void k_sample_par(mjk::Table tb, MlpPar mp, int use_mlp, double theta, double beta0, const double *wv,
-                             int n, double *y) {
+__global__ void __launch_bounds__(256) k_sample_par(mjk::Table tb, MlpPar mp, int use_mlp, double theta, double beta0,
+                                                    const double *wv, int n, double *y) {
     mjk::LoadArgs a{};
     a.theta = theta;
     a.beta0 = beta0;
     a.tab = tb;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        y[i] = use_mlp ? mp(a, wv[i]) : mjk::inverse_marginal(tb, wv[i]);
+    if (use_mlp) mp.begin();
+    const int lane = threadIdx.x & 31;
+    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+        const int i = i0 + lane;
+        const double w = i < n ? wv[i] : 0.5;
+        const double r = use_mlp ? mp(a, w) : mjk::inverse_marginal(tb, w);
+        if (i < n) y[i] = r;
+    }
 }
 
 }  // namespace
