@@ -41,6 +41,7 @@ struct SpeciesState {
     int tiled_ntiles = 0;       // tile count of the geometry that sort used
     int *counts = nullptr;      // mixed: key histogram / cursors of the sort, zero between sorts
     bool counted = false;       // the last push filled counts for the next sort
+    int lgw = 5;                // mixed: log2 of the walk length of the current layout
 };
 
 struct Run {
@@ -60,6 +61,9 @@ struct Run {
     bool tma = false;           // TMA descriptors of nfA/nfB for the current tile box are valid
     CUtensorMap tmA{}, tmB{};
     SpeciesState sp[PIC_MAX_SPECIES];
+    int2 *parts = nullptr;      // work list of the push (single runs): entries, their count, and its capacity
+    int *nparts = nullptr;
+    int parts_cap = 0, parts_bound = 0;
     int *offsets = nullptr, *block_sums = nullptr;
     int *perm = nullptr;        // sort scratch, max species capacity
     // FP64 path: node averages, and the sort's scratch (null when the allocator had no room: no sort then)
@@ -148,6 +152,9 @@ struct pic_ctx {
 namespace {
 
 constexpr int64_t kHistCap = 1 << 16;
+// Work list of the push (make_parts): parts aimed at, smallest part, most tiles listed.
+int part_slots(int ndim) { return 2 * 152 * (ndim == 3 ? 1 : 2); }
+constexpr int kPartMin = 512, kPartTiles = 65536;
 // The FP64 path sorts its particles where the arrays they gather from and add to (48 B
 // of node fields and 64 or 96 B of moments per cell) exceed what L2 holds besides the
 // particle stream.  Measured per step, sorted every 16 steps against never: 128^3 with 32
@@ -638,6 +645,12 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         int64_t capmax = 1;
         for (int s = 0; s < d.nspecies; ++s) capmax = std::max<int64_t>(capmax, d.species[s].capacity);
         r.perm = (int *)dev_alloc(ctx, sizeof(int) * capmax);
+        if (ctx->runs.size() == 1) {
+            r.parts_cap = std::min(max_tiles, kPartTiles) + part_slots(d.ndim) + 1;
+            r.parts = (int2 *)dev_alloc(ctx, sizeof(int2) * r.parts_cap);
+            r.nparts = (int *)dev_alloc(ctx, sizeof(int));
+            if (!r.parts || !r.nparts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
+        }
         if (!r.nfA || !r.nfB || !r.offsets || !r.block_sums || !r.perm)
             return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
     }
@@ -813,7 +826,47 @@ void prepare_counts(pic_ctx *ctx, Run &r) {
     }
 }
 
-SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S) {
+// Particles a lane of the push walks, as log2.  Long walks add fewer register sums to
+// shared memory, short ones leave the warps of a CTA more equal shares and order the sort
+// more finely; with few particles the longest walk is the kernel's time.  Push per step,
+// walks of 32 / 16 / 8 / 4: 128^3 (134M particles) 5.19 / 5.06 / 5.45 / 6.22 ms, 1024^2
+// (105M) 2.38 / 2.45 / 2.49 / 2.87; 45 x 37 x 51 (3.4M) 248 / 222 / 181 / 180 us, 251 x 130
+// sheet (0.7M) 87 / 71 / 58 / 52; 64^2 (0.13M), walks of 4 / 2 / 1: 18.7 / 16.4 / 18.8.
+int push_walk_lg(const pic_ctx *ctx) {
+    long long n = 0;
+    for (const Run &r : ctx->runs)
+        for (int q = 0; q < r.d.nspecies; ++q) n += r.sp[q].n;
+    const bool d3 = ctx->runs[0].d.ndim == 3;
+    int lg = d3 ? 4 : 5;
+    while (lg > 0 && (n >> (5 + lg)) < (d3 ? 8192 : 2048)) --lg;
+    return lg;
+}
+
+// Work list of a single run's push: tiles cut into parts, so that few or unequal tiles
+// still fill the GPU: two parts per resident CTA, none below kPartMin particles.  A CTA
+// per tile left 16 CTAs at 64^2 (53 us, in parts 16) and one dense column of tiles in a
+// Harris sheet (178 us, 58).  Parts cost a staging and a flush each: 512^2 takes 659 us
+// in 1024 tiles and 719 in twice the parts.
+void make_parts(pic_ctx *ctx, Run &r) {
+    r.parts_bound = r.t.ntiles;
+    if (!r.parts || r.t.ntiles > kPartTiles) return;
+    long long n = 0;
+    PushParts a{};
+    for (int q = 0; q < r.d.nspecies; ++q) {
+        a.tile_start[q] = r.sp[q].tile_start;
+        n += r.sp[q].n;
+    }
+    a.nspecies = r.d.nspecies;
+    a.ntiles = r.t.ntiles;
+    a.size = (int)std::min<long long>(INT32_MAX, std::max<long long>(kPartMin, n / part_slots(r.d.ndim) + 1));
+    a.cap = r.parts_cap;
+    a.list = r.parts;
+    a.count = r.nparts;
+    r.parts_bound = (int)std::min<long long>(r.t.ntiles, n) + (int)(n / a.size);
+    launch_push_parts(a, ctx->stream);
+}
+
+SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S, int lgw) {
     SortArgs a;
     a.g = r.g;
     a.t = r.t;
@@ -822,6 +875,8 @@ SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S) {
     a.dst = S.mb[1 - S.cur];
     a.counts = S.counts;
     a.counted = S.counted ? 1 : 0;
+    a.lgw = lgw;
+    a.lgw_src = S.lgw;
     a.offsets = r.offsets;
     a.block_sums = r.block_sums;
     // the old-tile walk is valid only for the tile geometry the layout was sorted with
@@ -833,8 +888,9 @@ SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S) {
 }
 
 // Host bookkeeping after the sort of S was enqueued: the sorted copy becomes current.
-void sort_done(Run &r, SpeciesState &S) {
+void sort_done(Run &r, SpeciesState &S, int lgw) {
     S.counted = false;
+    S.lgw = lgw;
     S.cur = 1 - S.cur;
     std::swap(S.tile_start, S.tile_start_alt);
     S.tiled = true;
@@ -842,8 +898,9 @@ void sort_done(Run &r, SpeciesState &S) {
 }
 
 void sort_species(pic_ctx *ctx, Run &r, SpeciesState &S) {
-    launch_sort(sort_args(ctx, r, S), ctx->stream);
-    sort_done(r, S);
+    const int lgw = push_walk_lg(ctx);
+    launch_sort(sort_args(ctx, r, S, lgw), ctx->stream);
+    sort_done(r, S, lgw);
 }
 
 HistRef hist_ref(Run &r) { return HistRef{r.hist, r.hist_idx, r.hist_cap}; }
@@ -861,10 +918,14 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
         SpeciesState &S = r.sp[q];
         a.sp[q] = S.mb[S.cur];
         a.tile_start[q] = S.tile_start;
+        a.lgw[q] = S.lgw;
         a.h[q] = (float)S.h;
         a.sgn[q] = S.q_over_e > 0 ? 1.f : -1.f;
         a.m_over_me[q] = S.m_over_me;
     }
+    a.parts = (r.parts && r.t.ntiles <= kPartTiles) ? r.parts : nullptr;
+    a.nparts = r.nparts;
+    a.parts_bound = r.parts_bound;
     a.dt = (float)r.d.dt;
     a.mode = 0;
     a.hist = hist_ref(r);
@@ -961,6 +1022,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
     const int nphase = (due.empty() ? 0 : 8 * maxsp) + 5 + (max_smooth > 0 ? 1 + max_smooth : 0);
     const bool walk = !(ctx->flags & (PIC_FLAG_PHASE_LAUNCHES | PIC_FLAG_TIMING)) && nphase <= kWalkMaxPhases &&
                       walk_ok(ctx, ndim, walls, count, push_smem);
+    const int lgw = push_walk_lg(ctx);
     // The walker sorts too unless one run holds more than a quarter of the particles: that run's
     // sort alone then sets the time, and its own launches per phase (more warps per SM for the
     // latency-bound gather and rank) finish it sooner.
@@ -977,8 +1039,8 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         for (int i : due) {
             Run &r = ctx->runs[i];
             for (int q = 0; q < r.d.nspecies; ++q) {
-                ctx->h_walk_sort[4 * i + q] = sort_args(ctx, r, r.sp[q]);
-                sort_done(r, r.sp[q]);
+                ctx->h_walk_sort[4 * i + q] = sort_args(ctx, r, r.sp[q], lgw);
+                sort_done(r, r.sp[q], lgw);
             }
             r.sorted = true;
             r.since_sort = 0;
@@ -990,7 +1052,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
             int ns = 0;
             for (int i : due) {
                 Run &r = ctx->runs[i];
-                if (q < r.d.nspecies) ctx->h_sort[ns++] = sort_args(ctx, r, r.sp[q]);
+                if (q < r.d.nspecies) ctx->h_sort[ns++] = sort_args(ctx, r, r.sp[q], lgw);
             }
             sort_multi_prefixes(ctx->h_sort.data(), ns, ctx->h_sort_prefix.data());
             CK(cudaMemcpyAsync(ctx->sort_args_dev, host_src(ctx, slot, soff, ctx->h_sort.data(), sizeof(SortArgs) * ns),
@@ -1002,7 +1064,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
                               ctx->runs[0].d.ndim, s);
             for (int i : due) {
                 Run &r = ctx->runs[i];
-                if (q < r.d.nspecies) sort_done(r, r.sp[q]);
+                if (q < r.d.nspecies) sort_done(r, r.sp[q], lgw);
             }
             launches += 8;
         }
@@ -1239,6 +1301,8 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
                 launches += r.sp[q].counted ? 6 : 8;
                 sort_species(ctx, r, r.sp[q]);
             }
+            make_parts(ctx, r);
+            launches += r.parts ? 1 : 0;
             r.sorted = true;
             r.since_sort = 0;
         }
@@ -1252,32 +1316,11 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         u64 *J[3] = {jplane<u64>(r, r.jcur, 0), jplane<u64>(r, r.jcur, 1), jplane<u64>(r, r.jcur, 2)};
         {
             KTimer t(ctx, PIC_KERNEL_PUSH);
-            MixedStepArgs a;
-            a.g = r.g;
-            a.t = r.t;
-            a.nfA = r.nfA;
-            a.nfB = r.nfB;
-            for (int c = 0; c < 3; ++c) a.J[c] = J[c];
-            a.nspecies = nsp;
-            for (int q = 0; q < nsp; ++q) {
-                SpeciesState &S = r.sp[q];
-                a.sp[q] = S.mb[S.cur];
-                a.tile_start[q] = S.tile_start;
-                a.h[q] = (float)S.h;
-                a.sgn[q] = S.q_over_e > 0 ? 1.f : -1.f;
-                a.m_over_me[q] = S.m_over_me;
-            }
-            a.dt = (float)r.d.dt;
-            a.mode = 0;
-            a.hist = hist_ref(r);
-            a.err = ctx->d_err;
-            a.use_tma = r.tma ? 1 : 0;
-            a.tmA = r.tmA;
-            a.tmB = r.tmB;
+            MixedStepArgs a = mixed_args(ctx, r);
             // when the next step sorts, this push counts its key histogram
             const bool count = r.since_sort + 1 >= r.sort_interval && r.t.lg[0] >= 0;
             prepare_counts(ctx, r);
-            for (int q = 0; q < 4; ++q) a.key_counts[q] = (count && q < nsp) ? r.sp[q].counts : nullptr;
+            for (int q = 0; q < nsp; ++q) a.key_counts[q] = count ? r.sp[q].counts : nullptr;
             launch_push_mixed(a, s);
             if (count)
                 for (int q = 0; q < nsp; ++q) r.sp[q].counted = true;
@@ -1351,6 +1394,7 @@ std::vector<long long> graph_signature(const pic_ctx *ctx) {
             v.push_back(S.n);
             v.push_back((long long)(uintptr_t)S.tile_start);
             v.push_back((long long)(uintptr_t)S.tile_start_alt);
+            v.push_back(S.lgw);
         }
     }
     return v;

@@ -279,6 +279,10 @@ struct MixedStepArgs {
     int nspecies;
     SpeciesMixed sp[4];
     const int *tile_start[4];       // per species: ntiles+1 offsets into the particle arrays
+    int lgw[4];                     // log2 of the particles a lane walks in a block of the layout
+    const int2 *parts;              // work list of the push (k_push_parts), null: one CTA per tile
+    const int *nparts;              // its length
+    int parts_bound;                // grid of the launch: a bound of that length, or the tile count
     float h[4];                     // (q/e)(m_e/m)
     float sgn[4];                   // sign of the charge
     double m_over_me[4];
@@ -381,8 +385,19 @@ struct SortArgs {
     int *perm;       // n scratch: source index of every destination slot
     int *err;
     int counted;     // counts already hold the key histogram of src (counted by the push)
+    int lgw, lgw_src;   // log2 of the walk length of the destination and of the source layout
 };
 void launch_sort(const SortArgs &a, cudaStream_t s);
+// The push's work list for the layout of the last sort (see k_push_parts).
+struct PushParts {
+    const int *tile_start[4];
+    int nspecies, ntiles;
+    int size;        // particles of a part at most
+    int cap;         // entries of list
+    int2 *list;
+    int *count;
+};
+void launch_push_parts(const PushParts &a, cudaStream_t s);
 // many independent sorts in one launch per phase: h_prefix (4 x (nsort + 1) ints)
 // is filled by sort_multi_prefixes from the host copy of the arguments and
 // uploaded to d_prefix next to d_args

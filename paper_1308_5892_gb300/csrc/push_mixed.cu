@@ -9,12 +9,20 @@ namespace pic {
 
 namespace {
 
-// One CTA per tile of one run; WALLS: conducting walls in x (a separate
+// One CTA per tile, or per entry of the work list, of one run; WALLS: conducting walls in x (a separate
 // instantiation keeps their register cost out of the periodic kernel); CT: the
 // fixed tile geometry code (fixed_tile), 0 for the run-time geometry.
 template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST, int CT>
 __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed(const __grid_constant__ MixedStepArgs a) {
-    push_tile<NDIM, THREADS, WALLS, HIST, CT>(a, blockIdx.x, &a);
+    int tile = blockIdx.x, part = 0, parts = 1;
+    if (a.parts) {
+        if ((int)blockIdx.x >= __ldg(a.nparts)) return;
+        const int2 e = __ldg(a.parts + blockIdx.x);
+        tile = e.x;
+        part = e.y & 0xffff;
+        parts = e.y >> 16;
+    }
+    push_tile<NDIM, THREADS, WALLS, HIST, CT>(a, tile, part, parts, &a);
 }
 
 // Persistent form for a batch of independent runs of uneven size: resident
@@ -41,7 +49,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed_multi(const MixedS
         int *dst = reinterpret_cast<int *>(&args_sh);
         for (int q = threadIdx.x; q < (int)(sizeof(MixedStepArgs) / sizeof(int)); q += THREADS) dst[q] = src[q];
         __syncthreads();
-        push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, item - tile_prefix[lo], runs + lo);
+        push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, item - tile_prefix[lo], 0, 1, runs + lo);
     }
 }
 
@@ -88,7 +96,7 @@ template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
 void launch_t(const MixedStepArgs &a, size_t smem, cudaStream_t s) {
     auto k = push_kernel<NDIM, THREADS, MINB, WALLS, HIST>(fixed_tile_code(a.t, NDIM));
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<a.t.ntiles, THREADS, smem, s>>>(a);
+    if (a.parts_bound > 0) k<<<a.parts_bound, THREADS, smem, s>>>(a);
 }
 
 }  // namespace

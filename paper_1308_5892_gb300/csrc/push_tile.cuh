@@ -33,8 +33,9 @@
 //    read 24 B (2D) / 28 B (3D) and written back.  Each warp prefetches the
 //    particles of its next iterations with cp.async into a ring of
 //    shared-memory stages, so the DRAM latency overlaps the arithmetic.
-// Work of a warp: 1024-particle blocks, which the sort stores 32 x 32
-// transposed, so lane a walks 32 consecutive cell-sorted particles (and keeps
+// Work of a warp: blocks of 32 W particles (W = 32; less for few particles, see
+// push_walk_lg), which the sort stores transposed, so lane a walks W consecutive
+// cell-sorted particles (and keeps
 // their start-cell current in registers until its cell changes) while one
 // load instruction still reads one contiguous 128-byte row.  The pieces of a
 // path after a node-plane crossing are queued per warp and deposited 32 at a
@@ -408,11 +409,14 @@ __device__ __forceinline__ void drain_one(const int *q_base, const float *q_d, c
 // Offset of the nfB stage after the nfA stage of `nodes` nodes (TMA destinations are 128-byte aligned).
 __host__ __device__ inline size_t node_b_offset(int nodes) { return ((size_t)nodes * 16 + 127) & ~size_t(127); }
 
+// part of parts: the share of the tile's work items this CTA takes (the parts of a
+// tile add their currents to the same global sums, exactly).
 // tmaps: the arguments' copy whose TMA descriptors are in parameter or global
 // memory (the multi-run kernel stages its arguments in shared memory).
 // CT: fixed tile geometry code (fixed_tile), 0 for the run-time geometry.
 template <int NDIM, int THREADS, bool WALLS, bool HIST, int CT = 0>
-__device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile, const MixedStepArgs *tmaps) {
+__device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile, const int part,
+                                          const int parts, const MixedStepArgs *tmaps) {
     extern __shared__ __align__(128) float4 smem4[];
     __shared__ __align__(8) unsigned long long tma_bar;
     constexpr int WARPS = THREADS / 32;
@@ -479,7 +483,19 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     const unsigned lt_mask = (1u << lane) - 1u;
     __shared__ int work_ctr[4];
     __shared__ double kin_sh[2][WARPS];
-    if (threadIdx.x < 4) work_ctr[threadIdx.x] = 0;
+    // work items of species sp: blocks, then 32-particle chunks of the tail; this part's share
+    auto item_range = [&](int sp, int &nblk, int &beg, int &end) {
+        const int nt = a.tile_start[sp][tile + 1] - a.tile_start[sp][tile], lgb = 5 + a.lgw[sp];
+        nblk = nt >> lgb;
+        const int nall = nblk + ((nt - (nblk << lgb)) + 31) / 32;
+        beg = (int)((long long)nall * part / parts);
+        end = (int)((long long)nall * (part + 1) / parts);
+    };
+    if ((int)threadIdx.x < a.nspecies) {
+        int nblk, beg, end;
+        item_range(threadIdx.x, nblk, beg, end);
+        work_ctr[threadIdx.x] = beg;
+    }
     if (lane == 0) { kin_sh[0][warp] = 0.0; kin_sh[1][warp] = 0.0; }
     // this warp's piece queue and particle stages
     int *wsm = Jlo + 3 * nodes + warp * warp_smem_words<NDIM>();
@@ -517,9 +533,9 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
         const SpeciesMixed &P = a.sp[sp];
         const float h = a.h[sp], alpha26 = a.sgn[sp] * kFx26;   // deposit prefactor in fixed-point units
         const int pbeg = a.tile_start[sp][tile], pend = a.tile_start[sp][tile + 1];
-        const int nt = pend - pbeg;
-        const int nblk = nt >> 10;                       // full 1024-blocks, stored transposed
-        const int nitems = nblk + ((nt - (nblk << 10)) + 31) / 32;   // + 32-particle tail chunks
+        const int lgb = 5 + a.lgw[sp];                   // log2 of a block: 2^lgw particles per lane
+        int nblk, ibeg, nitems;
+        item_range(sp, nblk, ibeg, nitems);
         // prefetch the particle of iteration j of an item into stage j % kStages (one group per iteration)
         auto issue = [&](int base, int j, int kn) {
             const int p = base + (j << 5) + lane;
@@ -546,10 +562,10 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                 qcount = 0;
             }
         };
-        for (int r0 = 0; r0 < nitems; r0 += kRoundItems) {
+        for (int r0 = ibeg; r0 < nitems; r0 += kRoundItems) {
         const int r1 = min(nitems, r0 + kRoundItems);
         const bool need_flush = since_flush + (long long)(r1 - r0) * 1024 >= (1LL << 17);   // uniform
-        if (r0 > 0 || need_flush) {
+        if (r0 > ibeg || need_flush) {
             // every warp has left the previous round; its pieces and register sums go to the limbs
             drain_queue();
             acc.flush(Jhi, Jlo, nodes, tc.sx, tc.sxy);
@@ -569,10 +585,10 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             if (lane == 0) item = atomicAdd(&work_ctr[sp], 1);
             item = __shfl_sync(kFull, item, 0);
             if (item >= r1) break;
-            // block item: lane walks base + 32k + lane, k = 0..31 (consecutive ranks);
+            // block item: lane walks base + 32k + lane, k = 0..kn-1 (consecutive ranks);
             // tail chunk: one element per lane in rank order
-            const int base = item < nblk ? pbeg + (item << 10) : pbeg + (nblk << 10) + ((item - nblk) << 5);
-            const int kn = item < nblk ? 32 : 1;
+            const int base = item < nblk ? pbeg + (item << lgb) : pbeg + (nblk << lgb) + ((item - nblk) << 5);
+            const int kn = item < nblk ? 1 << (lgb - 5) : 1;
             float kin0 = 0.f, kin1 = 0.f;
             int hk = -1, hn = 0;   // HIST: sort key of the lane's current run of particles, and its length
 #pragma unroll

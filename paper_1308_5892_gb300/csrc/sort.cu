@@ -42,7 +42,7 @@ __global__ void k_zero(SortArgs a) { zero_body(a.counts, nkeys_of(a), blockIdx.x
 
 template <int NDIM>
 __global__ void k_histogram(SortArgs a) {
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x};
+    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x, a.lgw_src};
     histogram_body<NDIM, 4>(a, w, nkeys_of(a));
 }
 
@@ -60,13 +60,52 @@ __global__ void k_scan_finish(SortArgs a) { scan_finish_body(a, nkeys_of(a), blo
 
 template <int NDIM>
 __global__ void k_rank(SortArgs a) {
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x};
+    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x, a.lgw_src};
     rank_body<NDIM, 4>(a, w, nkeys_of(a));
 }
 
 template <int NDIM>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(SortArgs a) {
     gather_body<NDIM, kGatherThreads, 4>(a.src, a.dst, a.n, a.perm, blockIdx.x);
+}
+
+// Work list of the push: every tile that holds particles, cut into parts of at most
+// `size` particles of all species.  list[c] = {tile, part | parts << 16}, list[count]
+// for c < *count.  One block.
+__global__ void __launch_bounds__(kScanThreads) k_push_parts(PushParts a) {
+    __shared__ int sh[kScanThreads / 32 + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int carry = 0;
+    for (int t0 = 0; t0 < a.ntiles; t0 += kScanThreads) {
+        const int t = t0 + threadIdx.x;
+        long long n = 0;
+        if (t < a.ntiles)
+            for (int q = 0; q < a.nspecies; ++q) n += a.tile_start[q][t + 1] - a.tile_start[q][t];
+        const int parts = (int)((n + a.size - 1) / a.size);
+        int incl = parts;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) sh[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            const int w = lane < kScanThreads / 32 ? sh[lane] : 0;
+            int wi = w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, wi, o);
+                if (lane >= o) wi += y;
+            }
+            sh[lane] = wi - w;
+            if (lane == 31) sh[32] = wi;
+        }
+        __syncthreads();
+        const int at = carry + sh[warp] + incl - parts;
+        for (int p = 0; p < parts && at + p < a.cap; ++p) a.list[at + p] = make_int2(t, p | parts << 16);
+        carry += sh[32];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *a.count = carry;
 }
 
 // ---- many independent sorts (one species of every run of an ensemble): one
@@ -95,7 +134,7 @@ __global__ void k_histogram_multi(const SortArgs *as, const int *prefix, int nso
     const int s = find_sort(prefix, nsort, blockIdx.x);
     const SortArgs &a = as[s];
     if (a.counted) return;
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s]};
+    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s], a.lgw_src};
     histogram_body<NDIM, 4>(a, w, nkeys_of(a));
 }
 
@@ -122,7 +161,7 @@ template <int NDIM>
 __global__ void k_rank_multi(const SortArgs *as, const int *prefix, int nsort) {
     const int s = find_sort(prefix, nsort, blockIdx.x);
     const SortArgs &a = as[s];
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s]};
+    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s], a.lgw_src};
     rank_body<NDIM, 4>(a, w, nkeys_of(a));
 }
 
@@ -158,6 +197,8 @@ void launch_sort(const SortArgs &a, cudaStream_t s) {
     // the counts end zeroed, ready for a push that counts the next sort's histogram
     k_zero<<<key_blocks(a), 256, 0, s>>>(a);
 }
+
+void launch_push_parts(const PushParts &a, cudaStream_t s) { k_push_parts<<<1, kScanThreads, 0, s>>>(a); }
 
 void sort_multi_prefixes(const SortArgs *h_args, int nsort, int *h_prefix) {
     int *pz = h_prefix, *pw = h_prefix + (nsort + 1), *pb = h_prefix + 2 * (nsort + 1),

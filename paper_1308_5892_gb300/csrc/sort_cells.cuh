@@ -29,15 +29,15 @@ __device__ inline int key_tile(const TileGeom &t, int key) {
 }
 
 // Position of cell-sorted rank r inside a tile of n_t particles: every full
-// block of 1024 is stored as a 32 x 32 transpose, so that lane a of a warp,
-// reading element base + 32k + a for k = 0..31, walks the 32 consecutive
-// ranks 32a .. 32a+31 (mostly one cell) while the 32 lanes of one load sit in
-// 32 different cells; the tail of the tile (n_t mod 1024) keeps rank order.
-__device__ __forceinline__ int interleaved_slot(int r, int n_t) {
-    const int nfull = n_t & ~1023;
-    if (r >= nfull) return r;
-    const int i = r & 1023;
-    return (r - i) + ((i & 31) << 5) + (i >> 5);
+// block of 32 W (W = 2^lgw) is stored as a transpose, so that lane a of a warp,
+// reading element base + 32k + a for k = 0..W-1, walks the W consecutive
+// ranks W a .. W a + W - 1 (mostly one cell) while the 32 lanes of one load sit in
+// different cells; the tail of the tile (n_t mod 32 W) keeps rank order.
+__device__ __forceinline__ int interleaved_slot(int r, int n_t, int lgw) {
+    const int block = 32 << lgw;
+    if (r >= (n_t & ~(block - 1))) return r;
+    const int i = r & (block - 1);
+    return (r - i) + ((i & ((1 << lgw) - 1)) << 5) + (i >> lgw);
 }
 
 // Source traversal: with a tiled source (sorted before), CTA b walks old tile b
@@ -50,6 +50,7 @@ struct SrcWalk {
     const int *old_start;   // old tile offsets, or nullptr when the source is untiled
     long long n;
     int b, nb;              // this block and the block count of the walk
+    int lgw;                // walk length of the source layout
     int parts = 1;          // blocks per old tile
     __device__ __forceinline__ void begin(long long &i, long long &end, int &t0, int &nt) const {
         if (old_start) {
@@ -69,7 +70,7 @@ struct SrcWalk {
         return old_start ? (long long)blockDim.x : (long long)nb * blockDim.x;
     }
     __device__ __forceinline__ long long pos(long long i, int t0, int nt) const {
-        return old_start ? (long long)t0 + interleaved_slot((int)i, nt) : i;
+        return old_start ? (long long)t0 + interleaved_slot((int)i, nt, lgw) : i;
     }
 };
 
@@ -238,7 +239,7 @@ __device__ inline void rank_body(const SortArgs &a, const SrcWalk &w, long long 
             if (key[v] < 0) continue;
             const int tile = key_tile(a.t, key[v]);
             const int t0 = ldro(a.tile_start + tile), t1 = ldro(a.tile_start + tile + 1);
-            const long long dst = (long long)t0 + interleaved_slot(base[v] - t0, t1 - t0);
+            const long long dst = (long long)t0 + interleaved_slot(base[v] - t0, t1 - t0, a.lgw);
             if (base[v] >= t0 && base[v] < t1 && dst < a.n) a.perm[dst] = (int)p[v];
             else atomicOr(a.err, ERR_SORT);   // counts inconsistent with the particles
         }

@@ -146,7 +146,7 @@ __device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, in
     if (kind == S_ZERO || kind == S_ZERO_AFTER) {
         zero_body(a.counts, nkeys, local, nitems);
     } else if (kind == S_HIST) {
-        const SrcWalk sw{a.old_tile_start, a.n, local, nitems, walk_tile_parts(a)};
+        const SrcWalk sw{a.old_tile_start, a.n, local, nitems, a.lgw_src, walk_tile_parts(a)};
         histogram_body<NDIM, 8>(a, sw, nkeys);
     } else if (kind == S_SCAN_BLOCKS) {
         scan_blocks_body<THREADS>(a.counts, a.offsets, a.block_sums, nkeys, local, sh);
@@ -155,7 +155,7 @@ __device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, in
     } else if (kind == S_SCAN_FINISH) {
         scan_finish_body(a, nkeys, local, nitems);
     } else if (kind == S_RANK) {
-        const SrcWalk sw{a.old_tile_start, a.n, local, nitems, walk_tile_parts(a)};
+        const SrcWalk sw{a.old_tile_start, a.n, local, nitems, a.lgw_src, walk_tile_parts(a)};
         rank_body<NDIM, 8>(a, sw, nkeys);
     } else {
         // fewer warps per SM than the sort's own gather launch: every array per
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
                 __syncthreads();
                 if (threadIdx.x == 0) args_sh.use_tma = 0;
                 __syncthreads();
-                push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, local, w.push + r);
+                push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, local, 0, 1, w.push + r);
             } else {
                 const FieldRunF *fsrc = kind == W_B_HALF_E ? w.fe + r : w.fp + r;
                 const int *src = reinterpret_cast<const int *>(fsrc);
