@@ -5,10 +5,10 @@
 //
 // One step of one run (main loop of App. A.3.1), state e^t, b^{t-dt/2}, x^t, u^{t-dt/2}:
 //   [re-sort particles by tile when due]                    (mixed path)
-//   b += -(dt/2) curl e            -> b^t; FP64 sums of e^2, b^2 at t recorded
+//   b += -(dt/2) curl e, twice     -> b^t (kept for the gather), b^{t+dt/2}   (steps 4, 5);
+//                                     FP64 sums of e^2, b^2 at t recorded
 //   node fields E, B at t            (mixed path, App. A.3.3 averages)
 //   per species: gather, Boris, move, deposit into J        (steps 2, 3, 8, 9)
-//   b += -(dt/2) curl e            -> b^{t+dt/2}            (steps 4, 5)
 //   e += dt curl b + J, zero the other J buffer             (steps 6, 7, 11, 12)
 #include <algorithm>
 #include <cmath>
@@ -113,7 +113,7 @@ struct pic_ctx {
     // batched ensemble (nruns > 1, mixed): per-run argument tables on the device
     bool multi = false;
     MixedStepArgs *multi_args = nullptr;
-    FieldRunF *multi_fe = nullptr, *multi_fp = nullptr;
+    FieldRunF *multi_fp = nullptr;
     int *multi_tiles = nullptr, *multi_blocks = nullptr, *multi_counter = nullptr;
     int *walk_tab = nullptr, *walk_ctl = nullptr;   // step walker: queue tables; head, abort, done[nruns]
     std::vector<int> h_walk;
@@ -141,7 +141,7 @@ struct pic_ctx {
     // with the conversion kernels through two halves of the staging buffer
     cudaStream_t io_stream = nullptr;
     cudaEvent_t io_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // start, loaded/filled[2], consumed/copied[2]
-    std::vector<FieldRunF> h_fe, h_fp;
+    std::vector<FieldRunF> h_fp;
     // PIC_FLAG_TIMING: event pairs per kernel class, resolved in pic_kernel_time
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending[kKernelClasses];
     std::vector<cudaEvent_t> ev_pool;
@@ -240,15 +240,18 @@ void dev_release(pic_ctx *ctx, void *p) {
 
 size_t real_size(const pic_ctx *ctx) { return ctx->precision == PIC_FP64 ? sizeof(double) : sizeof(float); }
 
+// mid: with the planes for b at t, within a step (they share the diagnostics' scratch)
 template <typename R>
-FieldPtrs<R> fields_of(Run &r) {
+FieldPtrs<R> fields_of(Run &r, bool mid = false) {
     FieldPtrs<R> f;
+    double *const scratch[3] = {r.rho_s, r.rho_tot, r.divb};
     R *F = (R *)r.F;
     for (int c = 0; c < 3; ++c) {
         f.e[c] = F + (size_t)c * r.g.pcells;
         f.b[c] = F + (size_t)(3 + c) * r.g.pcells;
         // the mixed path keeps the low-order part of e in planes 6..8 (see FieldPtrs)
         f.el[c] = sizeof(R) == sizeof(float) ? F + (size_t)(6 + c) * r.g.pcells : nullptr;
+        f.bt[c] = mid ? (R *)scratch[c] : nullptr;
     }
     return f;
 }
@@ -937,20 +940,19 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     return a;
 }
 
-// energy: record the e^2, b^2 sums (first b half advance); inc: advance the history counter (e advance)
-FieldRunF field_run(Run &r, bool energy, bool inc) {
+FieldRunF field_run(Run &r) {
     typedef unsigned long long u64;
     FieldRunF fr;
     fr.g = r.g;
-    fr.f = fields_of<float>(r);
+    fr.f = fields_of<float>(r, true);
     fr.nfA = r.nfA;
     fr.nfB = r.nfB;
     for (int c = 0; c < 3; ++c) {
         fr.J[c] = jplane<u64>(r, r.jcur, c);
         fr.Z[c] = jplane<u64>(r, 1 - r.jcur, c);
     }
-    fr.hist = energy ? hist_ref(r) : HistRef{nullptr, nullptr, 0};
-    fr.hist_inc = inc ? r.hist_idx : nullptr;
+    fr.hist = hist_ref(r);
+    fr.hist_inc = r.hist_idx;
     fr.scale = 2.0 / (r.d.n_x * r.d.n_x * r.d.rho_sp0) * 0x1p-36;
     fr.smooth = r.smooth;
     fr.sbuf[0] = (long long *)r.sbuf[0];
@@ -1019,7 +1021,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
     const int ndim = ctx->runs[0].d.ndim;
     const bool walls = ctx->runs[0].g.bcx == 1;
     const size_t push_smem = mixed_smem_bytes(ctx->runs[0].t, ndim);
-    const int nphase = (due.empty() ? 0 : 8 * maxsp) + 5 + (max_smooth > 0 ? 1 + max_smooth : 0);
+    const int nphase = (due.empty() ? 0 : 8 * maxsp) + 4 + (max_smooth > 0 ? 1 + max_smooth : 0);
     const bool walk = !(ctx->flags & (PIC_FLAG_PHASE_LAUNCHES | PIC_FLAG_TIMING)) && nphase <= kWalkMaxPhases &&
                       walk_ok(ctx, ndim, walls, count, push_smem);
     const int lgw = push_walk_lg(ctx);
@@ -1086,13 +1088,10 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         ctx->h_args[i] = mixed_args(ctx, r);
         if (count)
             for (int q = 0; q < r.d.nspecies; ++q) ctx->h_args[i].key_counts[q] = r.sp[q].counts;
-        ctx->h_fe[i] = field_run(r, true, false);
-        ctx->h_fp[i] = field_run(r, false, true);
+        ctx->h_fp[i] = field_run(r);
     }
     CK(cudaMemcpyAsync(ctx->multi_args, host_src(ctx, slot, soff, ctx->h_args.data(), sizeof(MixedStepArgs) * nr),
                        sizeof(MixedStepArgs) * nr, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(ctx->multi_fe, host_src(ctx, slot, soff, ctx->h_fe.data(), sizeof(FieldRunF) * nr),
-                       sizeof(FieldRunF) * nr, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(ctx->multi_fp, host_src(ctx, slot, soff, ctx->h_fp.data(), sizeof(FieldRunF) * nr),
                        sizeof(FieldRunF) * nr, cudaMemcpyHostToDevice, s));
     if (walk) {
@@ -1106,7 +1105,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
                     w.kind[np++] = k;
                 }
         const int ph_push = np + 2;
-        w.kind[np++] = W_B_HALF_E;
+        w.kind[np++] = W_B;
         w.kind[np++] = W_NODE;
         w.kind[np++] = W_PUSH;
         if (max_smooth > 0) {
@@ -1116,7 +1115,6 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
                 w.kind[np++] = W_SMOOTH_PASS;
             }
         }
-        w.kind[np++] = W_B_HALF;
         w.kind[np++] = W_E_FX;
         const int cpi = walk_cells_per_item(ndim);
         auto items = [&](int ph, int i) -> int {
@@ -1165,7 +1163,6 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         CK(cudaMemsetAsync(ctx->walk_ctl, 0, sizeof(int) * (2 + nr), s));
         w.sort = ctx->walk_sort_dev;
         w.push = ctx->multi_args;
-        w.fe = ctx->multi_fe;
         w.fp = ctx->multi_fp;
         w.prefix = ctx->walk_tab;
         w.base = ctx->walk_tab + np * nr + 1;
@@ -1198,7 +1195,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
     }
     {
         KTimer t(ctx, PIC_KERNEL_FIELD);
-        launch_fields_multi(FIELD_B_HALF, ctx->multi_fe, ctx->multi_blocks, ctx->multi_nblocks, nr, 0.5f * dt, dt, s);
+        launch_fields_multi(FIELD_B, ctx->multi_fp, ctx->multi_blocks, ctx->multi_nblocks, nr, 0.5f * dt, dt, s);
         launch_fields_multi(FIELD_NODE, ctx->multi_fp, ctx->multi_blocks, ctx->multi_nblocks, nr, 0.5f * dt, dt, s);
     }
     {
@@ -1219,7 +1216,6 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
     }
     {
         KTimer t(ctx, PIC_KERNEL_FIELD);
-        launch_fields_multi(FIELD_B_HALF, ctx->multi_fp, ctx->multi_blocks, ctx->multi_nblocks, nr, 0.5f * dt, dt, s);
         launch_fields_multi(FIELD_E_FX, ctx->multi_fp, ctx->multi_blocks, ctx->multi_nblocks, nr, 0.5f * dt, dt, s);
     }
     for (auto &r : ctx->runs) {
@@ -1228,7 +1224,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         r.step++;
         if (r.hist_n < r.hist_cap) r.hist_n++;
     }
-    ctx->launch_total += launches + 5;
+    ctx->launch_total += launches + 4;
     ctx->bytes_per_ps = ctx->runs[0].d.ndim == 2 ? 48.0 : 56.0;
     return PIC_OK;
 }
@@ -1250,7 +1246,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
     double *hslot = (r.hist_n < r.hist_cap) ? r.hist + 8 * r.hist_n : nullptr;
     const int nsp = r.d.nspecies;
     if (ctx->precision == PIC_FP64) {
-        FieldPtrs<double> f = fields_of<double>(r);
+        FieldPtrs<double> f = fields_of<double>(r, true);
         int launches = 0;
         if (r.spare64 && (!r.sorted || r.since_sort >= kSort64Interval)) {
             KTimer t(ctx, PIC_KERNEL_SORT);
@@ -1287,12 +1283,11 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         const double *Js = smooth_current<double>(ctx, r, J);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{nullptr, nullptr, 0}, nullptr, s);
             if (Js) launch_e_advance_smoothed<double, double, double>(r.g, f, Js, 1.0, Z, r.d.dt, nullptr, s);
             else launch_e_advance<double>(r.g, f, Jc, Z, r.d.dt, s);
         }
         ctx->bytes_per_ps = r.d.ndim == 2 ? 80.0 : 96.0;
-        ctx->launch_total += launches + 5 + nsp + (Js ? 1 + r.smooth : 0);   // shell fold + passes
+        ctx->launch_total += launches + 4 + nsp + (Js ? 1 + r.smooth : 0);   // shell fold + passes
     } else {
         int launches = 0;
         if (!r.sorted || r.since_sort >= r.sort_interval) {
@@ -1306,7 +1301,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
             r.sorted = true;
             r.since_sort = 0;
         }
-        FieldPtrs<float> f = fields_of<float>(r);
+        FieldPtrs<float> f = fields_of<float>(r, true);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
             launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, hist_ref(r), nullptr, s);
@@ -1331,14 +1326,13 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
             const double alpha_abs = 2.0 / (r.d.n_x * r.d.n_x * r.d.rho_sp0);
-            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, HistRef{nullptr, nullptr, 0}, nullptr, s);
             if (Js)
                 launch_e_advance_smoothed<float, u64, long long>(r.g, f, Js, alpha_abs * 0x1p-36, Z, (float)r.d.dt,
                                                                  r.hist_idx, s);
             else launch_e_advance_fx(r.g, f, Jc, Z, (float)r.d.dt, alpha_abs, r.hist_idx, s);
         }
         r.since_sort++;
-        launches += 5 + (Js ? 1 + r.smooth : 0);   // shell fold + passes
+        launches += 4 + (Js ? 1 + r.smooth : 0);   // shell fold + passes
         ctx->launch_total += launches;
         ctx->bytes_per_ps = r.d.ndim == 2 ? 48.0 : 56.0;
     }
@@ -1423,7 +1417,7 @@ pic_status capture_graph(pic_ctx *ctx) {
         for (auto &r : ctx->runs) maxsp = std::max(maxsp, r.d.nspecies);
         const size_t a = 256;
         auto up = [a](size_t b) { return (b + a - 1) & ~(a - 1); };
-        const size_t stride = up(sizeof(MixedStepArgs) * nr) + 2 * up(sizeof(FieldRunF) * nr) +
+        const size_t stride = up(sizeof(MixedStepArgs) * nr) + up(sizeof(FieldRunF) * nr) +
                               maxsp * (up(sizeof(SortArgs) * nr) + up(sizeof(int) * 4 * (nr + 1))) +
                               up(sizeof(int) * walk_tab_ints(nr)) + up(sizeof(SortArgs) * 4 * nr);
         if (ctx->gstage_bytes < stride * P) {
@@ -1528,7 +1522,6 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
         }
         ctx->multi = true;
         ctx->multi_args = (MixedStepArgs *)dev_alloc(ctx, sizeof(MixedStepArgs) * nruns);
-        ctx->multi_fe = (FieldRunF *)dev_alloc(ctx, sizeof(FieldRunF) * nruns);
         ctx->multi_fp = (FieldRunF *)dev_alloc(ctx, sizeof(FieldRunF) * nruns);
         ctx->multi_tiles = (int *)dev_alloc(ctx, sizeof(int) * (nruns + 1));
         ctx->multi_blocks = (int *)dev_alloc(ctx, sizeof(int) * (nruns + 1));
@@ -1542,7 +1535,7 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
         ctx->sort_prefix_dev = (int *)dev_alloc(ctx, sizeof(int) * 4 * (nruns + 1));
         ctx->h_sort.resize(nruns);
         ctx->h_sort_prefix.resize(4 * (nruns + 1));
-        if (!ctx->multi_args || !ctx->multi_fe || !ctx->multi_fp || !ctx->multi_tiles || !ctx->multi_blocks ||
+        if (!ctx->multi_args || !ctx->multi_fp || !ctx->multi_tiles || !ctx->multi_blocks ||
             !ctx->multi_counter || !ctx->sort_args_dev || !ctx->sort_prefix_dev || !ctx->walk_tab || !ctx->walk_ctl ||
             !ctx->walk_sort_dev) {
             pic_destroy(ctx);
@@ -1560,7 +1553,6 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
             return PIC_ECUDA;
         }
         ctx->h_args.resize(nruns);
-        ctx->h_fe.resize(nruns);
         ctx->h_fp.resize(nruns);
     }
     stage = std::max<size_t>(stage, 1 << 16);

@@ -2,8 +2,11 @@
 // A.3.2), the current fold and the node-averaged fields (App. A.3.3), shared
 // by the field kernels (fields.cu) and the persistent ensemble step (walk.cu).
 //
-// Each body updates one padded cell from the interior images of its
-// neighbours and writes only that cell (see fields.cu for the layout).
+// Each body updates one padded cell from its neighbours and writes only that cell
+// (see fields.cu for the layout).  Ghost cells hold the bits of the interior cells
+// they mirror, so a neighbour is the next padded cell, or the image one period away
+// for the outermost layer: one select per axis where wrapping the coordinates took
+// the kernels several times their memory time.
 #pragma once
 #include <type_traits>
 
@@ -31,8 +34,61 @@ __device__ inline void padded_coords(const Geom &g, long long p, int &pi, int &p
     pk = (int)(q / g.py);
 }
 
+// A padded cell: its coordinates, and its index modulo 2^32 (grids of more cells
+// than that do not fit the device's memory).
+struct CellAt {
+    int pi, pj, pk;
+    uint32_t p;
+    __device__ __forceinline__ CellAt(const Geom &g, long long at) : p((uint32_t)at) { padded_coords(g, at, pi, pj, pk); }
+    // cell q of plane pk
+    __device__ __forceinline__ CellAt(const Geom &g, uint32_t q, int k) : pk(k) {
+        pj = (int)g.fpx.div(q);
+        pi = (int)(q - (uint32_t)pj * (uint32_t)g.px);
+        p = (uint32_t)k * ((uint32_t)g.px * (uint32_t)g.py) + q;
+    }
+    __device__ __forceinline__ bool interior(const Geom &g) const {
+        return (unsigned)(pi - g.G) < (unsigned)g.nx && (unsigned)(pj - g.G) < (unsigned)g.ny &&
+               (unsigned)(pk - g.Gz) < (unsigned)g.nz;
+    }
+    // interior, and no other padded cell is its image
+    __device__ __forceinline__ bool deep(const Geom &g) const {
+        return pi >= 2 * g.G && pi < g.nx && pj >= 2 * g.G && pj < g.ny &&
+               (g.ndim == 2 || (pk >= 2 * g.Gz && pk < g.nz));
+    }
+    // padded index of the neighbour below and above on each axis (or of its image)
+    __device__ __forceinline__ uint32_t xm(const Geom &g) const { return p + (uint32_t)(pi > 0 ? -1 : g.nx - 1); }
+    __device__ __forceinline__ uint32_t xp(const Geom &g) const { return p + (uint32_t)(pi + 1 < g.px ? 1 : 1 - g.nx); }
+    __device__ __forceinline__ uint32_t ym(const Geom &g) const {
+        return p + (uint32_t)(pj > 0 ? -1 : g.ny - 1) * (uint32_t)g.px;
+    }
+    __device__ __forceinline__ uint32_t yp(const Geom &g) const {
+        return p + (uint32_t)(pj + 1 < g.py ? 1 : 1 - g.ny) * (uint32_t)g.px;
+    }
+    __device__ __forceinline__ uint32_t zm(const Geom &g) const {
+        return p + (uint32_t)(pk > 0 ? -1 : g.nz - 1) * ((uint32_t)g.px * (uint32_t)g.py);
+    }
+    __device__ __forceinline__ uint32_t zp(const Geom &g) const {
+        return p + (uint32_t)(pk + 1 < g.pz ? 1 : 1 - g.nz) * ((uint32_t)g.px * (uint32_t)g.py);
+    }
+    // index of the interior image in a compact plane
+    __device__ __forceinline__ uint32_t compact(const Geom &g) const {
+        return ((uint32_t)g.wz(pk - g.Gz) * (uint32_t)g.ny + (uint32_t)g.wy(pj - g.G)) * (uint32_t)g.nx +
+               (uint32_t)g.wx(pi - g.G);
+    }
+};
+
 template <typename R>
-__device__ inline R ld(const R *a, long long i) { return ldro(a + i); }
+__device__ inline R ld(const R *a, uint32_t i) { return ldro(a + i); }
+
+// A float as a double.  The hardware's conversion runs on the FP64 pipe (one warp
+// instruction per 16 clocks); normal values take a few integer instructions.
+__device__ __forceinline__ double widen(float x) {
+    const int b = __float_as_int(x);
+    if ((b & 0x7fffffff) == 0) return 0.0;
+    if ((unsigned)(b << 1) - 0x01000000u >= 0xfe000000u) return (double)x;   // subnormal, infinite, NaN
+    return __hiloint2double((b & (int)0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20)), b << 29);
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 
 // Block-wide FP64 sum of NV values, one atomicAdd per value per block.
 template <int NV>
@@ -57,37 +113,42 @@ __device__ inline void block_accumulate(double (&v)[NV], double *acc) {
     }
 }
 
-// b <- b - h curl e (Faraday, Eq. dyn3 on the Yee lattice).  When energy_acc
-// is given, the interior sums of e^2 and b^2 (after the update) are added to
-// energy_acc[0..5] in FP64.
+// The two half advances of b of one step, b <- b - h curl e (Faraday, Eq. dyn3 on
+// the Yee lattice): e does not change between them, so one pass forms its curl once,
+// stores b at t (for the gather) in the compact planes bt and b at t + dt/2 in b.
+// With energy, the sums of e^2 and b^2 at t over interior cells go to acc in FP64.
 template <typename R>
-__device__ __forceinline__ void b_advance_cell(const Geom &g, const FieldPtrs<R> &f, R h, long long p, bool energy,
+__device__ __forceinline__ void b_advance_cell(const Geom &g, const FieldPtrs<R> &f, R h, const CellAt &c, bool energy,
                                                double (&acc)[6]) {
-    {
-        int pi, pj, pk;
-        padded_coords(g, p, pi, pj, pk);
-        const int i = g.wx(pi - g.G), j = g.wy(pj - g.G), k = g.wz(pk - g.Gz);
-        const long long c = g.pidx(i, j, k);
-        const R ex = ld(f.e[0], c), ey = ld(f.e[1], c), ez = ld(f.e[2], c);
-        const R curl_x = (ld(f.e[2], g.widx(i, j + 1, k)) - ez) - (ld(f.e[1], g.widx(i, j, k + 1)) - ey);
-        const R curl_y = (ld(f.e[0], g.widx(i, j, k + 1)) - ex) - (ld(f.e[2], g.widx(i + 1, j, k)) - ez);
-        const R curl_z = (ld(f.e[1], g.widx(i + 1, j, k)) - ey) - (ld(f.e[0], g.widx(i, j + 1, k)) - ex);
-        R bx = f.b[0][p] - h * curl_x;
-        R by = f.b[1][p] - h * curl_y;
-        R bz = f.b[2][p] - h * curl_z;
-        if (g.bcx == 1 && i == 0) bx = R(0);   // normal b vanishes on the conductor wall (App. A.4)
-        f.b[0][p] = bx;
-        f.b[1][p] = by;
-        f.b[2][p] = bz;
-        if (energy && pi == i + g.G && pj == j + g.G && pk == k + g.Gz) {
-            acc[0] += (double)ex * (double)ex;
-            acc[1] += (double)ey * (double)ey;
-            acc[2] += (double)ez * (double)ez;
-            acc[3] += (double)bx * (double)bx;
-            acc[4] += (double)by * (double)by;
-            acc[5] += (double)bz * (double)bz;
+    const uint32_t p = c.p, xp = c.xp(g), yp = c.yp(g), zp = c.zp(g);
+    const R ex = ld(f.e[0], p), ey = ld(f.e[1], p), ez = ld(f.e[2], p);
+    const R curl_x = (ld(f.e[2], yp) - ez) - (ld(f.e[1], zp) - ey);
+    const R curl_y = (ld(f.e[0], zp) - ex) - (ld(f.e[2], xp) - ez);
+    const R curl_z = (ld(f.e[1], xp) - ey) - (ld(f.e[0], yp) - ex);
+    // normal b vanishes on the conductor wall (App. A.4)
+    const bool wall = g.bcx == 1 && g.wx(c.pi - g.G) == 0;
+    R bx = f.b[0][p] - h * curl_x;
+    R by = f.b[1][p] - h * curl_y;
+    R bz = f.b[2][p] - h * curl_z;
+    if (wall) bx = R(0);
+    if (c.interior(g)) {
+        const uint32_t q = c.compact(g);
+        f.bt[0][q] = bx;
+        f.bt[1][q] = by;
+        f.bt[2][q] = bz;
+        if (energy) {
+            const double v[6] = {widen(ex), widen(ey), widen(ez), widen(bx), widen(by), widen(bz)};
+#pragma unroll
+            for (int q6 = 0; q6 < 6; ++q6) acc[q6] += v[q6] * v[q6];
         }
     }
+    bx = bx - h * curl_x;
+    by = by - h * curl_y;
+    bz = bz - h * curl_z;
+    if (wall) bx = R(0);
+    f.b[0][p] = bx;
+    f.b[1][p] = by;
+    f.b[2][p] = bz;
 }
 
 // Padded coordinates of the images of interior coordinate i along one axis
@@ -115,6 +176,12 @@ __device__ inline R folded_current(const Geom &g, const R *J, int i, int j, int 
             for (int a = 0; a < nqx; ++a) s += J[row + qx[a]];
         }
     return s;
+}
+
+template <typename R>
+__device__ inline R folded_current(const Geom &g, const R *J, const CellAt &c) {
+    if (c.deep(g)) return J[c.p];
+    return folded_current(g, J, g.wx(c.pi - g.G), g.wy(c.pj - g.G), g.wz(c.pk - g.Gz));
 }
 
 // Mixed path: the same update with the fixed-point current (int64, units of
@@ -175,27 +242,22 @@ __device__ __forceinline__ void e_pair_store(const FieldPtrs<float> &f, int c, l
 __device__ __forceinline__ void e_fx_cell(const Geom &g, const FieldPtrs<float> &f, const unsigned long long *J0,
                                           const unsigned long long *J1, const unsigned long long *J2,
                                           unsigned long long *Z0, unsigned long long *Z1, unsigned long long *Z2,
-                                          float dt, F2 scale, long long p) {
-    {
-        int pi, pj, pk;
-        padded_coords(g, p, pi, pj, pk);
-        const int i = g.wx(pi - g.G), j = g.wy(pj - g.G), k = g.wz(pk - g.Gz);
-        const long long c = g.pidx(i, j, k);
-        const float bx = ld(f.b[0], c), by = ld(f.b[1], c), bz = ld(f.b[2], c);
-        const F2 curl_x = curl_pair(bz, ld(f.b[2], g.widx(i, j - 1, k)), by, ld(f.b[1], g.widx(i, j, k - 1)));
-        const F2 curl_y = curl_pair(bx, ld(f.b[0], g.widx(i, j, k - 1)), bz, ld(f.b[2], g.widx(i - 1, j, k)));
-        const F2 curl_z = curl_pair(by, ld(f.b[1], g.widx(i - 1, j, k)), bx, ld(f.b[0], g.widx(i, j - 1, k)));
-        F2 ex = e_pair_update(f, 0, p, dt, curl_x, scale, (long long)folded_current(g, J0, i, j, k));
-        F2 ey = e_pair_update(f, 1, p, dt, curl_y, scale, (long long)folded_current(g, J1, i, j, k));
-        F2 ez = e_pair_update(f, 2, p, dt, curl_z, scale, (long long)folded_current(g, J2, i, j, k));
-        if (g.bcx == 1 && i == 0) { ey = F2{0.f, 0.f}; ez = F2{0.f, 0.f}; }
-        e_pair_store(f, 0, p, ex);
-        e_pair_store(f, 1, p, ey);
-        e_pair_store(f, 2, p, ez);
-        Z0[p] = 0ull;
-        Z1[p] = 0ull;
-        Z2[p] = 0ull;
-    }
+                                          float dt, F2 scale, const CellAt &c) {
+    const uint32_t p = c.p, xm = c.xm(g), ym = c.ym(g), zm = c.zm(g);
+    const float bx = ld(f.b[0], p), by = ld(f.b[1], p), bz = ld(f.b[2], p);
+    const F2 curl_x = curl_pair(bz, ld(f.b[2], ym), by, ld(f.b[1], zm));
+    const F2 curl_y = curl_pair(bx, ld(f.b[0], zm), bz, ld(f.b[2], xm));
+    const F2 curl_z = curl_pair(by, ld(f.b[1], xm), bx, ld(f.b[0], ym));
+    F2 ex = e_pair_update(f, 0, p, dt, curl_x, scale, (long long)folded_current(g, J0, c));
+    F2 ey = e_pair_update(f, 1, p, dt, curl_y, scale, (long long)folded_current(g, J1, c));
+    F2 ez = e_pair_update(f, 2, p, dt, curl_z, scale, (long long)folded_current(g, J2, c));
+    if (g.bcx == 1 && g.wx(c.pi - g.G) == 0) { ey = F2{0.f, 0.f}; ez = F2{0.f, 0.f}; }
+    e_pair_store(f, 0, p, ex);
+    e_pair_store(f, 1, p, ey);
+    e_pair_store(f, 2, p, ez);
+    Z0[p] = 0ull;
+    Z1[p] = 0ull;
+    Z2[p] = 0ull;
 }
 
 // The same update with the smoothed current: Js holds 3 compact planes (nx*ny*nz
@@ -203,38 +265,36 @@ __device__ __forceinline__ void e_fx_cell(const Geom &g, const FieldPtrs<float> 
 // scale converts (1 in the FP64 path, |alpha| 2^-36 in the mixed path).
 template <typename R, typename ZT, typename CT>
 __device__ __forceinline__ void e_smoothed_cell(const Geom &g, const FieldPtrs<R> &f, const CT *Js, double scale,
-                                                ZT *Z0, ZT *Z1, ZT *Z2, R dt, long long p) {
-    int pi, pj, pk;
-    padded_coords(g, p, pi, pj, pk);
-    const int i = g.wx(pi - g.G), j = g.wy(pj - g.G), k = g.wz(pk - g.Gz);
-    const long long c = g.pidx(i, j, k);
+                                                ZT *Z0, ZT *Z1, ZT *Z2, R dt, const CellAt &c) {
+    const uint32_t p = c.p, xm = c.xm(g), ym = c.ym(g), zm = c.zm(g);
     const long long ncell = (long long)g.nx * g.ny * g.nz;
-    const long long q = ((long long)k * g.ny + j) * g.nx + i;
-    const R bx = ld(f.b[0], c), by = ld(f.b[1], c), bz = ld(f.b[2], c);
+    const uint32_t q = c.compact(g);
+    const bool wall = g.bcx == 1 && g.wx(c.pi - g.G) == 0;
+    const R bx = ld(f.b[0], p), by = ld(f.b[1], p), bz = ld(f.b[2], p);
     if constexpr (std::is_same<R, float>::value) {
         // the mixed path's FP32 pair, updated as in e_fx_cell (the smoothed current is int64 fixed point)
         const F2 sc = {(float)scale, (float)(scale - (double)(float)scale)};
-        const F2 curl_x = curl_pair(bz, ld(f.b[2], g.widx(i, j - 1, k)), by, ld(f.b[1], g.widx(i, j, k - 1)));
-        const F2 curl_y = curl_pair(bx, ld(f.b[0], g.widx(i, j, k - 1)), bz, ld(f.b[2], g.widx(i - 1, j, k)));
-        const F2 curl_z = curl_pair(by, ld(f.b[1], g.widx(i - 1, j, k)), bx, ld(f.b[0], g.widx(i, j - 1, k)));
+        const F2 curl_x = curl_pair(bz, ld(f.b[2], ym), by, ld(f.b[1], zm));
+        const F2 curl_y = curl_pair(bx, ld(f.b[0], zm), bz, ld(f.b[2], xm));
+        const F2 curl_z = curl_pair(by, ld(f.b[1], xm), bx, ld(f.b[0], ym));
         F2 ex = e_pair_update(f, 0, p, dt, curl_x, sc, (long long)ldro(Js + q));
         F2 ey = e_pair_update(f, 1, p, dt, curl_y, sc, (long long)ldro(Js + ncell + q));
         F2 ez = e_pair_update(f, 2, p, dt, curl_z, sc, (long long)ldro(Js + 2 * ncell + q));
-        if (g.bcx == 1 && i == 0) { ey = F2{0.f, 0.f}; ez = F2{0.f, 0.f}; }
+        if (wall) { ey = F2{0.f, 0.f}; ez = F2{0.f, 0.f}; }
         e_pair_store(f, 0, p, ex);
         e_pair_store(f, 1, p, ey);
         e_pair_store(f, 2, p, ez);
     } else {
-        const R curl_x = (bz - ld(f.b[2], g.widx(i, j - 1, k))) - (by - ld(f.b[1], g.widx(i, j, k - 1)));
-        const R curl_y = (bx - ld(f.b[0], g.widx(i, j, k - 1))) - (bz - ld(f.b[2], g.widx(i - 1, j, k)));
-        const R curl_z = (by - ld(f.b[1], g.widx(i - 1, j, k))) - (bx - ld(f.b[0], g.widx(i, j - 1, k)));
+        const R curl_x = (bz - ld(f.b[2], ym)) - (by - ld(f.b[1], zm));
+        const R curl_y = (bx - ld(f.b[0], zm)) - (bz - ld(f.b[2], xm));
+        const R curl_z = (by - ld(f.b[1], xm)) - (bx - ld(f.b[0], ym));
         const R jx = (R)(scale * (double)ldro(Js + q));
         const R jy = (R)(scale * (double)ldro(Js + ncell + q));
         const R jz = (R)(scale * (double)ldro(Js + 2 * ncell + q));
         R ex = f.e[0][p] + dt * curl_x + jx;
         R ey = f.e[1][p] + dt * curl_y + jy;
         R ez = f.e[2][p] + dt * curl_z + jz;
-        if (g.bcx == 1 && i == 0) { ey = R(0); ez = R(0); }
+        if (wall) { ey = R(0); ez = R(0); }
         f.e[0][p] = ex;
         f.e[1][p] = ey;
         f.e[2][p] = ez;
@@ -244,52 +304,75 @@ __device__ __forceinline__ void e_smoothed_cell(const Geom &g, const FieldPtrs<R
     Z2[p] = ZT(0);
 }
 
-// Staggered value read by the gather; with conductor walls a value located
-// inside the conductor, or a tangential e / normal b on the wall, reads zero.
+// Staggered value read by the gather between conductor walls: a value located inside
+// the conductor, or a tangential e / normal b on the wall, reads zero.
 template <typename R>
-__device__ inline R sval(const Geom &g, const R *a, bool xstag, int i, int j, int k) {
-    if (g.bcx == 1) {
-        if (xstag) { if (i < 0 || i > g.nx - 1) return R(0); }
-        else { if (i <= 0 || i >= g.nx) return R(0); }
-    }
+__device__ inline R sval(const Geom &g, const R *a, bool compact, bool xstag, int i, int j, int k) {
+    if (xstag) { if (i < 0 || i > g.nx - 1) return R(0); }
+    else { if (i <= 0 || i >= g.nx) return R(0); }
+    if (compact) return ldro(a + ((long long)g.wz(k) * g.ny + g.wy(j)) * g.nx + g.wx(i));
     return ldro(a + g.widx(i, j, k));
 }
 
-// Node-averaged fields (App. A.3.3) at padded node p: e over its two edge
-// neighbours, b over its four face neighbours.
+// Node-averaged fields (App. A.3.3) at a padded node: e over its two edge
+// neighbours, b over its four face neighbours.  b is that of the compact planes bt
+// when there are any (within a step), else the padded b.
 template <typename R>
-__device__ __forceinline__ void node_average(const Geom &g, const FieldPtrs<R> &f, long long p, R (&E)[3],
+__device__ __forceinline__ void node_average(const Geom &g, const FieldPtrs<R> &f, const CellAt &c, R (&E)[3],
                                              R (&B)[3]) {
-    int pi, pj, pk;
-    padded_coords(g, p, pi, pj, pk);
-    // node coordinate (not wrapped: the conductor masking needs the true x)
-    int i = pi - g.G;
-    const int j = pj - g.G, k = pk - g.Gz;
-    if (g.bcx == 0) i = g.wx(i);
-    E[0] = R(0.5) * (sval(g, f.e[0], true, i - 1, j, k) + sval(g, f.e[0], true, i, j, k));
-    E[1] = R(0.5) * (sval(g, f.e[1], false, i, j - 1, k) + sval(g, f.e[1], false, i, j, k));
-    E[2] = R(0.5) * (sval(g, f.e[2], false, i, j, k - 1) + sval(g, f.e[2], false, i, j, k));
-    B[0] = R(0.25) * (sval(g, f.b[0], false, i, j, k) + sval(g, f.b[0], false, i, j - 1, k) +
-                      sval(g, f.b[0], false, i, j, k - 1) + sval(g, f.b[0], false, i, j - 1, k - 1));
-    B[1] = R(0.25) * (sval(g, f.b[1], true, i, j, k) + sval(g, f.b[1], true, i - 1, j, k) +
-                      sval(g, f.b[1], true, i, j, k - 1) + sval(g, f.b[1], true, i - 1, j, k - 1));
-    B[2] = R(0.25) * (sval(g, f.b[2], true, i, j, k) + sval(g, f.b[2], true, i - 1, j, k) +
-                      sval(g, f.b[2], true, i - 1, j - 1, k) + sval(g, f.b[2], true, i, j - 1, k));
+    const bool mid = f.bt[0] != nullptr;
+    const R *const bx = mid ? f.bt[0] : f.b[0], *const by = mid ? f.bt[1] : f.b[1], *const bz = mid ? f.bt[2] : f.b[2];
+    if (g.bcx == 1) {
+        // node coordinate, not wrapped: the masking needs the true x
+        const int i = c.pi - g.G, j = c.pj - g.G, k = c.pk - g.Gz;
+        auto e = [&](int a, bool st, int ii, int jj, int kk) { return sval(g, f.e[a], false, st, ii, jj, kk); };
+        auto b = [&](const R *a, bool st, int ii, int jj, int kk) { return sval(g, a, mid, st, ii, jj, kk); };
+        E[0] = R(0.5) * (e(0, true, i - 1, j, k) + e(0, true, i, j, k));
+        E[1] = R(0.5) * (e(1, false, i, j - 1, k) + e(1, false, i, j, k));
+        E[2] = R(0.5) * (e(2, false, i, j, k - 1) + e(2, false, i, j, k));
+        B[0] = R(0.25) * (b(bx, false, i, j, k) + b(bx, false, i, j - 1, k) + b(bx, false, i, j, k - 1) +
+                          b(bx, false, i, j - 1, k - 1));
+        B[1] = R(0.25) * (b(by, true, i, j, k) + b(by, true, i - 1, j, k) + b(by, true, i, j, k - 1) +
+                          b(by, true, i - 1, j, k - 1));
+        B[2] = R(0.25) * (b(bz, true, i, j, k) + b(bz, true, i - 1, j, k) + b(bz, true, i - 1, j - 1, k) +
+                          b(bz, true, i, j - 1, k));
+        return;
+    }
+    E[0] = R(0.5) * (ld(f.e[0], c.xm(g)) + ld(f.e[0], c.p));
+    E[1] = R(0.5) * (ld(f.e[1], c.ym(g)) + ld(f.e[1], c.p));
+    E[2] = R(0.5) * (ld(f.e[2], c.zm(g)) + ld(f.e[2], c.p));
+    uint32_t q, x, y, z;   // the cell, and the way to its lower neighbours
+    if (mid) {
+        const int i = g.wx(c.pi - g.G), j = g.wy(c.pj - g.G), k = g.wz(c.pk - g.Gz);
+        q = ((uint32_t)k * (uint32_t)g.ny + (uint32_t)j) * (uint32_t)g.nx + (uint32_t)i;
+        x = (uint32_t)(i > 0 ? -1 : g.nx - 1);
+        y = (uint32_t)(j > 0 ? -1 : g.ny - 1) * (uint32_t)g.nx;
+        z = (uint32_t)(k > 0 ? -1 : g.nz - 1) * ((uint32_t)g.nx * (uint32_t)g.ny);
+    } else {
+        q = c.p;
+        x = c.xm(g) - q;
+        y = c.ym(g) - q;
+        z = c.zm(g) - q;
+    }
+    B[0] = R(0.25) * (ld(bx, q) + ld(bx, q + y) + ld(bx, q + z) + ld(bx, q + y + z));
+    B[1] = R(0.25) * (ld(by, q) + ld(by, q + x) + ld(by, q + z) + ld(by, q + x + z));
+    B[2] = R(0.25) * (ld(bz, q) + ld(bz, q + x) + ld(bz, q + x + y) + ld(bz, q + y));
 }
 
 // Mixed path: stored as {E_x,E_y,E_z,B_x} and {B_y,B_z}.
 __device__ __forceinline__ void node_cell(const Geom &g, const FieldPtrs<float> &f, float4 *nfA, float2 *nfB,
-                                          long long p) {
+                                          const CellAt &c) {
     float E[3], B[3];
-    node_average<float>(g, f, p, E, B);
-    nfA[p] = make_float4(E[0], E[1], E[2], B[0]);
-    nfB[p] = make_float2(B[1], B[2]);
+    node_average<float>(g, f, c, E, B);
+    nfA[c.p] = make_float4(E[0], E[1], E[2], B[0]);
+    nfB[c.p] = make_float2(B[1], B[2]);
 }
 
 // FP64 path: three planes of double2, {E_x,E_y} {E_z,B_x} {B_y,B_z}.
-__device__ __forceinline__ void node_cell64(const Geom &g, const FieldPtrs<double> &f, double2 *nf, long long p) {
+__device__ __forceinline__ void node_cell64(const Geom &g, const FieldPtrs<double> &f, double2 *nf, const CellAt &c) {
+    const size_t p = c.p;
     double E[3], B[3];
-    node_average<double>(g, f, p, E, B);
+    node_average<double>(g, f, c, E, B);
     nf[p] = make_double2(E[0], E[1]);
     nf[g.pcells + p] = make_double2(E[2], B[0]);
     nf[2 * g.pcells + p] = make_double2(B[1], B[2]);

@@ -2,16 +2,17 @@
 // used by the gather (App. A.3.3).
 //
 // Every kernel runs one thread per padded cell, ghosts included.  A thread
-// computes the update of its cell from the interior images of the
-// neighbours, so a ghost cell receives exactly the value of the interior cell
+// computes the update of its cell from neighbours that hold the bits of their
+// interior images, so a ghost cell receives exactly the value of the interior cell
 // it mirrors and the padded arrays stay periodic without a separate copy.
 // Each thread reads its own cell and neighbours, and writes only its own cell,
 // of arrays that are not read at neighbour positions in the same kernel, so
 // no two threads race.
 //
-// Roofline: HBM bound.  Algorithmic bytes per cell: b advance 6 reads +
-// 3 writes; e advance 6 + 3 (J) reads, 3 writes, 3 zero-writes; node fields 6
-// reads + 8 writes, in units of sizeof(Real) (float4 pairs for node fields).
+// Roofline: HBM bound.  Algorithmic bytes per cell: b advance (both halves) 6 reads +
+// 6 writes; e advance 6 + 3 (J) reads, 3 writes, 3 zero-writes; node fields 6
+// reads + 6 writes, in units of sizeof(Real) (J: 8 B).  Blocks of 256 cells of one
+// z plane, so that a thread divides once for its coordinates.
 #include <type_traits>
 
 #include "field_cells.cuh"
@@ -21,79 +22,77 @@ namespace pic {
 
 namespace {
 
-// b <- b - h curl e over every padded cell; with a history slot, the interior
-// sums of e^2 and b^2 are added to it.  kin_prev (nullable): the kinetic energy the
-// previous step recorded at u^{t-1/2}, which is this step's first entry.
+// Calls body(cell) for the cells of the blocks dealt to this thread block.
+template <typename F>
+__device__ __forceinline__ void for_cells(const Geom &g, F &&body) {
+    const uint32_t plane = (uint32_t)g.px * (uint32_t)g.py;
+    const int per = (int)((plane + 255) / 256), n = per * g.pz;
+    for (int b = blockIdx.x; b < n; b += gridDim.x) {
+        const int k = b / per;
+        const uint32_t q = (uint32_t)(b - k * per) * 256 + threadIdx.x;
+        if (q < plane) body(CellAt(g, q, k));
+    }
+}
+
+// Both half advances of b over every padded cell; with a history slot, the interior
+// sums of e^2 and b^2 at t are added to it.  kin_prev (nullable): the kinetic energy
+// the previous step recorded at u^{t-1/2}, which is this step's first entry.
 template <typename R>
-__global__ void k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, const double *kin_prev) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
+__global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, const double *kin_prev) {
     double *slot = hist.slot();
     if (slot && kin_prev && blockIdx.x == 0 && threadIdx.x == 0) slot[0] = *kin_prev;
     double *energy_acc = slot ? slot + 2 : nullptr;
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
-        b_advance_cell<R>(g, f, h, p, energy_acc != nullptr, acc);
+    for_cells(g, [&](const CellAt &c) { b_advance_cell<R>(g, f, h, c, energy_acc != nullptr, acc); });
     if (energy_acc) block_accumulate<6>(acc, energy_acc);
 }
 
 // e <- e + dt curl b + J (Ampere, Eq. dyn4 with the deposited current, main
 // loop steps 6, 11, 12), and zeroing of the other current buffer.
 template <typename R>
-__global__ void k_e_advance(Geom g, FieldPtrs<R> f, const R *J0, const R *J1, const R *J2, R *Z0, R *Z1, R *Z2,
-                            R dt) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride) {
-        int pi, pj, pk;
-        padded_coords(g, p, pi, pj, pk);
-        const int i = g.wx(pi - g.G), j = g.wy(pj - g.G), k = g.wz(pk - g.Gz);
-        const long long c = g.pidx(i, j, k);
-        const R bx = ld(f.b[0], c), by = ld(f.b[1], c), bz = ld(f.b[2], c);
-        const R curl_x = (bz - ld(f.b[2], g.widx(i, j - 1, k))) - (by - ld(f.b[1], g.widx(i, j, k - 1)));
-        const R curl_y = (bx - ld(f.b[0], g.widx(i, j, k - 1))) - (bz - ld(f.b[2], g.widx(i - 1, j, k)));
-        const R curl_z = (by - ld(f.b[1], g.widx(i - 1, j, k))) - (bx - ld(f.b[0], g.widx(i, j - 1, k)));
-        R ex = f.e[0][p] + dt * curl_x + folded_current(g, J0, i, j, k);
-        R ey = f.e[1][p] + dt * curl_y + folded_current(g, J1, i, j, k);
-        R ez = f.e[2][p] + dt * curl_z + folded_current(g, J2, i, j, k);
-        if (g.bcx == 1 && i == 0) { ey = R(0); ez = R(0); }   // tangential e vanishes on the wall
+__global__ void __launch_bounds__(256) k_e_advance(Geom g, FieldPtrs<R> f, const R *J0, const R *J1, const R *J2, R *Z0,
+                                                   R *Z1, R *Z2, R dt) {
+    for_cells(g, [&](const CellAt &c) {
+        const uint32_t p = c.p, xm = c.xm(g), ym = c.ym(g), zm = c.zm(g);
+        const R bx = ld(f.b[0], p), by = ld(f.b[1], p), bz = ld(f.b[2], p);
+        const R curl_x = (bz - ld(f.b[2], ym)) - (by - ld(f.b[1], zm));
+        const R curl_y = (bx - ld(f.b[0], zm)) - (bz - ld(f.b[2], xm));
+        const R curl_z = (by - ld(f.b[1], xm)) - (bx - ld(f.b[0], ym));
+        R ex = f.e[0][p] + dt * curl_x + folded_current(g, J0, c);
+        R ey = f.e[1][p] + dt * curl_y + folded_current(g, J1, c);
+        R ez = f.e[2][p] + dt * curl_z + folded_current(g, J2, c);
+        if (g.bcx == 1 && g.wx(c.pi - g.G) == 0) { ey = R(0); ez = R(0); }   // tangential e vanishes on the wall
         f.e[0][p] = ex;
         f.e[1][p] = ey;
         f.e[2][p] = ez;
         Z0[p] = R(0);
         Z1[p] = R(0);
         Z2[p] = R(0);
-    }
+    });
 }
 
-__global__ void k_e_advance_fx(Geom g, FieldPtrs<float> f, const unsigned long long *J0,
-                               const unsigned long long *J1, const unsigned long long *J2, unsigned long long *Z0,
-                               unsigned long long *Z1, unsigned long long *Z2, float dt, F2 scale,
-                               long long *hist_inc) {
+__global__ void __launch_bounds__(256) k_e_advance_fx(Geom g, FieldPtrs<float> f, const unsigned long long *J0,
+                                                      const unsigned long long *J1, const unsigned long long *J2,
+                                                      unsigned long long *Z0, unsigned long long *Z1,
+                                                      unsigned long long *Z2, float dt, F2 scale, long long *hist_inc) {
     // no kernel of this launch reads the counter; the next step's kernels see the new value
     if (hist_inc && blockIdx.x == 0 && threadIdx.x == 0) *hist_inc += 1;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
-        e_fx_cell(g, f, J0, J1, J2, Z0, Z1, Z2, dt, scale, p);
+    for_cells(g, [&](const CellAt &c) { e_fx_cell(g, f, J0, J1, J2, Z0, Z1, Z2, dt, scale, c); });
 }
 
 template <typename R, typename ZT, typename CT>
-__global__ void k_e_advance_smoothed(Geom g, FieldPtrs<R> f, const CT *Js, double scale, ZT *Z0, ZT *Z1, ZT *Z2,
-                                     R dt, long long *hist_inc) {
+__global__ void __launch_bounds__(256) k_e_advance_smoothed(Geom g, FieldPtrs<R> f, const CT *Js, double scale, ZT *Z0,
+                                                            ZT *Z1, ZT *Z2, R dt, long long *hist_inc) {
     if (hist_inc && blockIdx.x == 0 && threadIdx.x == 0) *hist_inc += 1;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
-        e_smoothed_cell<R, ZT, CT>(g, f, Js, scale, Z0, Z1, Z2, dt, p);
+    for_cells(g, [&](const CellAt &c) { e_smoothed_cell<R, ZT, CT>(g, f, Js, scale, Z0, Z1, Z2, dt, c); });
 }
 
-__global__ void k_node_fields(Geom g, FieldPtrs<float> f, float4 *nfA, float2 *nfB) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
-        node_cell(g, f, nfA, nfB, p);
+__global__ void __launch_bounds__(256) k_node_fields(Geom g, FieldPtrs<float> f, float4 *nfA, float2 *nfB) {
+    for_cells(g, [&](const CellAt &c) { node_cell(g, f, nfA, nfB, c); });
 }
 
-__global__ void k_node_fields64(Geom g, FieldPtrs<double> f, double2 *nf) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < g.pcells; p += stride)
-        node_cell64(g, f, nf, p);
+__global__ void __launch_bounds__(256) k_node_fields64(Geom g, FieldPtrs<double> f, double2 *nf) {
+    for_cells(g, [&](const CellAt &c) { node_cell64(g, f, nf, c); });
 }
 
 // Batched over runs: block b belongs to the run r with block_prefix[r] <= b <
@@ -120,23 +119,24 @@ __global__ void __launch_bounds__(256) k_fields_multi(const FieldRunF *runs, con
     __syncthreads();
     const long long p = (long long)(blockIdx.x - block_prefix[run_sh]) * blockDim.x + threadIdx.x;
     const bool in = p < r.g.pcells;
-    if (PHASE == FIELD_B_HALF) {
+    const CellAt c(r.g, in ? p : 0);
+    if (PHASE == FIELD_B) {
         double *slot = r.hist.slot();
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
-        if (in) b_advance_cell<float>(r.g, r.f, h, p, energy_acc != nullptr, acc);
+        if (in) b_advance_cell<float>(r.g, r.f, h, c, energy_acc != nullptr, acc);
         if (energy_acc) block_accumulate<6>(acc, energy_acc);
     } else if (PHASE == FIELD_NODE) {
-        if (in) node_cell(r.g, r.f, r.nfA, r.nfB, p);
+        if (in) node_cell(r.g, r.f, r.nfA, r.nfB, c);
     } else {
         if (r.hist_inc && blockIdx.x == block_prefix[run_sh] && threadIdx.x == 0) *r.hist_inc += 1;
         if (in) {
             if (r.smooth > 0)
                 e_smoothed_cell<float, unsigned long long, long long>(r.g, r.f, r.sbuf[r.smooth & 1], r.scale,
-                                                                      r.Z[0], r.Z[1], r.Z[2], dt, p);
+                                                                      r.Z[0], r.Z[1], r.Z[2], dt, c);
             else
                 e_fx_cell(r.g, r.f, r.J[0], r.J[1], r.J[2], r.Z[0], r.Z[1], r.Z[2], dt,
-                          F2{(float)r.scale, (float)(r.scale - (double)(float)r.scale)}, p);
+                          F2{(float)r.scale, (float)(r.scale - (double)(float)r.scale)}, c);
         }
     }
 }
@@ -170,32 +170,38 @@ inline int grid_for(long long n, int threads) {
     const long long cap = 152LL * 16;   // 16 resident 256-thread blocks per SM on 152 SMs
     return (int)(b < cap ? (b > 0 ? b : 1) : cap);
 }
+// grid of a for_cells kernel
+inline int cells_grid(const Geom &g, int per_sm) {
+    const long long n = ((long long)g.px * g.py + 255) / 256 * g.pz;
+    return (int)(n < 152LL * per_sm ? n : 152LL * per_sm);
+}
 
 }  // namespace
 
 template <typename R>
 void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s) {
-    k_b_advance<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, h, energy, kin_prev);
+    // (few blocks: each adds its six sums to the same addresses)
+    k_b_advance<R><<<cells_grid(g, 8), 256, 0, s>>>(g, f, h, energy, kin_prev);
 }
 
 template <typename R>
 void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *const Jzero[3], R dt,
                       cudaStream_t s) {
-    k_e_advance<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, J[0], J[1], J[2], Jzero[0], Jzero[1], Jzero[2],
+    k_e_advance<R><<<cells_grid(g, 16), 256, 0, s>>>(g, f, J[0], J[1], J[2], Jzero[0], Jzero[1], Jzero[2],
                                                            dt);
 }
 
 void launch_node_fields(const Geom &g, FieldPtrs<float> f, float4 *nfA, float2 *nfB, cudaStream_t s) {
-    k_node_fields<<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, nfA, nfB);
+    k_node_fields<<<cells_grid(g, 16), 256, 0, s>>>(g, f, nfA, nfB);
 }
 
 void launch_node_fields64(const Geom &g, FieldPtrs<double> f, double2 *nf, cudaStream_t s) {
-    k_node_fields64<<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, nf);
+    k_node_fields64<<<cells_grid(g, 16), 256, 0, s>>>(g, f, nf);
 }
 
 void launch_fields_multi(int phase, const FieldRunF *runs_dev, const int *block_prefix_dev, int nblocks, int nruns,
                          float h, float dt, cudaStream_t s) {
-    if (phase == FIELD_B_HALF) k_fields_multi<FIELD_B_HALF><<<nblocks, 256, 0, s>>>(runs_dev, block_prefix_dev, nruns, h, dt);
+    if (phase == FIELD_B) k_fields_multi<FIELD_B><<<nblocks, 256, 0, s>>>(runs_dev, block_prefix_dev, nruns, h, dt);
     else if (phase == FIELD_NODE) k_fields_multi<FIELD_NODE><<<nblocks, 256, 0, s>>>(runs_dev, block_prefix_dev, nruns, h, dt);
     else k_fields_multi<FIELD_E_FX><<<nblocks, 256, 0, s>>>(runs_dev, block_prefix_dev, nruns, h, dt);
 }
@@ -205,14 +211,14 @@ void launch_e_advance_fx(const Geom &g, FieldPtrs<float> f, const unsigned long 
                          cudaStream_t s) {
     const double scale = alpha_abs * 0x1p-36;
     const F2 sc = {(float)scale, (float)(scale - (double)(float)scale)};
-    k_e_advance_fx<<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, J[0], J[1], J[2], Jzero[0], Jzero[1], Jzero[2],
+    k_e_advance_fx<<<cells_grid(g, 16), 256, 0, s>>>(g, f, J[0], J[1], J[2], Jzero[0], Jzero[1], Jzero[2],
                                                            dt, sc, hist_inc);
 }
 
 template <typename R, typename ZT, typename CT>
 void launch_e_advance_smoothed(const Geom &g, FieldPtrs<R> f, const CT *Js, double scale, ZT *const Jzero[3],
                                R dt, long long *hist_inc, cudaStream_t s) {
-    k_e_advance_smoothed<R, ZT, CT><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, Js, scale, Jzero[0], Jzero[1],
+    k_e_advance_smoothed<R, ZT, CT><<<cells_grid(g, 16), 256, 0, s>>>(g, f, Js, scale, Jzero[0], Jzero[1],
                                                                             Jzero[2], dt, hist_inc);
 }
 

@@ -129,6 +129,7 @@ struct FieldPtrs {
     R *e[3];
     R *b[3];
     R *el[3];
+    R *bt[3];   // b at t between the b advance and the push of a step: compact interior planes (nullable)
 };
 
 // e_c at padded index p in FP64, with its low-order part when there is one.
@@ -208,7 +209,7 @@ struct HistRef {
 // ---- kernel launchers (implemented in the .cu files) ----
 
 // fields.cu
-// kin_prev (nullable): copied to slot[0] of the energy record
+// both half advances of b; b at t goes to f.bt.  kin_prev (nullable): copied to slot[0] of the energy record
 template <typename R>
 void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s);
 template <typename R>
@@ -319,7 +320,7 @@ struct FieldRunF {
     int smooth;             // current smoothing passes (0: off); the E_FX phase then reads sbuf[smooth & 1]
     long long *sbuf[2];     // compact fixed-point smoothing buffers, 3 planes of nx*ny*nz each
 };
-enum { FIELD_B_HALF = 0, FIELD_NODE = 1, FIELD_E_FX = 2 };
+enum { FIELD_B = 0, FIELD_NODE = 1, FIELD_E_FX = 2 };
 void launch_fields_multi(int phase, const FieldRunF *runs_dev, const int *block_prefix_dev, int nblocks, int nruns,
                          float h, float dt, cudaStream_t s);
 // smooth.cu, batched: phase 0 folds every smoothing run's J into sbuf[0]; phase 1 runs pass
@@ -338,12 +339,12 @@ enum WalkPhase {
     // the counting sort of one species (steps that sort)
     S_ZERO = 0, S_HIST, S_SCAN_BLOCKS, S_SCAN_SUMS, S_SCAN_FINISH, S_RANK, S_ZERO_AFTER, S_GATHER,
     // the main loop
-    W_B_HALF_E, W_NODE, W_PUSH, W_SMOOTH_FOLD, W_SMOOTH_PASS, W_B_HALF, W_E_FX
+    W_B, W_NODE, W_PUSH, W_SMOOTH_FOLD, W_SMOOTH_PASS, W_E_FX
 };
 constexpr int kWalkMaxPhases = 32;
 struct WalkArgs {
     const MixedStepArgs *push;     // per run
-    const FieldRunF *fe, *fp;      // per run: first b half advance (records the energies); other field phases
+    const FieldRunF *fp;           // per run: the field phases
     const SortArgs *sort;          // [nruns * 4]: run r, species q at 4 r + q (runs that sort this step)
     const int *prefix;             // [nphase * nruns + 1]: first queue item of (phase, slot), phase-major
     const int *base;               // [nruns * (nphase + 1)]: items of run r in the phases before each phase

@@ -2,9 +2,9 @@
 // phase of one step of every run: on the steps that re-sort a run, the phases
 // of the counting sort of each species (key histogram unless the previous push
 // counted it, block scans, rank, gather), then the main loop of App. A.3.1:
-// b half advance with the energy record, node-averaged fields,
-// gather-push-deposit, the optional current smoothing (step 10), b half
-// advance, e advance with the folded current.
+// both half advances of b with the energy record, node-averaged fields,
+// gather-push-deposit, the optional current smoothing (step 10), e advance with the
+// folded current.
 //
 // Work queue.  The items of phase ph of run r are the tiles of the run (push,
 // and parts of the old layout's tiles for the sort's histogram and rank),
@@ -89,17 +89,17 @@ __device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRun
     typedef unsigned long long u64;
     const Geom &g = fr.g;
     const long long p0 = (long long)local * w.cells_per_item;
-    if (kind == W_B_HALF_E || kind == W_B_HALF) {
+    if (kind == W_B) {
         const long long p1 = min(p0 + w.cells_per_item, g.pcells);
         double *slot = fr.hist.slot();
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         for (long long p = p0 + threadIdx.x; p < p1; p += THREADS)
-            b_advance_cell<float>(g, fr.f, w.h, p, energy_acc != nullptr, acc);
+            b_advance_cell<float>(g, fr.f, w.h, CellAt(g, p), energy_acc != nullptr, acc);
         if (energy_acc) block_accumulate<6>(acc, energy_acc);
     } else if (kind == W_NODE) {
         const long long p1 = min(p0 + w.cells_per_item, g.pcells);
-        for (long long p = p0 + threadIdx.x; p < p1; p += THREADS) node_cell(g, fr.f, fr.nfA, fr.nfB, p);
+        for (long long p = p0 + threadIdx.x; p < p1; p += THREADS) node_cell(g, fr.f, fr.nfA, fr.nfB, CellAt(g, p));
     } else if (kind == W_E_FX) {
         const long long p1 = min(p0 + w.cells_per_item, g.pcells);
         if (fr.hist_inc && local == 0 && threadIdx.x == 0) *fr.hist_inc += 1;
@@ -107,9 +107,9 @@ __device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRun
         for (long long p = p0 + threadIdx.x; p < p1; p += THREADS) {
             if (fr.smooth > 0)
                 e_smoothed_cell<float, u64, long long>(g, fr.f, fr.sbuf[fr.smooth & 1], fr.scale, fr.Z[0], fr.Z[1],
-                                                        fr.Z[2], w.dt, p);
+                                                        fr.Z[2], w.dt, CellAt(g, p));
             else
-                e_fx_cell(g, fr.f, fr.J[0], fr.J[1], fr.J[2], fr.Z[0], fr.Z[1], fr.Z[2], w.dt, sc, p);
+                e_fx_cell(g, fr.f, fr.J[0], fr.J[1], fr.J[2], fr.Z[0], fr.Z[1], fr.Z[2], w.dt, sc, CellAt(g, p));
         }
     } else {
         // smoothing: compact interior cells (k*ny + j)*nx + i
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
                 __syncthreads();
                 push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, local, 0, 1, w.push + r);
             } else {
-                const FieldRunF *fsrc = kind == W_B_HALF_E ? w.fe + r : w.fp + r;
+                const FieldRunF *fsrc = w.fp + r;
                 const int *src = reinterpret_cast<const int *>(fsrc);
                 int *dst = reinterpret_cast<int *>(&fr_sh);
                 for (int q = threadIdx.x; q < (int)(sizeof(FieldRunF) / sizeof(int)); q += THREADS) dst[q] = src[q];
