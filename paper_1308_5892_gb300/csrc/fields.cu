@@ -44,7 +44,8 @@ __global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, 
     double *energy_acc = slot ? slot + 2 : nullptr;
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for_cells(g, [&](const CellAt &c) { b_advance_cell<R>(g, f, h, c, energy_acc != nullptr, acc); });
-    if (energy_acc) block_accumulate<6>(acc, energy_acc);
+    __shared__ double sh[6 * 256];
+    if (energy_acc) block_accumulate<6, 256>(acc, energy_acc, sh);
 }
 
 // e <- e + dt curl b + J (Ampere, Eq. dyn4 with the deposited current, main
@@ -125,7 +126,8 @@ __global__ void __launch_bounds__(256) k_fields_multi(const FieldRunF *runs, con
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         if (in) b_advance_cell<float>(r.g, r.f, h, c, energy_acc != nullptr, acc);
-        if (energy_acc) block_accumulate<6>(acc, energy_acc);
+        __shared__ double sh[6 * 256];
+        if (energy_acc) block_accumulate<6, 256>(acc, energy_acc, sh);
     } else if (PHASE == FIELD_NODE) {
         if (in) node_cell(r.g, r.f, r.nfA, r.nfB, c);
     } else {
@@ -181,7 +183,7 @@ inline int cells_grid(const Geom &g, int per_sm) {
 template <typename R>
 void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s) {
     // (few blocks: each adds its six sums to the same addresses)
-    k_b_advance<R><<<cells_grid(g, 8), 256, 0, s>>>(g, f, h, energy, kin_prev);
+    k_b_advance<R><<<cells_grid(g, 4), 256, 0, s>>>(g, f, h, energy, kin_prev);
 }
 
 template <typename R>

@@ -83,9 +83,9 @@ __device__ bool wait_run(const WalkArgs &w, int r, int target) {
     }
 }
 
-// One field or smoothing item: cells [p0, p1) of run r.
+// One field or smoothing item: cells [p0, p1) of run r (sh: 6 THREADS doubles).
 template <int THREADS>
-__device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRunF &fr, int local) {
+__device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRunF &fr, int local, double *sh) {
     typedef unsigned long long u64;
     const Geom &g = fr.g;
     const long long p0 = (long long)local * w.cells_per_item;
@@ -96,7 +96,7 @@ __device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRun
         double acc[6] = {0, 0, 0, 0, 0, 0};
         for (long long p = p0 + threadIdx.x; p < p1; p += THREADS)
             b_advance_cell<float>(g, fr.f, w.h, CellAt(g, p), energy_acc != nullptr, acc);
-        if (energy_acc) block_accumulate<6>(acc, energy_acc);
+        if (energy_acc) block_accumulate<6, THREADS>(acc, energy_acc, sh);
     } else if (kind == W_NODE) {
         const long long p1 = min(p0 + w.cells_per_item, g.pcells);
         for (long long p = p0 + threadIdx.x; p < p1; p += THREADS) node_cell(g, fr.f, fr.nfA, fr.nfB, CellAt(g, p));
@@ -223,7 +223,9 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
                 int *dst = reinterpret_cast<int *>(&fr_sh);
                 for (int q = threadIdx.x; q < (int)(sizeof(FieldRunF) / sizeof(int)); q += THREADS) dst[q] = src[q];
                 __syncthreads();
-                field_item<THREADS>(w, kind, w.pass[ph], fr_sh, local);
+                // (the push's dynamic shared memory holds the sums)
+                extern __shared__ __align__(128) float4 smem4[];
+                field_item<THREADS>(w, kind, w.pass[ph], fr_sh, local, reinterpret_cast<double *>(smem4));
             }
         }
         __syncthreads();
@@ -311,6 +313,7 @@ int walk_sort_items(const SortArgs &a, int kind, int cpi) {
 }
 
 bool walk_fits(int ndim, bool walls, bool count, size_t push_smem) {
+    if (push_smem < sizeof(double) * 6 * (ndim == 3 ? 512 : 256)) return false;   // the energy sums live there
     return ndim == 3 ? fits_dim<3, 512, 1>(walls, count, push_smem) : fits_dim<2, 256, 2>(walls, count, push_smem);
 }
 
