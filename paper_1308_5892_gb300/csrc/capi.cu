@@ -39,8 +39,9 @@ struct SpeciesState {
     int *tile_start_alt = nullptr;
     bool tiled = false;         // current layout comes from a sort
     int tiled_ntiles = 0;       // tile count of the geometry that sort used
-    int *counts = nullptr;      // mixed: key histogram / cursors of the sort, zero between sorts
-    bool counted = false;       // the last push filled counts for the next sort
+    int *counts = nullptr;      // mixed: key histogram / cursors of the sort
+    int *perm = nullptr;        // mixed: source slot of every slot of the layout being sorted to; id index elsewhere
+    bool moving = false;        // mixed: sorted, and the next push moves the particles to the new layout
     int lgw = 5;                // mixed: log2 of the walk length of the current layout
 };
 
@@ -65,7 +66,7 @@ struct Run {
     int *nparts = nullptr;
     int parts_cap = 0, parts_bound = 0;
     int *offsets = nullptr, *block_sums = nullptr;
-    int *perm = nullptr;        // sort scratch, max species capacity
+    int *perm = nullptr;        // FP64: sort scratch, max species capacity
     // FP64 path: node averages, and the sort's scratch (null when the allocator had no room: no sort then)
     double2 *nf64 = nullptr;
     double *M64 = nullptr;      // moment planes of the current
@@ -119,13 +120,13 @@ struct pic_ctx {
     std::vector<int> h_walk;
     SortArgs *walk_sort_dev = nullptr;              // step walker: sort arguments, [nruns * 4]
     std::vector<SortArgs> h_walk_sort;
-    int walk_fit[2][2] = {{-1, -1}, {-1, -1}};      // walk_fits() by (walls, count) for walk_fit_smem
+    int walk_fit[2][2] = {{-1, -1}, {-1, -1}};      // walk_fits() by (walls, move) for walk_fit_smem
     size_t walk_fit_smem = 0;
     int multi_nblocks = 0;
     bool multi_tiles_dirty = false;
     std::vector<MixedStepArgs> h_args;
     SortArgs *sort_args_dev = nullptr;    // one species of every run, for the batched sort
-    int *sort_prefix_dev = nullptr;       // 4 x (nruns + 1) block prefixes of its phases
+    int *sort_prefix_dev = nullptr;       // 3 x (nruns + 1) block prefixes of its phases
     std::vector<SortArgs> h_sort;
     std::vector<int> h_sort_prefix;
     // CUDA graph of one period of steps (mixed path): captured on a private stream,
@@ -339,14 +340,9 @@ __global__ void k_upload_mixed(Geom g, const double *st, long long stride, long 
         }
         for (int comp = 3; comp < 6; ++comp)
             if (!isfinite(st[comp * stride + q])) atomicOr(err, ERR_NONFINITE);
-        d.cell[a + q] = pack_cell(g.ndim, c[0], c[1], c[2]);
-        d.off[0][a + q] = o[0];
-        d.off[1][a + q] = o[1];
-        if (g.ndim == 3) d.off[2][a + q] = o[2];
-        d.u[0][a + q] = (float)st[3 * stride + q];
-        d.u[1][a + q] = (float)st[4 * stride + q];
-        d.u[2][a + q] = (float)st[5 * stride + q];
-        d.id[a + q] = (int32_t)(a + q);
+        const float u[3] = {(float)st[3 * stride + q], (float)st[4 * stride + q], (float)st[5 * stride + q]};
+        put_particle(g.ndim, d, a + q, pack_cell(g.ndim, c[0], c[1], c[2]), o, u, __int_as_float((int)(a + q)));
+        if (g.ndim == 2) d.id[a + q] = (int32_t)(a + q);
     }
 }
 
@@ -355,18 +351,25 @@ __global__ void k_id_index(const int32_t *id, long long n, int *inv) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x)
         if ((unsigned long long)id[p] < (unsigned long long)n) inv[id[p]] = (int)p;   // ids are 0 .. n-1
 }
+__global__ void k_id_index_mixed(int ndim, SpeciesMixed s, long long n, int *inv) {
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
+        const int id = get_id(ndim, s, p);
+        if ((unsigned long long)id < (unsigned long long)n) inv[id] = (int)p;
+    }
+}
 
 __global__ void k_pick_mixed(Geom g, SpeciesMixed s, const int *inv, const long long *ids, long long m, double *st) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
         const int p = inv[ids[q]];
         int i, j, k;
-        unpack_cell(g.ndim, s.cell[p], i, j, k);
-        st[q] = (double)i + (double)s.off[0][p];
-        st[m + q] = (double)j + (double)s.off[1][p];
-        st[2 * m + q] = g.ndim == 3 ? (double)k + (double)s.off[2][p] : 0.0;
-        st[3 * m + q] = s.u[0][p];
-        st[4 * m + q] = s.u[1][p];
-        st[5 * m + q] = s.u[2][p];
+        float off[3], u[3];
+        unpack_cell(g.ndim, get_particle(g.ndim, s, p, off, u), i, j, k);
+        st[q] = (double)i + (double)off[0];
+        st[m + q] = (double)j + (double)off[1];
+        st[2 * m + q] = g.ndim == 3 ? (double)k + (double)off[2] : 0.0;
+        st[3 * m + q] = u[0];
+        st[4 * m + q] = u[1];
+        st[5 * m + q] = u[2];
     }
 }
 
@@ -389,13 +392,14 @@ __global__ void k_download_by_id(Geom g, SpeciesMixed s, const int *inv, long lo
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
         const int p = inv[a + q];
         int i, j, k;
-        unpack_cell(g.ndim, s.cell[p], i, j, k);
-        st[q] = (double)i + (double)s.off[0][p];
-        st[stride + q] = (double)j + (double)s.off[1][p];
-        st[2 * stride + q] = g.ndim == 3 ? (double)k + (double)s.off[2][p] : 0.0;
-        st[3 * stride + q] = s.u[0][p];
-        st[4 * stride + q] = s.u[1][p];
-        st[5 * stride + q] = s.u[2][p];
+        float off[3], u[3];
+        unpack_cell(g.ndim, get_particle(g.ndim, s, p, off, u), i, j, k);
+        st[q] = (double)i + (double)off[0];
+        st[stride + q] = (double)j + (double)off[1];
+        st[2 * stride + q] = g.ndim == 3 ? (double)k + (double)off[2] : 0.0;
+        st[3 * stride + q] = u[0];
+        st[4 * stride + q] = u[1];
+        st[5 * stride + q] = u[2];
     }
 }
 
@@ -645,16 +649,13 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         r.block_sums = (int *)dev_alloc(ctx, sizeof(int) * sort_scan_scratch(nkeys));
         r.max_tiles = max_tiles;
         r.max_keys = max_keys;
-        int64_t capmax = 1;
-        for (int s = 0; s < d.nspecies; ++s) capmax = std::max<int64_t>(capmax, d.species[s].capacity);
-        r.perm = (int *)dev_alloc(ctx, sizeof(int) * capmax);
         if (ctx->runs.size() == 1) {
             r.parts_cap = std::min(max_tiles, kPartTiles) + part_slots(d.ndim) + 1;
             r.parts = (int2 *)dev_alloc(ctx, sizeof(int2) * r.parts_cap);
             r.nparts = (int *)dev_alloc(ctx, sizeof(int));
             if (!r.parts || !r.nparts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
         }
-        if (!r.nfA || !r.nfB || !r.offsets || !r.block_sums || !r.perm)
+        if (!r.nfA || !r.nfB || !r.offsets || !r.block_sums)
             return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
     }
     if (!mixed) {
@@ -698,18 +699,16 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         } else {
             for (int b = 0; b < 2; ++b) {
                 SpeciesMixed &m = S.mb[b];
-                m.cell = (uint32_t *)dev_alloc(ctx, sizeof(uint32_t) * cap);
-                m.id = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * cap);
-                for (int a = 0; a < 3; ++a) {
-                    m.off[a] = (a < d.ndim) ? (float *)dev_alloc(ctx, sizeof(float) * cap) : nullptr;
-                    m.u[a] = (float *)dev_alloc(ctx, sizeof(float) * cap);
-                    if ((a < d.ndim && !m.off[a]) || !m.u[a]) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for particles");
-                }
-                if (!m.cell || !m.id) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for particles");
+                m.a = (float4 *)dev_alloc(ctx, sizeof(float4) * cap);
+                m.b = (float *)dev_alloc(ctx, sizeof(float) * (d.ndim == 3 ? 4 : 2) * cap);
+                m.id = d.ndim == 3 ? nullptr : (int32_t *)dev_alloc(ctx, sizeof(int32_t) * cap);
+                if (!m.a || !m.b || (d.ndim == 2 && !m.id))
+                    return fail(ctx, PIC_ENOMEM, "allocator returned NULL for particles");
             }
+            S.perm = (int *)dev_alloc(ctx, sizeof(int) * cap);
+            if (!S.perm) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort");
             S.counts = (int *)dev_alloc(ctx, sizeof(int) * (r.max_keys + 1));
             if (!S.counts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort counts");
-            CK(cudaMemsetAsync(S.counts, 0, sizeof(int) * (r.max_keys + 1), ctx->stream));
             S.tile_start = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             S.tile_start_alt = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             if (!S.tile_start || !S.tile_start_alt) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for tile offsets");
@@ -814,21 +813,6 @@ pic_status read_err(pic_ctx *ctx) {
 
 // ------------------------------------------------------------ stepping
 
-// Invariant: at a push, counts are zero unless counted.  Sorts leave them
-// zero, and every other change of the particles or of the tile geometry is
-// followed by a sort before the next push.  Counts left by an earlier
-// counting push whose sort never came (the sort interval grew in between) no
-// longer describe the particles, so they are cleared here.
-void prepare_counts(pic_ctx *ctx, Run &r) {
-    for (int q = 0; q < r.d.nspecies; ++q) {
-        SpeciesState &S = r.sp[q];
-        if (!S.counted) continue;
-        (void)cudaMemsetAsync(S.counts, 0, sizeof(int) * ((size_t)r.t.ntiles * r.t.cells_per_tile + 1),
-                              ctx->stream);   // a failure surfaces at the step's error check
-        S.counted = false;
-    }
-}
-
 // Particles a lane of the push walks, as log2.  Long walks add fewer register sums to
 // shared memory, short ones leave the warps of a CTA more equal shares and order the sort
 // more finely; with few particles the longest walk is the kernel's time.  Push per step,
@@ -875,9 +859,7 @@ SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S, int lgw) {
     a.t = r.t;
     a.n = S.n;
     a.src = S.mb[S.cur];
-    a.dst = S.mb[1 - S.cur];
     a.counts = S.counts;
-    a.counted = S.counted ? 1 : 0;
     a.lgw = lgw;
     a.lgw_src = S.lgw;
     a.offsets = r.offsets;
@@ -885,16 +867,17 @@ SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S, int lgw) {
     // the old-tile walk is valid only for the tile geometry the layout was sorted with
     a.old_tile_start = (S.tiled && S.tiled_ntiles == r.t.ntiles) ? S.tile_start : nullptr;
     a.tile_start = S.tile_start_alt;
-    a.perm = r.perm;
+    a.perm = S.perm;
     a.err = ctx->d_err;
     return a;
 }
 
-// Host bookkeeping after the sort of S was enqueued: the sorted copy becomes current.
+// Host bookkeeping after the sort of S was enqueued: the other buffer becomes current,
+// and the next push fills it.
 void sort_done(Run &r, SpeciesState &S, int lgw) {
-    S.counted = false;
     S.lgw = lgw;
     S.cur = 1 - S.cur;
+    S.moving = true;
     std::swap(S.tile_start, S.tile_start_alt);
     S.tiled = true;
     S.tiled_ntiles = r.t.ntiles;
@@ -908,6 +891,7 @@ void sort_species(pic_ctx *ctx, Run &r, SpeciesState &S) {
 
 HistRef hist_ref(Run &r) { return HistRef{r.hist, r.hist_idx, r.hist_cap}; }
 
+// Arguments of the push of this step (once per step: it takes over a sort's move).
 MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     typedef unsigned long long u64;
     MixedStepArgs a;
@@ -920,6 +904,10 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     for (int q = 0; q < r.d.nspecies; ++q) {
         SpeciesState &S = r.sp[q];
         a.sp[q] = S.mb[S.cur];
+        a.src[q] = S.mb[1 - S.cur];
+        a.perm[q] = S.moving ? S.perm : nullptr;
+        S.moving = false;
+        a.n[q] = (int)S.n;
         a.tile_start[q] = S.tile_start;
         a.lgw[q] = S.lgw;
         a.h[q] = (float)S.h;
@@ -933,7 +921,6 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     a.mode = 0;
     a.hist = hist_ref(r);
     a.err = ctx->d_err;
-    for (int q = 0; q < 4; ++q) a.key_counts[q] = nullptr;
     a.use_tma = r.tma ? 1 : 0;
     a.tmA = r.tmA;
     a.tmB = r.tmB;
@@ -965,13 +952,13 @@ FieldRunF field_run(Run &r) {
 size_t walk_tab_ints(int nr) { return (size_t)kWalkMaxPhases * nr + 1 + (size_t)nr * (kWalkMaxPhases + 2); }
 
 // Can the step walker run with this push shared memory (cached per context)?
-bool walk_ok(pic_ctx *ctx, int ndim, bool walls, bool count, size_t smem) {
+bool walk_ok(pic_ctx *ctx, int ndim, bool walls, bool move, size_t smem) {
     if (smem != ctx->walk_fit_smem) {
         ctx->walk_fit[0][0] = ctx->walk_fit[0][1] = ctx->walk_fit[1][0] = ctx->walk_fit[1][1] = -1;
         ctx->walk_fit_smem = smem;
     }
-    int &f = ctx->walk_fit[walls ? 1 : 0][count ? 1 : 0];
-    if (f < 0) f = walk_fits(ndim, walls, count, smem) ? 1 : 0;
+    int &f = ctx->walk_fit[walls ? 1 : 0][move ? 1 : 0];
+    if (f < 0) f = walk_fits(ndim, walls, move, smem) ? 1 : 0;
     return f == 1;
 }
 
@@ -1008,22 +995,16 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
             maxsp = std::max(maxsp, r.d.nspecies);
         }
     }
-    // when the next step sorts every run, this step's push counts their key histograms
-    bool count = true;
-    for (int i = 0; i < nr; ++i) {
-        const Run &r = ctx->runs[i];
-        const int since = is_due[i] ? 0 : r.since_sort;
-        if (!(since + 1 >= r.sort_interval && r.t.lg[0] >= 0)) count = false;
-    }
+    const bool move = !due.empty();
     const float dt = (float)ctx->runs[0].d.dt;
     int max_smooth = 0;
     for (auto &r : ctx->runs) max_smooth = std::max(max_smooth, r.smooth);
     const int ndim = ctx->runs[0].d.ndim;
     const bool walls = ctx->runs[0].g.bcx == 1;
     const size_t push_smem = mixed_smem_bytes(ctx->runs[0].t, ndim);
-    const int nphase = (due.empty() ? 0 : 8 * maxsp) + 4 + (max_smooth > 0 ? 1 + max_smooth : 0);
+    const int nphase = (due.empty() ? 0 : 6 * maxsp) + 4 + (max_smooth > 0 ? 1 + max_smooth : 0);
     const bool walk = !(ctx->flags & (PIC_FLAG_PHASE_LAUNCHES | PIC_FLAG_TIMING)) && nphase <= kWalkMaxPhases &&
-                      walk_ok(ctx, ndim, walls, count, push_smem);
+                      walk_ok(ctx, ndim, walls, move, push_smem);
     const int lgw = push_walk_lg(ctx);
     // The walker sorts too unless one run holds more than a quarter of the particles: that run's
     // sort alone then sets the time, and its own launches per phase (more warps per SM for the
@@ -1060,15 +1041,15 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
             CK(cudaMemcpyAsync(ctx->sort_args_dev, host_src(ctx, slot, soff, ctx->h_sort.data(), sizeof(SortArgs) * ns),
                                sizeof(SortArgs) * ns, cudaMemcpyHostToDevice, s));
             CK(cudaMemcpyAsync(ctx->sort_prefix_dev,
-                               host_src(ctx, slot, soff, ctx->h_sort_prefix.data(), sizeof(int) * 4 * (ns + 1)),
-                               sizeof(int) * 4 * (ns + 1), cudaMemcpyHostToDevice, s));
+                               host_src(ctx, slot, soff, ctx->h_sort_prefix.data(), sizeof(int) * 3 * (ns + 1)),
+                               sizeof(int) * 3 * (ns + 1), cudaMemcpyHostToDevice, s));
             launch_sort_multi(ctx->sort_args_dev, ctx->sort_prefix_dev, ctx->h_sort_prefix.data(), ns,
                               ctx->runs[0].d.ndim, s);
             for (int i : due) {
                 Run &r = ctx->runs[i];
                 if (q < r.d.nspecies) sort_done(r, r.sp[q], lgw);
             }
-            launches += 8;
+            launches += 6;
         }
         for (int i : due) {
             ctx->runs[i].sorted = true;
@@ -1082,12 +1063,9 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         CK(cudaStreamSynchronize(s));
         ctx->multi_tiles_dirty = false;
     }
-    for (auto &r : ctx->runs) prepare_counts(ctx, r);
     for (int i = 0; i < nr; ++i) {
         Run &r = ctx->runs[i];
         ctx->h_args[i] = mixed_args(ctx, r);
-        if (count)
-            for (int q = 0; q < r.d.nspecies; ++q) ctx->h_args[i].key_counts[q] = r.sp[q].counts;
         ctx->h_fp[i] = field_run(r);
     }
     CK(cudaMemcpyAsync(ctx->multi_args, host_src(ctx, slot, soff, ctx->h_args.data(), sizeof(MixedStepArgs) * nr),
@@ -1100,7 +1078,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         int np = 0;
         if (!due.empty() && walk_sort)
             for (int q = 0; q < maxsp; ++q)
-                for (int k = S_ZERO; k <= S_GATHER; ++k) {
+                for (int k = S_ZERO; k <= S_RANK; ++k) {
                     w.species[np] = q;
                     w.kind[np++] = k;
                 }
@@ -1120,7 +1098,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         auto items = [&](int ph, int i) -> int {
             const Run &r = ctx->runs[i];
             const long long ncell = (long long)r.g.nx * r.g.ny * r.g.nz;
-            if (w.kind[ph] <= S_GATHER)
+            if (w.kind[ph] <= S_RANK)
                 return (is_due[i] && w.species[ph] < r.d.nspecies)
                            ? walk_sort_items(ctx->h_walk_sort[4 * i + w.species[ph]], w.kind[ph], cpi) : 0;
             switch (w.kind[ph]) {
@@ -1178,11 +1156,8 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         w.h = 0.5f * dt;
         w.dt = dt;
         w.wait_ns = (ctx->flags & PIC_FLAG_INJECT_STALL) ? 20000000LL : 2000000000LL;
-        launch_walk(w, ndim, walls, count, push_smem, fixed_tile_code(ctx->runs[0].t, ndim), s);
+        launch_walk(w, ndim, walls, move, push_smem, fixed_tile_code(ctx->runs[0].t, ndim), s);
         CK(cudaGetLastError());
-        if (count)
-            for (auto &r : ctx->runs)
-                for (int q = 0; q < r.d.nspecies; ++q) r.sp[q].counted = true;
         for (auto &r : ctx->runs) {
             r.since_sort++;
             r.jcur = 1 - r.jcur;
@@ -1202,10 +1177,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         KTimer t(ctx, PIC_KERNEL_PUSH);
         CK(cudaMemsetAsync(ctx->multi_counter, 0, sizeof(int), s));
         launch_push_mixed_multi(ctx->multi_args, ctx->multi_tiles, nr, ctx->runs[0].d.ndim, ctx->runs[0].t,
-                                ctx->runs[0].g.bcx == 1, count, ctx->multi_counter, s);
-        if (count)
-            for (auto &r : ctx->runs)
-                for (int q = 0; q < r.d.nspecies; ++q) r.sp[q].counted = true;
+                                ctx->runs[0].g.bcx == 1, move, ctx->multi_counter, s);
     }
     if (max_smooth > 0) {
         KTimer t(ctx, PIC_KERNEL_SMOOTH);
@@ -1293,7 +1265,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         if (!r.sorted || r.since_sort >= r.sort_interval) {
             KTimer t(ctx, PIC_KERNEL_SORT);
             for (int q = 0; q < nsp; ++q) {
-                launches += r.sp[q].counted ? 6 : 8;
+                launches += 5;
                 sort_species(ctx, r, r.sp[q]);
             }
             make_parts(ctx, r);
@@ -1312,13 +1284,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         {
             KTimer t(ctx, PIC_KERNEL_PUSH);
             MixedStepArgs a = mixed_args(ctx, r);
-            // when the next step sorts, this push counts its key histogram
-            const bool count = r.since_sort + 1 >= r.sort_interval && r.t.lg[0] >= 0;
-            prepare_counts(ctx, r);
-            for (int q = 0; q < nsp; ++q) a.key_counts[q] = count ? r.sp[q].counts : nullptr;
             launch_push_mixed(a, s);
-            if (count)
-                for (int q = 0; q < nsp; ++q) r.sp[q].counted = true;
         }
         u64 *Z[3] = {jplane<u64>(r, 1 - r.jcur, 0), jplane<u64>(r, 1 - r.jcur, 1), jplane<u64>(r, 1 - r.jcur, 2)};
         const u64 *Jc[3] = {J[0], J[1], J[2]};
@@ -1384,7 +1350,6 @@ std::vector<long long> graph_signature(const pic_ctx *ctx) {
         for (int q = 0; q < r.d.nspecies; ++q) {
             const SpeciesState &S = r.sp[q];
             v.push_back(S.cur);
-            v.push_back(S.counted);
             v.push_back(S.n);
             v.push_back((long long)(uintptr_t)S.tile_start);
             v.push_back((long long)(uintptr_t)S.tile_start_alt);
@@ -1418,7 +1383,7 @@ pic_status capture_graph(pic_ctx *ctx) {
         const size_t a = 256;
         auto up = [a](size_t b) { return (b + a - 1) & ~(a - 1); };
         const size_t stride = up(sizeof(MixedStepArgs) * nr) + up(sizeof(FieldRunF) * nr) +
-                              maxsp * (up(sizeof(SortArgs) * nr) + up(sizeof(int) * 4 * (nr + 1))) +
+                              maxsp * (up(sizeof(SortArgs) * nr) + up(sizeof(int) * 3 * (nr + 1))) +
                               up(sizeof(int) * walk_tab_ints(nr)) + up(sizeof(SortArgs) * 4 * nr);
         if (ctx->gstage_bytes < stride * P) {
             if (ctx->gstage) cudaFreeHost(ctx->gstage);
@@ -1532,9 +1497,9 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
         ctx->walk_sort_dev = (SortArgs *)dev_alloc(ctx, sizeof(SortArgs) * 4 * nruns);
         ctx->h_walk_sort.assign(4 * (size_t)nruns, SortArgs{});
         ctx->sort_args_dev = (SortArgs *)dev_alloc(ctx, sizeof(SortArgs) * nruns);
-        ctx->sort_prefix_dev = (int *)dev_alloc(ctx, sizeof(int) * 4 * (nruns + 1));
+        ctx->sort_prefix_dev = (int *)dev_alloc(ctx, sizeof(int) * 3 * (nruns + 1));
         ctx->h_sort.resize(nruns);
-        ctx->h_sort_prefix.resize(4 * (nruns + 1));
+        ctx->h_sort_prefix.resize(3 * (nruns + 1));
         if (!ctx->multi_args || !ctx->multi_fp || !ctx->multi_tiles || !ctx->multi_blocks ||
             !ctx->multi_counter || !ctx->sort_args_dev || !ctx->sort_prefix_dev || !ctx->walk_tab || !ctx->walk_ctl ||
             !ctx->walk_sort_dev) {
@@ -1648,6 +1613,7 @@ pic_status pic_set_state(pic_ctx *ctx, int run, const pic_state_view *in) {
         const int64_t n = in->count[s];
         S.n = n;
         S.sorted64 = false;
+        S.moving = false;
         const double *P = in->particles[s];
         if (ctx->precision == PIC_FP64) {
             for (int a = 0; a < 3; ++a) {
@@ -1660,7 +1626,6 @@ pic_status pic_set_state(pic_ctx *ctx, int run, const pic_state_view *in) {
         } else {
             S.cur = 0;
             S.tiled = false;
-            S.counted = false;
             if (const double *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n)) {
                 k_upload_mixed<<<nblk(n), 256, 0, sm>>>(g, Pm, n, n, 0, S.mb[0], ctx->d_err);
                 CK(cudaGetLastError());
@@ -1757,16 +1722,16 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
             // conversion and copy in turn on the context stream (a copy stream of
             // its own measured slower here than this serial form); the id -> storage
             // index map lets each chunk touch only its own particles
-            k_id_index<<<nblk(n), 256, 0, sm>>>(S.mb[S.cur].id, n, r.perm);
+            k_id_index_mixed<<<nblk(n), 256, 0, sm>>>(g.ndim, S.mb[S.cur], n, S.perm);
             if (double *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n)) {
-                k_download_by_id<<<nblk(n), 256, 0, sm>>>(g, S.mb[S.cur], r.perm, 0, n, Pm, n);
+                k_download_by_id<<<nblk(n), 256, 0, sm>>>(g, S.mb[S.cur], S.perm, 0, n, Pm, n);
                 CK(cudaGetLastError());
                 continue;
             }
             const int64_t chunk = (int64_t)(ctx->staging_bytes / (6 * sizeof(double)));
             for (int64_t a0 = 0; a0 < n; a0 += chunk) {
                 const int64_t m = std::min(chunk, n - a0);
-                k_download_by_id<<<nblk(m), 256, 0, sm>>>(g, S.mb[S.cur], r.perm, a0, m, stg, m);
+                k_download_by_id<<<nblk(m), 256, 0, sm>>>(g, S.mb[S.cur], S.perm, a0, m, stg, m);
                 CK(cudaGetLastError());
                 for (int a = 0; a < 6; ++a)
                     CK(cudaMemcpyAsync(P + a * n + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
@@ -1792,13 +1757,15 @@ pic_status pic_get_particles(pic_ctx *ctx, int run, int species, const int64_t *
     // chunk are copied behind them
     const int64_t chunk = (int64_t)(ctx->staging_bytes / (7 * sizeof(double)));
     double *stg = (double *)ctx->staging;
-    if (S.n > 0 && (ctx->precision == PIC_MIXED || S.sorted64))
-        k_id_index<<<nblk(S.n), 256, 0, sm>>>(ctx->precision == PIC_MIXED ? S.mb[S.cur].id : S.id64, S.n, r.perm);
+    if (S.n > 0 && ctx->precision == PIC_MIXED)
+        k_id_index_mixed<<<nblk(S.n), 256, 0, sm>>>(r.d.ndim, S.mb[S.cur], S.n, S.perm);
+    else if (S.n > 0 && S.sorted64)
+        k_id_index<<<nblk(S.n), 256, 0, sm>>>(S.id64, S.n, r.perm);
     for (int64_t a0 = 0; a0 < nids; a0 += chunk) {
         const int64_t m = std::min(chunk, nids - a0);
         long long *dids = reinterpret_cast<long long *>(stg + 6 * m);
         CK(cudaMemcpyAsync(dids, ids + a0, sizeof(long long) * m, cudaMemcpyHostToDevice, sm));
-        if (ctx->precision == PIC_MIXED) k_pick_mixed<<<nblk(m), 256, 0, sm>>>(r.g, S.mb[S.cur], r.perm, dids, m, stg);
+        if (ctx->precision == PIC_MIXED) k_pick_mixed<<<nblk(m), 256, 0, sm>>>(r.g, S.mb[S.cur], S.perm, dids, m, stg);
         else k_pick64<<<nblk(m), 256, 0, sm>>>(S.s64, S.sorted64 ? r.perm : nullptr, dids, m, r.d.ndim, stg);
         CK(cudaGetLastError());
         for (int a = 0; a < 6; ++a)
@@ -1990,7 +1957,6 @@ void apply_tuning(pic_ctx *ctx, const int T[3], int K) {
             r.sorted = false;
             for (int q = 0; q < r.d.nspecies; ++q) {
                 r.sp[q].tiled = false;
-                r.sp[q].counted = false;
             }
         }
     }
@@ -2183,8 +2149,8 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
     CK(cudaGetLastError());
     S.n = n;
     S.tiled = false;
-    S.counted = false;
     S.sorted64 = false;
+    S.moving = false;
     r.sorted = false;
     r.since_sort = 0;
     // initial staggering of the momenta: one Boris step of -dt/2 (App. A.3.1)
@@ -2284,8 +2250,8 @@ pic_status mlp_load(pic_ctx *ctx, int run, int species, long long n, double thet
     CK(cudaGetLastError());
     S.n = n;
     S.tiled = false;
-    S.counted = false;
     S.sorted64 = false;
+    S.moving = false;
     r.sorted = false;
     r.since_sort = 0;
     if (mixed) {

@@ -101,14 +101,16 @@ __global__ void k_particle_diag64(Species64 sp, long long n, double *acc, unsign
     block_sum_atomic<6>(v, acc);
 }
 
-__global__ void k_particle_diag_mixed(SpeciesMixed sp, long long n, double *acc, unsigned long long *nonfinite) {
+__global__ void k_particle_diag_mixed(int ndim, SpeciesMixed sp, long long n, double *acc, unsigned long long *nonfinite) {
     double v[6] = {0, 0, 0, 0, 0, 0};
     unsigned long long bad = 0;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        const double ux = sp.u[0][p], uy = sp.u[1][p], uz = sp.u[2][p];
+        float off[3], u[3];
+        get_particle(ndim, sp, p, off, u);
+        const double ux = u[0], uy = u[1], uz = u[2];
         const double u2 = ux * ux + uy * uy + uz * uz;
         const double gam = sqrt(1.0 + u2);
-        if (!isfinite(u2) || !isfinite(sp.off[0][p]) || !isfinite(sp.off[1][p])) ++bad;
+        if (!isfinite(u2) || !isfinite(off[0]) || !isfinite(off[1])) ++bad;
         v[0] += u2 / (1.0 + gam);
         v[1] += ux; v[2] += uy; v[3] += uz;
         v[4] += u2 / gam;
@@ -154,8 +156,9 @@ template <int NDIM>
 __global__ void k_rho_mixed(Geom g, SpeciesMixed sp, long long n, double alpha, double *rho) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         int i, j, k;
-        unpack_cell(NDIM, sp.cell[p], i, j, k);
-        double d[3] = {sp.off[0][p], sp.off[1][p], NDIM == 3 ? sp.off[2][p] : 0.0};
+        float off[3], u[3];
+        unpack_cell(NDIM, get_particle(NDIM, sp, p, off, u), i, j, k);
+        const double d[3] = {off[0], off[1], off[2]};
         rho_one<NDIM>(g, i, j, k, d, alpha, rho);
     }
 }
@@ -201,9 +204,9 @@ void launch_particle_diag64(const Geom &g, Species64 sp, long long n, double m_o
 
 void launch_particle_diag_mixed(const Geom &g, SpeciesMixed sp, long long n, double m_over_me, double *acc,
                                 long long *nonfinite, cudaStream_t s) {
-    (void)g; (void)m_over_me;
+    (void)m_over_me;
     if (n > 0)
-        k_particle_diag_mixed<<<blocks_for(n), 256, 0, s>>>(sp, n, acc, reinterpret_cast<unsigned long long *>(nonfinite));
+        k_particle_diag_mixed<<<blocks_for(n), 256, 0, s>>>(g.ndim, sp, n, acc, reinterpret_cast<unsigned long long *>(nonfinite));
 }
 
 template <typename R>

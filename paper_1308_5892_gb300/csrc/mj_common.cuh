@@ -229,14 +229,14 @@ __global__ void __launch_bounds__(256) k_load_mj(LoadArgs a, Par par_of) {
             if (a.x64[1][p] >= a.g.ny) a.x64[1][p] = 0.0;
             if (a.ndim == 3 && a.x64[2][p] >= a.g.nz) a.x64[2][p] = 0.0;
         } else {
+            const float um[3] = {(float)mom[0], (float)mom[1], (float)mom[2]};
+            float of[3] = {0.f, 0.f, 0.f};
+            uint32_t cell;
             if (a.colocate) {
-                a.mx.cell[p] = a.cmx.cell[p];
-                a.mx.off[0][p] = a.cmx.off[0][p];
-                a.mx.off[1][p] = a.cmx.off[1][p];
-                if (a.ndim == 3) a.mx.off[2][p] = a.cmx.off[2][p];
+                float uc[3];
+                cell = get_particle(a.ndim, a.cmx, p, of, uc);
             } else {
                 int ci[3] = {0, 0, 0};
-                float of[3] = {0.f, 0.f, 0.f};
                 const int n3[3] = {a.g.nx, a.g.ny, a.g.nz};
                 for (int c = 0; c < a.ndim; ++c) {
                     const double f = floor(pos[c]);
@@ -249,15 +249,10 @@ __global__ void __launch_bounds__(256) k_load_mj(LoadArgs a, Par par_of) {
                     ci[c] = k;
                     of[c] = o;
                 }
-                a.mx.cell[p] = pack_cell(a.ndim, ci[0], ci[1], ci[2]);
-                a.mx.off[0][p] = of[0];
-                a.mx.off[1][p] = of[1];
-                if (a.ndim == 3) a.mx.off[2][p] = of[2];
+                cell = pack_cell(a.ndim, ci[0], ci[1], ci[2]);
             }
-            a.mx.u[0][p] = (float)mom[0];
-            a.mx.u[1][p] = (float)mom[1];
-            a.mx.u[2][p] = (float)mom[2];
-            a.mx.id[p] = (int32_t)p;
+            put_particle(a.ndim, a.mx, p, cell, of, um, __int_as_float((int)p));
+            if (a.ndim == 2) a.mx.id[p] = (int32_t)p;
         }
     }
 }

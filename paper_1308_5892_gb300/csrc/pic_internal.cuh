@@ -18,7 +18,7 @@
 //    current (push_fp64.cu).
 //  - particles, FP64 path: SoA planes x,y,z,u_x,u_y,u_z of double (absolute
 //    positions), sorted by cell every few steps (then with an int32 id); mixed path: packed cell coordinates (uint32), FP32 offsets
-//    (SoA), FP32 momenta (SoA) and an int32 id, kept sorted by tile.
+//    and momenta, and an int32 id (SpeciesMixed), kept sorted by tile.
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -145,12 +145,46 @@ struct Species64 {
     double *u[3];
 };
 
+// A mixed-path species, in words of 16 + 16 B per particle in 3D, a = {packed cell, off
+// x, y, z}, b = {u_x, u_y, u_z, id}, and 16 + 8 B in 2D, a = {packed cell, off x, y, u_x},
+// b = {u_y, u_z}, with the ids apart.  Wide words make a particle two loads and two
+// stores, and the scattered reads of a sort's move two (2D three) sectors instead of
+// eight.
 struct SpeciesMixed {
-    uint32_t *cell;
-    float *off[3];
-    float *u[3];
-    int32_t *id;
+    float4 *a;
+    float *b;
+    int32_t *id;    // 2D
 };
+__device__ __forceinline__ const uint32_t *cell_ptr(const SpeciesMixed &s, long long p) {
+    return reinterpret_cast<const uint32_t *>(s.a + p);
+}
+__device__ __forceinline__ int32_t get_id(int ndim, const SpeciesMixed &s, long long p) {
+    return ndim == 3 ? __float_as_int(reinterpret_cast<const float4 *>(s.b)[p].w) : s.id[p];
+}
+__device__ __forceinline__ uint32_t get_particle(int ndim, const SpeciesMixed &s, long long p, float off[3], float u[3]) {
+    const float4 a = s.a[p];
+    off[0] = a.y;
+    off[1] = a.z;
+    if (ndim == 3) {
+        const float4 b = reinterpret_cast<const float4 *>(s.b)[p];
+        off[2] = a.w; u[0] = b.x; u[1] = b.y; u[2] = b.z;
+    } else {
+        const float2 b = reinterpret_cast<const float2 *>(s.b)[p];
+        off[2] = 0.f; u[0] = a.w; u[1] = b.x; u[2] = b.y;
+    }
+    return __float_as_uint(a.x);
+}
+// id: bits of the id (3D; the 2D ids are stored apart)
+__device__ __forceinline__ void put_particle(int ndim, const SpeciesMixed &s, long long p, uint32_t cell,
+                                             const float off[3], const float u[3], float id) {
+    if (ndim == 3) {
+        s.a[p] = make_float4(__uint_as_float(cell), off[0], off[1], off[2]);
+        reinterpret_cast<float4 *>(s.b)[p] = make_float4(u[0], u[1], u[2], id);
+    } else {
+        s.a[p] = make_float4(__uint_as_float(cell), off[0], off[1], u[0]);
+        reinterpret_cast<float2 *>(s.b)[p] = make_float2(u[1], u[2]);
+    }
+}
 
 struct TileGeom {
     int T[3];        // tile extent in cells (T[2] = 1 in 2D)
@@ -279,6 +313,11 @@ struct MixedStepArgs {
     unsigned long long *J[3];       // padded int64 fixed-point current planes (units 2^-36 of sgn(q) flux)
     int nspecies;
     SpeciesMixed sp[4];
+    // on the step of a sort: the source slot of every slot of the new layout; the push
+    // reads particle perm[p] of src and writes it to slot p of sp (null: in place)
+    const int *perm[4];
+    SpeciesMixed src[4];
+    int n[4];                       // particles
     const int *tile_start[4];       // per species: ntiles+1 offsets into the particle arrays
     int lgw[4];                     // log2 of the particles a lane walks in a block of the layout
     const int2 *parts;              // work list of the push (k_push_parts), null: one CTA per tile
@@ -291,9 +330,6 @@ struct MixedStepArgs {
     int mode;                       // 0 step, 1 half step back (momenta only)
     HistRef hist;                   // slot[0..1]: kinetic energy of u^{t-1/2} and u^{t+1/2}
     int *err;
-    // when non-null: per species, the push adds to key_counts[s][key] the number of
-    // particles whose new cell has that sort key (the next sort's histogram)
-    int *key_counts[4];
     // TMA descriptors of the node-field arrays nfA (4 floats per node) and nfB
     // (2 floats per node) with a box of one tile + halo; use_tma = 0 when the
     // geometry breaks a TMA alignment rule (odd tile width or odd padded x extent)
@@ -302,9 +338,9 @@ struct MixedStepArgs {
 };
 void launch_push_mixed(const MixedStepArgs &a, cudaStream_t s);
 // persistent launch over the tiles of many runs (same ndim and tile shape)
-// count: every run's args carry key_counts (the next sort's histogram)
+// move: some run's particles move to a new layout (perm)
 void launch_push_mixed_multi(const MixedStepArgs *runs_dev, const int *tile_prefix_dev, int nruns, int ndim,
-                             const TileGeom &t, bool walls, bool count, int *counter, cudaStream_t s);
+                             const TileGeom &t, bool walls, bool move, int *counter, cudaStream_t s);
 
 // fields.cu, batched over runs: one launch updates every run's grid
 struct FieldRunF {
@@ -337,7 +373,7 @@ size_t mixed_smem_bytes(const TileGeom &t, int ndim);
 struct SortArgs;
 enum WalkPhase {
     // the counting sort of one species (steps that sort)
-    S_ZERO = 0, S_HIST, S_SCAN_BLOCKS, S_SCAN_SUMS, S_SCAN_FINISH, S_RANK, S_ZERO_AFTER, S_GATHER,
+    S_ZERO = 0, S_HIST, S_SCAN_BLOCKS, S_SCAN_SUMS, S_SCAN_FINISH, S_RANK,
     // the main loop
     W_B, W_NODE, W_PUSH, W_SMOOTH_FOLD, W_SMOOTH_PASS, W_E_FX
 };
@@ -365,9 +401,9 @@ int walk_cells_per_item(int ndim);
 // Items of sort phase `kind` of one species' sort in the walker.
 int walk_sort_items(const SortArgs &a, int kind, int cells_per_item);
 // Can the walker run a step with this push shared memory on this device?
-bool walk_fits(int ndim, bool walls, bool count, size_t push_smem);
+bool walk_fits(int ndim, bool walls, bool move, size_t push_smem);
 // tile_code: fixed_tile_code of the runs' (common) tile geometry
-void launch_walk(const WalkArgs &w, int ndim, bool walls, bool count, size_t push_smem, int tile_code,
+void launch_walk(const WalkArgs &w, int ndim, bool walls, bool move, size_t push_smem, int tile_code,
                  cudaStream_t s);
 // dynamic shared memory a push CTA may use (227 KB per block, less the kernels' static shared memory)
 constexpr size_t kMaxPushSmem = 224 * 1024;
@@ -377,7 +413,7 @@ struct SortArgs {
     Geom g;
     TileGeom t;
     long long n;
-    SpeciesMixed src, dst;
+    SpeciesMixed src;
     int *counts;     // ntiles*cells_per_tile + 1 scratch
     int *offsets;    // same size: exclusive scan; offsets[key] start of key
     int *block_sums; // scratch for the scan
@@ -385,7 +421,6 @@ struct SortArgs {
     const int *old_tile_start;  // tile offsets of the source layout, or nullptr if untiled
     int *perm;       // n scratch: source index of every destination slot
     int *err;
-    int counted;     // counts already hold the key histogram of src (counted by the push)
     int lgw, lgw_src;   // log2 of the walk length of the destination and of the source layout
 };
 void launch_sort(const SortArgs &a, cudaStream_t s);
@@ -399,7 +434,7 @@ struct PushParts {
     int *count;
 };
 void launch_push_parts(const PushParts &a, cudaStream_t s);
-// many independent sorts in one launch per phase: h_prefix (4 x (nsort + 1) ints)
+// many independent sorts in one launch per phase: h_prefix (3 x (nsort + 1) ints)
 // is filled by sort_multi_prefixes from the host copy of the arguments and
 // uploaded to d_prefix next to d_args
 void sort_multi_prefixes(const SortArgs *h_args, int nsort, int *h_prefix);

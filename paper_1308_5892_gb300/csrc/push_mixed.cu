@@ -12,7 +12,7 @@ namespace {
 // One CTA per tile, or per entry of the work list, of one run; WALLS: conducting walls in x (a separate
 // instantiation keeps their register cost out of the periodic kernel); CT: the
 // fixed tile geometry code (fixed_tile), 0 for the run-time geometry.
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST, int CT>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE, int CT>
 __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed(const __grid_constant__ MixedStepArgs a) {
     int tile = blockIdx.x, part = 0, parts = 1;
     if (a.parts) {
@@ -22,14 +22,14 @@ __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed(const __grid_const
         part = e.y & 0xffff;
         parts = e.y >> 16;
     }
-    push_tile<NDIM, THREADS, WALLS, HIST, CT>(a, tile, part, parts, &a);
+    push_tile<NDIM, THREADS, WALLS, MOVE, CT>(a, tile, part, parts, &a);
 }
 
 // Persistent form for a batch of independent runs of uneven size: resident
 // CTAs take (run, tile) work items from one counter until all tiles of all
 // runs are done, so small runs do not leave most of the GPU idle.
 // tile_prefix[r] is the number of tiles of runs 0..r-1.
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST, int CT>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE, int CT>
 __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed_multi(const MixedStepArgs *runs, const int *tile_prefix,
                                                                     int nruns, int *counter) {
     __shared__ int item_sh;
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_push_mixed_multi(const MixedS
         int *dst = reinterpret_cast<int *>(&args_sh);
         for (int q = threadIdx.x; q < (int)(sizeof(MixedStepArgs) / sizeof(int)); q += THREADS) dst[q] = src[q];
         __syncthreads();
-        push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, item - tile_prefix[lo], 0, 1, runs + lo);
+        push_tile<NDIM, THREADS, WALLS, MOVE, CT>(args_sh, item - tile_prefix[lo], 0, 1, runs + lo);
     }
 }
 
@@ -60,41 +60,41 @@ __global__ void k_half_back_mixed(Geom g, const float4 *nfA, const float2 *nfB, 
                                   float h, float dt) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         int ci, cj, ck;
-        unpack_cell(NDIM, P.cell[p], ci, cj, ck);
-        const float d[3] = {P.off[0][p], P.off[1][p], NDIM == 3 ? P.off[2][p] : 0.f};
-        float u[3] = {P.u[0][p], P.u[1][p], P.u[2][p]};
+        float d[3], u[3];
+        const uint32_t c = get_particle(NDIM, P, p, d, u);
+        unpack_cell(NDIM, c, ci, cj, ck);
         float E[3], B[3];
         gather_global<NDIM>(g, nfA, nfB, ci, cj, ck, d, E, B);
         boris<float>(u, E, B, h, -0.5f * dt);
-        P.u[0][p] = u[0]; P.u[1][p] = u[1]; P.u[2][p] = u[2];
+        put_particle(NDIM, P, p, c, d, u, __int_as_float(get_id(NDIM, P, p)));
     }
 }
 
 // The kernel instance for a tile geometry code: the fixed form where one exists
 // for NDIM (periodic runs), else the run-time one.
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 auto push_kernel(int ct) {
-    auto k = k_push_mixed<NDIM, THREADS, MINB, WALLS, HIST, 0>;
+    auto k = k_push_mixed<NDIM, THREADS, MINB, WALLS, MOVE, 0>;
     if constexpr (!WALLS && NDIM == 3) {
-        if (ct == 1) k = k_push_mixed<NDIM, THREADS, MINB, WALLS, HIST, 1>;
+        if (ct == 1) k = k_push_mixed<NDIM, THREADS, MINB, WALLS, MOVE, 1>;
     } else if constexpr (!WALLS) {
-        if (ct == 2) k = k_push_mixed<NDIM, THREADS, MINB, WALLS, HIST, 2>;
+        if (ct == 2) k = k_push_mixed<NDIM, THREADS, MINB, WALLS, MOVE, 2>;
     }
     return k;
 }
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 auto push_multi_kernel(int ct) {
-    auto k = k_push_mixed_multi<NDIM, THREADS, MINB, WALLS, HIST, 0>;
+    auto k = k_push_mixed_multi<NDIM, THREADS, MINB, WALLS, MOVE, 0>;
     // (the 3D fixed form spills a few registers in this kernel: the run-time one is kept)
     if constexpr (!WALLS && NDIM == 2) {
-        if (ct == 2) k = k_push_mixed_multi<NDIM, THREADS, MINB, WALLS, HIST, 2>;
+        if (ct == 2) k = k_push_mixed_multi<NDIM, THREADS, MINB, WALLS, MOVE, 2>;
     }
     return k;
 }
 
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 void launch_t(const MixedStepArgs &a, size_t smem, cudaStream_t s) {
-    auto k = push_kernel<NDIM, THREADS, MINB, WALLS, HIST>(fixed_tile_code(a.t, NDIM));
+    auto k = push_kernel<NDIM, THREADS, MINB, WALLS, MOVE>(fixed_tile_code(a.t, NDIM));
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (a.parts_bound > 0) k<<<a.parts_bound, THREADS, smem, s>>>(a);
 }
@@ -116,10 +116,10 @@ void launch_half_back_mixed(const Geom &g, const float4 *nfA, const float2 *nfB,
     else k_half_back_mixed<2><<<blocks, 256, 0, s>>>(g, nfA, nfB, sp, n, h, dt);
 }
 
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 void launch_multi_t(const MixedStepArgs *runs, const int *tile_prefix, int nruns, int *counter, size_t smem, int ct,
                     cudaStream_t s) {
-    auto k = push_multi_kernel<NDIM, THREADS, MINB, WALLS, HIST>(ct);
+    auto k = push_multi_kernel<NDIM, THREADS, MINB, WALLS, MOVE>(ct);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem);
@@ -131,32 +131,34 @@ void launch_multi_t(const MixedStepArgs *runs, const int *tile_prefix, int nruns
 
 template <int NDIM, int THREADS, int MINB>
 void launch_multi_dim(const MixedStepArgs *runs, const int *tile_prefix, int nruns, int *counter, size_t smem,
-                      bool walls, bool count, int ct, cudaStream_t s) {
+                      bool walls, bool move, int ct, cudaStream_t s) {
     if (walls) {
-        if (count) launch_multi_t<NDIM, THREADS, MINB, true, true>(runs, tile_prefix, nruns, counter, smem, ct, s);
+        if (move) launch_multi_t<NDIM, THREADS, MINB, true, true>(runs, tile_prefix, nruns, counter, smem, ct, s);
         else launch_multi_t<NDIM, THREADS, MINB, true, false>(runs, tile_prefix, nruns, counter, smem, ct, s);
     } else {
-        if (count) launch_multi_t<NDIM, THREADS, MINB, false, true>(runs, tile_prefix, nruns, counter, smem, ct, s);
+        if (move) launch_multi_t<NDIM, THREADS, MINB, false, true>(runs, tile_prefix, nruns, counter, smem, ct, s);
         else launch_multi_t<NDIM, THREADS, MINB, false, false>(runs, tile_prefix, nruns, counter, smem, ct, s);
     }
 }
 
 void launch_push_mixed_multi(const MixedStepArgs *runs_dev, const int *tile_prefix_dev, int nruns, int ndim,
-                             const TileGeom &t, bool walls, bool count, int *counter, cudaStream_t s) {
+                             const TileGeom &t, bool walls, bool move, int *counter, cudaStream_t s) {
     const size_t smem = mixed_smem_bytes(t, ndim);
     const int ct = fixed_tile_code(t, ndim);
-    if (ndim == 3) launch_multi_dim<3, 512, 1>(runs_dev, tile_prefix_dev, nruns, counter, smem, walls, count, ct, s);
-    else launch_multi_dim<2, 256, 2>(runs_dev, tile_prefix_dev, nruns, counter, smem, walls, count, ct, s);
+    if (ndim == 3) launch_multi_dim<3, 512, 1>(runs_dev, tile_prefix_dev, nruns, counter, smem, walls, move, ct, s);
+    else launch_multi_dim<2, 256, 2>(runs_dev, tile_prefix_dev, nruns, counter, smem, walls, move, ct, s);
 }
 
 template <int NDIM, int THREADS, int MINB>
 void launch_dim(const MixedStepArgs &a, size_t smem, cudaStream_t s) {
-    const bool walls = a.g.bcx == 1, count = a.key_counts[0] != nullptr;
+    const bool walls = a.g.bcx == 1;
+    bool move = false;
+    for (int q = 0; q < a.nspecies; ++q) move = move || a.perm[q];
     if (walls) {
-        if (count) launch_t<NDIM, THREADS, MINB, true, true>(a, smem, s);
+        if (move) launch_t<NDIM, THREADS, MINB, true, true>(a, smem, s);
         else launch_t<NDIM, THREADS, MINB, true, false>(a, smem, s);
     } else {
-        if (count) launch_t<NDIM, THREADS, MINB, false, true>(a, smem, s);
+        if (move) launch_t<NDIM, THREADS, MINB, false, true>(a, smem, s);
         else launch_t<NDIM, THREADS, MINB, false, false>(a, smem, s);
     }
 }

@@ -32,7 +32,10 @@
 //  - particles (packed cell, FP32 offsets, FP32 momenta) are streamed once:
 //    read 24 B (2D) / 28 B (3D) and written back.  Each warp prefetches the
 //    particles of its next iterations with cp.async into a ring of
-//    shared-memory stages, so the DRAM latency overlaps the arithmetic.
+//    shared-memory stages, so the DRAM latency overlaps the arithmetic.  On the
+//    step of a sort the prefetch reads through the sort's permutation from the old
+//    layout and the push writes the new one: the sort needs no pass of its own over
+//    the particles (2 x 67M on 128^3: 3.1 ms a sort).
 // Work of a warp: blocks of 32 W particles (W = 32; less for few particles, see
 // push_walk_lg), which the sort stores transposed, so lane a walks W consecutive
 // cell-sorted particles (and keeps
@@ -44,7 +47,6 @@
 // last sort), or that a conducting wall reflects, takes a slow path that
 // gathers from global memory and deposits with global int64 atomics of the
 // same fixed-point values, so the result never depends on the sort interval.
-// On the step before a sort the kernel also counts the sort's key histogram.
 //
 // Roofline: HBM bound at 2 x 24 B (2D) or 2 x 28 B (3D) per particle-step;
 // field and current traffic per cell is amortised over the particles per cell.
@@ -247,9 +249,17 @@ struct SmemSinkFx {
     }
 };
 
-// cp.async of one 4-byte word, global -> shared, and its group fences.
-__device__ __forceinline__ void cp_async4(uint32_t saddr, const void *gptr) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(saddr), "l"(__cvta_generic_to_global(gptr))
+// cp.async of N bytes, global -> shared, and its group fences.  16 bytes go past L1
+// (.cg): beside the push's shared memory L1 has lines for about 200 misses in flight,
+// which held the scattered reads of a move to a quarter of a word per clock and SM
+// (128^3: 12.4 ms for the push of the move, in words of 16 + 8 + 4 + 4 B through L1).
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void *gptr) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr), "l"(__cvta_generic_to_global(gptr))
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async(uint32_t saddr, const void *gptr) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(saddr), "l"(__cvta_generic_to_global(gptr)), "n"(N)
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
@@ -297,13 +307,13 @@ __device__ __forceinline__ void tma_load(int ndim, uint32_t dst, const CUtensorM
 
 constexpr int kQueue = 64;      // per-warp ring of waiting pieces (at most 63 wait at any time)
 constexpr int kRoundItems = 64; // work items per round of a tile (at most 64 x 1024 particles)
-constexpr int kStages = 3;      // per-warp particle prefetch ring
-// words of one particle in a stage: cell, NDIM offsets, 3 momenta
-template <int NDIM> __host__ __device__ constexpr int words_per_particle() { return NDIM + 4; }
+constexpr int kStages = 2;      // per-warp particle prefetch ring (an iteration lasts several DRAM latencies)
+// words of one particle in a stage: 32 a, then 32 b
+template <int NDIM> __host__ __device__ constexpr int words_per_particle() { return NDIM == 3 ? 8 : 6; }
 
 // Shared memory of one warp after the node fields and the current limbs: the
 // piece queue (cell base, d[3], D[3]: 7 x kQueue words) and the particle
-// stages (kStages x words_per_particle x 32 words, word-major).
+// stages (kStages x words_per_particle x 32 words; 16-byte aligned).
 template <int NDIM>
 __host__ __device__ constexpr int warp_smem_words() { return 7 * kQueue + kStages * words_per_particle<NDIM>() * 32; }
 
@@ -413,8 +423,9 @@ __host__ __device__ inline size_t node_b_offset(int nodes) { return ((size_t)nod
 // tile add their currents to the same global sums, exactly).
 // tmaps: the arguments' copy whose TMA descriptors are in parameter or global
 // memory (the multi-run kernel stages its arguments in shared memory).
+// MOVE: a species may have a permutation (the step of a sort).
 // CT: fixed tile geometry code (fixed_tile), 0 for the run-time geometry.
-template <int NDIM, int THREADS, bool WALLS, bool HIST, int CT = 0>
+template <int NDIM, int THREADS, bool WALLS, bool MOVE, int CT = 0>
 __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile, const int part,
                                           const int parts, const MixedStepArgs *tmaps) {
     extern __shared__ __align__(128) float4 smem4[];
@@ -502,8 +513,8 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     int *q_base = wsm;
     float *q_d = reinterpret_cast<float *>(wsm + kQueue);        // [3][kQueue]
     float *q_D = q_d + 3 * kQueue;                               // [3][kQueue]
-    const uint32_t *stage = reinterpret_cast<const uint32_t *>(wsm + 7 * kQueue);   // [kStages][NW][32]
-    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage) + 4u * lane;
+    const uint32_t *stage = reinterpret_cast<const uint32_t *>(wsm + 7 * kQueue);   // [kStages][NW * 32]
+    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(stage);
     __syncthreads();
     if (a.use_tma && !mbar_wait_bounded(bar, 0, 1 << 22)) {
         // the copy did not land in time: flag it, give it a second bounded wait, go on
@@ -536,18 +547,34 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
         const int lgb = 5 + a.lgw[sp];                   // log2 of a block: 2^lgw particles per lane
         int nblk, ibeg, nitems;
         item_range(sp, nblk, ibeg, nitems);
-        // prefetch the particle of iteration j of an item into stage j % kStages (one group per iteration)
-        auto issue = [&](int base, int j, int kn) {
+        const int *const perm = MOVE ? a.perm[sp] : nullptr;
+        const SpeciesMixed &Q = perm ? a.src[sp] : a.sp[sp];   // where the particles are read
+        // source of the particle of iteration j of an item, -1 past its end
+        auto source = [&](int base, int j, int kn) -> int {
             const int p = base + (j << 5) + lane;
-            if (j < kn && p < pend) {
-                const uint32_t sa = stage_s + (uint32_t)((j % kStages) * NW * 128);
-                cp_async4(sa, P.cell + p);
-                cp_async4(sa + 128, P.off[0] + p);
-                cp_async4(sa + 256, P.off[1] + p);
-                if (NDIM == 3) cp_async4(sa + 384, P.off[2] + p);
-                cp_async4(sa + (NDIM + 1) * 128, P.u[0] + p);
-                cp_async4(sa + (NDIM + 2) * 128, P.u[1] + p);
-                cp_async4(sa + (NDIM + 3) * 128, P.u[2] + p);
+            if (j >= kn || p >= pend) return -1;
+            if (!perm) return p;
+            const int q = ldro(perm + p);
+            return (unsigned)q < (unsigned)a.n[sp] ? q : 0;   // (out of range only after a key that the sort has flagged)
+        };
+        // prefetch it into stage j % kStages (one group per iteration).  On a move, the 2D words below
+        // 16 bytes go through registers past L1: b is used, and the id stored, an iteration later.
+        int id = 0, id_slot = -1;
+        float2 wb_next = make_float2(0.f, 0.f);
+        auto issue = [&](int base, int j, int q) {
+            if (NDIM == 2 && MOVE && perm) {
+                if (id_slot >= 0) P.id[id_slot] = id;
+                id_slot = -1;
+            }
+            if (q >= 0) {
+                const uint32_t st = stage_s + (uint32_t)((j % kStages) * NW * 128) + 16u * lane;
+                cp_async16(st, Q.a + q);
+                if (NDIM == 3) cp_async16(st + 512u, reinterpret_cast<const float4 *>(Q.b) + q);
+                else if (MOVE && perm) {
+                    wb_next = __ldcg(reinterpret_cast<const float2 *>(Q.b) + q);
+                    id = __ldcg(Q.id + q);
+                    id_slot = base + (j << 5) + lane;
+                } else cp_async<8>(st + 512u - 8u * lane, reinterpret_cast<const float2 *>(Q.b) + q);
             }
             cp_async_commit();
         };
@@ -590,44 +617,35 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             const int base = item < nblk ? pbeg + (item << lgb) : pbeg + (nblk << lgb) + ((item - nblk) << 5);
             const int kn = item < nblk ? 1 << (lgb - 5) : 1;
             float kin0 = 0.f, kin1 = 0.f;
-            int hk = -1, hn = 0;   // HIST: sort key of the lane's current run of particles, and its length
 #pragma unroll
-            for (int j = 0; j < kStages - 1; ++j) issue(base, j, kn);
+            for (int j = 0; j < kStages - 1; ++j) issue(base, j, source(base, j, kn));
+            int next = source(base, kStages - 1, kn);   // a permutation entry is read one iteration ahead of its use
 #pragma unroll 1
             for (int k = 0; k < kn; ++k) {
-                issue(base, k + kStages - 1, kn);
+                const float2 wb_now = wb_next;
+                issue(base, k + kStages - 1, next);
+                next = source(base, k + kStages, kn);
                 cp_async_wait<kStages - 1>();   // this lane's words of iteration k have landed
                 const int p = base + (k << 5) + lane;
                 int nc = 0, q0 = 0;
                 PathSplit<NDIM, float> ps;
                 if (p < pend) {
-                    const uint32_t *st = stage + (k % kStages) * NW * 32 + lane;
-                    uint32_t c = st[0];
-                    float d[3] = {__uint_as_float(st[32]), __uint_as_float(st[64]),
-                                  NDIM == 3 ? __uint_as_float(st[96]) : 0.f};
-                    float u[3] = {__uint_as_float(st[(NDIM + 1) * 32]), __uint_as_float(st[(NDIM + 2) * 32]),
-                                  __uint_as_float(st[(NDIM + 3) * 32])};
+                    const uint32_t *st = stage + (k % kStages) * NW * 32;
+                    const float4 wa = reinterpret_cast<const float4 *>(st)[lane];
+                    uint32_t c = __float_as_uint(wa.x);
+                    float d[3] = {wa.y, wa.z, 0.f}, u[3], id_bits = 0.f;
+                    if (NDIM == 3) {
+                        const float4 wb = reinterpret_cast<const float4 *>(st + 128)[lane];
+                        d[2] = wa.w; u[0] = wb.x; u[1] = wb.y; u[2] = wb.z; id_bits = wb.w;
+                    } else {
+                        const float2 wb = (MOVE && perm) ? wb_now : reinterpret_cast<const float2 *>(st + 128)[lane];
+                        u[0] = wa.w; u[1] = wb.x; u[2] = wb.y;
+                    }
                     float d0[3], D[3];
                     int s[3], ci, cj, ck, side;
                     bool fast;
                     push_one<NDIM, WALLS>(a, tc, h, c, d, u, d0, s, D, fast, q0, ci, cj, ck, kin0, kin1, side);
-                    P.cell[p] = c;
-                    P.off[0][p] = d[0];
-                    P.off[1][p] = d[1];
-                    if (NDIM == 3) P.off[2][p] = d[2];
-                    P.u[0][p] = u[0]; P.u[1][p] = u[1]; P.u[2][p] = u[2];
-                    if (HIST) {
-                        // histogram of the next sort: consecutive particles of a lane mostly share a key
-                        int ki, kj, kk;
-                        unpack_cell(NDIM, c, ki, kj, kk);
-                        const int key = tile_key_pow2(a.t, ki, kj, kk);
-                        if (key != hk) {
-                            if (hn) atomicAdd(a.key_counts[sp] + hk, hn);
-                            hk = key;
-                            hn = 0;
-                        }
-                        ++hn;
-                    }
+                    put_particle(NDIM, P, p, c, d, u, id_bits);
                     if (fast) {
                         // the start-cell piece goes to the register accumulator
                         if (acc.q0 != q0) {
@@ -675,7 +693,6 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                     }
                 }
             }
-            if (HIST && hn) atomicAdd(a.key_counts[sp] + hk, hn);
             // kinetic energy of the item (at most 32 values per lane in FP32), summed per warp in FP64
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -688,6 +705,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             }
         }
         }   // rounds
+        if (NDIM == 2 && id_slot >= 0) P.id[id_slot] = id;
         drain_queue();
     }
     acc.flush(Jhi, Jlo, nodes, tc.sx, tc.sxy);

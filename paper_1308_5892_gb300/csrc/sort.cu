@@ -2,21 +2,16 @@
 //
 // key(cell) = tile_index * cells_per_tile + index of the cell inside its tile,
 // so particles end up grouped by tile and, inside a tile, by cell; the cell
-// order inside a tile is then stored block-transposed (interleaved_slot).  The sort
-// is out of place (src -> dst, the caller swaps the buffers): histogram of the
-// keys (unless the preceding push counted it), exclusive scan, a rank pass
-// whose per-key cursors are advanced with warp-aggregated atomics (lanes of a
-// warp that share a key take consecutive slots with one atomic) and which
-// writes only the 4-byte inverse permutation, then a gather pass that writes
-// every particle array in destination order (coalesced stores; scattered
-// partial-sector stores of the full particle state cost several times its size
-// in DRAM traffic).  The tile offsets are read from the scanned counts, and
-// the counts are left zeroed for the next push to count into.  Every phase also
+// order inside a tile is then stored block-transposed (interleaved_slot).  Histogram
+// of the keys, exclusive scan, and a rank pass
+// that writes the inverse permutation (4 bytes per particle); the push that follows
+// reads the particles through it and writes them to the other buffer, so the sort
+// moves no particle itself.  The tile offsets are read from the scanned counts.
+// Every phase also
 // has a batched form that sorts one species of many runs in one launch.
 //
-// Roofline: HBM bound; per particle 4 B (histogram) + 8 B (rank) +
-// 4 + 2 x (24..28 + 4) B (gather) plus per key 3 x 4 B.  Particle counts are
-// int32 (at most 2^31 - 1 particles per species).
+// Roofline: HBM bound; per particle 4 B (histogram) + 8 B (rank) plus per key
+// 3 x 4 B.  Particle counts are int32 (at most 2^31 - 1 particles per species).
 #include "pic_internal.cuh"
 #include "sort_cells.cuh"
 
@@ -34,11 +29,16 @@ inline int blocks_for(long long n, int threads) {
 constexpr int kWalkThreads = 512;
 inline int walk_blocks(const SortArgs &a) { return a.old_tile_start ? a.t.ntiles : blocks_for(a.n, kWalkThreads); }
 inline int key_blocks(const SortArgs &a) { return blocks_for(nkeys_of(a), 256); }
-inline int gather_blocks(const SortArgs &a) { return (int)((a.n + kGatherChunk - 1) / kGatherChunk); }
+// The box passes (sort_cells.cuh) take sorted sources whose tile box fits.
+inline bool boxed(const SortArgs &a) { return a.old_tile_start && box_fits(a.t, a.g.ndim); }
 
 // ---- one sort: one launch per phase ----
 
-__global__ void k_zero(SortArgs a) { zero_body(a.counts, nkeys_of(a), blockIdx.x, gridDim.x); }
+template <int NDIM, bool RANK>
+__global__ void __launch_bounds__(kWalkThreads, 3) k_box(const __grid_constant__ SortArgs a) {
+    __shared__ int box[box_max<NDIM>()];
+    box_body<NDIM, kWalkThreads, RANK>(a, blockIdx.x, 0, 1, box);
+}
 
 template <int NDIM>
 __global__ void k_histogram(SortArgs a) {
@@ -62,11 +62,6 @@ template <int NDIM>
 __global__ void k_rank(SortArgs a) {
     const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x, a.lgw_src};
     rank_body<NDIM, 4>(a, w, nkeys_of(a));
-}
-
-template <int NDIM>
-__global__ void __launch_bounds__(kGatherThreads) k_gather(SortArgs a) {
-    gather_body<NDIM, kGatherThreads, 4>(a.src, a.dst, a.n, a.perm, blockIdx.x);
 }
 
 // Work list of the push: every tile that holds particles, cut into parts of at most
@@ -121,19 +116,20 @@ __device__ inline int find_sort(const int *prefix, int nsort, int B) {
     return lo;
 }
 
-// always: zero the counts of every sort (after its rank pass); otherwise skip sorts counted by the push
-__global__ void k_zero_multi(const SortArgs *as, const int *prefix, int nsort, int always) {
+__global__ void k_zero_multi(const SortArgs *as, const int *prefix, int nsort) {
     const int s = find_sort(prefix, nsort, blockIdx.x);
-    const SortArgs &a = as[s];
-    if (a.counted && !always) return;
-    zero_body(a.counts, nkeys_of(a), blockIdx.x - prefix[s], prefix[s + 1] - prefix[s]);
+    zero_body(as[s].counts, nkeys_of(as[s]), blockIdx.x - prefix[s], prefix[s + 1] - prefix[s]);
 }
 
 template <int NDIM>
-__global__ void k_histogram_multi(const SortArgs *as, const int *prefix, int nsort) {
+__global__ void __launch_bounds__(kWalkThreads) k_histogram_multi(const SortArgs *as, const int *prefix, int nsort) {
     const int s = find_sort(prefix, nsort, blockIdx.x);
     const SortArgs &a = as[s];
-    if (a.counted) return;
+    if (a.old_tile_start && box_fits(a.t, NDIM)) {
+        __shared__ int box[box_max<NDIM>()];
+        box_body<NDIM, kWalkThreads, false>(a, blockIdx.x - prefix[s], 0, 1, box);
+        return;
+    }
     const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s], a.lgw_src};
     histogram_body<NDIM, 4>(a, w, nkeys_of(a));
 }
@@ -158,18 +154,16 @@ __global__ void k_scan_finish_multi(const SortArgs *as, const int *prefix, int n
 }
 
 template <int NDIM>
-__global__ void k_rank_multi(const SortArgs *as, const int *prefix, int nsort) {
+__global__ void __launch_bounds__(kWalkThreads) k_rank_multi(const SortArgs *as, const int *prefix, int nsort) {
     const int s = find_sort(prefix, nsort, blockIdx.x);
     const SortArgs &a = as[s];
+    if (a.old_tile_start && box_fits(a.t, NDIM)) {
+        __shared__ int box[box_max<NDIM>()];
+        box_body<NDIM, kWalkThreads, true>(a, blockIdx.x - prefix[s], 0, 1, box);
+        return;
+    }
     const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x - prefix[s], prefix[s + 1] - prefix[s], a.lgw_src};
     rank_body<NDIM, 4>(a, w, nkeys_of(a));
-}
-
-template <int NDIM>
-__global__ void __launch_bounds__(kGatherThreads) k_gather_multi(const SortArgs *as, const int *prefix, int nsort) {
-    const int s = find_sort(prefix, nsort, blockIdx.x);
-    const SortArgs &a = as[s];
-    gather_body<NDIM, kGatherThreads, 4>(a.src, a.dst, a.n, a.perm, blockIdx.x - prefix[s]);
 }
 
 }  // namespace
@@ -177,50 +171,41 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_multi(const SortArgs 
 size_t sort_scan_scratch(long long nkeys) { return (size_t)((nkeys + kScanTile - 1) / kScanTile + 1); }
 
 void launch_sort(const SortArgs &a, cudaStream_t s) {
-    if (!a.counted) k_zero<<<key_blocks(a), 256, 0, s>>>(a);
-    if (a.n > 0 && !a.counted) {
-        if (a.g.ndim == 3) k_histogram<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
+    cudaMemsetAsync(a.counts, 0, sizeof(int) * nkeys_of(a), s);
+    if (a.n > 0) {
+        if (boxed(a)) (a.g.ndim == 3 ? k_box<3, false> : k_box<2, false>)<<<a.t.ntiles, kWalkThreads, 0, s>>>(a);
+        else if (a.g.ndim == 3) k_histogram<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
         else k_histogram<2><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
     }
     k_scan_blocks<<<scan_blocks(a), kScanThreads, 0, s>>>(a);
     k_scan_sums<<<1, kScanThreads, 0, s>>>(a);
     k_scan_finish<<<key_blocks(a), 256, 0, s>>>(a);
     if (a.n > 0) {
-        if (a.g.ndim == 3) {
-            k_rank<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
-            k_gather<3><<<gather_blocks(a), kGatherThreads, 0, s>>>(a);
-        } else {
-            k_rank<2><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
-            k_gather<2><<<gather_blocks(a), kGatherThreads, 0, s>>>(a);
-        }
+        if (boxed(a)) (a.g.ndim == 3 ? k_box<3, true> : k_box<2, true>)<<<a.t.ntiles, kWalkThreads, 0, s>>>(a);
+        else if (a.g.ndim == 3) k_rank<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
+        else k_rank<2><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
     }
-    // the counts end zeroed, ready for a push that counts the next sort's histogram
-    k_zero<<<key_blocks(a), 256, 0, s>>>(a);
 }
 
 void launch_push_parts(const PushParts &a, cudaStream_t s) { k_push_parts<<<1, kScanThreads, 0, s>>>(a); }
 
 void sort_multi_prefixes(const SortArgs *h_args, int nsort, int *h_prefix) {
-    int *pz = h_prefix, *pw = h_prefix + (nsort + 1), *pb = h_prefix + 2 * (nsort + 1),
-        *pg = h_prefix + 3 * (nsort + 1);
-    pz[0] = pw[0] = pb[0] = pg[0] = 0;
+    int *pz = h_prefix, *pw = h_prefix + (nsort + 1), *pb = h_prefix + 2 * (nsort + 1);
+    pz[0] = pw[0] = pb[0] = 0;
     for (int i = 0; i < nsort; ++i) {
         const SortArgs &a = h_args[i];
         pz[i + 1] = pz[i] + key_blocks(a);
         pw[i + 1] = pw[i] + (a.n > 0 ? walk_blocks(a) : 0);
         pb[i + 1] = pb[i] + scan_blocks(a);
-        pg[i + 1] = pg[i] + gather_blocks(a);
     }
 }
 
 void launch_sort_multi(const SortArgs *d_args, const int *d_prefix, const int *h_prefix, int nsort, int ndim,
                        cudaStream_t s) {
     if (nsort <= 0) return;
-    const int *pz = d_prefix, *pw = d_prefix + (nsort + 1), *pb = d_prefix + 2 * (nsort + 1),
-              *pg = d_prefix + 3 * (nsort + 1);
-    const int nz = h_prefix[nsort], nw = h_prefix[2 * (nsort + 1) - 1], nb = h_prefix[3 * (nsort + 1) - 1],
-              ng = h_prefix[4 * (nsort + 1) - 1];
-    k_zero_multi<<<nz, 256, 0, s>>>(d_args, pz, nsort, 0);
+    const int *pz = d_prefix, *pw = d_prefix + (nsort + 1), *pb = d_prefix + 2 * (nsort + 1);
+    const int nz = h_prefix[nsort], nw = h_prefix[2 * (nsort + 1) - 1], nb = h_prefix[3 * (nsort + 1) - 1];
+    k_zero_multi<<<nz, 256, 0, s>>>(d_args, pz, nsort);
     if (nw > 0) {
         if (ndim == 3) k_histogram_multi<3><<<nw, kWalkThreads, 0, s>>>(d_args, pw, nsort);
         else k_histogram_multi<2><<<nw, kWalkThreads, 0, s>>>(d_args, pw, nsort);
@@ -231,12 +216,6 @@ void launch_sort_multi(const SortArgs *d_args, const int *d_prefix, const int *h
     if (nw > 0) {
         if (ndim == 3) k_rank_multi<3><<<nw, kWalkThreads, 0, s>>>(d_args, pw, nsort);
         else k_rank_multi<2><<<nw, kWalkThreads, 0, s>>>(d_args, pw, nsort);
-    }
-    // the counts end zeroed, ready for a push that counts the next sort's histogram
-    k_zero_multi<<<nz, 256, 0, s>>>(d_args, pz, nsort, 1);
-    if (ng > 0) {
-        if (ndim == 3) k_gather_multi<3><<<ng, kGatherThreads, 0, s>>>(d_args, pg, nsort);
-        else k_gather_multi<2><<<ng, kGatherThreads, 0, s>>>(d_args, pg, nsort);
     }
 }
 

@@ -1,5 +1,5 @@
 // sort_cells.cuh -- phase bodies of the counting sort of the mixed-path
-// particles (see sort.cu): key histogram, block scans, rank pass and gather,
+// particles (see sort.cu): key histogram, block scans and rank pass,
 // each written for block b of nb blocks of one sort.  Shared by the sort
 // kernels (sort.cu) and the persistent ensemble step (walk.cu).
 #pragma once
@@ -89,7 +89,7 @@ __device__ __forceinline__ void walk_keys(const SortArgs &a, const SrcWalk &w, l
     for (int v = 0; v < V; ++v) {
         const long long iv = i + v * w.step();
         p[v] = iv < end ? w.pos(iv, t0, nt) : -1;
-        c[v] = p[v] >= 0 ? ldro(a.src.cell + p[v]) : 0u;
+        c[v] = p[v] >= 0 ? ldro(cell_ptr(a.src, p[v])) : 0u;
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -100,6 +100,120 @@ __device__ __forceinline__ void walk_keys(const SortArgs &a, const SrcWalk &w, l
         }
     }
 }
+
+// ---- key passes over a tiled source ----
+//
+// A block of THREADS threads takes a share of one old tile.  Most of its particles
+// are still in the tile or within the halo H of it, a box of cells that fits shared
+// memory: they are counted there (a shared atomic that returns the particle's rank in
+// its cell), and one global atomic per occupied cell of the box then adds the count,
+// or reserves that many slots.  A particle beyond the box takes a global atomic of its
+// own.
+constexpr int kBoxRounds = 16;     // particles a thread holds per round, one register each
+constexpr int kBoxMax3 = 4096, kBoxMax2 = 2048;   // cells of a box the shared array holds
+template <int NDIM> __host__ __device__ constexpr int box_max() { return NDIM == 3 ? kBoxMax3 : kBoxMax2; }
+// Does the tile's box fit, so that the box passes can run?
+__host__ __device__ inline bool box_fits(const TileGeom &t, int ndim) {
+    return (long long)t.R[0] * t.R[1] * t.R[2] <= (ndim == 3 ? kBoxMax3 : kBoxMax2);
+}
+
+// The histogram (RANK false), or the rank pass (RANK true: the inverse permutation
+// perm[slot] = source index), of part `part` of `parts` of old tile `tile`.  box:
+// box_max ints of shared memory; all threads of the block take part.
+template <int NDIM, int THREADS, bool RANK>
+__device__ inline void box_body(const SortArgs &a, int tile, int part, int parts, int *box) {
+    const Geom &g = a.g;
+    const TileGeom &t = a.t;
+    const int t0 = ldro(a.old_tile_start + tile), nt = ldro(a.old_tile_start + tile + 1) - t0;
+    const int end = t0 + (int)((long long)nt * (part + 1) / parts);
+    const int tx = tile % t.ntile[0], tyz = tile / t.ntile[0];
+    const int x0 = tx * t.T[0] - t.H, y0 = (tyz % t.ntile[1]) * t.T[1] - t.H,
+              z0 = NDIM == 3 ? (tyz / t.ntile[1]) * t.T[2] - t.H : 0;
+    const int Rx = t.R[0], Ry = t.R[1], nb = Rx * Ry * (NDIM == 3 ? t.R[2] : 1);
+    const long long nkeys = (long long)t.ntiles * t.cells_per_tile;
+    // the new layout of the block's own tile, where most particles stay
+    const int own0 = RANK ? ldro(a.tile_start + tile) : 0, own1 = RANK ? ldro(a.tile_start + tile + 1) : 0;
+    auto place = [&](int r, int d0, int d1, int p) {
+        const long long dst = (long long)d0 + interleaved_slot(r - d0, d1 - d0, a.lgw);
+        if (r >= d0 && r < d1 && dst < a.n) a.perm[dst] = p;
+        else atomicOr(a.err, ERR_SORT);   // counts inconsistent with the particles
+    };
+    auto place_key = [&](int r, int key, int p) {
+        const int dt = key_tile(t, key);
+        place(r, ldro(a.tile_start + dt), ldro(a.tile_start + dt + 1), p);
+    };
+    for (int base = t0 + (int)((long long)nt * part / parts); base < end; base += kBoxRounds * THREADS) {
+        for (int q = threadIdx.x; q < nb; q += THREADS) box[q] = 0;
+        __syncthreads();
+        // rank in the cell << 17 | cell in the tile << 16 | box cell, -1 when there is nothing left to place
+        int held[kBoxRounds];
+#pragma unroll
+        for (int v0 = 0; v0 < kBoxRounds; v0 += 8) {
+            uint32_t c[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int p = base + (v0 + v) * THREADS + threadIdx.x;
+                c[v] = p < end ? ldro(cell_ptr(a.src, p)) : 0u;
+            }
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int p = base + (v0 + v) * THREADS + threadIdx.x;
+                held[v0 + v] = -1;
+                if (p >= end) continue;
+                // the cell, or its image, in the box
+                int i, j, k;
+                unpack_cell(NDIM, c[v], i, j, k);
+                i -= x0; j -= y0; k -= z0;
+                i += i < 0 ? g.nx : (i >= g.nx ? -g.nx : 0);
+                j += j < 0 ? g.ny : (j >= g.ny ? -g.ny : 0);
+                if (NDIM == 3) k += k < 0 ? g.nz : (k >= g.nz ? -g.nz : 0);
+                if ((unsigned)i < (unsigned)Rx && (unsigned)j < (unsigned)Ry && (NDIM == 2 || (unsigned)k < (unsigned)t.R[2])) {
+                    const int b = (NDIM == 3 ? k * Ry + j : j) * Rx + i;
+                    const int rank = atomicAdd(box + b, 1);
+                    if (RANK) {
+                        // (the last tile of an axis may stick out of the grid: those cells are others' images)
+                        const bool own = (unsigned)(i - t.H) < (unsigned)min(t.T[0], g.nx - x0 - t.H) &&
+                                         (unsigned)(j - t.H) < (unsigned)min(t.T[1], g.ny - y0 - t.H) &&
+                                         (NDIM == 2 || (unsigned)(k - t.H) < (unsigned)min(t.T[2], g.nz - z0 - t.H));
+                        held[v0 + v] = rank << 17 | (own ? 1 << 16 : 0) | b;
+                    }
+                } else {
+                    const int key = cell_key<NDIM>(t, c[v]);
+                    if (key < 0 || key >= nkeys) {
+                        atomicOr(a.err, ERR_SORT);
+                        continue;
+                    }
+                    const int r = atomicAdd(a.counts + key, 1);
+                    if (RANK) place_key(r, key, p);
+                }
+            }
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < nb; q += THREADS) {
+            const int n = box[q];
+            if (n > 0) {
+                const int i = q % Rx, r = q / Rx, k = NDIM == 3 ? r / Ry : 0, j = r - k * Ry;
+                const uint32_t c = pack_cell(NDIM, g.wx(x0 + i), g.wy(y0 + j), NDIM == 3 ? g.wz(z0 + k) : 0);
+                const int b = atomicAdd(a.counts + cell_key<NDIM>(t, c), n);
+                if (RANK) box[q] = b;
+            }
+        }
+        if (RANK) {
+            __syncthreads();
+#pragma unroll
+            for (int v = 0; v < kBoxRounds; ++v) {
+                if (held[v] < 0) continue;
+                const int p = base + v * THREADS + threadIdx.x;
+                const int r = box[held[v] & 0xffff] + (held[v] >> 17);
+                if (held[v] & (1 << 16)) place(r, own0, own1, p);
+                else place_key(r, cell_key<NDIM>(t, ldro(cell_ptr(a.src, p))), p);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---- key passes over any source ----
 
 // V elements per thread and iteration (independent loads in flight).
 template <int NDIM, int V>
@@ -243,100 +357,6 @@ __device__ inline void rank_body(const SortArgs &a, const SrcWalk &w, long long 
             if (base[v] >= t0 && base[v] < t1 && dst < a.n) a.perm[dst] = (int)p[v];
             else atomicOr(a.err, ERR_SORT);   // counts inconsistent with the particles
         }
-    }
-}
-
-// Gather pass in destination order.  One CTA per chunk of kGatherChunk
-// destination slots, one particle array at a time: the sources of a chunk lie
-// in the same tile of the previous layout (plus the few particles that changed
-// tile), so while the resident CTAs work on one array the source regions they
-// read stay in L2 and every source sector comes from DRAM about once.  (A
-// grid-stride loop over the whole array spreads the resident threads over all
-// of it and fetches each 32-byte sector many times for its 4 used bytes.)
-// THREADS threads, LOADS independent loads in flight per thread.
-constexpr int kGatherThreads = 256;
-constexpr int kGatherChunk = 4096;
-
-template <int NDIM, int THREADS, int LOADS>
-__device__ inline void gather_body(const SpeciesMixed &src, const SpeciesMixed &dst, long long n, const int *perm,
-                                   int b) {
-    constexpr int NA = NDIM + 5;   // cell, offsets, 3 momenta, id
-    const long long q0 = (long long)b * kGatherChunk;
-    const long long q1 = q0 + kGatherChunk < n ? q0 + kGatherChunk : n;
-#pragma unroll 1
-    for (int a = 0; a < NA; ++a) {
-        const uint32_t *sa;
-        uint32_t *da;
-        if (a == 0) { sa = src.cell; da = dst.cell; }
-        else if (a <= NDIM) { sa = reinterpret_cast<const uint32_t *>(src.off[a - 1]);
-                              da = reinterpret_cast<uint32_t *>(dst.off[a - 1]); }
-        else if (a < NA - 1) { sa = reinterpret_cast<const uint32_t *>(src.u[a - 1 - NDIM]);
-                               da = reinterpret_cast<uint32_t *>(dst.u[a - 1 - NDIM]); }
-        else { sa = reinterpret_cast<const uint32_t *>(src.id); da = reinterpret_cast<uint32_t *>(dst.id); }
-        for (long long q = q0 + threadIdx.x; q < q1; q += LOADS * THREADS) {
-            int p[LOADS];
-#pragma unroll
-            for (int v = 0; v < LOADS; ++v) {
-                const long long qq = q + v * THREADS;
-                p[v] = qq < q1 ? ldro(perm + qq) : -1;
-            }
-            uint32_t x[LOADS];
-            // an out-of-range entry exists only after a bad key, which the sort has flagged
-#pragma unroll
-            for (int v = 0; v < LOADS; ++v) x[v] = (p[v] >= 0 && p[v] < n) ? ldro(sa + p[v]) : 0u;
-#pragma unroll
-            for (int v = 0; v < LOADS; ++v) {
-                const long long qq = q + v * THREADS;
-                if (qq < q1) da[qq] = x[v];
-            }
-        }
-    }
-}
-
-// Gather of one chunk with every array per read of the permutation: LOADS
-// slots per thread, all NDIM + 5 arrays loaded before any is stored (more
-// independent loads in flight for a block that runs at few warps per SM).
-template <int NDIM, int THREADS, int LOADS>
-__device__ inline void gather_all_body(const SpeciesMixed &src, const SpeciesMixed &dst, long long n, const int *perm,
-                                       int b) {
-    constexpr int NA = NDIM + 5;   // cell, offsets, 3 momenta, id
-    const uint32_t *sa[NA];
-    uint32_t *da[NA];
-    sa[0] = src.cell; da[0] = dst.cell;
-#pragma unroll
-    for (int a = 0; a < NDIM; ++a) {
-        sa[1 + a] = reinterpret_cast<const uint32_t *>(src.off[a]);
-        da[1 + a] = reinterpret_cast<uint32_t *>(dst.off[a]);
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        sa[1 + NDIM + a] = reinterpret_cast<const uint32_t *>(src.u[a]);
-        da[1 + NDIM + a] = reinterpret_cast<uint32_t *>(dst.u[a]);
-    }
-    sa[NA - 1] = reinterpret_cast<const uint32_t *>(src.id);
-    da[NA - 1] = reinterpret_cast<uint32_t *>(dst.id);
-    const long long q0 = (long long)b * kGatherChunk;
-    const long long q1 = q0 + kGatherChunk < n ? q0 + kGatherChunk : n;
-    for (long long q = q0 + threadIdx.x; q < q1; q += LOADS * THREADS) {
-        int p[LOADS];
-#pragma unroll
-        for (int v = 0; v < LOADS; ++v) {
-            const long long qq = q + v * THREADS;
-            p[v] = qq < q1 ? ldro(perm + qq) : -1;
-        }
-        uint32_t x[NA][LOADS];
-        // an out-of-range entry exists only after a bad key, which the sort has flagged
-#pragma unroll
-        for (int a = 0; a < NA; ++a)
-#pragma unroll
-            for (int v = 0; v < LOADS; ++v) x[a][v] = (p[v] >= 0 && p[v] < n) ? ldro(sa[a] + p[v]) : 0u;
-#pragma unroll
-        for (int a = 0; a < NA; ++a)
-#pragma unroll
-            for (int v = 0; v < LOADS; ++v) {
-                const long long qq = q + v * THREADS;
-                if (qq < q1) da[a][qq] = x[a][v];
-            }
     }
 }
 

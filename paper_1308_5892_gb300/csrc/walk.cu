@@ -1,7 +1,6 @@
 // walk.cu -- the persistent step of a mixed ensemble: one launch runs every
 // phase of one step of every run: on the steps that re-sort a run, the phases
-// of the counting sort of each species (key histogram unless the previous push
-// counted it, block scans, rank, gather), then the main loop of App. A.3.1:
+// of the counting sort of each species (key histogram, block scans, rank), then the main loop of App. A.3.1:
 // both half advances of b with the energy record, node-averaged fields,
 // gather-push-deposit, the optional current smoothing (step 10), e advance with the
 // folded current.
@@ -9,8 +8,7 @@
 // Work queue.  The items of phase ph of run r are the tiles of the run (push,
 // and parts of the old layout's tiles for the sort's histogram and rank),
 // chunks of cells_per_item cells or keys (field, smoothing, zeroing and
-// scan-finish phases), scan blocks of 4096 keys, or gather chunks of 4096
-// particles.  The queue order is phase-major; inside a phase the runs with the
+// scan-finish phases), or scan blocks of 4096 keys.  The queue order is phase-major; inside a phase the runs with the
 // most particles per tile come first, so the longest items do not start last.
 // Resident CTAs take items from one counter.  Before an item of phase ph of
 // run r starts, every item of run r in the phases before ph must be done:
@@ -139,12 +137,16 @@ __host__ __device__ inline int walk_tile_parts(const SortArgs &a) {
 }
 
 // One item of a sort phase: block `local` of the `nitems` blocks of that phase
-// of species q's sort (sh: 33 ints of scratch for the scans).
+// of species q's sort (sh: 33 ints of scratch for the scans, box: box_max ints).
 template <int NDIM, int THREADS>
-__device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, int *sh) {
+__device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, int *sh, int *box) {
     const long long nkeys = nkeys_of(a);
-    if (kind == S_ZERO || kind == S_ZERO_AFTER) {
+    if (kind == S_ZERO) {
         zero_body(a.counts, nkeys, local, nitems);
+    } else if ((kind == S_HIST || kind == S_RANK) && a.old_tile_start && box_fits(a.t, NDIM)) {
+        const int parts = walk_tile_parts(a), tile = local / parts;
+        if (kind == S_HIST) box_body<NDIM, THREADS, false>(a, tile, local - tile * parts, parts, box);
+        else box_body<NDIM, THREADS, true>(a, tile, local - tile * parts, parts, box);
     } else if (kind == S_HIST) {
         const SrcWalk sw{a.old_tile_start, a.n, local, nitems, a.lgw_src, walk_tile_parts(a)};
         histogram_body<NDIM, 8>(a, sw, nkeys);
@@ -154,17 +156,13 @@ __device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, in
         scan_sums_body<THREADS>(a.block_sums, scan_blocks(a), sh);
     } else if (kind == S_SCAN_FINISH) {
         scan_finish_body(a, nkeys, local, nitems);
-    } else if (kind == S_RANK) {
+    } else {
         const SrcWalk sw{a.old_tile_start, a.n, local, nitems, a.lgw_src, walk_tile_parts(a)};
         rank_body<NDIM, 8>(a, sw, nkeys);
-    } else {
-        // fewer warps per SM than the sort's own gather launch: every array per
-        // read of the permutation, more loads in flight per thread
-        gather_all_body<NDIM, THREADS, 4>(a.src, a.dst, a.n, a.perm, local);
     }
 }
 
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST, int CT>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE, int CT>
 __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ WalkArgs w) {
     __shared__ int item_sh, go_sh;
     __shared__ int scan_sh[33];
@@ -203,12 +201,15 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
         }
         __syncthreads();
         if (go_sh) {
-            if (kind <= S_GATHER) {
+            if (kind <= S_RANK) {
                 const int *src = reinterpret_cast<const int *>(w.sort + 4 * r + w.species[ph]);
                 int *dst = reinterpret_cast<int *>(&sort_sh);
                 for (int q = threadIdx.x; q < (int)(sizeof(SortArgs) / sizeof(int)); q += THREADS) dst[q] = src[q];
                 __syncthreads();
-                sort_item<NDIM, THREADS>(sort_sh, kind, local, w.prefix[lo + 1] - w.prefix[lo], scan_sh);
+                // (the push's dynamic shared memory holds the box)
+                extern __shared__ __align__(128) float4 smem4[];
+                sort_item<NDIM, THREADS>(sort_sh, kind, local, w.prefix[lo + 1] - w.prefix[lo], scan_sh,
+                                         reinterpret_cast<int *>(smem4));
             } else if (kind == W_PUSH) {
                 const int *src = reinterpret_cast<const int *>(w.push + r);
                 int *dst = reinterpret_cast<int *>(&args_sh);
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
                 __syncthreads();
                 if (threadIdx.x == 0) args_sh.use_tma = 0;
                 __syncthreads();
-                push_tile<NDIM, THREADS, WALLS, HIST, CT>(args_sh, local, 0, 1, w.push + r);
+                push_tile<NDIM, THREADS, WALLS, MOVE, CT>(args_sh, local, 0, 1, w.push + r);
             } else {
                 const FieldRunF *fsrc = w.fp + r;
                 const int *src = reinterpret_cast<const int *>(fsrc);
@@ -238,21 +239,21 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
 
 // The walker instance for a tile geometry code (fixed_tile): the fixed form where
 // one exists for NDIM (periodic runs), else the run-time one.
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 auto walk_kernel(int ct) {
-    auto k = k_walk<NDIM, THREADS, MINB, WALLS, HIST, 0>;
+    auto k = k_walk<NDIM, THREADS, MINB, WALLS, MOVE, 0>;
     // (the 3D fixed form spills a few registers in this kernel: the run-time one is kept)
     if constexpr (!WALLS && NDIM == 2) {
-        if (ct == 2) k = k_walk<NDIM, THREADS, MINB, WALLS, HIST, 2>;
+        if (ct == 2) k = k_walk<NDIM, THREADS, MINB, WALLS, MOVE, 2>;
     }
     return k;
 }
 
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 bool fits_t(size_t smem) {
     cudaFuncAttributes attr;
     // the fixed-geometry forms hold the same static shared memory
-    if (cudaFuncGetAttributes(&attr, k_walk<NDIM, THREADS, MINB, WALLS, HIST, 0>) != cudaSuccess) {
+    if (cudaFuncGetAttributes(&attr, k_walk<NDIM, THREADS, MINB, WALLS, MOVE, 0>) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -262,9 +263,9 @@ bool fits_t(size_t smem) {
     return attr.sharedSizeBytes + smem <= (size_t)optin;
 }
 
-template <int NDIM, int THREADS, int MINB, bool WALLS, bool HIST>
+template <int NDIM, int THREADS, int MINB, bool WALLS, bool MOVE>
 void launch_t(const WalkArgs &w, size_t smem, int ct, cudaStream_t s) {
-    auto k = walk_kernel<NDIM, THREADS, MINB, WALLS, HIST>(ct);
+    auto k = walk_kernel<NDIM, THREADS, MINB, WALLS, MOVE>(ct);
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0, dev = 0, sms = 152;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem);
@@ -275,20 +276,20 @@ void launch_t(const WalkArgs &w, size_t smem, int ct, cudaStream_t s) {
 }
 
 template <int NDIM, int THREADS, int MINB>
-void launch_dim(const WalkArgs &w, bool walls, bool count, size_t smem, int ct, cudaStream_t s) {
+void launch_dim(const WalkArgs &w, bool walls, bool move, size_t smem, int ct, cudaStream_t s) {
     if (walls) {
-        if (count) launch_t<NDIM, THREADS, MINB, true, true>(w, smem, ct, s);
+        if (move) launch_t<NDIM, THREADS, MINB, true, true>(w, smem, ct, s);
         else launch_t<NDIM, THREADS, MINB, true, false>(w, smem, ct, s);
     } else {
-        if (count) launch_t<NDIM, THREADS, MINB, false, true>(w, smem, ct, s);
+        if (move) launch_t<NDIM, THREADS, MINB, false, true>(w, smem, ct, s);
         else launch_t<NDIM, THREADS, MINB, false, false>(w, smem, ct, s);
     }
 }
 
 template <int NDIM, int THREADS, int MINB>
-bool fits_dim(bool walls, bool count, size_t smem) {
-    if (walls) return count ? fits_t<NDIM, THREADS, MINB, true, true>(smem) : fits_t<NDIM, THREADS, MINB, true, false>(smem);
-    return count ? fits_t<NDIM, THREADS, MINB, false, true>(smem) : fits_t<NDIM, THREADS, MINB, false, false>(smem);
+bool fits_dim(bool walls, bool move, size_t smem) {
+    if (walls) return move ? fits_t<NDIM, THREADS, MINB, true, true>(smem) : fits_t<NDIM, THREADS, MINB, true, false>(smem);
+    return move ? fits_t<NDIM, THREADS, MINB, false, true>(smem) : fits_t<NDIM, THREADS, MINB, false, false>(smem);
 }
 
 }  // namespace
@@ -300,28 +301,28 @@ int walk_sort_items(const SortArgs &a, int kind, int cpi) {
     const long long nkeys = nkeys_of(a);
     auto chunks = [](long long n, long long per) { return (int)std::max<long long>(1, (n + per - 1) / per); };
     switch (kind) {
-    case S_ZERO: return a.counted ? 0 : chunks(nkeys, cpi);
-    case S_HIST: return (a.counted || a.n == 0) ? 0 : (a.old_tile_start ? a.t.ntiles * walk_tile_parts(a) : chunks(a.n, cpi));
+    case S_ZERO: return chunks(nkeys, cpi);
+    case S_HIST: return a.n == 0 ? 0 : (a.old_tile_start ? a.t.ntiles * walk_tile_parts(a) : chunks(a.n, cpi));
     case S_SCAN_BLOCKS: return scan_blocks(a);
     case S_SCAN_SUMS: return 1;
     case S_SCAN_FINISH: return chunks(nkeys, cpi);
     case S_RANK: return a.n == 0 ? 0 : (a.old_tile_start ? a.t.ntiles * walk_tile_parts(a) : chunks(a.n, cpi));
-    case S_ZERO_AFTER: return chunks(nkeys, cpi);
-    case S_GATHER: return a.n == 0 ? 0 : chunks(a.n, kGatherChunk);
     default: return 0;
     }
 }
 
-bool walk_fits(int ndim, bool walls, bool count, size_t push_smem) {
-    if (push_smem < sizeof(double) * 6 * (ndim == 3 ? 512 : 256)) return false;   // the energy sums live there
-    return ndim == 3 ? fits_dim<3, 512, 1>(walls, count, push_smem) : fits_dim<2, 256, 2>(walls, count, push_smem);
+bool walk_fits(int ndim, bool walls, bool move, size_t push_smem) {
+    // the energy sums and the sort's boxes live there
+    if (push_smem < std::max(sizeof(double) * 6 * (ndim == 3 ? 512 : 256), sizeof(int) * (ndim == 3 ? kBoxMax3 : kBoxMax2)))
+        return false;
+    return ndim == 3 ? fits_dim<3, 512, 1>(walls, move, push_smem) : fits_dim<2, 256, 2>(walls, move, push_smem);
 }
 
-void launch_walk(const WalkArgs &w, int ndim, bool walls, bool count, size_t push_smem, int tile_code,
+void launch_walk(const WalkArgs &w, int ndim, bool walls, bool move, size_t push_smem, int tile_code,
                  cudaStream_t s) {
     if (w.total <= 0) return;
-    if (ndim == 3) launch_dim<3, 512, 1>(w, walls, count, push_smem, tile_code, s);
-    else launch_dim<2, 256, 2>(w, walls, count, push_smem, tile_code, s);
+    if (ndim == 3) launch_dim<3, 512, 1>(w, walls, move, push_smem, tile_code, s);
+    else launch_dim<2, 256, 2>(w, walls, move, push_smem, tile_code, s);
 }
 
 }  // namespace pic
