@@ -320,6 +320,7 @@ __host__ __device__ constexpr int warp_smem_words() { return 7 * kQueue + kStage
 // Per-CTA constants of the tile.
 struct TileCtx {
     int x0, y0, z0, Rx, Ry, Rz, sx, sxy, nodes, H, T0, T1, T2;
+    int lx, ly, lz;   // local cells 1..l of each axis take the fast path
     const float4 *nA;
     const float2 *nB;
     int *Jhi, *Jlo;
@@ -335,17 +336,16 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
                                          int &ci, int &cj, int &ck, float &kin0, float &kin1, int &side) {
     const Geom &g = a.g;
     unpack_cell(NDIM, c, ci, cj, ck);
-    // local cell in the staged box, nearest periodic image of the tile
+    // local cell in the staged box, nearest periodic image of the tile; the fast path
+    // needs nodes l-1..l+2 of the box (the gather reads l..l+1, the deposit writes all),
+    // inside the padded grid: 1 <= l <= tc.l{x,y,z}
     int lx = ci - tc.x0, ly = cj - tc.y0, lz = NDIM == 3 ? ck - tc.z0 : 0;
     if (lx >= tc.T0 + tc.H) lx -= g.nx; else if (lx < -tc.H) lx += g.nx;
     if (ly >= tc.T1 + tc.H) ly -= g.ny; else if (ly < -tc.H) ly += g.ny;
     if (NDIM == 3) { if (lz >= tc.T2 + tc.H) lz -= g.nz; else if (lz < -tc.H) lz += g.nz; }
     lx += tc.H; ly += tc.H; lz += NDIM == 3 ? tc.H : 0;
-    // fast path: the gather reads nodes l..l+1 and the deposit writes nodes
-    // l-1..l+2 of the staged box, all of which must also lie in the padded grid
-    fast = lx >= 1 && lx <= tc.Rx - 3 && ly >= 1 && ly <= tc.Ry - 3 && tc.x0 + lx + 2 < g.px &&
-           tc.y0 + ly + 2 < g.py;
-    if (NDIM == 3) fast = fast && lz >= 1 && lz <= tc.Rz - 3 && tc.z0 + lz + 2 < g.pz;
+    fast = (unsigned)(lx - 1) < (unsigned)tc.lx && (unsigned)(ly - 1) < (unsigned)tc.ly &&
+           (NDIM == 2 || (unsigned)(lz - 1) < (unsigned)tc.lz);
     q0 = lx + ly * tc.sx + lz * tc.sxy;
     float E[3], B[3];
     if (fast) gather_nodes<NDIM>(tc.nA, tc.nB, q0, tc.sx, tc.sxy, d, E, B);
@@ -356,9 +356,9 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
     const float dt = a.dt;
     boris<float>(u, E, B, h, dt);
     const float u2 = __fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmul_rn(u[0], u[0])));
-    const float inv_gam = rsqrtf(__fadd_rn(1.f, u2));
+    const float inv_gam = rsqrt_<float>(__fadd_rn(1.f, u2));
     // gamma - 1 = u^2 / (1 + gamma), free of cancellation
-    kin0 = __fadd_rn(kin0, __fdividef(u2_0, __fmaf_rn(__fadd_rn(1.f, u2_0), rsqrtf(__fadd_rn(1.f, u2_0)), 1.f)));
+    kin0 = __fadd_rn(kin0, __fdividef(u2_0, __fmaf_rn(__fadd_rn(1.f, u2_0), rsqrt_<float>(__fadd_rn(1.f, u2_0)), 1.f)));
     kin1 = __fadd_rn(kin1, __fdividef(u2, __fmaf_rn(__fadd_rn(1.f, u2), inv_gam, 1.f)));
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
@@ -378,7 +378,7 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
         float sa = floorf(pa);
         float da = snap_offset<float>(pa - sa);   // the end offset on the 2^-24 grid
         if (da >= 1.f) { da = 0.f; sa += 1.f; }
-        if (!(sa >= -1.f && sa <= 1.f)) {   // faster than one cell per step, or not finite:
+        if (!(fabsf(sa) <= 1.f)) {   // faster than one cell per step, or not finite:
             atomicOr(a.err, ERR_FAST_MOVE);  // flag it and keep every index in bounds
             sa = 0.f;
             da = d[ax];
@@ -398,8 +398,9 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
         d[0] = 1.f;
     }
     // with walls, x is never wrapped (cell 0 and nx - 1 hold the particles at the walls)
-    const int ni = WALLS ? ci + s[0] : g.wx(ci + s[0]);
-    const int nj = g.wy(cj + s[1]), nk = NDIM == 3 ? g.wz(ck + s[2]) : 0;
+    auto wrap1 = [](int i, int n) { return i < 0 ? n - 1 : (i >= n ? 0 : i); };   // one cell beyond [0, n)
+    const int ni = WALLS ? ci + s[0] : wrap1(ci + s[0], g.nx);
+    const int nj = wrap1(cj + s[1], g.ny), nk = NDIM == 3 ? wrap1(ck + s[2], g.nz) : 0;
     c = pack_cell(NDIM, ni, nj, nk);
 }
 
@@ -452,6 +453,9 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
         tc.sx = Rx; tc.sxy = Rx * Ry; tc.nodes = Rx * Ry * Rz;
         tc.H = F.H; tc.T0 = F.T0; tc.T1 = F.T1; tc.T2 = F.T2;
     }
+    tc.lx = max(0, min(tc.Rx - 3, g.px - 3 - tc.x0));
+    tc.ly = max(0, min(tc.Ry - 3, g.py - 3 - tc.y0));
+    tc.lz = NDIM == 3 ? max(0, min(tc.Rz - 3, g.pz - 3 - tc.z0)) : 0;
     const int nodes = tc.nodes;
     float4 *nA = smem4;
     float2 *nB = reinterpret_cast<float2 *>(reinterpret_cast<char *>(smem4) + node_b_offset(nodes));
