@@ -362,19 +362,21 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
     kin1 = __fadd_rn(kin1, __fdividef(u2, __fmaf_rn(__fadd_rn(1.f, u2), inv_gam, 1.f)));
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
-        D[ax] = dt * u[ax] * inv_gam;
+        D[ax] = __fmul_rn(__fmul_rn(dt, u[ax]), inv_gam);
         d0[ax] = d[ax];
         s[ax] = 0;
     }
     // conducting walls in x (App. A.4): a particle that would cross a wall is reflected
     side = 0;
     if (WALLS) {
-        const float px = d[0] + D[0];
+        const float px = __fadd_rn(d[0], D[0]);
         side = (ci == 0 && px < 0.f) ? -1 : ((ci == g.nx - 1 && px > 1.f) ? 1 : 0);
     }
 #pragma unroll
     for (int ax = 0; ax < NDIM; ++ax) {
-        const float pa = d[ax] + D[ax];
+        // The roundings of the end position are part of the result and must not depend on what the
+        // compiler contracts in an instance: x without walls takes one rounding, the others two.
+        const float pa = ax == 0 && !WALLS ? __fmaf_rn(__fmul_rn(dt, u[0]), inv_gam, d[0]) : __fadd_rn(d[ax], D[ax]);
         float sa = floorf(pa);
         float da = snap_offset<float>(pa - sa);   // the end offset on the 2^-24 grid
         if (da >= 1.f) { da = 0.f; sa += 1.f; }
