@@ -918,8 +918,8 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     a.nparts = r.nparts;
     a.parts_bound = r.parts_bound;
     a.dt = (float)r.d.dt;
-    a.mode = 0;
     a.hist = hist_ref(r);
+    a.kin0 = r.hist_n == 0 ? 1 : 0;
     a.err = ctx->d_err;
     a.use_tma = r.tma ? 1 : 0;
     a.tmA = r.tmA;
@@ -939,6 +939,7 @@ FieldRunF field_run(Run &r) {
         fr.Z[c] = jplane<u64>(r, 1 - r.jcur, c);
     }
     fr.hist = hist_ref(r);
+    fr.carry = r.hist_n > 0 ? 1 : 0;
     fr.hist_inc = r.hist_idx;
     fr.scale = 2.0 / (r.d.n_x * r.d.n_x * r.d.rho_sp0) * 0x1p-36;
     fr.smooth = r.smooth;
@@ -1235,7 +1236,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
             KTimer t(ctx, PIC_KERNEL_FIELD);
             // after the first step the energy at u^{t-1/2} is what the step before recorded
             launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{hslot, nullptr, 0},
-                                     hslot && r.hist_n > 0 ? hslot - 7 : nullptr, s);
+                                     r.hist_n > 0, s);
             launch_node_fields64(r.g, f, r.nf64, s);
         }
         double *J[3] = {jplane<double>(r, r.jcur, 0), jplane<double>(r, r.jcur, 1), jplane<double>(r, r.jcur, 2)};
@@ -1276,7 +1277,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         FieldPtrs<float> f = fields_of<float>(r, true);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, hist_ref(r), nullptr, s);
+            launch_b_advance<float>(r.g, f, 0.5f * (float)r.d.dt, hist_ref(r), r.hist_n > 0, s);
             launch_node_fields(r.g, f, r.nfA, r.nfB, s);
         }
         typedef unsigned long long u64;

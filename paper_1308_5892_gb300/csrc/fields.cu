@@ -35,12 +35,11 @@ __device__ __forceinline__ void for_cells(const Geom &g, F &&body) {
 }
 
 // Both half advances of b over every padded cell; with a history slot, the interior
-// sums of e^2 and b^2 at t are added to it.  kin_prev (nullable): the kinetic energy
-// the previous step recorded at u^{t-1/2}, which is this step's first entry.
+// sums of e^2 and b^2 at t are added to it.  carry: see launch_b_advance.
 template <typename R>
-__global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, const double *kin_prev) {
+__global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, bool carry) {
     double *slot = hist.slot();
-    if (slot && kin_prev && blockIdx.x == 0 && threadIdx.x == 0) slot[0] = *kin_prev;
+    if (slot && carry && blockIdx.x == 0 && threadIdx.x == 0) slot[0] = slot[-7];
     double *energy_acc = slot ? slot + 2 : nullptr;
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for_cells(g, [&](const CellAt &c) { b_advance_cell<R>(g, f, h, c, energy_acc != nullptr, acc); });
@@ -123,6 +122,7 @@ __global__ void __launch_bounds__(256) k_fields_multi(const FieldRunF *runs, con
     const CellAt c(r.g, in ? p : 0);
     if (PHASE == FIELD_B) {
         double *slot = r.hist.slot();
+        if (slot && r.carry && p == 0) slot[0] = slot[-7];
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         if (in) b_advance_cell<float>(r.g, r.f, h, c, energy_acc != nullptr, acc);
@@ -181,9 +181,9 @@ inline int cells_grid(const Geom &g, int per_sm) {
 }  // namespace
 
 template <typename R>
-void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s) {
+void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, bool carry, cudaStream_t s) {
     // (few blocks: each adds its six sums to the same addresses)
-    k_b_advance<R><<<cells_grid(g, 4), 256, 0, s>>>(g, f, h, energy, kin_prev);
+    k_b_advance<R><<<cells_grid(g, 4), 256, 0, s>>>(g, f, h, energy, carry);
 }
 
 template <typename R>
@@ -229,9 +229,8 @@ void launch_add_uniform(const Geom &g, FieldPtrs<R> f, const double e0[3], const
     k_add_uniform<R><<<grid_for(g.pcells, 256), 256, 0, s>>>(g, f, e0[0], e0[1], e0[2], b0[0], b0[1], b0[2]);
 }
 
-template void launch_b_advance<float>(const Geom &, FieldPtrs<float>, float, HistRef, const double *, cudaStream_t);
-template void launch_b_advance<double>(const Geom &, FieldPtrs<double>, double, HistRef, const double *,
-                                       cudaStream_t);
+template void launch_b_advance<float>(const Geom &, FieldPtrs<float>, float, HistRef, bool, cudaStream_t);
+template void launch_b_advance<double>(const Geom &, FieldPtrs<double>, double, HistRef, bool, cudaStream_t);
 template void launch_e_advance<float>(const Geom &, FieldPtrs<float>, const float *const[3], float *const[3], float,
                                       cudaStream_t);
 template void launch_e_advance<double>(const Geom &, FieldPtrs<double>, const double *const[3], double *const[3],

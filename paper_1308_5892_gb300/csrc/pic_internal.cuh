@@ -243,9 +243,10 @@ struct HistRef {
 // ---- kernel launchers (implemented in the .cu files) ----
 
 // fields.cu
-// both half advances of b; b at t goes to f.bt.  kin_prev (nullable): copied to slot[0] of the energy record
+// both half advances of b; b at t goes to f.bt.  carry: slot[0] of the energy record, the kinetic
+// energy at u^{t-1/2}, is what the step before recorded at its u^{t+1/2}
 template <typename R>
-void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, const double *kin_prev, cudaStream_t s);
+void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, bool carry, cudaStream_t s);
 template <typename R>
 void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *const Jzero[3], R dt,
                       cudaStream_t s);
@@ -327,8 +328,8 @@ struct MixedStepArgs {
     float sgn[4];                   // sign of the charge
     double m_over_me[4];
     float dt;
-    int mode;                       // 0 step, 1 half step back (momenta only)
     HistRef hist;                   // slot[0..1]: kinetic energy of u^{t-1/2} and u^{t+1/2}
+    int kin0;                       // record the first (no step before has; such a step moves every particle)
     int *err;
     // TMA descriptors of the node-field arrays nfA (4 floats per node) and nfB
     // (2 floats per node) with a box of one tile + halo; use_tma = 0 when the
@@ -351,6 +352,7 @@ struct FieldRunF {
     const unsigned long long *J[3];
     unsigned long long *Z[3];
     HistRef hist;           // slot[2..7]: e^2, b^2 sums of the step (null base: none)
+    int carry;              // slot[0] is the kinetic energy at u^{t+1/2} of the slot before
     long long *hist_inc;    // E_FX phase: step counter of the history, incremented once (nullable)
     double scale;           // |alpha| 2^-36
     int smooth;             // current smoothing passes (0: off); the E_FX phase then reads sbuf[smooth & 1]

@@ -330,7 +330,7 @@ struct TileCtx {
 // state; d0, s, D describe the path for the deposit; fast tells whether the
 // stencil stays in the staged box, and q0 is then the local node index of the
 // start cell.
-template <int NDIM, bool WALLS>
+template <int NDIM, bool WALLS, bool MOVE>
 __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &tc, float h, uint32_t &c, float d[3],
                                          float u[3], float d0[3], int s[3], float D[3], bool &fast, int &q0,
                                          int &ci, int &cj, int &ck, float &kin0, float &kin1, int &side) {
@@ -352,13 +352,17 @@ __device__ __forceinline__ void push_one(const MixedStepArgs &a, const TileCtx &
     else gather_global<NDIM>(g, a.nfA, a.nfB, ci, cj, ck, d, E, B);
     // explicit roundings (nothing left to contract), so that every kernel that
     // inlines this body computes the same bits
-    const float u2_0 = __fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmul_rn(u[0], u[0])));
+    // u^{t-1/2}: its energy was recorded by the step before, except on the first step of a
+    // state, which sorts
+    if (MOVE) {
+        const float u2_0 = __fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmul_rn(u[0], u[0])));
+        kin0 = __fadd_rn(kin0, __fdividef(u2_0, __fmaf_rn(__fadd_rn(1.f, u2_0), rsqrt_<float>(__fadd_rn(1.f, u2_0)), 1.f)));
+    }
     const float dt = a.dt;
     boris<float>(u, E, B, h, dt);
     const float u2 = __fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmul_rn(u[0], u[0])));
     const float inv_gam = rsqrt_<float>(__fadd_rn(1.f, u2));
     // gamma - 1 = u^2 / (1 + gamma), free of cancellation
-    kin0 = __fadd_rn(kin0, __fdividef(u2_0, __fmaf_rn(__fadd_rn(1.f, u2_0), rsqrt_<float>(__fadd_rn(1.f, u2_0)), 1.f)));
     kin1 = __fadd_rn(kin1, __fdividef(u2, __fmaf_rn(__fadd_rn(1.f, u2), inv_gam, 1.f)));
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
@@ -650,7 +654,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                     float d0[3], D[3];
                     int s[3], ci, cj, ck, side;
                     bool fast;
-                    push_one<NDIM, WALLS>(a, tc, h, c, d, u, d0, s, D, fast, q0, ci, cj, ck, kin0, kin1, side);
+                    push_one<NDIM, WALLS, MOVE>(a, tc, h, c, d, u, d0, s, D, fast, q0, ci, cj, ck, kin0, kin1, side);
                     put_particle(NDIM, P, p, c, d, u, id_bits);
                     if (fast) {
                         // the start-cell piece goes to the register accumulator
@@ -702,7 +706,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             // kinetic energy of the item (at most 32 values per lane in FP32), summed per warp in FP64
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                kin0 += __shfl_xor_sync(kFull, kin0, o);
+                if (MOVE) kin0 += __shfl_xor_sync(kFull, kin0, o);
                 kin1 += __shfl_xor_sync(kFull, kin1, o);
             }
             if (lane == 0) {
@@ -718,7 +722,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     __syncthreads();
     flush_limbs(false);
     double *slot = a.hist.slot();
-    if (slot && threadIdx.x < 2) {
+    if (slot && threadIdx.x < 2 && (threadIdx.x == 1 || (MOVE && a.kin0))) {
         double t = 0.0;
         for (int w = 0; w < WARPS; ++w) t += kin_sh[threadIdx.x][w];
         atomicAdd(slot + threadIdx.x, t);
