@@ -96,6 +96,7 @@ struct pic_ctx {
     bool have_alloc = false;
     std::vector<Run> runs;
     int *d_err = nullptr;
+    int *h_err = nullptr;       // page-locked copy for read_err
     void *staging = nullptr;
     size_t staging_bytes = 0;
     double *mj_table = nullptr;     // cumulative marginal of the loader, kMjTable + 1 values
@@ -302,10 +303,14 @@ __global__ void k_check64(Geom g, Species64 s, long long n, int *err) {
     }
 }
 
-// src_lo (nullable): the low-order part added to src (e in the mixed path).
+// The six field planes c0 .. c0 + gridDim.y - 1 of F into compact planes of dst (F holds the
+// low-order part of e in planes 6 .. 8 in the mixed path).
 template <typename R>
-__global__ void k_unpad_field(Geom g, const R *src, const R *src_lo, double *dst) {
+__global__ void k_unpad_fields(Geom g, const R *F, int c0, double *dst) {
     const long long n = (long long)g.nx * g.ny * g.nz;
+    const int c = c0 + blockIdx.y;
+    const R *src = F + c * g.pcells, *src_lo = sizeof(R) == sizeof(float) && c < 3 ? F + (6 + c) * g.pcells : nullptr;
+    dst += blockIdx.y * n;
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(q % g.nx);
         const long long r = q / g.nx;
@@ -351,7 +356,18 @@ __global__ void k_id_index(const int32_t *id, long long n, int *inv) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x)
         if ((unsigned long long)id[p] < (unsigned long long)n) inv[id[p]] = (int)p;   // ids are 0 .. n-1
 }
-__global__ void k_id_index_mixed(int ndim, SpeciesMixed s, long long n, int *inv) {
+// Species of a download by id, one per blockIdx.y: storage, count, index map and
+// destination (6 planes `stride` doubles apart).
+struct Download {
+    SpeciesMixed s[PIC_MAX_SPECIES];
+    long long n[PIC_MAX_SPECIES];
+    int *inv[PIC_MAX_SPECIES];
+    double *dst[PIC_MAX_SPECIES];
+};
+__global__ void k_id_index_mixed(int ndim, Download d) {
+    const SpeciesMixed s = d.s[blockIdx.y];
+    const long long n = d.n[blockIdx.y];
+    int *inv = d.inv[blockIdx.y];
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         const int id = get_id(ndim, s, p);
         if ((unsigned long long)id < (unsigned long long)n) inv[id] = (int)p;
@@ -384,11 +400,14 @@ __global__ void k_pick64(Species64 s, const int *inv, const long long *ids, long
     }
 }
 
-// Download of ids [a, a+m) through the id -> storage index map inv: coalesced
-// staging writes, one pass over the chunk's own particles.
-// st: 6 planes `stride` doubles apart, written for ids [a, a+m)
-__global__ void k_download_by_id(Geom g, SpeciesMixed s, const int *inv, long long a, long long m, double *st,
-                                 long long stride) {
+// Download of ids [a, a+m) through the id -> storage index map: coalesced staging
+// writes, one pass over the chunk's own particles.
+__global__ void k_download_by_id(Geom g, Download d, long long a, long long chunk, long long stride) {
+    const SpeciesMixed s = d.s[blockIdx.y];
+    const int *inv = d.inv[blockIdx.y];
+    double *st = d.dst[blockIdx.y];
+    const long long m = min(chunk, d.n[blockIdx.y] - a);
+    if (stride == 0) stride = d.n[blockIdx.y];
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
         const int p = inv[a + q];
         int i, j, k;
@@ -797,9 +816,11 @@ pic_status io_ready(pic_ctx *ctx) {
 }
 
 pic_status read_err(pic_ctx *ctx) {
-    int e = 0;
-    CK(cudaMemcpyAsync(&e, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    // (a copy into pageable memory goes through the driver's staging first)
+    if (!ctx->h_err) CK(cudaMallocHost((void **)&ctx->h_err, sizeof(int)));
+    CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    const int e = *ctx->h_err;
     if (e) {
         CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
         if (e & ERR_TIMEOUT) return fail(ctx, PIC_ETIMEOUT, "a bounded device wait gave up");
@@ -1561,6 +1582,7 @@ void pic_destroy(pic_ctx *ctx) {
     for (auto e : ctx->io_ev)
         if (e) cudaEventDestroy(e);
     if (ctx->gstage) cudaFreeHost(ctx->gstage);
+    if (ctx->h_err) cudaFreeHost(ctx->h_err);
     for (int k = 0; k < kKernelClasses; ++k)
         for (auto &pr : ctx->ev_pending[k]) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
     for (auto e : ctx->ev_pool) cudaEventDestroy(e);
@@ -1685,15 +1707,61 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
     double *stg = (double *)ctx->staging;
     // page-locked host buffers are written by the conversion kernels directly
     double *fmap = mapped_host(out->fields, sizeof(double) * 6 * ncell);
-    for (int c = 0; c < 6; ++c) {
-        double *dst = fmap ? fmap + c * ncell : stg;
-        if (ctx->precision == PIC_FP64)
-            k_unpad_field<double><<<nblk(ncell), 256, 0, sm>>>(g, (double *)r.F + c * g.pcells, nullptr, dst);
-        else
-            k_unpad_field<float><<<nblk(ncell), 256, 0, sm>>>(
-                g, (float *)r.F + c * g.pcells, c < 3 ? (float *)r.F + (6 + c) * g.pcells : nullptr, dst);
+    // all planes in one launch where the destination holds them
+    const int planes = fmap || ctx->staging_bytes >= sizeof(double) * 6 * (size_t)ncell ? 6 : 1;
+    for (int c = 0; c < 6; c += planes) {
+        double *dst = fmap ? fmap : stg;
+        const dim3 grid(nblk(ncell), planes);
+        if (ctx->precision == PIC_FP64) k_unpad_fields<double><<<grid, 256, 0, sm>>>(g, (double *)r.F, c, dst);
+        else k_unpad_fields<float><<<grid, 256, 0, sm>>>(g, (float *)r.F, c, dst);
+        CK(cudaGetLastError());
         if (!fmap)
-            CK(cudaMemcpyAsync(out->fields + c * ncell, stg, sizeof(double) * ncell, cudaMemcpyDeviceToHost, sm));
+            CK(cudaMemcpyAsync(out->fields + c * ncell, stg, sizeof(double) * planes * ncell, cudaMemcpyDeviceToHost, sm));
+    }
+    if (ctx->precision == PIC_MIXED) {
+        // conversion and copy in turn on the context stream (a copy stream of its own
+        // measured slower here than this serial form); the id -> storage index map lets
+        // each chunk touch only its own particles.  Page-locked buffers of all species are
+        // written by one launch (at small sizes the launches are the time).
+        Download dl{}, direct{};
+        int ns = 0, nd = 0;
+        long long most = 0, most_direct = 0;
+        for (int s = 0; s < r.d.nspecies; ++s) {
+            SpeciesState &S = r.sp[s];
+            out->count[s] = S.n;
+            if (S.n == 0 || !out->particles[s]) continue;
+            dl.s[ns] = S.mb[S.cur];
+            dl.n[ns] = S.n;
+            dl.inv[ns] = S.perm;
+            dl.dst[ns++] = out->particles[s];
+            most = std::max<long long>(most, S.n);
+        }
+        if (ns > 0) k_id_index_mixed<<<dim3(nblk(most), ns), 256, 0, sm>>>(g.ndim, dl);
+        for (int q = 0; q < ns; ++q) {
+            const int64_t n = dl.n[q];
+            double *P = dl.dst[q], *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n);
+            if (Pm) {
+                direct.s[nd] = dl.s[q];
+                direct.n[nd] = n;
+                direct.inv[nd] = dl.inv[q];
+                direct.dst[nd++] = Pm;
+                most_direct = std::max<long long>(most_direct, n);
+                continue;
+            }
+            const int64_t chunk = (int64_t)(ctx->staging_bytes / (6 * sizeof(double)));
+            for (int64_t a0 = 0; a0 < n; a0 += chunk) {
+                const int64_t m = std::min(chunk, n - a0);
+                k_download_by_id<<<nblk(m), 256, 0, sm>>>(g, Download{{dl.s[q]}, {dl.n[q]}, {dl.inv[q]}, {stg}}, a0, m, m);
+                CK(cudaGetLastError());
+                for (int a = 0; a < 6; ++a)
+                    CK(cudaMemcpyAsync(P + a * n + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
+            }
+        }
+        if (nd > 0) k_download_by_id<<<dim3(nblk(most_direct), nd), 256, 0, sm>>>(g, direct, 0, INT64_MAX, 0);
+        CK(cudaGetLastError());
+        out->step = r.step;
+        CK(cudaStreamSynchronize(sm));
+        return PIC_OK;
     }
     for (int s = 0; s < r.d.nspecies; ++s) {
         SpeciesState &S = r.sp[s];
@@ -1701,8 +1769,8 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
         out->count[s] = n;
         double *P = out->particles[s];
         if (n == 0 || !P) continue;
-        if (ctx->precision == PIC_FP64 && S.sorted64) {
-            // as the mixed path below: by id, straight into page-locked buffers or through the staging buffer
+        if (S.sorted64) {
+            // as the mixed path above: by id, straight into page-locked buffers or through the staging buffer
             k_id_index<<<nblk(n), 256, 0, sm>>>(S.id64, n, r.perm);
             double *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n);
             const int64_t chunk = Pm ? n : (int64_t)(ctx->staging_bytes / (6 * sizeof(double)));
@@ -1719,24 +1787,6 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
                 CK(cudaMemcpyAsync(P + (3 + a) * n, S.s64.u[a], sizeof(double) * n, cudaMemcpyDeviceToHost, sm));
             }
             if (g.ndim == 2) std::memset(P + 2 * n, 0, sizeof(double) * n);
-        } else {
-            // conversion and copy in turn on the context stream (a copy stream of
-            // its own measured slower here than this serial form); the id -> storage
-            // index map lets each chunk touch only its own particles
-            k_id_index_mixed<<<nblk(n), 256, 0, sm>>>(g.ndim, S.mb[S.cur], n, S.perm);
-            if (double *Pm = mapped_host(P, sizeof(double) * 6 * (size_t)n)) {
-                k_download_by_id<<<nblk(n), 256, 0, sm>>>(g, S.mb[S.cur], S.perm, 0, n, Pm, n);
-                CK(cudaGetLastError());
-                continue;
-            }
-            const int64_t chunk = (int64_t)(ctx->staging_bytes / (6 * sizeof(double)));
-            for (int64_t a0 = 0; a0 < n; a0 += chunk) {
-                const int64_t m = std::min(chunk, n - a0);
-                k_download_by_id<<<nblk(m), 256, 0, sm>>>(g, S.mb[S.cur], S.perm, a0, m, stg, m);
-                CK(cudaGetLastError());
-                for (int a = 0; a < 6; ++a)
-                    CK(cudaMemcpyAsync(P + a * n + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
-            }
         }
     }
     out->step = r.step;
@@ -1759,7 +1809,7 @@ pic_status pic_get_particles(pic_ctx *ctx, int run, int species, const int64_t *
     const int64_t chunk = (int64_t)(ctx->staging_bytes / (7 * sizeof(double)));
     double *stg = (double *)ctx->staging;
     if (S.n > 0 && ctx->precision == PIC_MIXED)
-        k_id_index_mixed<<<nblk(S.n), 256, 0, sm>>>(r.d.ndim, S.mb[S.cur], S.n, S.perm);
+        k_id_index_mixed<<<nblk(S.n), 256, 0, sm>>>(r.d.ndim, Download{{S.mb[S.cur]}, {S.n}, {S.perm}, {nullptr}});
     else if (S.n > 0 && S.sorted64)
         k_id_index<<<nblk(S.n), 256, 0, sm>>>(S.id64, S.n, r.perm);
     for (int64_t a0 = 0; a0 < nids; a0 += chunk) {
