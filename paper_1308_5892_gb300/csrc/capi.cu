@@ -664,8 +664,7 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         r.nfB = (float2 *)dev_alloc(ctx, sizeof(float2) * g.pcells);
         node_maps(r);
         const long long nkeys = max_keys;
-        r.offsets = (int *)dev_alloc(ctx, sizeof(int) * (nkeys + 1));
-        r.block_sums = (int *)dev_alloc(ctx, sizeof(int) * sort_scan_scratch(nkeys));
+        r.block_sums = (int *)dev_alloc(ctx, sizeof(int) * d.nspecies * sort_scan_scratch(nkeys));
         r.max_tiles = max_tiles;
         r.max_keys = max_keys;
         if (ctx->runs.size() == 1) {
@@ -674,7 +673,7 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
             r.nparts = (int *)dev_alloc(ctx, sizeof(int));
             if (!r.parts || !r.nparts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
         }
-        if (!r.nfA || !r.nfB || !r.offsets || !r.block_sums)
+        if (!r.nfA || !r.nfB || !r.block_sums)
             return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
     }
     if (!mixed) {
@@ -883,8 +882,7 @@ SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S, int lgw) {
     a.counts = S.counts;
     a.lgw = lgw;
     a.lgw_src = S.lgw;
-    a.offsets = r.offsets;
-    a.block_sums = r.block_sums;
+    a.block_sums = r.block_sums + (&S - r.sp) * sort_scan_scratch(r.max_keys);
     // the old-tile walk is valid only for the tile geometry the layout was sorted with
     a.old_tile_start = (S.tiled && S.tiled_ntiles == r.t.ntiles) ? S.tile_start : nullptr;
     a.tile_start = S.tile_start_alt;
@@ -904,10 +902,16 @@ void sort_done(Run &r, SpeciesState &S, int lgw) {
     S.tiled_ntiles = r.t.ntiles;
 }
 
-void sort_species(pic_ctx *ctx, Run &r, SpeciesState &S) {
+// Sort of all species of a single run; returns the launches.
+int sort_run(pic_ctx *ctx, Run &r) {
     const int lgw = push_walk_lg(ctx);
-    launch_sort(sort_args(ctx, r, S, lgw), ctx->stream);
-    sort_done(r, S, lgw);
+    SortPack a{};
+    for (a.n = 0; a.n < r.d.nspecies; ++a.n) {
+        SpeciesState &S = r.sp[a.n];
+        a.s[a.n] = sort_args(ctx, r, S, lgw);
+        sort_done(r, S, lgw);
+    }
+    return launch_sort(a, ctx->stream);
 }
 
 HistRef hist_ref(Run &r) { return HistRef{r.hist, r.hist_idx, r.hist_cap}; }
@@ -1286,10 +1290,7 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         int launches = 0;
         if (!r.sorted || r.since_sort >= r.sort_interval) {
             KTimer t(ctx, PIC_KERNEL_SORT);
-            for (int q = 0; q < nsp; ++q) {
-                launches += 5;
-                sort_species(ctx, r, r.sp[q]);
-            }
+            launches += sort_run(ctx, r);
             make_parts(ctx, r);
             launches += r.parts ? 1 : 0;
             r.sorted = true;
@@ -1781,7 +1782,7 @@ pic_status pic_get_state(pic_ctx *ctx, int run, pic_state_view *out) {
                 for (int a = 0; !Pm && a < 6; ++a)
                     CK(cudaMemcpyAsync(P + a * n + a0, stg + a * m, sizeof(double) * m, cudaMemcpyDeviceToHost, sm));
             }
-        } else if (ctx->precision == PIC_FP64) {
+        } else {
             for (int a = 0; a < 3; ++a) {
                 if (a < g.ndim) CK(cudaMemcpyAsync(P + a * n, S.s64.x[a], sizeof(double) * n, cudaMemcpyDeviceToHost, sm));
                 CK(cudaMemcpyAsync(P + (3 + a) * n, S.s64.u[a], sizeof(double) * n, cudaMemcpyDeviceToHost, sm));

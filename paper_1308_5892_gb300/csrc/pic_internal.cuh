@@ -416,8 +416,7 @@ struct SortArgs {
     TileGeom t;
     long long n;
     SpeciesMixed src;
-    int *counts;     // ntiles*cells_per_tile + 1 scratch
-    int *offsets;    // same size: exclusive scan; offsets[key] start of key
+    int *counts;     // ntiles*cells_per_tile + 1 scratch: counts, scanned in place to the cursors
     int *block_sums; // scratch for the scan
     int *tile_start; // ntiles+1 output
     const int *old_tile_start;  // tile offsets of the source layout, or nullptr if untiled
@@ -425,7 +424,12 @@ struct SortArgs {
     int *err;
     int lgw, lgw_src;   // log2 of the walk length of the destination and of the source layout
 };
-void launch_sort(const SortArgs &a, cudaStream_t s);
+// the species of one run (same grid and tiles), one launch per phase
+struct SortPack {
+    SortArgs s[4];
+    int n;
+};
+int launch_sort(const SortPack &a, cudaStream_t s);   // returns the launches
 // The push's work list for the layout of the last sort (see k_push_parts).
 struct PushParts {
     const int *tile_start[4];

@@ -12,6 +12,8 @@
 //
 // Roofline: HBM bound; per particle 4 B (histogram) + 8 B (rank) plus per key
 // 3 x 4 B.  Particle counts are int32 (at most 2^31 - 1 particles per species).
+#include <algorithm>
+
 #include "pic_internal.cuh"
 #include "sort_cells.cuh"
 
@@ -21,47 +23,68 @@ namespace {
 
 // ---- block counts of the phases of one sort ----
 
-inline int blocks_for(long long n, int threads) {
+__host__ __device__ inline int blocks_for(long long n, int threads) {
     long long b = (n + threads - 1) / threads;
     const long long cap = 152LL * 32;
     return (int)(b < 1 ? 1 : (b < cap ? b : cap));
 }
 constexpr int kWalkThreads = 512;
-inline int walk_blocks(const SortArgs &a) { return a.old_tile_start ? a.t.ntiles : blocks_for(a.n, kWalkThreads); }
+__host__ __device__ inline int walk_blocks(const SortArgs &a) { return a.old_tile_start ? a.t.ntiles : blocks_for(a.n, kWalkThreads); }
 inline int key_blocks(const SortArgs &a) { return blocks_for(nkeys_of(a), 256); }
 // The box passes (sort_cells.cuh) take sorted sources whose tile box fits.
-inline bool boxed(const SortArgs &a) { return a.old_tile_start && box_fits(a.t, a.g.ndim); }
+__host__ __device__ inline bool boxed(const SortArgs &a) { return a.old_tile_start && box_fits(a.t, a.g.ndim); }
 
-// ---- one sort: one launch per phase ----
+// ---- one run: one launch per phase ----
 
-template <int NDIM, bool RANK>
-__global__ void __launch_bounds__(kWalkThreads, 3) k_box(const __grid_constant__ SortArgs a) {
-    __shared__ int box[box_max<NDIM>()];
-    box_body<NDIM, kWalkThreads, RANK>(a, blockIdx.x, 0, 1, box);
+// blockIdx.y is the species of the run.
+
+__global__ void k_zero(const __grid_constant__ SortPack a) {
+    zero_body(a.s[blockIdx.y].counts, nkeys_of(a.s[blockIdx.y]), blockIdx.x, gridDim.x);
 }
 
-template <int NDIM>
-__global__ void k_histogram(SortArgs a) {
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x, a.lgw_src};
-    histogram_body<NDIM, 4>(a, w, nkeys_of(a));
+// Histogram (RANK false) or rank pass; ONE: of the first species alone.
+template <int NDIM, bool RANK, bool ONE>
+__global__ void __launch_bounds__(kWalkThreads, 3) k_keys(const __grid_constant__ SortPack pack) {
+    const SortArgs &a = pack.s[ONE ? 0 : blockIdx.y];
+    const int nb = walk_blocks(a);
+    if (a.n == 0 || (int)blockIdx.x >= nb) return;
+    if (boxed(a)) {
+        __shared__ int box[box_max<NDIM>()];
+        box_body<NDIM, kWalkThreads, RANK>(a, blockIdx.x, 0, 1, box);
+        return;
+    }
+    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, nb, a.lgw_src};
+    if (RANK) rank_body<NDIM, 4>(a, w, nkeys_of(a));
+    else histogram_body<NDIM, 4>(a, w, nkeys_of(a));
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(SortArgs a) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(const __grid_constant__ SortPack pack) {
     __shared__ int sh[33];
-    scan_blocks_body<kScanThreads>(a.counts, a.offsets, a.block_sums, nkeys_of(a), blockIdx.x, sh);
+    const SortArgs &a = pack.s[blockIdx.y];
+    scan_blocks_body<kScanThreads>(a.counts, a.counts, a.block_sums, nkeys_of(a), blockIdx.x, sh);
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(SortArgs a) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const __grid_constant__ SortPack pack) {
     __shared__ int sh[33];
+    const SortArgs &a = pack.s[blockIdx.y];
     scan_sums_body<kScanThreads>(a.block_sums, scan_blocks(a), sh);
 }
 
-__global__ void k_scan_finish(SortArgs a) { scan_finish_body(a, nkeys_of(a), blockIdx.x, gridDim.x); }
-
-template <int NDIM>
-__global__ void k_rank(SortArgs a) {
-    const SrcWalk w{a.old_tile_start, a.n, (int)blockIdx.x, (int)gridDim.x, a.lgw_src};
-    rank_body<NDIM, 4>(a, w, nkeys_of(a));
+// Blocks of kScanTile keys.  With few blocks (kFewBlocks) the sums are not scanned by a
+// launch of their own: every block adds up those before it.
+constexpr int kFewBlocks = kScanThreads;
+__global__ void __launch_bounds__(kScanThreads) k_scan_finish(const __grid_constant__ SortPack pack) {
+    __shared__ int sh[33];
+    const SortArgs &a = pack.s[blockIdx.y];
+    const int b = blockIdx.x;
+    int sum;
+    if (gridDim.x <= kFewBlocks) {
+        int v[kScanTile / kScanThreads] = {(int)threadIdx.x < b ? a.block_sums[threadIdx.x] : 0};
+        sum = block_scan<kScanThreads>(v, sh);
+    } else sum = a.block_sums[b];
+    const long long nkeys = nkeys_of(a), k0 = (long long)b * kScanTile;
+    for (long long i = k0 + threadIdx.x; i < min(k0 + kScanTile, nkeys); i += kScanThreads) scan_finish_one(a, i, sum);
+    if (b == 0 && threadIdx.x == 0) a.tile_start[a.t.ntiles] = (int)a.n;
 }
 
 // Work list of the push: every tile that holds particles, cut into parts of at most
@@ -139,7 +162,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_blocks_multi(const SortAr
     __shared__ int sh[33];
     const int s = find_sort(prefix, nsort, blockIdx.x);
     const SortArgs &a = as[s];
-    scan_blocks_body<kScanThreads>(a.counts, a.offsets, a.block_sums, nkeys_of(a), blockIdx.x - prefix[s], sh);
+    scan_blocks_body<kScanThreads>(a.counts, a.counts, a.block_sums, nkeys_of(a), blockIdx.x - prefix[s], sh);
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums_multi(const SortArgs *as) {
@@ -170,21 +193,43 @@ __global__ void __launch_bounds__(kWalkThreads) k_rank_multi(const SortArgs *as,
 
 size_t sort_scan_scratch(long long nkeys) { return (size_t)((nkeys + kScanTile - 1) / kScanTile + 1); }
 
-void launch_sort(const SortArgs &a, cudaStream_t s) {
-    cudaMemsetAsync(a.counts, 0, sizeof(int) * nkeys_of(a), s);
-    if (a.n > 0) {
-        if (boxed(a)) (a.g.ndim == 3 ? k_box<3, false> : k_box<2, false>)<<<a.t.ntiles, kWalkThreads, 0, s>>>(a);
-        else if (a.g.ndim == 3) k_histogram<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
-        else k_histogram<2><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
+constexpr long long kApart = 1 << 25;
+int launch_sort(const SortPack &a, cudaStream_t s) {
+    const SortArgs &a0 = a.s[0];
+    int nw = 0;
+    long long most = 0;
+    for (int q = 0; q < a.n; ++q) {
+        nw = std::max(nw, a.s[q].n > 0 ? walk_blocks(a.s[q]) : 0);
+        most = std::max(most, a.s[q].n);
     }
-    k_scan_blocks<<<scan_blocks(a), kScanThreads, 0, s>>>(a);
-    k_scan_sums<<<1, kScanThreads, 0, s>>>(a);
-    k_scan_finish<<<key_blocks(a), 256, 0, s>>>(a);
-    if (a.n > 0) {
-        if (boxed(a)) (a.g.ndim == 3 ? k_box<3, true> : k_box<2, true>)<<<a.t.ntiles, kWalkThreads, 0, s>>>(a);
-        else if (a.g.ndim == 3) k_rank<3><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
-        else k_rank<2><<<walk_blocks(a), kWalkThreads, 0, s>>>(a);
-    }
+    const int nb = scan_blocks(a0);
+    int launches = 3;
+    // one launch for all species fills the GPU better; large ones each have a launch of their
+    // own, whose arguments are at fixed places (128^3, 2 x 67M particles: 1.72 against 1.86 ms a
+    // sort; 64^3, 2 x 8.4M: 0.35 against 0.30; 45 x 37 x 51, 2 x 1.7M: 0.125 against 0.092)
+    auto keys = [&](auto one, auto all) {
+        if (nw == 0) return;
+        if (most <= kApart) {
+            all<<<dim3(nw, a.n), kWalkThreads, 0, s>>>(a);
+            ++launches;
+            return;
+        }
+        for (int q = 0; q < a.n; ++q) {
+            SortPack p{};
+            p.n = 1;
+            p.s[0] = a.s[q];
+            if (a.s[q].n > 0) one<<<walk_blocks(a.s[q]), kWalkThreads, 0, s>>>(p), ++launches;
+        }
+    };
+    k_zero<<<dim3(key_blocks(a0), a.n), 256, 0, s>>>(a);
+    if (a0.g.ndim == 3) keys(k_keys<3, false, true>, k_keys<3, false, false>);
+    else keys(k_keys<2, false, true>, k_keys<2, false, false>);
+    k_scan_blocks<<<dim3(nb, a.n), kScanThreads, 0, s>>>(a);
+    if (nb > kFewBlocks) k_scan_sums<<<dim3(1, a.n), kScanThreads, 0, s>>>(a);
+    k_scan_finish<<<dim3(nb, a.n), kScanThreads, 0, s>>>(a);
+    if (a0.g.ndim == 3) keys(k_keys<3, true, true>, k_keys<3, true, false>);
+    else keys(k_keys<2, true, true>, k_keys<2, true, false>);
+    return launches + (nb > kFewBlocks ? 1 : 0);
 }
 
 void launch_push_parts(const PushParts &a, cudaStream_t s) { k_push_parts<<<1, kScanThreads, 0, s>>>(a); }

@@ -272,7 +272,7 @@ __device__ inline int block_scan(int (&v)[kScanTile / THREADS], int *sh) {
     return total;
 }
 
-// Scan of block b's kScanTile counts into offsets; the block total goes to block_sums[b].
+// Scan of block b's kScanTile counts (out may be in); the block total goes to block_sums[b].
 template <int THREADS>
 __device__ inline void scan_blocks_body(const int *in, int *out, int *block_sums, long long n, int b, int *sh) {
     constexpr int kScanItems = kScanTile / THREADS;
@@ -305,18 +305,19 @@ __device__ inline void scan_sums_body(int *block_sums, int nb, int *sh) {
     }
 }
 
-// Add block offsets; copy to the cursors (counts array); extract tile offsets.
-__device__ inline void scan_finish_body(const SortArgs &a, long long nkeys, int b, int nb) {
-    for (long long i = (long long)b * blockDim.x + threadIdx.x; i < nkeys; i += (long long)nb * blockDim.x) {
-        int v = a.offsets[i] + a.block_sums[i / kScanTile];
-        if (v < 0 || v > a.n) {   // counts inconsistent with the particles: flag, keep offsets in range
-            atomicOr(a.err, ERR_SORT);
-            v = v < 0 ? 0 : (int)a.n;
-        }
-        a.offsets[i] = v;
-        a.counts[i] = v;
-        if (i % a.t.cells_per_tile == 0) a.tile_start[i / a.t.cells_per_tile] = v;
+// Add block offsets to the scanned counts (the cursors); extract tile offsets.
+__device__ inline void scan_finish_one(const SortArgs &a, long long i, int sum) {
+    int v = a.counts[i] + sum;
+    if (v < 0 || v > a.n) {   // counts inconsistent with the particles: flag, keep offsets in range
+        atomicOr(a.err, ERR_SORT);
+        v = v < 0 ? 0 : (int)a.n;
     }
+    a.counts[i] = v;
+    if (i % a.t.cells_per_tile == 0) a.tile_start[i / a.t.cells_per_tile] = v;
+}
+__device__ inline void scan_finish_body(const SortArgs &a, long long nkeys, int b, int nb) {
+    for (long long i = (long long)b * blockDim.x + threadIdx.x; i < nkeys; i += (long long)nb * blockDim.x)
+        scan_finish_one(a, i, a.block_sums[i / kScanTile]);
     if (b == 0 && threadIdx.x == 0) a.tile_start[a.t.ntiles] = (int)a.n;
 }
 

@@ -152,7 +152,7 @@ __device__ void sort_item(const SortArgs &a, int kind, int local, int nitems, in
         const SrcWalk sw{a.old_tile_start, a.n, local, nitems, a.lgw_src, walk_tile_parts(a)};
         histogram_body<NDIM, 8>(a, sw, nkeys);
     } else if (kind == S_SCAN_BLOCKS) {
-        scan_blocks_body<THREADS>(a.counts, a.offsets, a.block_sums, nkeys, local, sh);
+        scan_blocks_body<THREADS>(a.counts, a.counts, a.block_sums, nkeys, local, sh);
     } else if (kind == S_SCAN_SUMS) {
         scan_sums_body<THREADS>(a.block_sums, scan_blocks(a), sh);
     } else if (kind == S_SCAN_FINISH) {
