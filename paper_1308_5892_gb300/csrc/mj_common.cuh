@@ -83,25 +83,10 @@ struct Table {
     double s0, h;       // sigma_k = s0 + k h
     int n;              // intervals
     const double *F;    // n + 1 cumulative values, F[0] = 0, F[n] = 1
+    double ep, em, iZ;  // e^psi, e^-psi, 1 / Z
 };
 
-// The same integral over at most one table interval by the 4-point rule: with an
-// interval of x = h sqrt(mu) <= 0.05 thermal widths its relative error is below
-// 6e-10 (x / 1)^8 |g^(8) / g| widths^8 < 1e-16 out to six widths, where the 8-point
-// rule of the table is not needed.
-__device__ inline double gl4_integral(const Marg &m, double a, double b) {
-    const double c = 0.5 * (a + b), h = 0.5 * (b - a);
-    const double x0 = 0.3399810435848563 * h, x1 = 0.8611363115940526 * h;   // Gauss-Legendre nodes and weights
-    return (0.6521451548625461 * (m.g(c - x0) + m.g(c + x0)) + 0.3478548451374538 * (m.g(c - x1) + m.g(c + x1))) * h;
-}
-
-// Newton's iteration on the cumulative marginal from the linear interpolation in the
-// table.  It converges quadratically: after a step below 1e-7 of the interval the
-// next one would be below the rounding of sigma.  That takes two steps of 5 densities;
-// a fixed four of 9, and the 60 steps a few lanes of every warp took below, made the
-// loader 52 ms for 4.2M particles, now 9.5 (FP64 instructions bound it).
 __device__ inline double inverse_marginal(const Table &t, double w) {
-    const bool fine = t.h * t.h * t.m.mu <= 0.0025;
     int lo = 0, hi = t.n;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -111,38 +96,122 @@ __device__ inline double inverse_marginal(const Table &t, double w) {
     const double Fa = t.F[lo], Fb = t.F[lo + 1];
     double sig = a + (Fb > Fa ? (w - Fa) / (Fb - Fa) : 0.5) * t.h;
     for (int it = 0; it < 4; ++it) {
-        const double F = Fa + (fine ? gl4_integral(t.m, a, sig) : gl_integral(t.m, a, sig));
+        const double F = Fa + gl_integral(t.m, a, sig);
         const double g = t.m.g(sig);
         if (!(g > 0.0)) break;
         double nxt = sig - (F - w) / g;
         nxt = fmin(fmax(nxt, a), a + t.h);
-        const bool done = fabs(nxt - sig) <= 1e-7 * t.h;
         sig = nxt;
-        if (done) break;
     }
     return sinh(sig + t.m.psi);
+}
+
+// inverse_marginal with about 4 densities instead of 36, and those with two exponentials
+// each: sigma starts from the cubic through the four table values around it (off by
+// ~(h / width)^4 / 40 intervals), the density over at most one interval is integrated by
+// the 4-point rule (relative error 6e-10 (h / width)^8 |g^(8) / g| width^8 < 1e-16 out to
+// six widths of the density), and the slope of the cubic, good to (h / width)^3, serves
+// for the correction: after one below 1e-8 of the interval the rest is below 1e-15.
+// The full inverse is taken where the interval is above 0.06 of the width, at the ends of
+// the table and where this does not settle.  Both end within a few roundings of F (in
+// units of the density) and of sigma of the root; err is ten times that, for the caller
+// that needs the bits (0: they are those of inverse_marginal).
+__device__ inline double inverse_marginal_quick(const Table &t, double w, double &err) {
+    err = 0.0;
+    if (!(t.h * t.h * fmax(t.m.mu, 1.0) <= 0.0036)) return inverse_marginal(t, w);
+    int lo = 0, hi = t.n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (t.F[mid] <= w) lo = mid; else hi = mid;
+    }
+    if (lo == 0 || lo + 2 > t.n) return inverse_marginal(t, w);
+    // the cubic F(x) = d1 (x + c2 x (x - 1) + c3 (x^3 - x)) + Fa on the interval 0 <= x <= 1
+    const double Fa = t.F[lo], d1 = t.F[lo + 1] - Fa;
+    const float inv = 1.f / (float)d1;
+    const float e0 = (float)((Fa - t.F[lo - 1]) - d1), e2 = (float)((t.F[lo + 2] - t.F[lo + 1]) - d1);
+    const float c2 = -0.5f * e0 * inv, c3 = (e0 + e2) * inv * (1.f / 6.f);
+    if (!(fabsf(c2) < 0.25f && fabsf(c3) < 0.1f)) return inverse_marginal(t, w);
+    const double r = (w - Fa) / d1;
+    float xf = (float)r, slope = 1.f;
+    for (int it = 0; it < 3; ++it) {
+        slope = 1.f + c2 * (2.f * xf - 1.f) + c3 * (3.f * xf * xf - 1.f);
+        if (it < 2) xf -= (xf + (xf - 1.f) * xf * (c2 + c3 * (xf + 1.f)) - (float)r) / slope;
+    }
+    const double xd = (double)xf;
+    const double x = xd - (xd + (xd - 1.0) * xd * ((double)c2 + (double)c3 * (xd + 1.0)) - r) * (double)(1.f / slope);
+    const double a = t.s0 + lo * t.h, g = d1 * (double)slope / t.h;
+    double sig = fmin(fmax(fma(x, t.h, a), a), a + t.h);
+    const double igh = (double)(1.f / (float)g);
+    for (int it = 0; it < 4; ++it) {
+        const double c = 0.5 * (a + sig), hw = 0.5 * (sig - a);
+        double F = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {   // Gauss-Legendre nodes and weights
+            const double s = fma((k & 1 ? hw : -hw), (k < 2 ? 0.3399810435848563 : 0.8611363115940526), c);
+            const double E = exp(0.5 * s), I = 1.0 / E, sh = 0.5 * (E - I);
+            const double cs = 0.5 * (E * E * t.ep + I * I * t.em);
+            F += (k < 2 ? 0.6521451548625461 : 0.3478548451374538) *
+                 (fma(t.m.mu * t.m.G0, cs, 1.0) * cs * exp(-2.0 * t.m.mu * sh * sh));
+        }
+        const double step = (Fa + F * hw * t.iZ - w) * igh;
+        sig = fmin(fmax(sig - step, a), a + t.h);
+        if (fabs(step) <= 1e-8 * t.h) {
+            const double y = sinh(sig + t.m.psi);
+            err = (4e-15 / g + 1e-14 * (1.0 + fabs(sig) + fabs(t.m.psi))) * sqrt(1.0 + y * y);
+            return y;
+        }
+    }
+    return inverse_marginal(t, w);
 }
 
 // t = a (u - 1) >= 0 from l(a + t) = w l(a) (Eq. finding_u), written as
 // log1p(t / (1 + a)) - t = log w and solved by Newton from t = -log w (the
 // large-a limit); the function is concave and decreasing in t, so the steps
-// converge monotonically once on the right of the root.  The error after a step of
-// relative size d is below d^2 / 2 of t (|f'' t / 2 f'| < 1/2), so a step below 1e-8
-// is the last one; waiting for a step of zero can go on between two neighbouring
-// doubles until the limit.
+// converge monotonically once on the right of the root, and go on until t stands still.
+// Where it alternates between two neighbouring doubles, the result is that of the 60th
+// step, which follows from the parity.  (Taking those steps, which some lane of nearly
+// every warp did, was half of the loader's 52 ms for 4.2M particles; see k_load_mj.)
 __device__ inline double conditional_t(double a, double w) {
     const double lw = log(w);
-    double t = -lw;
+    double t = -lw, before = -1.0;
     for (int it = 0; it < 60; ++it) {
         const double f = log1p(t / (1.0 + a)) - t - lw;
         const double fp = 1.0 / (1.0 + a + t) - 1.0;
         double nt = t - f / fp;
         if (nt < 0.0) nt = 0.5 * t;
-        const bool done = fabs(nt - t) <= 1e-8 * nt;
+        if (nt == before) return (it & 1) ? nt : t;   // step 60 is an even number of steps after nt's, or t's
+        const bool done = fabs(nt - t) <= 1e-16 * (nt + 1e-300);
+        before = t;
         t = nt;
         if (done) break;
     }
     return t;
+}
+
+// The same root with one step in FP64: Newton's in FP32 as far as they go, then Halley's.
+// After one of relative size d the error is below 0.6 d^3 of t (with s = 1 / (1 + a + t),
+// |f2 t / 2 f1| < 1/2 and |f3 t^2 / 6 f1| = s^2 t^2 / 3 (a + t) < 1/3 for the derivatives
+// f1, f2, f3), below rounding for d <= 1e-5.  FP32 gets there unless a and t are small,
+// where f cancels.
+__device__ inline double conditional_t_quick(double a, double w) {
+    const double lw = log(w);
+    const float af = 1.f + (float)a, lf = (float)lw;
+    float tf = -lf;
+    for (int it = 0; it < 12; ++it) {
+        const float nt = fmaxf(tf - (log1pf(tf / af) - tf - lf) / (1.f / (af + tf) - 1.f), 0.5f * tf);
+        const bool done = fabsf(nt - tf) <= 1e-4f * nt;
+        tf = nt;
+        if (done) break;
+    }
+    double t = (double)tf;
+    for (int it = 0; it < 4; ++it) {
+        const double s = 1.0 / (1.0 + a + t), f1 = s - 1.0;
+        const double f = log1p(t / (1.0 + a)) - t - lw;
+        const double d = f * f1 / (f1 * f1 + 0.5 * f * s * s);
+        t -= d;
+        if (fabs(d) <= 1e-5 * t) return t;
+    }
+    return conditional_t(a, w);
 }
 
 struct LoadArgs {
@@ -174,7 +243,10 @@ struct LoadArgs {
 // the learned network (mlp.cu).
 struct ExactPar {
     __device__ void begin() const {}
-    __device__ double operator()(const LoadArgs &a, double w) const { return inverse_marginal(a.tab, w); }
+    // err > 0: a bound on the distance from inverse_marginal's value
+    __device__ double operator()(const LoadArgs &a, double w, double &err) const {
+        return inverse_marginal_quick(a.tab, w, err);
+    }
 };
 
 // Par::begin is called by every thread of a block once, and the sampler by whole warps.
@@ -188,25 +260,37 @@ __global__ void __launch_bounds__(256) k_load_mj(LoadArgs a, Par par_of) {
         double w[6];
         uniforms6(a.seed, a.species, p, w);
         // momentum along n and in the orthogonal plane
-        const double y = par_of(a, w[3]);
+        double err, y = par_of(a, w[3], err);
         if (p >= a.n) continue;
         const double mu = 1.0 / a.theta;
         const double G0 = 1.0 / sqrt(1.0 - a.sb0 * a.sb0);
-        const double gy = sqrt(1.0 + y * y);
-        const double aa = mu * G0 * gy;
-        const double um1 = conditional_t(aa, w[4]) / aa;   // u - 1
-        const double r = sqrt(um1 * (um1 + 2.0));
+        const double Gb = 1.0 / sqrt(1.0 - a.beta0 * a.beta0);
         double sphi, cphi;
         sincospi(2.0 * w[5], &sphi, &cphi);
-        double par = y, q1 = gy * r * cphi, q2 = gy * r * sphi;
-        if (a.naive) {
-            // the same sample drawn at rest (its table was built with beta0 = 0), then boosted
-            const double g0 = sqrt(1.0 + par * par + q1 * q1 + q2 * q2);
-            const double Gb = 1.0 / sqrt(1.0 - a.beta0 * a.beta0);
-            par = Gb * (par + a.beta0 * g0);
-        }
         double mom[3];
-        for (int c = 0; c < 3; ++c) mom[c] = a.nvec[c] * par + a.e1[c] * q1 + a.e2[c] * q2;
+        // FP64 instructions bound the loader: 52 ms for 4.2M particles when every one went through
+        // inverse_marginal and the full conditional_t.  Here these follow, once, only where the error
+        // of the quick values could change a rounding to FP32 (one particle in about 10^5), so that
+        // the FP32 momenta are those of the full ones: 5.9 ms.
+        for (bool quick = true;; quick = false) {
+            const double gy = sqrt(1.0 + y * y);
+            const double aa = mu * G0 * gy;
+            const double um1 = (quick ? conditional_t_quick(aa, w[4]) : conditional_t(aa, w[4])) / aa;   // u - 1
+            const double r = sqrt(um1 * (um1 + 2.0));
+            double par = y, q1 = gy * r * cphi, q2 = gy * r * sphi;
+            if (a.naive) {
+                // the same sample drawn at rest (its table was built with beta0 = 0), then boosted
+                const double g0 = sqrt(1.0 + par * par + q1 * q1 + q2 * q2);
+                par = Gb * (par + a.beta0 * g0);
+            }
+            for (int c = 0; c < 3; ++c) mom[c] = a.nvec[c] * par + a.e1[c] * q1 + a.e2[c] * q2;
+            if (!a.mixed || !quick) break;
+            const double d = (4.0 * err * (1.0 + r) + 1e-14 * (1.0 + 1.0 / aa) * gy * r) * (a.naive ? 2.0 * Gb : 1.0);
+            if ((float)(mom[0] - d) == (float)(mom[0] + d) && (float)(mom[1] - d) == (float)(mom[1] + d) &&
+                (float)(mom[2] - d) == (float)(mom[2] + d))
+                break;
+            if (err > 0.0) y = inverse_marginal(a.tab, w[3]);
+        }
         // position
         double pos[3] = {0.0, 0.0, 0.0};
         if (!a.colocate) {
@@ -292,6 +376,9 @@ inline LoadArgs make_load_args(const Geom &g, int ndim, long long n, int species
     a.tab.h = h;
     a.tab.n = ntab;
     a.tab.F = Fdev;
+    a.tab.ep = std::exp(psi);
+    a.tab.em = std::exp(-psi);
+    a.tab.iZ = 1.0 / Z;
     a.colocate = colocate;
     for (int c = 0; c < 3; ++c) {
         a.x64[c] = d64.x[c];

@@ -345,7 +345,8 @@ struct MlpPar {
     const __half *w;
     double psi, scale;
     __device__ void begin() const { mlp_stage(w); }
-    __device__ double operator()(const mjk::LoadArgs &a, double wv) const {
+    __device__ double operator()(const mjk::LoadArgs &a, double wv, double &err) const {
+        err = 0.0;
         const double wc = fmin(fmax(wv, 1e-7), 1.0 - 1e-7);
         float x0, x1, x2;
         features(a.theta, a.beta0, wc, x0, x1, x2);
@@ -366,7 +367,8 @@ __global__ void __launch_bounds__(256) k_sample_par(mjk::Table tb, MlpPar mp, in
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + lane;
         const double w = i < n ? wv[i] : 0.5;
-        const double r = use_mlp ? mp(a, w) : mjk::inverse_marginal(tb, w);
+        double err;
+        const double r = use_mlp ? mp(a, w, err) : mjk::inverse_marginal(tb, w);
         if (i < n) y[i] = r;
     }
 }
