@@ -873,6 +873,21 @@ void make_parts(pic_ctx *ctx, Run &r) {
     launch_push_parts(a, ctx->stream);
 }
 
+// Push items per tile of run r in the step walker: parts of about 1/8 of a resident CTA's
+// share of all particles, at most 32768 (a part costs a staging and a flush, a few us).
+// Whole tiles of a dense run (256 particles per cell and species, 262144 in a 32 x 16
+// tile) take a CTA 3 ms, longer than the step of a 16-run ensemble should be.
+int walk_push_parts(const pic_ctx *ctx, const Run &r) {
+    long long all = 0, n = 0;
+    for (const Run &q : ctx->runs)
+        for (int k = 0; k < q.d.nspecies; ++k) all += q.sp[k].n;
+    for (int k = 0; k < r.d.nspecies; ++k) n += r.sp[k].n;
+    const int slots = 152 * (r.d.ndim == 3 ? 1 : 2);
+    const long long size = std::min(32768LL, std::max(1024LL, all / (8 * slots)));
+    const long long per_tile = (n + r.t.ntiles - 1) / r.t.ntiles;
+    return (int)std::max(1LL, std::min(64LL, (per_tile + size / 2) / size));
+}
+
 SortArgs sort_args(pic_ctx *ctx, Run &r, SpeciesState &S, int lgw) {
     SortArgs a;
     a.g = r.g;
@@ -1092,6 +1107,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
     for (int i = 0; i < nr; ++i) {
         Run &r = ctx->runs[i];
         ctx->h_args[i] = mixed_args(ctx, r);
+        ctx->h_args[i].walk_parts = walk_push_parts(ctx, r);
         ctx->h_fp[i] = field_run(r);
     }
     CK(cudaMemcpyAsync(ctx->multi_args, host_src(ctx, slot, soff, ctx->h_args.data(), sizeof(MixedStepArgs) * nr),
@@ -1128,19 +1144,19 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
                 return (is_due[i] && w.species[ph] < r.d.nspecies)
                            ? walk_sort_items(ctx->h_walk_sort[4 * i + w.species[ph]], w.kind[ph], cpi) : 0;
             switch (w.kind[ph]) {
-            case W_PUSH: return r.t.ntiles;
+            case W_PUSH: return r.t.ntiles * ctx->h_args[i].walk_parts;
             case W_SMOOTH_FOLD: return r.smooth > 0 ? (int)((ncell + cpi - 1) / cpi) : 0;
             case W_SMOOTH_PASS: return r.smooth > w.pass[ph] ? (int)((ncell + cpi - 1) / cpi) : 0;
             default: return (int)((r.g.pcells + cpi - 1) / cpi);
             }
         };
         int *prefix = ctx->h_walk.data(), *base = prefix + np * nr + 1, *order = base + nr * (np + 1);
-        // slots of a phase: runs by decreasing particles per tile (the longest push items first)
+        // slots of a phase: runs by decreasing particles per push item (the longest first)
         std::vector<double> load(nr, 0.0);
         for (int i = 0; i < nr; ++i) {
             const Run &r = ctx->runs[i];
             for (int q = 0; q < r.d.nspecies; ++q) load[i] += (double)r.sp[q].n;
-            load[i] /= std::max(1, r.t.ntiles);
+            load[i] /= std::max(1, r.t.ntiles * ctx->h_args[i].walk_parts);
             order[i] = i;
         }
         std::stable_sort(order, order + nr, [&](int a, int b) { return load[a] > load[b]; });

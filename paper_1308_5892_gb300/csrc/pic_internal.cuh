@@ -324,6 +324,7 @@ struct MixedStepArgs {
     const int2 *parts;              // work list of the push (k_push_parts), null: one CTA per tile
     const int *nparts;              // its length
     int parts_bound;                // grid of the launch: a bound of that length, or the tile count
+    int walk_parts;                 // step walker: push items per tile
     float h[4];                     // (q/e)(m_e/m)
     float sgn[4];                   // sign of the charge
     double m_over_me[4];

@@ -5,8 +5,8 @@
 // gather-push-deposit, the optional current smoothing (step 10), e advance with the
 // folded current.
 //
-// Work queue.  The items of phase ph of run r are the tiles of the run (push,
-// and parts of the old layout's tiles for the sort's histogram and rank),
+// Work queue.  The items of phase ph of run r are parts of the tiles of the run (push;
+// walk_push_parts) and of the old layout's tiles (the sort's histogram and rank),
 // chunks of cells_per_item cells or keys (field, smoothing, zeroing and
 // scan-finish phases), or scan blocks of 4096 keys.  The queue order is phase-major; inside a phase the runs with the
 // most particles per tile come first, so the longest items do not start last.
@@ -218,7 +218,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_walk(const __grid_constant__ 
                 __syncthreads();
                 if (threadIdx.x == 0) args_sh.use_tma = 0;
                 __syncthreads();
-                push_tile<NDIM, THREADS, WALLS, MOVE, CT>(args_sh, local, 0, 1, w.push + r);
+                const int parts = args_sh.walk_parts, tile = local / parts;
+                push_tile<NDIM, THREADS, WALLS, MOVE, CT>(args_sh, tile, local - tile * parts, parts, w.push + r);
             } else {
                 const FieldRunF *fsrc = w.fp + r;
                 const int *src = reinterpret_cast<const int *>(fsrc);
