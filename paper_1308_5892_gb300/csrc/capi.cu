@@ -838,14 +838,18 @@ pic_status read_err(pic_ctx *ctx) {
 // more finely; with few particles the longest walk is the kernel's time.  Push per step,
 // walks of 32 / 16 / 8 / 4: 128^3 (134M particles) 5.19 / 5.06 / 5.45 / 6.22 ms, 1024^2
 // (105M) 2.38 / 2.45 / 2.49 / 2.87; 45 x 37 x 51 (3.4M) 248 / 222 / 181 / 180 us, 251 x 130
-// sheet (0.7M) 87 / 71 / 58 / 52; 64^2 (0.13M), walks of 4 / 2 / 1: 18.7 / 16.4 / 18.8.
+// sheet (0.7M) 87 / 71 / 58 / 50; 64^2 (0.13M), walks of 4 / 2 / 1: 18.7 / 16.4 / 18.2;
+// 128^2 of 0.66M, 8 / 4 / 2: 46 / 39 / 43, of 0.26M, 4 / 2 / 1: 26 / 22 / 25; 256^2 of 1.05M,
+// 16 / 8 / 4: 76 / 52 / 52; 512^2 of 4.2M, 32 / 16: 190 / 128 (2.4K warps: a second round of
+// blocks for a few of them doubles the time).
 int push_walk_lg(const pic_ctx *ctx) {
     long long n = 0;
     for (const Run &r : ctx->runs)
         for (int q = 0; q < r.d.nspecies; ++q) n += r.sp[q].n;
+    static const int least2[6] = {0, 2048, 4096, 4096, 4096, 8192};   // blocks of 32 walks in all
     const bool d3 = ctx->runs[0].d.ndim == 3;
     int lg = d3 ? 4 : 5;
-    while (lg > 0 && (n >> (5 + lg)) < (d3 ? 8192 : 2048)) --lg;
+    while (lg > 0 && (n >> (5 + lg)) < (d3 ? 8192 : least2[lg])) --lg;
     return lg;
 }
 
@@ -960,6 +964,10 @@ MixedStepArgs mixed_args(pic_ctx *ctx, Run &r) {
     a.dt = (float)r.d.dt;
     a.hist = hist_ref(r);
     a.kin0 = r.hist_n == 0 ? 1 : 0;
+    // The rest of a tile after its full blocks in small items: they even out the warps of a CTA
+    // at its end (512^2, items of 1 / 2 / 4 / 16 rows: 627 / 617 / 616 / 645 us per step; 256^2
+    // of 8 particles per cell 84 / 85 / 94 / 100).
+    a.tail_lg = 1;
     a.err = ctx->d_err;
     a.use_tma = r.tma ? 1 : 0;
     a.tmA = r.tmA;
@@ -1108,6 +1116,7 @@ pic_status step_multi(pic_ctx *ctx, int slot) {
         Run &r = ctx->runs[i];
         ctx->h_args[i] = mixed_args(ctx, r);
         ctx->h_args[i].walk_parts = walk_push_parts(ctx, r);
+        ctx->h_args[i].tail_lg = 4;   // (other CTAs fill the gaps: 2 / 8 / 16 rows 2582 / 2508 / 2468 us per step)
         ctx->h_fp[i] = field_run(r);
     }
     CK(cudaMemcpyAsync(ctx->multi_args, host_src(ctx, slot, soff, ctx->h_args.data(), sizeof(MixedStepArgs) * nr),

@@ -325,6 +325,7 @@ struct MixedStepArgs {
     const int *nparts;              // its length
     int parts_bound;                // grid of the launch: a bound of that length, or the tile count
     int walk_parts;                 // step walker: push items per tile
+    int tail_lg;                    // 2D: log2 of the rows per work item after a tile's last full block
     float h[4];                     // (q/e)(m_e/m)
     float sgn[4];                   // sign of the charge
     double m_over_me[4];

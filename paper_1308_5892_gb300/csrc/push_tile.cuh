@@ -38,8 +38,8 @@
 //    the particles (2 x 67M on 128^3: 3.1 ms a sort).
 // Work of a warp: blocks of 32 W particles (W = 32; less for few particles, see
 // push_walk_lg), which the sort stores transposed, so lane a walks W consecutive
-// cell-sorted particles (and keeps
-// their start-cell current in registers until its cell changes) while one
+// cell-sorted particles (and keeps their start-cell current in registers until its
+// cell changes) while one
 // load instruction still reads one contiguous 128-byte row.  The pieces of a
 // path after a node-plane crossing are queued per warp and deposited 32 at a
 // time by all lanes together.
@@ -504,17 +504,17 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     const unsigned lt_mask = (1u << lane) - 1u;
     __shared__ int work_ctr[4];
     __shared__ double kin_sh[2][WARPS];
-    // work items of species sp: blocks, then 32-particle chunks of the tail; this part's share
-    auto item_range = [&](int sp, int &nblk, int &beg, int &end) {
-        const int nt = a.tile_start[sp][tile + 1] - a.tile_start[sp][tile], lgb = 5 + a.lgw[sp];
-        nblk = nt >> lgb;
-        const int nall = nblk + ((nt - (nblk << lgb)) + 31) / 32;
+    // work items of species sp, of 2^lgw rows of 32 particles and of 2^lgt at the end; this part's share
+    auto item_range = [&](int sp, int &rows, int &beg, int &end) {
+        const int lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
+        rows = (a.tile_start[sp][tile + 1] - a.tile_start[sp][tile] + 31) >> 5;
+        const int nall = (rows >> lgw) + (((rows & ((1 << lgw) - 1)) + (1 << lgt) - 1) >> lgt);
         beg = (int)((long long)nall * part / parts);
         end = (int)((long long)nall * (part + 1) / parts);
     };
     if ((int)threadIdx.x < a.nspecies) {
-        int nblk, beg, end;
-        item_range(threadIdx.x, nblk, beg, end);
+        int rows, beg, end;
+        item_range(threadIdx.x, rows, beg, end);
         work_ctr[threadIdx.x] = beg;
     }
     if (lane == 0) { kin_sh[0][warp] = 0.0; kin_sh[1][warp] = 0.0; }
@@ -554,9 +554,9 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
         const SpeciesMixed &P = a.sp[sp];
         const float h = a.h[sp], alpha26 = a.sgn[sp] * kFx26;   // deposit prefactor in fixed-point units
         const int pbeg = a.tile_start[sp][tile], pend = a.tile_start[sp][tile + 1];
-        const int lgb = 5 + a.lgw[sp];                   // log2 of a block: 2^lgw particles per lane
-        int nblk, ibeg, nitems;
-        item_range(sp, nblk, ibeg, nitems);
+        const int lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
+        int rows, ibeg, nitems;
+        item_range(sp, rows, ibeg, nitems);
         const int *const perm = MOVE ? a.perm[sp] : nullptr;
         const SpeciesMixed &Q = perm ? a.src[sp] : a.sp[sp];   // where the particles are read
         // source of the particle of iteration j of an item, -1 past its end
@@ -622,10 +622,10 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             if (lane == 0) item = atomicAdd(&work_ctr[sp], 1);
             item = __shfl_sync(kFull, item, 0);
             if (item >= r1) break;
-            // block item: lane walks base + 32k + lane, k = 0..kn-1 (consecutive ranks);
-            // tail chunk: one element per lane in rank order
-            const int base = item < nblk ? pbeg + (item << lgb) : pbeg + (nblk << lgb) + ((item - nblk) << 5);
-            const int kn = item < nblk ? 1 << (lgb - 5) : 1;
+            // the lane walks base + 32k + lane, k = 0..kn-1 (consecutive ranks)
+            const int nfull = rows >> lgw, row = item < nfull ? item << lgw : (nfull << lgw) + ((item - nfull) << lgt);
+            const int base = pbeg + (row << 5);
+            const int kn = item < nfull ? 1 << lgw : min(1 << lgt, rows - row);
             float kin0 = 0.f, kin1 = 0.f;
 #pragma unroll
             for (int j = 0; j < kStages - 1; ++j) issue(base, j, source(base, j, kn));

@@ -30,7 +30,8 @@ def _arrays(ndim, shape, n, seed, dense):
 
 @pytest.mark.parametrize("ndim,shape,n,dense", [
     (2, (40, 24, 1), 5, False), (2, (40, 24, 1), 256, True), (2, (64, 48, 1), 32768, False), (2, (64, 48, 1), 40001, True),
-    (2, (33, 50, 1), 140000, True), (2, (9, 7, 1), 3000, False), (3, (12, 17, 9), 6001, False),
+    (2, (33, 50, 1), 140000, True), (2, (33, 50, 1), 262144 + 77, True), (2, (70, 61, 1), 1100003, False),
+    (2, (70, 61, 1), 4300007, False), (2, (9, 7, 1), 3000, False), (3, (12, 17, 9), 6001, False),
     (3, (24, 16, 16), 70000, True), (3, (24, 16, 16), 262144, False), (3, (5, 4, 6), 20000, False)])
 def test_parts_and_walks_equal_whole_tiles_bitwise(ndim, shape, n, dense):
     f, parts = _arrays(ndim, shape, n, 17 + n, dense)
