@@ -446,19 +446,21 @@ def _e2e(pic, torch, desc, w, seed, args, barrier):
 # FP64 path: particle state read + written per particle-step (x, u as doubles)
 FP64_BYTES_PER_PARTICLE = {2: 80.0, 3: 96.0}
 # FP64 flops per particle-step of k_push_fp64 (dadd + dmul + 2 dfma) and FP64
-# instructions (dadd + dmul + dfma), from ncu instruction counts on the 64^3 and 512^2
-# thermal workloads divided by the particles pushed: 3D 108 + 80 + 86, 2D 58 + 50 + 62
-FP64_FLOPS_PER_PARTICLE = {3: 360.0, 2: 232.0}
-FP64_INST_PER_PARTICLE = {3: 274.0, 2: 170.0}
+# instructions (dadd + dmul + dfma), from ncu instruction counts on a 64^3 (theta 1) and a
+# 300 x 211 (theta 0.1) plasma divided by the particles pushed: 3D 30.0 + 45.2 + 110.8,
+# 2D 17.7 + 22.7 + 72.8
+FP64_FLOPS_PER_PARTICLE = {3: 296.8, 2: 186.0}
+FP64_INST_PER_PARTICLE = {3: 186.0, 2: 113.2}
 # FP32 flops per particle-step of the mixed 3D push (fadd + fmul + 2 ffma: 32.4 + 92.8 +
 # 103.3 per particle, ncu on the 64^3 workload)
 MIXED_FP32_FLOPS_PER_PARTICLE = {3: 331.8}
 # DRAM bytes (read + written) per particle-step of the 3D push kernel, from one
 # ncu capture of the same kernel and tiling (16x8x4, sort interval 3) on the
-# 64^3 case (profiles/push_mixed_thermal3d_64.md: 917.2 MB for 16,777,216
+# 64^3 case (profiles/push_mixed_thermal3d_64.md: 1413.5 MB on the step of a sort,
+# whose push moves the particles, and 1051.5 on the two others, for 16,777,216
 # particles), scaled to a launch by the particles it processes.  None where no
 # capture exists.
-PUSH_TRAFFIC_B_PER_PARTICLE = {3: 917.2e6 / 16777216}
+PUSH_TRAFFIC_B_PER_PARTICLE = {3: (1413.5e6 + 2 * 1051.5e6) / 3 / 16777216}
 PUSH_TRAFFIC_TILING = {3: ([16, 8, 4], 3)}   # (tile, sort interval) of that capture
 
 

@@ -132,8 +132,8 @@ __device__ __forceinline__ void deposit_segment(const R d[3], const R D[3], R al
 // displacement.  There are no data-dependent branches: every candidate value is
 // computed and the right one selected, so the lanes of a warp whose particles cross
 // different planes stay converged.  Both forms compute the same values.  Push per step:
-// 1024^2 2.31 ms by rank, 2.20 by the minimum; 128^3 4.98 by rank, 5.22 by the minimum
-// (more state per axis, which spills).
+// 128^3 4.80 ms by rank, 5.22 by the minimum (more state per axis, which spills); 1024^2 2.20
+// by the minimum, 2.31 by rank and with the longer approximations it had then.
 //
 // 3D: the rank of each crossing is set up once.
 template <typename R>

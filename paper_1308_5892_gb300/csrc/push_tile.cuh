@@ -30,7 +30,7 @@
 //    on the address conflicts that cell-sorted particles cause on every
 //    deposit; integer atomics and the register accumulation below avoid that.)
 //  - particles (packed cell, FP32 offsets, FP32 momenta) are streamed once:
-//    read 24 B (2D) / 28 B (3D) and written back.  Each warp prefetches the
+//    read 24 B (2D) / 32 B with the id (3D) in 16-byte words and written back.  Each warp prefetches the
 //    particles of its next iterations with cp.async into a ring of
 //    shared-memory stages, so the DRAM latency overlaps the arithmetic.  On the
 //    step of a sort the prefetch reads through the sort's permutation from the old

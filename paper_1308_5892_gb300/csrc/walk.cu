@@ -8,8 +8,9 @@
 // Work queue.  The items of phase ph of run r are parts of the tiles of the run (push;
 // walk_push_parts) and of the old layout's tiles (the sort's histogram and rank),
 // chunks of cells_per_item cells or keys (field, smoothing, zeroing and
-// scan-finish phases), or scan blocks of 4096 keys.  The queue order is phase-major; inside a phase the runs with the
-// most particles per tile come first, so the longest items do not start last.
+// scan-finish phases), or scan blocks of 4096 keys.  The queue order is phase-major; inside
+// a phase the runs with the most particles per push item come first, so the longest items
+// do not start last.
 // Resident CTAs take items from one counter.  Before an item of phase ph of
 // run r starts, every item of run r in the phases before ph must be done:
 // thread 0 waits until the run's done counter reaches that count
