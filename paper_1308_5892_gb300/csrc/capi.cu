@@ -96,7 +96,7 @@ struct pic_ctx {
     bool have_alloc = false;
     std::vector<Run> runs;
     int *d_err = nullptr;
-    int *h_err = nullptr;       // page-locked copy for read_err
+    int *h_err = nullptr;       // page-locked copy for read_err (null: pageable)
     void *staging = nullptr;
     size_t staging_bytes = 0;
     double *mj_table = nullptr;     // cumulative marginal of the loader, kMjTable + 1 values
@@ -815,11 +815,11 @@ pic_status io_ready(pic_ctx *ctx) {
 }
 
 pic_status read_err(pic_ctx *ctx) {
-    // (a copy into pageable memory goes through the driver's staging first)
-    if (!ctx->h_err) CK(cudaMallocHost((void **)&ctx->h_err, sizeof(int)));
-    CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    // (a copy into pageable memory goes through a staging buffer of CUDA's first)
+    int word = 0, *const host = ctx->h_err ? ctx->h_err : &word;
+    CK(cudaMemcpyAsync(host, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    const int e = *ctx->h_err;
+    const int e = *host;
     if (e) {
         CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
         if (e & ERR_TIMEOUT) return fail(ctx, PIC_ETIMEOUT, "a bounded device wait gave up");
@@ -1510,6 +1510,10 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
     ctx->runs.resize(nruns);
     ctx->d_err = (int *)dev_alloc(ctx, sizeof(int));
     if (!ctx->d_err) { pic_destroy(ctx); return PIC_ENOMEM; }
+    if (cudaMallocHost((void **)&ctx->h_err, sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->h_err = nullptr;
+    }
     if (cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream) != cudaSuccess) { pic_destroy(ctx); return PIC_ECUDA; }
     size_t stage = 0;
     for (int r = 0; r < nruns; ++r) {
