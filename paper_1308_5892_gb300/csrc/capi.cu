@@ -290,14 +290,17 @@ __device__ inline bool in_domain(const Geom &g, int ax, double x) {
 }
 
 // Validation of an uploaded FP64 particle array (the mixed upload checks as it converts).
+// A position that fails is replaced by 0: the kernels index by cell without a check, and
+// a rejected run stays in its context, whose other runs may go on.
 __global__ void k_check64(Geom g, Species64 s, long long n, int *err) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         for (int a = 0; a < 3; ++a) {
             if (!isfinite(s.u[a][p])) atomicOr(err, ERR_NONFINITE);
             if (a < g.ndim) {
                 const double x = s.x[a][p];
-                if (!isfinite(x)) atomicOr(err, ERR_NONFINITE);
-                else if (!in_domain(g, a, x)) atomicOr(err, ERR_RANGE);
+                if (isfinite(x) && in_domain(g, a, x)) continue;
+                atomicOr(err, isfinite(x) ? ERR_RANGE : ERR_NONFINITE);
+                s.x[a][p] = 0.0;
             }
         }
     }
