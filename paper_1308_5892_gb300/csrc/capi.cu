@@ -825,7 +825,16 @@ pic_status read_err(pic_ctx *ctx) {
     const int e = *host;
     if (e) {
         CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
-        if (e & ERR_TIMEOUT) return fail(ctx, PIC_ETIMEOUT, "a bounded device wait gave up");
+        if (e & ERR_TIMEOUT) {
+            // steps that did not end are in nobody's record: host and device start it again together
+            for (auto &r : ctx->runs) {
+                r.hist_n = 0;
+                CK(cudaMemsetAsync(r.hist, 0, sizeof(double) * 8 * r.hist_cap, ctx->stream));
+                CK(cudaMemsetAsync(r.hist_idx, 0, sizeof(long long), ctx->stream));
+                r.sorted = false;   // the record's first step sorts
+            }
+            return fail(ctx, PIC_ETIMEOUT, "a bounded device wait gave up");
+        }
         if (e & ERR_FAST_MOVE) return fail(ctx, PIC_ESTATE, "a particle moved more than one cell in one step");
         if (e & ERR_SORT) return fail(ctx, PIC_ESTATE, "particle cell outside the grid during sort");
         if (e & ERR_NONFINITE) return fail(ctx, PIC_ENUMERIC, "non-finite value in the state");

@@ -39,7 +39,7 @@ __device__ __forceinline__ void for_cells(const Geom &g, F &&body) {
 template <typename R>
 __global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, HistRef hist, bool carry) {
     double *slot = hist.slot();
-    if (slot && carry && blockIdx.x == 0 && threadIdx.x == 0) slot[0] = slot[-7];
+    if (slot && carry && blockIdx.x == 0 && threadIdx.x == 0 && hist.has_previous()) slot[0] = slot[-7];
     double *energy_acc = slot ? slot + 2 : nullptr;
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for_cells(g, [&](const CellAt &c) { b_advance_cell<R>(g, f, h, c, energy_acc != nullptr, acc); });
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256) k_fields_multi(const FieldRunF *runs, con
     const CellAt c(r.g, in ? p : 0);
     if (PHASE == FIELD_B) {
         double *slot = r.hist.slot();
-        if (slot && r.carry && p == 0) slot[0] = slot[-7];
+        if (slot && r.carry && p == 0 && r.hist.has_previous()) slot[0] = slot[-7];
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         if (in) b_advance_cell<float>(r.g, r.f, h, c, energy_acc != nullptr, acc);

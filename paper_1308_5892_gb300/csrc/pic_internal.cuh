@@ -238,6 +238,9 @@ struct HistRef {
         const long long i = *idx;
         return i < cap ? base + 8 * i : nullptr;
     }
+    // Is the slot before this step's inside the record?  (A step that a timeout ends does not
+    // count, so that steps queued behind it may start the record again.)
+    __device__ inline bool has_previous() const { return !idx || *idx > 0; }
 };
 
 // ---- kernel launchers (implemented in the .cu files) ----

@@ -91,7 +91,7 @@ __device__ void field_item(const WalkArgs &w, int kind, int pass, const FieldRun
     if (kind == W_B) {
         const long long p1 = min(p0 + w.cells_per_item, g.pcells);
         double *slot = fr.hist.slot();
-        if (slot && fr.carry && p0 == 0 && threadIdx.x == 0) slot[0] = __ldcg(slot - 7);
+        if (slot && fr.carry && p0 == 0 && threadIdx.x == 0 && fr.hist.has_previous()) slot[0] = __ldcg(slot - 7);
         double *energy_acc = slot ? slot + 2 : nullptr;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         for (long long p = p0 + threadIdx.x; p < p1; p += THREADS)
