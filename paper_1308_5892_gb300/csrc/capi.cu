@@ -728,12 +728,21 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
             }
             S.perm = (int *)dev_alloc(ctx, sizeof(int) * cap);
             if (!S.perm) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort");
+            // A step that a timeout ends early leaves any of these as they were, and calls after it
+            // index by their contents: everything in them is a valid particle from the start.
+            for (int b = 0; b < 2; ++b) {
+                CK(cudaMemsetAsync(S.mb[b].a, 0, sizeof(float4) * cap, ctx->stream));
+                CK(cudaMemsetAsync(S.mb[b].b, 0, sizeof(float) * (d.ndim == 3 ? 4 : 2) * cap, ctx->stream));
+                if (S.mb[b].id) CK(cudaMemsetAsync(S.mb[b].id, 0, sizeof(int32_t) * cap, ctx->stream));
+            }
+            CK(cudaMemsetAsync(S.perm, 0, sizeof(int) * cap, ctx->stream));
             S.counts = (int *)dev_alloc(ctx, sizeof(int) * (r.max_keys + 1));
             if (!S.counts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort counts");
             S.tile_start = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             S.tile_start_alt = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             if (!S.tile_start || !S.tile_start_alt) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for tile offsets");
             CK(cudaMemsetAsync(S.tile_start, 0, sizeof(int) * (r.max_tiles + 1), ctx->stream));
+            CK(cudaMemsetAsync(S.tile_start_alt, 0, sizeof(int) * (r.max_tiles + 1), ctx->stream));
         }
     }
     return PIC_OK;
@@ -826,12 +835,14 @@ pic_status read_err(pic_ctx *ctx) {
     if (e) {
         CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
         if (e & ERR_TIMEOUT) {
-            // steps that did not end are in nobody's record: host and device start it again together
+            // Steps that did not end are in nobody's record: host and device start it again together.
+            // The sort or the push of any run may be missing: the next step sorts from storage order.
             for (auto &r : ctx->runs) {
                 r.hist_n = 0;
                 CK(cudaMemsetAsync(r.hist, 0, sizeof(double) * 8 * r.hist_cap, ctx->stream));
                 CK(cudaMemsetAsync(r.hist_idx, 0, sizeof(long long), ctx->stream));
-                r.sorted = false;   // the record's first step sorts
+                r.sorted = false;
+                for (int q = 0; q < r.d.nspecies; ++q) r.sp[q].tiled = r.sp[q].moving = false;
             }
             return fail(ctx, PIC_ETIMEOUT, "a bounded device wait gave up");
         }
