@@ -504,18 +504,20 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     const unsigned lt_mask = (1u << lane) - 1u;
     __shared__ int work_ctr[4];
     __shared__ double kin_sh[2][WARPS];
-    // work items of species sp, of 2^lgw rows of 32 particles and of 2^lgt at the end; this part's share
-    auto item_range = [&](int sp, int &rows, int &beg, int &end) {
-        const int lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
-        rows = (a.tile_start[sp][tile + 1] - a.tile_start[sp][tile] + 31) >> 5;
-        const int nall = (rows >> lgw) + (((rows & ((1 << lgw) - 1)) + (1 << lgt) - 1) >> lgt);
-        beg = (int)((long long)nall * part / parts);
-        end = (int)((long long)nall * (part + 1) / parts);
-    };
+    // Particles and work items (of 2^lgw rows of 32 particles, and of 2^lgt at the end) of a
+    // species in the tile, and this part's share of the items.  In shared memory: the
+    // registers of the tile and of the part are free for the particles.
+    __shared__ int span_sh[4][5];   // particles begin, end; rows; items begin, end
     if ((int)threadIdx.x < a.nspecies) {
-        int rows, beg, end;
-        item_range(threadIdx.x, rows, beg, end);
-        work_ctr[threadIdx.x] = beg;
+        const int sp = threadIdx.x, lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
+        const int p0 = a.tile_start[sp][tile], p1 = a.tile_start[sp][tile + 1], rows = (p1 - p0 + 31) >> 5;
+        const int nall = (rows >> lgw) + (((rows & ((1 << lgw) - 1)) + (1 << lgt) - 1) >> lgt);
+        const int beg = (int)((long long)nall * part / parts);
+        span_sh[sp][0] = p0;
+        span_sh[sp][1] = p1;
+        span_sh[sp][2] = rows;
+        span_sh[sp][3] = work_ctr[sp] = beg;
+        span_sh[sp][4] = (int)((long long)nall * (part + 1) / parts);
     }
     if (lane == 0) { kin_sh[0][warp] = 0.0; kin_sh[1][warp] = 0.0; }
     // this warp's piece queue and particle stages
@@ -546,17 +548,14 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                 atomicAdd(a.J[comp] + ((long long)gz * g.py + gy) * g.px + gx, (unsigned long long)v);
         }
     };
-    long long since_flush = 0;   // particles summed into the limbs since they were last cleared (uniform)
+    int since_flush = 0;   // particles summed into the limbs since they were last cleared (uniform)
     RegAcc<NDIM> acc;
     acc.q0 = -1;
     int qhead = 0, qcount = 0;   // warp-uniform state of the piece ring
     for (int sp = 0; sp < a.nspecies; ++sp) {
         const SpeciesMixed &P = a.sp[sp];
         const float h = a.h[sp], alpha26 = a.sgn[sp] * kFx26;   // deposit prefactor in fixed-point units
-        const int pbeg = a.tile_start[sp][tile], pend = a.tile_start[sp][tile + 1];
-        const int lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
-        int rows, ibeg, nitems;
-        item_range(sp, rows, ibeg, nitems);
+        const int pend = span_sh[sp][1];
         const int *const perm = MOVE ? a.perm[sp] : nullptr;
         const SpeciesMixed &Q = perm ? a.src[sp] : a.sp[sp];   // where the particles are read
         // source of the particle of iteration j of an item, -1 past its end
@@ -599,10 +598,10 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                 qcount = 0;
             }
         };
-        for (int r0 = ibeg; r0 < nitems; r0 += kRoundItems) {
-        const int r1 = min(nitems, r0 + kRoundItems);
-        const bool need_flush = since_flush + (long long)(r1 - r0) * 1024 >= (1LL << 17);   // uniform
-        if (r0 > ibeg || need_flush) {
+        for (int r0 = span_sh[sp][3]; r0 < span_sh[sp][4]; r0 += kRoundItems) {
+        const int r1 = min(span_sh[sp][4], r0 + kRoundItems);
+        const bool need_flush = since_flush + (r1 - r0) * 1024 >= 1 << 17;   // uniform
+        if (r0 > span_sh[sp][3] || need_flush) {
             // every warp has left the previous round; its pieces and register sums go to the limbs
             drain_queue();
             acc.flush(Jhi, Jlo, nodes, tc.sx, tc.sxy);
@@ -615,7 +614,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             if (threadIdx.x == 0) work_ctr[sp] = r0;
             __syncthreads();
         }
-        since_flush += (long long)(r1 - r0) * 1024;
+        since_flush += (r1 - r0) * 1024;
         // work items of the round are taken by whole warps from a shared counter
         for (;;) {
             int item = 0;
@@ -623,8 +622,9 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             item = __shfl_sync(kFull, item, 0);
             if (item >= r1) break;
             // the lane walks base + 32k + lane, k = 0..kn-1 (consecutive ranks)
+            const int lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw), rows = span_sh[sp][2];
             const int nfull = rows >> lgw, row = item < nfull ? item << lgw : (nfull << lgw) + ((item - nfull) << lgt);
-            const int base = pbeg + (row << 5);
+            const int base = span_sh[sp][0] + (row << 5);
             const int kn = item < nfull ? 1 << lgw : min(1 << lgt, rows - row);
             float kin0 = 0.f, kin1 = 0.f;
 #pragma unroll
