@@ -57,6 +57,7 @@
 #pragma once
 #include "particle_core.cuh"
 #include "pic_internal.cuh"
+#include "span.cuh"
 
 namespace pic {
 
@@ -510,7 +511,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     __shared__ int span_sh[4][5];   // particles begin, end; rows; items begin, end
     if ((int)threadIdx.x < a.nspecies) {
         const int sp = threadIdx.x, lgw = a.lgw[sp], lgt = NDIM == 3 ? 0 : min(a.tail_lg, lgw);
-        const int p0 = a.tile_start[sp][tile], p1 = a.tile_start[sp][tile + 1], rows = (p1 - p0 + 31) >> 5;
+        const int p0 = a.tile_start[sp][tile], p1 = a.tile_start[sp][tile + 1], rows = slot_rows(p1 - p0);
         const int nall = (rows >> lgw) + (((rows & ((1 << lgw) - 1)) + (1 << lgt) - 1) >> lgt);
         const int beg = (int)((long long)nall * part / parts);
         span_sh[sp][0] = p0;
@@ -560,9 +561,9 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
         const SpeciesMixed &Q = perm ? a.src[sp] : a.sp[sp];   // where the particles are read
         // source of the particle of iteration j of an item, -1 past its end
         auto source = [&](int base, int j, int kn) -> int {
-            const int p = base + (j << 5) + lane;
-            if (j >= kn || p >= pend) return -1;
-            if (!perm) return p;
+            const Slot p = slot_at(base, (j << 5) + lane);
+            if (j >= kn || !slot_before(p, pend)) return -1;
+            if (!perm) return (int)p;
             const int q = ldro(perm + p);
             return (unsigned)q < (unsigned)a.n[sp] ? q : 0;   // (out of range only after a key that the sort has flagged)
         };
@@ -636,10 +637,10 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
                 issue(base, k + kStages - 1, next);
                 next = source(base, k + kStages, kn);
                 cp_async_wait<kStages - 1>();   // this lane's words of iteration k have landed
-                const int p = base + (k << 5) + lane;
+                const Slot p = slot_at(base, (k << 5) + lane);
                 int nc = 0, q0 = 0;
                 PathSplit<NDIM, float> ps;
-                if (p < pend) {
+                if (slot_before(p, pend)) {
                     const uint32_t *st = stage + (k % kStages) * NW * 32;
                     const float4 wa = reinterpret_cast<const float4 *>(st)[lane];
                     uint32_t c = __float_as_uint(wa.x);

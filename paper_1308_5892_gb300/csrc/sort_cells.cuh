@@ -4,6 +4,7 @@
 // kernels (sort.cu) and the persistent ensemble step (walk.cu).
 #pragma once
 #include "pic_internal.cuh"
+#include "span.cuh"
 
 namespace pic {
 
@@ -153,7 +154,8 @@ __device__ inline void box_body(const SortArgs &a, int tile, int part, int parts
         const int dt = key_tile(t, key);
         place(r, ldro(a.tile_start + dt), ldro(a.tile_start + dt + 1), p);
     };
-    for (int base = t0 + (int)((long long)nt * part / parts); base < end; base += kBoxRounds * THREADS) {
+    for (Slot base = t0 + (int)((long long)nt * part / parts); slot_before(base, end);
+         base = slot_at(base, kBoxRounds * THREADS)) {
         for (int q = threadIdx.x; q < nb; q += THREADS) box[q] = 0;
         __syncthreads();
         // rank in the cell << 17 | cell in the tile << 16 | box cell, -1 when there is nothing left to place
@@ -163,14 +165,14 @@ __device__ inline void box_body(const SortArgs &a, int tile, int part, int parts
             uint32_t c[8];
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
-                const int p = base + (v0 + v) * THREADS + threadIdx.x;
-                c[v] = p < end ? ldro(cell_ptr(a.src, p)) : 0u;
+                const Slot p = slot_at(base, (v0 + v) * THREADS + threadIdx.x);
+                c[v] = slot_before(p, end) ? ldro(cell_ptr(a.src, p)) : 0u;
             }
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
-                const int p = base + (v0 + v) * THREADS + threadIdx.x;
+                const Slot p = slot_at(base, (v0 + v) * THREADS + threadIdx.x);
                 held[v0 + v] = -1;
-                if (p >= end) continue;
+                if (!slot_before(p, end)) continue;
                 // the cell, or its image, in the box
                 int i, j, k;
                 unpack_cell(NDIM, c[v], i, j, k);
@@ -195,7 +197,7 @@ __device__ inline void box_body(const SortArgs &a, int tile, int part, int parts
                         continue;
                     }
                     const int r = atomicAdd(a.counts + key, 1);
-                    if (RANK) place_key(r, key, p);
+                    if (RANK) place_key(r, key, (int)p);
                 }
             }
         }
@@ -214,7 +216,7 @@ __device__ inline void box_body(const SortArgs &a, int tile, int part, int parts
 #pragma unroll
             for (int v = 0; v < kBoxRounds; ++v) {
                 if (held[v] < 0) continue;
-                const int p = base + v * THREADS + threadIdx.x;
+                const int p = (int)slot_at(base, v * THREADS + threadIdx.x);
                 const int r = box[held[v] & 0xffff] + (held[v] >> 17);
                 if (held[v] & (1 << 16)) place(r, own0, own1, p);
                 else place_key(r, cell_key<NDIM>(t, ldro(cell_ptr(a.src, p))), p);
