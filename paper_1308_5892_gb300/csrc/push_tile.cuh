@@ -552,6 +552,7 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
     int since_flush = 0;   // particles summed into the limbs since they were last cleared (uniform)
     RegAcc<NDIM> acc;
     acc.q0 = -1;
+    int held = 0;   // rows of particles since the register sums were last cleared (warp-uniform)
     int qhead = 0, qcount = 0;   // warp-uniform state of the piece ring
     for (int sp = 0; sp < a.nspecies; ++sp) {
         const SpeciesMixed &P = a.sp[sp];
@@ -627,6 +628,12 @@ __device__ __forceinline__ void push_tile(const MixedStepArgs &a, const int tile
             const int nfull = rows >> lgw, row = item < nfull ? item << lgw : (nfull << lgw) + ((item - nfull) << lgt);
             const int base = span_sh[sp][0] + (row << 5);
             const int kn = item < nfull ? 1 << lgw : min(1 << lgt, rows - row);
+            // no register sum takes more than 32 particles, however many of its cell's items a warp takes
+            if (held + kn > 32) {
+                acc.flush(Jhi, Jlo, nodes, tc.sx, tc.sxy);
+                held = 0;
+            }
+            held += kn;
             float kin0 = 0.f, kin1 = 0.f;
 #pragma unroll
             for (int j = 0; j < kStages - 1; ++j) issue(base, j, source(base, j, kn));
