@@ -264,6 +264,8 @@ R *jplane(Run &r, int buf, int c) {
     static_assert(sizeof(R) == 8, "current planes are 8-byte values");
     return (R *)r.J + ((size_t)buf * 3 + c) * r.g.pcells;
 }
+// The mixed path has two current buffers (one filled while the other is zeroed), FP64 one.
+size_t jplanes(const pic_ctx *ctx) { return ctx->precision == PIC_MIXED ? 6 : 3; }
 
 // ------------------------------------------------------------ conversion kernels
 
@@ -658,10 +660,10 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
     const long long ncell = (long long)g.nx * g.ny * g.nz;
     const size_t fplanes = mixed ? 9 : 6;   // mixed: e, b and the low-order part of e
     r.F = dev_alloc(ctx, fplanes * rs * g.pcells);
-    r.J = dev_alloc(ctx, 6 * 8 * g.pcells);
+    r.J = dev_alloc(ctx, jplanes(ctx) * 8 * g.pcells);
     if (!r.F || !r.J) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the field arrays");
     CK(cudaMemsetAsync(r.F, 0, fplanes * rs * g.pcells, ctx->stream));
-    CK(cudaMemsetAsync(r.J, 0, 6 * 8 * g.pcells, ctx->stream));
+    CK(cudaMemsetAsync(r.J, 0, jplanes(ctx) * 8 * g.pcells, ctx->stream));
     if (mixed) {
         r.nfA = (float4 *)dev_alloc(ctx, sizeof(float4) * g.pcells);
         r.nfB = (float2 *)dev_alloc(ctx, sizeof(float2) * g.pcells);
@@ -678,11 +680,6 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
         }
         if (!r.nfA || !r.nfB || !r.block_sums)
             return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the tile buffers");
-    }
-    if (!mixed) {
-        r.nf64 = (double2 *)dev_alloc(ctx, 3 * sizeof(double2) * g.pcells);
-        r.M64 = (double *)dev_alloc(ctx, moment_planes64(d.ndim) * sizeof(double) * g.pcells);
-        if (!r.nf64 || !r.M64) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the node fields");
     }
     r.rho_s = (double *)dev_alloc(ctx, sizeof(double) * ncell);
     r.rho_tot = (double *)dev_alloc(ctx, sizeof(double) * ncell);
@@ -748,12 +745,26 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
     return PIC_OK;
 }
 
+// Node averages and moment planes of the FP64 push: allocated after everything a context
+// needs.  Without room for them (112 or 144 B per cell, beside 96 for fields, current and
+// diagnostics) the push gathers from the fields and adds to the current itself: the same
+// result in two to three times the time (64^3 with 32 particles per cell and species 14.1
+// against 7.05 ms per step, 128^3 115 against 56.4, 400^3 with one 342 against 111).
+void setup_moments64(pic_ctx *ctx, Run &r) {
+    r.nf64 = (double2 *)dev_try_alloc(ctx, 3 * sizeof(double2) * r.g.pcells);
+    if (!r.nf64) return;
+    r.M64 = (double *)dev_try_alloc(ctx, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells);
+    if (r.M64) return;
+    dev_release(ctx, r.nf64);
+    r.nf64 = nullptr;
+}
+
 // Scratch of the FP64 sort: an id per particle, and for the largest species one
 // spare array and the permutation.  Allocated after everything a context needs; a
 // context that gets none of it steps unsorted (slower, the same result).
 void setup_sort64(pic_ctx *ctx, Run &r) {
     const long long ncell = (long long)r.g.nx * r.g.ny * r.g.nz;
-    if ((size_t)r.g.pcells * (48 + 8 * moment_planes64(r.d.ndim)) <= kSort64Bytes || ncell > INT32_MAX) return;
+    if (!r.nf64 || (size_t)r.g.pcells * (48 + 8 * moment_planes64(r.d.ndim)) <= kSort64Bytes || ncell > INT32_MAX) return;
     int64_t cap = 0;
     bool equal = true;
     for (int s = 0; s < r.d.nspecies; ++s) {
@@ -1287,12 +1298,24 @@ const typename SmoothValue<JT>::type *smooth_current(pic_ctx *ctx, Run &r, JT *c
     return launch_smooth_current<JT>(r.g, J, r.smooth, buf, ctx->stream);
 }
 
+Cells64 cells64(Run &r, const FieldPtrs<double> &f, bool direct) {
+    return Cells64{direct ? nullptr : r.nf64, r.M64, f, (double *)r.J};
+}
+
+// Initial staggering of newly loaded momenta of the FP64 path (App. A.3.1).
+void half_back64(Run &r, SpeciesState &S, cudaStream_t s) {
+    const FieldPtrs<double> f = fields_of<double>(r);
+    if (r.nf64) launch_node_fields64(r.g, f, r.nf64, s);
+    launch_half_back64(r.g, cells64(r, f, !r.nf64), S.s64, S.n, S.h, r.d.dt, s);
+}
+
 pic_status step_run(pic_ctx *ctx, Run &r) {
     cudaStream_t s = ctx->stream;
     double *hslot = (r.hist_n < r.hist_cap) ? r.hist + 8 * r.hist_n : nullptr;
     const int nsp = r.d.nspecies;
     if (ctx->precision == PIC_FP64) {
         FieldPtrs<double> f = fields_of<double>(r, true);
+        const bool direct = !r.nf64;
         int launches = 0;
         if (r.spare64 && (!r.sorted || r.since_sort >= kSort64Interval)) {
             KTimer t(ctx, PIC_KERNEL_SORT);
@@ -1310,30 +1333,29 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
             // after the first step the energy at u^{t-1/2} is what the step before recorded
             launch_b_advance<double>(r.g, f, 0.5 * r.d.dt, HistRef{hslot, nullptr, 0},
                                      r.hist_n > 0, s);
-            launch_node_fields64(r.g, f, r.nf64, s);
+            if (!direct) launch_node_fields64(r.g, f, r.nf64, s);
         }
-        double *J[3] = {jplane<double>(r, r.jcur, 0), jplane<double>(r, r.jcur, 1), jplane<double>(r, r.jcur, 2)};
+        double *J[3] = {jplane<double>(r, 0, 0), jplane<double>(r, 0, 1), jplane<double>(r, 0, 2)};
         {
             KTimer t(ctx, PIC_KERNEL_PUSH);
-            CK(cudaMemsetAsync(r.M64, 0, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells, s));
+            if (direct) CK(cudaMemsetAsync(r.J, 0, jplanes(ctx) * 8 * r.g.pcells, s));
+            else CK(cudaMemsetAsync(r.M64, 0, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells, s));
             for (int q = 0; q < nsp; ++q) {
                 SpeciesState &S = r.sp[q];
-                launch_push_fp64(r.g, r.nf64, r.M64, S.s64, S.n, S.sorted64, S.h, S.q_over_e < 0, r.d.dt,
-                                 S.m_over_me, hslot, r.hist_n == 0, ctx->d_err, s);
+                launch_push_fp64(r.g, cells64(r, f, direct), S.s64, S.n, S.sorted64, S.h, S.alpha, r.d.dt, S.m_over_me,
+                                 hslot, r.hist_n == 0, ctx->d_err, s);
             }
-            launch_current64(r.g, r.M64, J, std::fabs(r.sp[0].alpha), s);
+            if (!direct) launch_current64(r.g, r.M64, J, std::fabs(r.sp[0].alpha), s);
         }
-        double *Z[3] = {jplane<double>(r, 1 - r.jcur, 0), jplane<double>(r, 1 - r.jcur, 1),
-                        jplane<double>(r, 1 - r.jcur, 2)};
         const double *Jc[3] = {J[0], J[1], J[2]};
         const double *Js = smooth_current<double>(ctx, r, J);
         {
             KTimer t(ctx, PIC_KERNEL_FIELD);
-            if (Js) launch_e_advance_smoothed<double, double, double>(r.g, f, Js, 1.0, Z, r.d.dt, nullptr, s);
-            else launch_e_advance<double>(r.g, f, Jc, Z, r.d.dt, s);
+            if (Js) launch_e_advance_smoothed<double, double, double>(r.g, f, Js, 1.0, nullptr, r.d.dt, nullptr, s);
+            else launch_e_advance<double>(r.g, f, Jc, r.d.dt, s);
         }
         ctx->bytes_per_ps = r.d.ndim == 2 ? 80.0 : 96.0;
-        ctx->launch_total += launches + 4 + nsp + (Js ? 1 + r.smooth : 0);   // shell fold + passes
+        ctx->launch_total += launches + (direct ? 2 : 4) + nsp + (Js ? 1 + r.smooth : 0);   // shell fold + passes
     } else {
         int launches = 0;
         if (!r.sorted || r.since_sort >= r.sort_interval) {
@@ -1610,8 +1632,10 @@ pic_status pic_init(const pic_run_desc *runs, int nruns, const pic_opts *opts, p
     ctx->mlpLoss = (double *)dev_alloc(ctx, sizeof(double));
     ctx->mlpF = (double *)dev_alloc(ctx, sizeof(double) * (size_t)ncombo * (kMjTable + 1));
     ctx->mlpPar = (double *)dev_alloc(ctx, sizeof(double) * 8 * ncombo);
-    if (precision == PIC_FP64)
+    if (precision == PIC_FP64) {
+        for (auto &r : ctx->runs) setup_moments64(ctx, r);
         for (auto &r : ctx->runs) setup_sort64(ctx, r);
+    }
     if (!ctx->staging || !ctx->mj_table || !ctx->mlpW || !ctx->mlpG || !ctx->mlpM || !ctx->mlpV || !ctx->mlpWh ||
         !ctx->mlpX || !ctx->mlpT || !ctx->mlpLoss || !ctx->mlpF || !ctx->mlpPar) {
         pic_destroy(ctx);
@@ -1682,7 +1706,7 @@ pic_status pic_set_state(pic_ctx *ctx, int run, const pic_state_view *in) {
                 g, src, (float *)r.F + c * g.pcells, c < 3 ? (float *)r.F + (6 + c) * g.pcells : nullptr, ctx->d_err);
         CK(cudaGetLastError());
     }
-    CK(cudaMemsetAsync(r.J, 0, 6 * 8 * g.pcells, sm));
+    CK(cudaMemsetAsync(r.J, 0, jplanes(ctx) * 8 * g.pcells, sm));
     r.jcur = 0;
     for (int s = 0; s < r.d.nspecies; ++s) {
         SpeciesState &S = r.sp[s];
@@ -2263,8 +2287,7 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
         launch_node_fields(g, f, r.nfA, r.nfB, sm);
         launch_half_back_mixed(g, r.nfA, r.nfB, S.mb[S.cur], n, (float)S.h, (float)r.d.dt, sm);
     } else {
-        launch_node_fields64(g, fields_of<double>(r), r.nf64, sm);
-        launch_half_back64(g, r.nf64, S.s64, n, S.h, r.d.dt, sm);
+        half_back64(r, S, sm);
     }
     CK(cudaGetLastError());
     r.step = 0;
@@ -2363,8 +2386,7 @@ pic_status mlp_load(pic_ctx *ctx, int run, int species, long long n, double thet
         launch_node_fields(r.g, f, r.nfA, r.nfB, sm);
         launch_half_back_mixed(r.g, r.nfA, r.nfB, S.mb[S.cur], n, (float)S.h, (float)r.d.dt, sm);
     } else {
-        launch_node_fields64(r.g, fields_of<double>(r), r.nf64, sm);
-        launch_half_back64(r.g, r.nf64, S.s64, n, S.h, r.d.dt, sm);
+        half_back64(r, S, sm);
     }
     CK(cudaGetLastError());
     r.step = 0;

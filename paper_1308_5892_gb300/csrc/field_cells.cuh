@@ -40,6 +40,8 @@ struct CellAt {
     int pi, pj, pk;
     uint32_t p;
     __device__ __forceinline__ CellAt(const Geom &g, long long at) : p((uint32_t)at) { padded_coords(g, at, pi, pj, pk); }
+    __device__ __forceinline__ CellAt(const Geom &g, int i, int j, int k)
+        : pi(i), pj(j), pk(k), p(((uint32_t)k * (uint32_t)g.py + (uint32_t)j) * (uint32_t)g.px + (uint32_t)i) {}
     // cell q of plane pk
     __device__ __forceinline__ CellAt(const Geom &g, uint32_t q, int k) : pk(k) {
         pj = (int)g.fpx.div(q);
@@ -296,9 +298,11 @@ __device__ __forceinline__ void e_smoothed_cell(const Geom &g, const FieldPtrs<R
         f.e[1][p] = ey;
         f.e[2][p] = ez;
     }
-    Z0[p] = ZT(0);
-    Z1[p] = ZT(0);
-    Z2[p] = ZT(0);
+    if constexpr (std::is_same<R, float>::value) {   // (the FP64 path has one current buffer)
+        Z0[p] = ZT(0);
+        Z1[p] = ZT(0);
+        Z2[p] = ZT(0);
+    }
 }
 
 // Staggered value read by the gather between conductor walls: a value located inside

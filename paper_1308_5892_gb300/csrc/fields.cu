@@ -47,11 +47,10 @@ __global__ void __launch_bounds__(256) k_b_advance(Geom g, FieldPtrs<R> f, R h, 
     if (energy_acc) block_accumulate<6, 256>(acc, energy_acc, sh);
 }
 
-// e <- e + dt curl b + J (Ampere, Eq. dyn4 with the deposited current, main
-// loop steps 6, 11, 12), and zeroing of the other current buffer.
+// FP64 path: e <- e + dt curl b + J (Ampere, Eq. dyn4 with the deposited current, main
+// loop steps 6, 11, 12).
 template <typename R>
-__global__ void __launch_bounds__(256) k_e_advance(Geom g, FieldPtrs<R> f, const R *J0, const R *J1, const R *J2, R *Z0,
-                                                   R *Z1, R *Z2, R dt) {
+__global__ void __launch_bounds__(256) k_e_advance(Geom g, FieldPtrs<R> f, const R *J0, const R *J1, const R *J2, R dt) {
     for_cells(g, [&](const CellAt &c) {
         const uint32_t p = c.p, xm = c.xm(g), ym = c.ym(g), zm = c.zm(g);
         const R bx = ld(f.b[0], p), by = ld(f.b[1], p), bz = ld(f.b[2], p);
@@ -65,9 +64,6 @@ __global__ void __launch_bounds__(256) k_e_advance(Geom g, FieldPtrs<R> f, const
         f.e[0][p] = ex;
         f.e[1][p] = ey;
         f.e[2][p] = ez;
-        Z0[p] = R(0);
-        Z1[p] = R(0);
-        Z2[p] = R(0);
     });
 }
 
@@ -187,10 +183,8 @@ void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, bool c
 }
 
 template <typename R>
-void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *const Jzero[3], R dt,
-                      cudaStream_t s) {
-    k_e_advance<R><<<cells_grid(g, 16), 256, 0, s>>>(g, f, J[0], J[1], J[2], Jzero[0], Jzero[1], Jzero[2],
-                                                           dt);
+void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R dt, cudaStream_t s) {
+    k_e_advance<R><<<cells_grid(g, 16), 256, 0, s>>>(g, f, J[0], J[1], J[2], dt);
 }
 
 void launch_node_fields(const Geom &g, FieldPtrs<float> f, float4 *nfA, float2 *nfB, cudaStream_t s) {
@@ -220,8 +214,8 @@ void launch_e_advance_fx(const Geom &g, FieldPtrs<float> f, const unsigned long 
 template <typename R, typename ZT, typename CT>
 void launch_e_advance_smoothed(const Geom &g, FieldPtrs<R> f, const CT *Js, double scale, ZT *const Jzero[3],
                                R dt, long long *hist_inc, cudaStream_t s) {
-    k_e_advance_smoothed<R, ZT, CT><<<cells_grid(g, 16), 256, 0, s>>>(g, f, Js, scale, Jzero[0], Jzero[1],
-                                                                            Jzero[2], dt, hist_inc);
+    ZT *const Z[3] = {Jzero ? Jzero[0] : nullptr, Jzero ? Jzero[1] : nullptr, Jzero ? Jzero[2] : nullptr};
+    k_e_advance_smoothed<R, ZT, CT><<<cells_grid(g, 16), 256, 0, s>>>(g, f, Js, scale, Z[0], Z[1], Z[2], dt, hist_inc);
 }
 
 template <typename R>
@@ -231,10 +225,7 @@ void launch_add_uniform(const Geom &g, FieldPtrs<R> f, const double e0[3], const
 
 template void launch_b_advance<float>(const Geom &, FieldPtrs<float>, float, HistRef, bool, cudaStream_t);
 template void launch_b_advance<double>(const Geom &, FieldPtrs<double>, double, HistRef, bool, cudaStream_t);
-template void launch_e_advance<float>(const Geom &, FieldPtrs<float>, const float *const[3], float *const[3], float,
-                                      cudaStream_t);
-template void launch_e_advance<double>(const Geom &, FieldPtrs<double>, const double *const[3], double *const[3],
-                                       double, cudaStream_t);
+template void launch_e_advance<double>(const Geom &, FieldPtrs<double>, const double *const[3], double, cudaStream_t);
 template void launch_e_advance_smoothed<double, double, double>(const Geom &, FieldPtrs<double>, const double *,
                                                                double, double *const[3], double, long long *,
                                                                cudaStream_t);

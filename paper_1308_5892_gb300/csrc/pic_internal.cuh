@@ -14,8 +14,8 @@
 //    accumulated while the other is zeroed); node fields (mixed path): one
 //    float4 pair per padded cell, {E_x,E_y,E_z,B_x} {B_y,B_z,0,0}, the node
 //    averages of App. A.3.3 at time t.
-//  - FP64 path: node fields, three planes of double2, and the moment planes of the
-//    current (push_fp64.cu).
+//  - FP64 path: one current buffer; where there is room, node fields, three planes of
+//    double2, and the moment planes of the current (push_fp64.cu).
 //  - particles, FP64 path: SoA planes x,y,z,u_x,u_y,u_z of double (absolute
 //    positions), sorted by cell every few steps (then with an int32 id); mixed path: packed cell coordinates (uint32), FP32 offsets
 //    and momenta, and an int32 id (SpeciesMixed), kept sorted by tile.
@@ -251,8 +251,7 @@ struct HistRef {
 template <typename R>
 void launch_b_advance(const Geom &g, FieldPtrs<R> f, R h, HistRef energy, bool carry, cudaStream_t s);
 template <typename R>
-void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R *const Jzero[3], R dt,
-                      cudaStream_t s);
+void launch_e_advance(const Geom &g, FieldPtrs<R> f, const R *const J[3], R dt, cudaStream_t s);
 void launch_node_fields(const Geom &g, FieldPtrs<float> f, float4 *nfA, float2 *nfB, cudaStream_t s);
 void launch_node_fields64(const Geom &g, FieldPtrs<double> f, double2 *nf, cudaStream_t s);
 // e += dt curl b + |alpha| * J for the fixed-point current of the mixed path
@@ -264,7 +263,8 @@ template <typename R>
 void launch_add_uniform(const Geom &g, FieldPtrs<R> f, const double e0[3], const double b0[3], cudaStream_t s);
 // e += dt curl b + scale * Js with the smoothed compact current Js (3 planes of
 // nx*ny*nz values: double in the FP64 path, int64 fixed point in the mixed
-// path, in the units of the path's current), and zeroing of Jzero
+// path, in the units of the path's current), and zeroing of Jzero (mixed path; null in the
+// FP64 path)
 template <typename R, typename ZT, typename CT>
 void launch_e_advance_smoothed(const Geom &g, FieldPtrs<R> f, const CT *Js, double scale, ZT *const Jzero[3],
                                R dt, long long *hist_inc, cudaStream_t s);
@@ -286,17 +286,26 @@ const typename SmoothValue<JT>::type *launch_smooth_current(const Geom &g, JT *c
 // one smoothing pass of one compact plane, in -> out (distinct arrays)
 void launch_smooth(const Geom &g, const double *in, double *out, cudaStream_t s);
 
-// push_fp64.cu: nf holds the node averages (three planes of double2); M the moment planes
-// of the current (moment_planes64 of them, zero before the first species), to which a
-// species adds with the sign of its charge; kin_acc (nullable): kinetic energy at
-// u^{t-1/2} (only with kin0) and at u^{t+1/2}
+// push_fp64.cu
+// What a species' push reads and adds to.  By moments: nf holds the node averages (three
+// planes of double2), M the moment planes of the current (moment_planes64 of them, zero
+// before the first species).  Direct (nf null): the fields f, with b at t, and the three
+// padded planes of the current from J on (zero before the first species).
+struct Cells64 {
+    const double2 *nf;
+    double *M;
+    FieldPtrs<double> f;
+    double *J;
+};
 int moment_planes64(int ndim);
-void launch_push_fp64(const Geom &g, const double2 *nf, double *M, Species64 sp, long long n, bool sorted, double h,
-                      bool negative, double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s);
+// alpha: that of the species; kin_acc (nullable): kinetic energy at u^{t-1/2} (only with
+// kin0) and at u^{t+1/2}
+void launch_push_fp64(const Geom &g, const Cells64 &io, Species64 sp, long long n, bool sorted, double h, double alpha,
+                      double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s);
 // the interior of the padded current planes J from the moments
 void launch_current64(const Geom &g, const double *M, double *const J[3], double alpha_abs, cudaStream_t s);
-// initial staggering of the momenta by -dt/2
-void launch_half_back64(const Geom &g, const double2 *nf, Species64 sp, long long n, double h, double dt,
+// initial staggering of the momenta by -dt/2 (io.f then has b at t - dt/2 alone)
+void launch_half_back64(const Geom &g, const Cells64 &io, Species64 sp, long long n, double h, double dt,
                         cudaStream_t s);
 // log2 of the particles a lane of the push walks in a sorted block of 32 << lg particles
 int walk_lg64(long long n);

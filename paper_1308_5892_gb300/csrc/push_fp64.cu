@@ -92,6 +92,60 @@ struct CellSums64 {
     }
 };
 
+// The push reads node averages and adds moments, or gathers and deposits at the particle
+// itself (direct): a cell's node averages and moments take 112 (2D) or 144 B beside the 96 B
+// of its fields, current and diagnostics, and a grid that fills the memory has no room for
+// them.  No sums are kept per lane then, and the loop over the nodes stays a loop: unrolled
+// by 2, 4 and 8 it is as fast (400^3 cells with 2 particles each: 341, 340, 357 ms per step,
+// looped 342).
+struct MomentCells64 {
+    static constexpr bool kDirect = false;
+    const double2 *nf;
+    double *M;
+};
+struct DirectCells64 {
+    static constexpr bool kDirect = true;
+    FieldPtrs<double> f;
+    double *J;
+    double scale;   // minus alpha (Ampere's law takes minus alpha times the flux)
+};
+
+// Fluxes of a segment through the faces of its cell (deposit_segment), scaled, into the
+// three padded planes from J (the cell's entry of the first) on.
+template <int NDIM>
+__device__ __forceinline__ void fluxes64(double *J, size_t plane, unsigned sx, unsigned sxy, const double d[3],
+                                         const double D[3], double scale) {
+    double w0[3], w1[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        w1[a] = fma(0.5, D[a], d[a]);
+        w0[a] = 1.0 - w1[a];
+    }
+    const double ax = scale * D[0], ay = scale * D[1], az = scale * D[2];
+    const double cxy = D[0] * D[1] * (1.0 / 12.0);
+    double *const Jx = J, *const Jy = J + plane, *const Jz = J + 2 * plane;
+    if (NDIM == 3) {
+        const double cyz = D[1] * D[2] * (1.0 / 12.0), czx = D[2] * D[0] * (1.0 / 12.0);
+        atomicAdd(Jx, ax * fma(w0[1], w0[2], cyz));
+        atomicAdd(Jx + sx, ax * fma(w1[1], w0[2], -cyz));
+        atomicAdd(Jx + sxy, ax * fma(w0[1], w1[2], -cyz));
+        atomicAdd(Jx + sx + sxy, ax * fma(w1[1], w1[2], cyz));
+        atomicAdd(Jy, ay * fma(w0[2], w0[0], czx));
+        atomicAdd(Jy + 1, ay * fma(w0[2], w1[0], -czx));
+        atomicAdd(Jy + sxy, ay * fma(w1[2], w0[0], -czx));
+        atomicAdd(Jy + 1 + sxy, ay * fma(w1[2], w1[0], czx));
+    } else {
+        atomicAdd(Jx, ax * w0[1]);
+        atomicAdd(Jx + sx, ax * w1[1]);
+        atomicAdd(Jy, ay * w0[0]);
+        atomicAdd(Jy + 1, ay * w1[0]);
+    }
+    atomicAdd(Jz, az * fma(w0[0], w0[1], cxy));
+    atomicAdd(Jz + 1, az * fma(w1[0], w0[1], -cxy));
+    atomicAdd(Jz + sx, az * fma(w0[0], w1[1], -cxy));
+    atomicAdd(Jz + 1 + sx, az * fma(w1[0], w1[1], cxy));
+}
+
 // Reciprocal and reciprocal square root of normal x > 0 to the last bit or so: the FP32
 // value of the hardware (relative error e0 < 2^-22) corrected by one third-order
 // step of Householder's iteration, r (1 + e + e^2) with e = 1 - x r, and
@@ -176,6 +230,36 @@ __device__ __forceinline__ void gather64(const double2 *__restrict__ nf, size_t 
             }
 }
 
+// The same with the averages of the cell's nodes formed on the way (c: the cell).
+template <int NDIM>
+__device__ __forceinline__ void gather_direct64(const Geom &g, const FieldPtrs<double> &f, const int c[3],
+                                                const double d[3], double E[3], double B[3]) {
+    E[0] = E[1] = E[2] = B[0] = B[1] = B[2] = 0.0;
+#pragma unroll 1
+    for (int q = 0; q < (NDIM == 3 ? 8 : 4); ++q) {
+        const int eps = q & 1, eta = (q >> 1) & 1, xi = q >> 2;
+        double w = (eps ? d[0] : 1.0 - d[0]) * (eta ? d[1] : 1.0 - d[1]);
+        if (NDIM == 3) w *= xi ? d[2] : 1.0 - d[2];
+        double e[3], b[3];
+        node_average<double>(g, f, CellAt(g, c[0] + g.G + eps, c[1] + g.G + eta, c[2] + g.Gz + xi), e, b);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            E[a] += w * e[a];
+            B[a] += w * b[a];
+        }
+    }
+}
+template <int NDIM>
+__device__ __forceinline__ void gather_cell64(const Geom &g, const MomentCells64 &io, const int *, unsigned q,
+                                              const double d[3], double E[3], double B[3]) {
+    gather64<NDIM>(io.nf, (size_t)g.pcells, q, (unsigned)g.px, (unsigned)g.px * (unsigned)g.py, d, E, B);
+}
+template <int NDIM>
+__device__ __forceinline__ void gather_cell64(const Geom &g, const DirectCells64 &io, const int *c, unsigned,
+                                              const double d[3], double E[3], double B[3]) {
+    gather_direct64<NDIM>(g, io.f, c, d, E, B);
+}
+
 // One axis of a move: start offset d, displacement D; the cell shift sa and the end
 // offset da, by comparisons of the upper word (pa < 0 or -0, pa >= 1).
 __device__ __forceinline__ void end_of_move(double d, double D, int &sa, double &da, int *err) {
@@ -205,14 +289,27 @@ struct MomentSink64 {
     __device__ __forceinline__ void add(int v, double a, double b) { atomicAdd(m + v * plane, a * b); }
 };
 
-// All pieces of a path into the moment planes; cell: padded index of the start cell.
+// A segment in the cell of padded index `cell`, into memory.
+template <int NDIM>
+__device__ __forceinline__ void segment64(const MomentCells64 &io, size_t plane, unsigned cell, unsigned, unsigned,
+                                          const double d[3], const double D[3], int sign) {
+    MomentSink64 m{io.M + cell, plane};
+    moments64<NDIM>(d, D, sign, m);
+}
+template <int NDIM>
+__device__ __forceinline__ void segment64(const DirectCells64 &io, size_t plane, unsigned cell, unsigned sx,
+                                          unsigned sxy, const double d[3], const double D[3], int) {
+    fluxes64<NDIM>(io.J + cell, plane, sx, sxy, d, D, io.scale);
+}
+
+// All pieces of a path; cell: padded index of the start cell.
 // The path from d0 to the end d1 in the cell shifted by s is cut at the planes it
 // crosses, at most one per axis, in the order of the crossing parameters t (ties in
 // axis order).  Breakpoints on the crossed axis are the plane's exact value and the
 // last piece ends at d1, so the pieces sum to the stored move.  t >= 0, so the
 // integer pipe compares them.
-template <int NDIM>
-__device__ __forceinline__ void deposit_path64(double *M, size_t plane, unsigned cell, unsigned sx, unsigned sxy,
+template <int NDIM, class IO>
+__device__ __forceinline__ void deposit_path64(const IO &io, size_t plane, unsigned cell, unsigned sx, unsigned sxy,
                                                const double d0[3], const int s[3], const double d1[3], double dz,
                                                int sign) {
     double cur[3], dv[3];
@@ -258,8 +355,7 @@ __device__ __forceinline__ void deposit_path64(double *M, size_t plane, unsigned
                 next += up ? stride[a] : 0u - stride[a];
             }
         }
-        MomentSink64 m{M + cell, plane};
-        moments64<NDIM>(pd, pD, sign, m);
+        segment64<NDIM>(io, plane, cell, sx, sxy, pd, pD, sign);
         if (last) break;
         tprev = __longlong_as_double(tmin);
         cell = next;
@@ -268,8 +364,8 @@ __device__ __forceinline__ void deposit_path64(double *M, size_t plane, unsigned
 
 // Conductor walls (App. A.4): the path to the wall and the mirrored remainder are
 // deposited as two legs; x returns the end.  Slow path of the few particles at a wall.
-template <int NDIM>
-__device__ __noinline__ void reflect64(const Geom &g, double *M, const int c[3], const double d[3], const double D[3],
+template <int NDIM, class IO>
+__device__ __noinline__ void reflect64(const Geom &g, const IO &io, const int c[3], const double d[3], const double D[3],
                                        int sign, double x[3], int *err) {
     const double xs = c[0] + d[0];
     const double wall = xs + D[0] < 0.0 ? 0.0 : (double)g.nx;
@@ -290,7 +386,7 @@ __device__ __noinline__ void reflect64(const Geom &g, double *M, const int c[3],
             x[a] = (double)(c0[a] + s[a]) + d1[a];
         }
         // the second leg may start in the image of a cell beyond a periodic edge
-        deposit_path64<NDIM>(M, (size_t)g.pcells,
+        deposit_path64<NDIM>(io, (size_t)g.pcells,
                              (unsigned)g.pidx(min(max(c0[0], 0), g.nx - 1), g.wy(c0[1]), NDIM == 3 ? g.wz(c0[2]) : 0),
                              (unsigned)g.px, (unsigned)g.px * (unsigned)g.py, d0, s, d1, L[2], sign);
         for (int a = 0; a < 3; ++a) {
@@ -311,10 +407,9 @@ __device__ __noinline__ void reflect64(const Geom &g, double *M, const int c[3],
 // flight work on neighbouring blocks; lane a walks the slots base + 32 k + a, which
 // after a sort are consecutive cell-sorted particles.
 // KIN0: also sum the energy at u^{t-1/2} (first step after a new state).
-template <int NDIM, bool WALLS, bool KIN0>
+template <int NDIM, bool WALLS, bool KIN0, class IO>
 __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
-    k_push_fp64(const __grid_constant__ Geom g, const double2 *__restrict__ nf, double *M, Species64 sp, long long n,
-                int lgw, double h, int sign, double dt, double m_over_me, double *kin_acc, int *err) {
+    k_push_fp64(const __grid_constant__ Geom g, const __grid_constant__ IO io, Species64 sp, long long n, int lgw, double h, int sign, double dt, double m_over_me, double *kin_acc, int *err) {
     constexpr int ND = NDIM == 3 ? 6 : 5;   // doubles of a queued path: start, end (and D_z in 2D)
     __shared__ double q_val[kThreads64 / 32][ND][kQueue64];
     __shared__ uint2 q_cell[kThreads64 / 32][kQueue64];
@@ -340,7 +435,7 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
             d0[a] = qv[a][idx];
             d1[a] = qv[NDIM + a][idx];
         }
-        deposit_path64<NDIM>(M, plane, cc.x, sx, sxy, d0, s, d1, NDIM == 2 ? qv[4][idx] : 0.0, sign);
+        deposit_path64<NDIM>(io, plane, cc.x, sx, sxy, d0, s, d1, NDIM == 2 ? qv[4][idx] : 0.0, sign);
     };
 
     // (step i of a warp is unit i mod 2^lgw of its block i >> lgw)
@@ -367,7 +462,7 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
             q = ((unsigned)(c[2] + g.Gz) * (unsigned)g.py + (unsigned)(c[1] + g.G)) * (unsigned)g.px +
                 (unsigned)(c[0] + g.G);
             double E[3], B[3];
-            gather64<NDIM>(nf, plane, q, sx, sxy, d, E, B);
+            gather_cell64<NDIM>(g, io, c, q, d, E, B);
             if (KIN0) kin0 += sqrt(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) - 1.0;
             boris64(u, E, B, qe);
             const double g2 = fma(u[2], u[2], fma(u[1], u[1], fma(u[0], u[0], 1.0)));
@@ -384,7 +479,7 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
             if (WALLS && reflect) {
                 u[0] = -u[0];
                 double x[3];
-                reflect64<NDIM>(g, M, c, d, D, sign, x, err);
+                reflect64<NDIM>(g, io, c, d, D, sign, x, err);
 #pragma unroll
                 for (int a = 0; a < NDIM; ++a) sp.x[a][p] = x[a];
             } else {
@@ -401,13 +496,17 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
                 }
                 queued = (s[0] | s[1] | s[2]) != 0;
                 if (!queued) {
-                    if (acc.q != q) {
-                        acc.flush(M, plane);
-                        acc.reset(q);
-                    }
                     // the end minus the start is the stored move
                     const double Dp[3] = {d1[0] - d[0], d1[1] - d[1], NDIM == 3 ? d1[2] - d[2] : D[2]};
-                    moments64<NDIM>(d, Dp, sign, acc);
+                    if constexpr (IO::kDirect) {
+                        segment64<NDIM>(io, plane, q, sx, sxy, d, Dp, sign);
+                    } else {
+                        if (acc.q != q) {
+                            acc.flush(io.M, plane);
+                            acc.reset(q);
+                        }
+                        moments64<NDIM>(d, Dp, sign, acc);
+                    }
                 }
             }
             sp.u[0][p] = u[0]; sp.u[1][p] = u[1]; sp.u[2][p] = u[2];
@@ -434,7 +533,7 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
     }
     __syncwarp();
     if (lane < qcount) drain_one((qhead + lane) & (kQueue64 - 1));
-    acc.flush(M, plane);
+    if constexpr (!IO::kDirect) acc.flush(io.M, plane);
     if (kin_acc) {
         for (int o = 16; o > 0; o >>= 1) {
             if (KIN0) kin0 += __shfl_xor_sync(kFull, kin0, o);
@@ -448,17 +547,16 @@ __global__ void __launch_bounds__(kThreads64, 512 / kThreads64)
 }
 
 // Initial staggering: u^0 -> u^{-dt/2} by one Boris step of -dt/2, no move.
-template <int NDIM>
-__global__ void __launch_bounds__(256) k_half_back64(Geom g, const double2 *__restrict__ nf, Species64 sp, long long n,
-                                                     double qe) {
+template <int NDIM, class IO>
+__global__ void __launch_bounds__(256) k_half_back64(const __grid_constant__ Geom g, const __grid_constant__ IO io,
+                                                     Species64 sp, long long n, double qe) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         int c[3] = {0, 0, 0};
         double d[3] = {0, 0, 0}, u[3] = {sp.u[0][p], sp.u[1][p], sp.u[2][p]};
         for (int a = 0; a < NDIM; ++a) split_bits(sp.x[a][p], c[a], d[a]);
         if (g.bcx == 1 && c[0] >= g.nx) { c[0] = g.nx - 1; d[0] = 1.0; }
         double E[3], B[3];
-        gather64<NDIM>(nf, (size_t)g.pcells, (unsigned)g.pidx(c[0], c[1], c[2]), (unsigned)g.px,
-                       (unsigned)g.px * (unsigned)g.py, d, E, B);
+        gather_cell64<NDIM>(g, io, c, (unsigned)g.pidx(c[0], c[1], c[2]), d, E, B);
         boris64(u, E, B, qe);
         sp.u[0][p] = u[0]; sp.u[1][p] = u[1]; sp.u[2][p] = u[2];
     }
@@ -511,30 +609,37 @@ int walk_lg64(long long n) {
 
 namespace {
 
-template <int NDIM, bool WALLS>
-void launch_dim(const Geom &g, const double2 *nf, double *M, Species64 sp, long long n, bool sorted, double h, int sign,
-                double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s) {
+template <int NDIM, bool WALLS, class IO>
+void launch_dim(const Geom &g, const IO &io, Species64 sp, long long n, bool sorted, double h, int sign, double dt,
+                double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s) {
     // The pipe is the bound, so every SM gets the same share in one wave of all resident
     // warps, and each warp as many particles as that allows (its last drain is part filled).
     const int lgw = sorted ? walk_lg64(n) : 0;
     const long long nblk = (n + (32LL << lgw) - 1) >> (5 + lgw);
     const int grid = (int)((std::min<long long>(nblk, kWarps64) + kThreads64 / 32 - 1) / (kThreads64 / 32));
-    auto k = kin0 ? k_push_fp64<NDIM, WALLS, true> : k_push_fp64<NDIM, WALLS, false>;
-    k<<<grid, kThreads64, 0, s>>>(g, nf, M, sp, n, lgw, h, sign, dt, m_over_me, kin_acc, err);
+    auto k = kin0 ? k_push_fp64<NDIM, WALLS, true, IO> : k_push_fp64<NDIM, WALLS, false, IO>;
+    k<<<grid, kThreads64, 0, s>>>(g, io, sp, n, lgw, h, sign, dt, m_over_me, kin_acc, err);
+}
+
+template <class IO>
+void launch_push(const Geom &g, const IO &io, Species64 sp, long long n, bool sorted, double h, int sign, double dt,
+                 double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s) {
+    const bool walls = g.bcx == 1;
+    auto f = g.ndim == 3 ? (walls ? launch_dim<3, true, IO> : launch_dim<3, false, IO>)
+                         : (walls ? launch_dim<2, true, IO> : launch_dim<2, false, IO>);
+    f(g, io, sp, n, sorted, h, sign, dt, m_over_me, kin_acc, kin0, err, s);
 }
 
 }  // namespace
 
 int moment_planes64(int ndim) { return ndim == 3 ? nmoments<3>() : nmoments<2>(); }
 
-void launch_push_fp64(const Geom &g, const double2 *nf, double *M, Species64 sp, long long n, bool sorted, double h,
-                      bool negative, double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s) {
+void launch_push_fp64(const Geom &g, const Cells64 &io, Species64 sp, long long n, bool sorted, double h, double alpha,
+                      double dt, double m_over_me, double *kin_acc, bool kin0, int *err, cudaStream_t s) {
     if (n <= 0) return;
-    const int sign = negative ? (int)0x80000000 : 0;
-    const bool walls = g.bcx == 1;
-    auto f = g.ndim == 3 ? (walls ? launch_dim<3, true> : launch_dim<3, false>)
-                         : (walls ? launch_dim<2, true> : launch_dim<2, false>);
-    f(g, nf, M, sp, n, sorted, h, sign, dt, m_over_me, kin_acc, kin0, err, s);
+    const int sign = alpha < 0 ? (int)0x80000000 : 0;
+    if (io.nf) launch_push(g, MomentCells64{io.nf, io.M}, sp, n, sorted, h, sign, dt, m_over_me, kin_acc, kin0, err, s);
+    else launch_push(g, DirectCells64{io.f, io.J, -alpha}, sp, n, sorted, h, sign, dt, m_over_me, kin_acc, kin0, err, s);
 }
 
 void launch_current64(const Geom &g, const double *M, double *const J[3], double alpha_abs, cudaStream_t s) {
@@ -545,12 +650,20 @@ void launch_current64(const Geom &g, const double *M, double *const J[3], double
     else k_current64<2><<<blocks, 256, 0, s>>>(g, M, J[0], J[1], J[2], -alpha_abs);
 }
 
-void launch_half_back64(const Geom &g, const double2 *nf, Species64 sp, long long n, double h, double dt,
+void launch_half_back64(const Geom &g, const Cells64 &io, Species64 sp, long long n, double h, double dt,
                         cudaStream_t s) {
     if (n <= 0) return;
     const int blocks = (int)std::min<long long>((n + 255) / 256, 152LL * 16);
-    if (g.ndim == 3) k_half_back64<3><<<blocks, 256, 0, s>>>(g, nf, sp, n, -0.25 * h * dt);
-    else k_half_back64<2><<<blocks, 256, 0, s>>>(g, nf, sp, n, -0.25 * h * dt);
+    const double qe = -0.25 * h * dt;
+    const MomentCells64 m{io.nf, io.M};
+    const DirectCells64 d{io.f, nullptr, 0.0};
+    if (g.ndim == 3) {
+        if (io.nf) k_half_back64<3><<<blocks, 256, 0, s>>>(g, m, sp, n, qe);
+        else k_half_back64<3><<<blocks, 256, 0, s>>>(g, d, sp, n, qe);
+    } else {
+        if (io.nf) k_half_back64<2><<<blocks, 256, 0, s>>>(g, m, sp, n, qe);
+        else k_half_back64<2><<<blocks, 256, 0, s>>>(g, d, sp, n, qe);
+    }
 }
 
 }  // namespace pic
