@@ -72,6 +72,7 @@ struct Run {
     double *M64 = nullptr;      // moment planes of the current
     int *counts64 = nullptr;
     double *spare64 = nullptr;  // one particle array of the largest capacity
+    bool ghosts64 = false;      // the current's ghosts are not zero (left so by a direct push)
     bool rotate64 = false;      // equal capacities: a gathered array trades places with the spare one
     double *rho_s = nullptr, *rho_tot = nullptr, *divb = nullptr;
     int smooth = 0;             // current smoothing passes per step (App. A.3.4)
@@ -165,6 +166,12 @@ constexpr int kPartMin = 512, kPartTiles = 65536;
 // against 7.45, 300 x 211 0.83 against 0.82.  An interval of 4 costs 58.7 ms at 128^3.
 constexpr int kSort64Interval = 16;
 constexpr size_t kSort64Bytes = 100u << 20;
+// With fewer particles than a fifth of the cells the FP64 push gathers and deposits at the
+// particle (push_fp64.cu), as node averages and moments cost by the cell.  Per step, direct
+// against by moments, at 0.04 / 0.2 / 0.4 / 1 particles per cell: 200^3 1.22 / 3.31 / 5.85 / 13.5
+// against 2.87 / 3.67 / 4.43 / 6.46 ms, 3000^2 0.93 / 1.76 / 2.79 / 5.87 against 1.92 / 2.40 / 2.66 / 3.95,
+// 96^3 170 / 303 / 437 / 887 against 398 / 488 / 548 / 744 us, 256^2 59 / 58 / 61 / 77 against 69 / 70 / 73 / 82.
+constexpr int kDirect64Cells = 5;
 
 pic_status fail(pic_ctx *c, pic_status st, const char *fmt, ...) {
     char buf[512];
@@ -1298,6 +1305,11 @@ const typename SmoothValue<JT>::type *smooth_current(pic_ctx *ctx, Run &r, JT *c
     return launch_smooth_current<JT>(r.g, J, r.smooth, buf, ctx->stream);
 }
 
+// Does the push of n particles of r gather and deposit at the particle?
+bool direct64(const Run &r, long long n) {
+    return !r.nf64 || n * kDirect64Cells < (long long)r.g.nx * r.g.ny * r.g.nz;
+}
+
 Cells64 cells64(Run &r, const FieldPtrs<double> &f, bool direct) {
     return Cells64{direct ? nullptr : r.nf64, r.M64, f, (double *)r.J};
 }
@@ -1305,8 +1317,9 @@ Cells64 cells64(Run &r, const FieldPtrs<double> &f, bool direct) {
 // Initial staggering of newly loaded momenta of the FP64 path (App. A.3.1).
 void half_back64(Run &r, SpeciesState &S, cudaStream_t s) {
     const FieldPtrs<double> f = fields_of<double>(r);
-    if (r.nf64) launch_node_fields64(r.g, f, r.nf64, s);
-    launch_half_back64(r.g, cells64(r, f, !r.nf64), S.s64, S.n, S.h, r.d.dt, s);
+    const bool direct = direct64(r, S.n);
+    if (!direct) launch_node_fields64(r.g, f, r.nf64, s);
+    launch_half_back64(r.g, cells64(r, f, direct), S.s64, S.n, S.h, r.d.dt, s);
 }
 
 pic_status step_run(pic_ctx *ctx, Run &r) {
@@ -1315,9 +1328,11 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
     const int nsp = r.d.nspecies;
     if (ctx->precision == PIC_FP64) {
         FieldPtrs<double> f = fields_of<double>(r, true);
-        const bool direct = !r.nf64;
+        long long particles = 0;
+        for (int q = 0; q < nsp; ++q) particles += r.sp[q].n;
+        const bool direct = direct64(r, particles);
         int launches = 0;
-        if (r.spare64 && (!r.sorted || r.since_sort >= kSort64Interval)) {
+        if (r.spare64 && !direct && (!r.sorted || r.since_sort >= kSort64Interval)) {
             KTimer t(ctx, PIC_KERNEL_SORT);
             for (int q = 0; q < nsp; ++q)
                 if (r.sp[q].n > 0) {
@@ -1338,8 +1353,9 @@ pic_status step_run(pic_ctx *ctx, Run &r) {
         double *J[3] = {jplane<double>(r, 0, 0), jplane<double>(r, 0, 1), jplane<double>(r, 0, 2)};
         {
             KTimer t(ctx, PIC_KERNEL_PUSH);
-            if (direct) CK(cudaMemsetAsync(r.J, 0, jplanes(ctx) * 8 * r.g.pcells, s));
-            else CK(cudaMemsetAsync(r.M64, 0, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells, s));
+            if (direct || r.ghosts64) CK(cudaMemsetAsync(r.J, 0, jplanes(ctx) * 8 * r.g.pcells, s));
+            r.ghosts64 = direct;
+            if (!direct) CK(cudaMemsetAsync(r.M64, 0, moment_planes64(r.d.ndim) * sizeof(double) * r.g.pcells, s));
             for (int q = 0; q < nsp; ++q) {
                 SpeciesState &S = r.sp[q];
                 launch_push_fp64(r.g, cells64(r, f, direct), S.s64, S.n, S.sorted64, S.h, S.alpha, r.d.dt, S.m_over_me,

@@ -95,7 +95,8 @@ struct CellSums64 {
 // The push reads node averages and adds moments, or gathers and deposits at the particle
 // itself (direct): a cell's node averages and moments take 112 (2D) or 144 B beside the 96 B
 // of its fields, current and diagnostics, and a grid that fills the memory has no room for
-// them.  No sums are kept per lane then, and the loop over the nodes stays a loop: unrolled
+// them; and they cost by the cell, which is more than they save where particles are few
+// (kDirect64Cells).  No sums are kept per lane then, and the loop over the nodes stays a loop: unrolled
 // by 2, 4 and 8 it is as fast (400^3 cells with 2 particles each: 341, 340, 357 ms per step,
 // looped 342).
 struct MomentCells64 {

@@ -1,8 +1,9 @@
 """A rejected FP64 upload leaves its run in the context, and pic_step advances every
 run: the positions that failed must index inside the grid, and the other runs go on
-as without it.  Over the plain and the sorted path (grids of about 10^6 cells), in
-2D and 3D, periodic and between walls.  Bound: the order of the current sums, a few
-1e-16 of each array's largest value per step."""
+as without it.  Over the plain, the sorted (grids of about 10^6 cells) and the direct
+path (fewer particles than a fifth of the cells), in 2D and 3D, periodic and between
+walls.  Bound: the order of the current sums, a few 1e-16 of each array's largest value
+per step."""
 import numpy as np
 import pytest
 
@@ -15,7 +16,8 @@ BAD = [np.nan, np.inf, -np.inf, -1.0, -1e-300, -3e9, 1e300, 2.0 ** 21, 2.0 ** 40
 
 
 @pytest.mark.parametrize("ndim,shape,ppc,bc", [(2, (16, 12, 1), 4, 0), (3, (7, 9, 8), 2, 0), (2, (21, 12, 1), 4, 1),
-                                               (2, (1100, 900, 1), 0.01, 0), (3, (91, 100, 88), 0.01, 1)])
+                                               (2, (1100, 900, 1), 0.01, 0), (3, (91, 100, 88), 0.01, 1),
+                                               (2, (1100, 900, 1), 0.15, 0), (3, (91, 100, 88), 0.15, 1)])
 def test_other_runs_go_on_after_a_rejected_fp64_state(ndim, shape, ppc, bc):
     desc, fields, parts, _ = _make(ndim, shape, ppc, seed=61 + ndim, spread=0.5, amp=0.01, colocate=False, bc=(bc, 0, 0))
     if bc:   # what vanishes on the wall
