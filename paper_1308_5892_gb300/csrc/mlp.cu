@@ -355,7 +355,8 @@ struct MlpPar {
     }
 };
 
-// Drift component of given uniforms, exact or learned (tests and the gain measurement).
+// Drift component of given uniforms, exact or learned (tests and the gain measurement):
+// both as the loader draws it.
 __global__ void __launch_bounds__(256) k_sample_par(mjk::Table tb, MlpPar mp, int use_mlp, double theta, double beta0,
                                                     const double *wv, int n, double *y) {
     mjk::LoadArgs a{};
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(256) k_sample_par(mjk::Table tb, MlpPar mp, in
         const int i = i0 + lane;
         const double w = i < n ? wv[i] : 0.5;
         double err;
-        const double r = use_mlp ? mp(a, w, err) : mjk::inverse_marginal(tb, w);
+        const double r = use_mlp ? mp(a, w, err) : mjk::ExactPar()(a, w, err);
         if (i < n) y[i] = r;
     }
 }
@@ -417,6 +418,9 @@ void launch_sample_par(const double *F, double s0, double h, double psi, double 
     tb.h = h;
     tb.n = kMjTable;
     tb.F = F;
+    tb.ep = std::exp(psi);
+    tb.em = std::exp(-psi);
+    tb.iZ = 1.0 / Z;
     MlpPar mp{(const __half *)Wh, std::atanh(beta0), std::asinh(std::sqrt(theta))};
     const int blocks = std::max(1, std::min((n + 255) / 256, 152 * 16));
     k_sample_par<<<blocks, 256, 0, s>>>(tb, mp, use_mlp, theta, beta0, w, n, y);
