@@ -68,7 +68,11 @@ typedef enum { PIC_MJ_EXACT = 0, PIC_MJ_MLP = 1, PIC_MJ_NAIVE_BOOST = 2 } pic_mj
 typedef enum { PIC_KERNEL_PUSH = 0, PIC_KERNEL_FIELD = 1, PIC_KERNEL_SORT = 2, PIC_KERNEL_SMOOTH = 3 } pic_kernel_class;
 
 /* Device memory provider.  alloc returns a device pointer of at least `bytes`
- * bytes aligned to 256 bytes, or NULL; free receives the same pointer and size. */
+ * bytes aligned to 256 bytes, or NULL; free receives the same pointer and size.
+ * NULL makes pic_init return PIC_ENOMEM, but for what PIC_FP64 asks for last and
+ * can do without: node averages and moment planes (112 B per cell in 2D, 144 in
+ * 3D), and on large grids the scratch of a sort.  Without it steps give the same
+ * result to rounding in two to three times the time. */
 typedef struct {
     void *(*alloc)(size_t bytes, void *user);
     void (*free)(void *ptr, size_t bytes, void *user);
@@ -111,14 +115,15 @@ typedef struct {
 } pic_run_desc;
 
 /* Options of a context.
- *  precision      PIC_FP64: every quantity in double precision, plain
- *                 one-thread-per-particle kernel with global atomics.
+ *  precision      PIC_FP64: every quantity in double precision; currents summed
+ *                 with FP64 reductions in global memory, whose order (and with
+ *                 it the last bits) may differ between two runs.
  *                 PIC_MIXED: positions as cell index + FP32 offset (on a
  *                 grid of 2^-24 cells), FP32 momenta and fields, currents
  *                 summed exactly in fixed point (each flux rounded once to
  *                 2^-26 of a particle's volume flux, integer sums), e carried
  *                 as a pair of FP32 words (value and rounding remainder)
- *                 updated in FP64 so that its rounding does not accumulate
+ *                 updated by error-free FP32 operations, so that its rounding does not accumulate
  *                 in div e, particles kept sorted by tile; FP64 for
  *                 diagnostics.
  *  sort_interval  steps between re-sorts in PIC_MIXED (0: chosen by the autotuner)
@@ -248,7 +253,8 @@ pic_status pic_load_maxwell_juttner(pic_ctx *ctx, int run, int species, double p
 /* Advance every run by nsteps steps of the main loop (App. A.3.1).  Queued
  * on the context stream; unless PIC_FLAG_ASYNC, synchronises and reports a
  * device-side error flag (PIC_ESTATE when a particle moved more than one cell
- * in a step, PIC_ETIMEOUT when a bounded wait gave up).
+ * in a step, PIC_ETIMEOUT when a bounded wait gave up: the state is then
+ * undefined, every call on it stays valid, and the energy history starts again).
  * PIC_MIXED without PIC_FLAG_NO_GRAPH or PIC_FLAG_TIMING: once the runs are
  * sorted and a sort is due, one period of 2K steps (K = sort interval) is
  * captured as a CUDA graph (on a stream of the context's own; the capture
@@ -331,8 +337,8 @@ pic_status pic_mlp_gradients(pic_ctx *ctx, const float *x, const float *target, 
 /* FP16 inference (FP32 accumulation) of n host inputs (3 planes) into out. */
 pic_status pic_mlp_infer(pic_ctx *ctx, const float *x, int64_t n, float *out);
 /* Drift component p_par of given uniforms w (host, n values) for one
- * (theta, beta0), by method PIC_MJ_EXACT or PIC_MJ_MLP, into y (host);
- * *device_ms receives the kernel time. */
+ * (theta, beta0), by method PIC_MJ_EXACT or PIC_MJ_MLP, as the loader draws
+ * them, into y (host); *device_ms receives the kernel time. */
 pic_status pic_mj_sample_marginal(pic_ctx *ctx, double theta, double beta0, const double *w, int64_t n, double *y,
                                   int method, double *device_ms);
 

@@ -653,7 +653,8 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
             return fail(ctx, PIC_EINVAL, "tile %dx%dx%d needs more shared memory than a CTA has", r.t.T[0], r.t.T[1],
                         r.t.T[2]);
     }
-    // FP64: the cells around the box that a path or its faces reach (one below, two above)
+    // FP64: the cells around the box that a path or its faces reach: one below and two above
+    // by fluxes (the direct push), one on each side by moments
     const int G = mixed ? r.t.H : 2;
     Geom &g = r.g;
     g.ndim = d.ndim; g.nx = d.nx; g.ny = d.ny; g.nz = d.ndim == 2 ? 1 : d.nz;

@@ -10,15 +10,16 @@
 //    simulated axis (z is not padded in 2D); padded index of interior (i,j,k)
 //    is ((k+Gz)*py + (j+G))*px + (i+G), px = nx+2G, ...  Ghost cells hold the
 //    periodic images of the interior, so a tile plus halo is one contiguous box.
-//  - fields: 6 planes e_x..b_z of Real; currents: 2 buffers x 3 planes (one is
-//    accumulated while the other is zeroed); node fields (mixed path): one
-//    float4 pair per padded cell, {E_x,E_y,E_z,B_x} {B_y,B_z,0,0}, the node
-//    averages of App. A.3.3 at time t.
+//  - fields: 6 planes e_x..b_z of Real (mixed path: and the low-order part of e).
+//  - mixed path: currents in 2 buffers x 3 planes (one is accumulated while the other is
+//    zeroed); node fields, the node averages of App. A.3.3 at time t: one float4
+//    {E_x,E_y,E_z,B_x} and one float2 {B_y,B_z} per padded cell.
 //  - FP64 path: one current buffer; where there is room, node fields, three planes of
 //    double2, and the moment planes of the current (push_fp64.cu).
-//  - particles, FP64 path: SoA planes x,y,z,u_x,u_y,u_z of double (absolute
-//    positions), sorted by cell every few steps (then with an int32 id); mixed path: packed cell coordinates (uint32), FP32 offsets
-//    and momenta, and an int32 id (SpeciesMixed), kept sorted by tile.
+//  - particles, FP64 path: SoA planes x,y,z,u_x,u_y,u_z of double (absolute positions), on
+//    grids beyond L2 sorted by cell every few steps (then with an int32 id); mixed path:
+//    packed cell coordinates (uint32), FP32 offsets and momenta, and an int32 id
+//    (SpeciesMixed), kept sorted by tile.
 #pragma once
 #include <cstdint>
 #include <vector>
@@ -99,15 +100,6 @@ struct Geom {
     __host__ __device__ inline int wz(int k) const { return wrap_index(k, nz); }
     // padded index of the interior image of any integer coordinate
     __host__ __device__ inline long long widx(int i, int j, int k) const { return pidx(wx(i), wy(j), wz(k)); }
-    // the same with plain modulo wraps: smaller code where a kernel makes many such
-    // calls and registers are short (the FP64 push kernel spills with the selects)
-    __host__ __device__ inline long long widx_mod(int i, int j, int k) const {
-        int a = i % nx, b = j % ny, c = k % nz;
-        a += a < 0 ? nx : 0;
-        b += b < 0 ? ny : 0;
-        c += c < 0 ? nz : 0;
-        return pidx(a, b, c);
-    }
 };
 
 // Packed cell coordinates of the mixed path: 2D i | j<<16; 3D i | j<<11 | k<<22.

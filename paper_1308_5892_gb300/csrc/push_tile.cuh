@@ -17,8 +17,8 @@
 //    than 1 in magnitude, and one slot receives at most 4 pieces of it.  A
 //    tile of N particles (all species) therefore puts |hi| < N 2^14 and
 //    lo < 4 N 2^12 into a slot: both stay below 2^31 while N < 2^17 = 131072.
-//    A tile works through its particles in rounds of at most 64 work items
-//    (65536 particles), and before a round that could bring the particles
+//    A tile works through its particles in rounds of at most 64 work items (of at
+//    most 1024 particles, for which each is counted), and before a round that could bring the particles
 //    summed since the last flush to 2^17 the limbs are added to the global
 //    current and cleared, so no tile size or particle density can overflow
 //    them (dense filaments put several times the mean count into a tile).
