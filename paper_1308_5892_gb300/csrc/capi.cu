@@ -368,6 +368,23 @@ __global__ void k_id_index(const int32_t *id, long long n, int *inv) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x)
         if ((unsigned long long)id[p] < (unsigned long long)n) inv[id[p]] = (int)p;   // ids are 0 .. n-1
 }
+// Replaces what is no particle of the grid (storage that was never written) by one at rest in cell 0.
+__global__ void k_make_valid(Geom g, SpeciesMixed s, long long n) {
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
+        int i, j, k;
+        float off[3], u[3];
+        unpack_cell(g.ndim, get_particle(g.ndim, s, p, off, u), i, j, k);
+        bool ok = i < g.nx && j < g.ny && k < g.nz;
+        for (int a = 0; a < 3; ++a) ok = ok && off[a] >= 0.f && off[a] <= 1.f && isfinite(u[a]);
+        const float zero[3] = {0.f, 0.f, 0.f};
+        if (!ok) put_particle(g.ndim, s, p, 0u, zero, zero, __int_as_float(get_id(g.ndim, s, p)));
+    }
+}
+// Storage slot of an id by its index map; slot 0 where the map has no entry (as above).
+__device__ __forceinline__ int slot_of(const int *inv, long long id, long long n) {
+    const int p = inv[id];
+    return (unsigned long long)p < (unsigned long long)n ? p : 0;
+}
 // Species of a download by id, one per blockIdx.y: storage, count, index map and
 // destination (6 planes `stride` doubles apart).
 struct Download {
@@ -386,9 +403,10 @@ __global__ void k_id_index_mixed(int ndim, Download d) {
     }
 }
 
-__global__ void k_pick_mixed(Geom g, SpeciesMixed s, const int *inv, const long long *ids, long long m, double *st) {
+__global__ void k_pick_mixed(Geom g, SpeciesMixed s, long long n, const int *inv, const long long *ids, long long m,
+                             double *st) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
-        const int p = inv[ids[q]];
+        const int p = slot_of(inv, ids[q], n);
         int i, j, k;
         float off[3], u[3];
         unpack_cell(g.ndim, get_particle(g.ndim, s, p, off, u), i, j, k);
@@ -421,7 +439,7 @@ __global__ void k_download_by_id(Geom g, Download d, long long a, long long chun
     const long long m = min(chunk, d.n[blockIdx.y] - a);
     if (stride == 0) stride = d.n[blockIdx.y];
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x) {
-        const int p = inv[a + q];
+        const int p = slot_of(inv, a + q, d.n[blockIdx.y]);
         int i, j, k;
         float off[3], u[3];
         unpack_cell(g.ndim, get_particle(g.ndim, s, p, off, u), i, j, k);
@@ -733,20 +751,13 @@ pic_status setup_run(pic_ctx *ctx, Run &r, const pic_opts *o) {
             }
             S.perm = (int *)dev_alloc(ctx, sizeof(int) * cap);
             if (!S.perm) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort");
-            // A step that a timeout ends early leaves any of these as they were, and calls after it
-            // index by their contents: everything in them is a valid particle from the start.
-            for (int b = 0; b < 2; ++b) {
-                CK(cudaMemsetAsync(S.mb[b].a, 0, sizeof(float4) * cap, ctx->stream));
-                CK(cudaMemsetAsync(S.mb[b].b, 0, sizeof(float) * (d.ndim == 3 ? 4 : 2) * cap, ctx->stream));
-                if (S.mb[b].id) CK(cudaMemsetAsync(S.mb[b].id, 0, sizeof(int32_t) * cap, ctx->stream));
-            }
-            CK(cudaMemsetAsync(S.perm, 0, sizeof(int) * cap, ctx->stream));
             S.counts = (int *)dev_alloc(ctx, sizeof(int) * (r.max_keys + 1));
             if (!S.counts) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for the sort counts");
             S.tile_start = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             S.tile_start_alt = (int *)dev_alloc(ctx, sizeof(int) * (r.max_tiles + 1));
             if (!S.tile_start || !S.tile_start_alt) return fail(ctx, PIC_ENOMEM, "allocator returned NULL for tile offsets");
             CK(cudaMemsetAsync(S.tile_start, 0, sizeof(int) * (r.max_tiles + 1), ctx->stream));
+            // (a step that a timeout ends early may leave these as they are)
             CK(cudaMemsetAsync(S.tile_start_alt, 0, sizeof(int) * (r.max_tiles + 1), ctx->stream));
         }
     }
@@ -855,8 +866,13 @@ pic_status read_err(pic_ctx *ctx) {
         CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
         if (e & ERR_TIMEOUT) {
             // Steps that did not end are in nobody's record: host and device start it again together.
-            // The sort or the push of any run may be missing: the next step sorts from storage order.
+            // The sort or the push of any run may be missing: what is no particle becomes one, and
+            // the next step sorts from storage order.  (Steps queued behind stay inside their arrays
+            // whatever the storage holds: keys and sources are checked, cells wrap or are clamped.)
             for (auto &r : ctx->runs) {
+                for (int q = 0; ctx->precision == PIC_MIXED && q < r.d.nspecies; ++q)
+                    if (r.sp[q].n > 0)
+                        k_make_valid<<<nblk(r.sp[q].n), 256, 0, ctx->stream>>>(r.g, r.sp[q].mb[r.sp[q].cur], r.sp[q].n);
                 r.hist_n = 0;
                 CK(cudaMemsetAsync(r.hist, 0, sizeof(double) * 8 * r.hist_cap, ctx->stream));
                 CK(cudaMemsetAsync(r.hist_idx, 0, sizeof(long long), ctx->stream));
@@ -1910,7 +1926,7 @@ pic_status pic_get_particles(pic_ctx *ctx, int run, int species, const int64_t *
         const int64_t m = std::min(chunk, nids - a0);
         long long *dids = reinterpret_cast<long long *>(stg + 6 * m);
         CK(cudaMemcpyAsync(dids, ids + a0, sizeof(long long) * m, cudaMemcpyHostToDevice, sm));
-        if (ctx->precision == PIC_MIXED) k_pick_mixed<<<nblk(m), 256, 0, sm>>>(r.g, S.mb[S.cur], S.perm, dids, m, stg);
+        if (ctx->precision == PIC_MIXED) k_pick_mixed<<<nblk(m), 256, 0, sm>>>(r.g, S.mb[S.cur], S.n, S.perm, dids, m, stg);
         else k_pick64<<<nblk(m), 256, 0, sm>>>(S.s64, S.sorted64 ? r.perm : nullptr, dids, m, r.d.ndim, stg);
         CK(cudaGetLastError());
         for (int a = 0; a < 6; ++a)

@@ -173,8 +173,9 @@ __device__ __noinline__ void gather_global(const Geom &g, const float4 *nA, cons
                 float w = (eps ? d[0] : 1.f - d[0]) * (eta ? d[1] : 1.f - d[1]);
                 if (NDIM == 3) w *= (xi ? d[2] : 1.f - d[2]);
                 // with walls the x node is not wrapped: node nx lies in the padding and holds the
-                // masked averages of the high wall, which differ from node 0's
-                const long long q = g.bcx == 1 ? g.pidx(ci + eps, g.wy(cj + eta), g.wz(ck + xi))
+                // masked averages of the high wall, which differ from node 0's (a cell beyond the
+                // walls is in storage that a timeout left unwritten)
+                const long long q = g.bcx == 1 ? g.pidx(min(ci, g.nx - 1) + eps, g.wy(cj + eta), g.wz(ck + xi))
                                                : g.widx(ci + eps, cj + eta, ck + xi);
                 const float4 a = ldro(nA + q);
                 const float2 b = ldro(nB + q);

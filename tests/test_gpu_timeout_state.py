@@ -29,11 +29,12 @@ def _stalled_step(ctx, n):
 
 @pytest.mark.parametrize("runs,wall", [(BALANCED_RUNS, 0), (ORACLE_RUNS[:3], 0), (BALANCED_WALL_RUNS, 1),
                                        (BALANCED_3D_RUNS, 0), (BALANCED_3D_RUNS[::2], 1)])
-@pytest.mark.parametrize("before,steps", [(0, 1), (0, 3), (4, 1), (6, 2)])   # the hook hits the first sort, a later one, none
-def test_calls_after_a_timeout_stay_in_range(runs, wall, before, steps):
+# the hook hits the first sort, a later one, none; and sorts queued behind one
+@pytest.mark.parametrize("before,steps,interval", [(0, 1, 4), (0, 3, 4), (4, 1, 4), (6, 2, 4), (0, 3, 1), (2, 4, 1)])
+def test_calls_after_a_timeout_stay_in_range(runs, wall, before, steps, interval):
     runs = [r[:-1] + (0,) for r in runs] if wall else runs   # (no smoothing between walls)
     descs, states = _random_ensemble(runs, (wall, 0, 0), 950)
-    with pic.Context(descs, precision=pic.PIC_MIXED, sort_interval=4) as ens:
+    with pic.Context(descs, precision=pic.PIC_MIXED, sort_interval=interval) as ens:
         _set(ens, states)
         ens.step(before)
         _stalled_step(ens, steps)
@@ -53,7 +54,7 @@ def test_calls_after_a_timeout_stay_in_range(runs, wall, before, steps):
         _set(ens, states)
         ens.step(5)
         got = [ens.get_state(r) for r in range(len(descs))]
-    with pic.Context(descs, precision=pic.PIC_MIXED, sort_interval=4) as ref:
+    with pic.Context(descs, precision=pic.PIC_MIXED, sort_interval=interval) as ref:
         _set(ref, states)
         ref.step(5)
         for r in range(len(descs)):
