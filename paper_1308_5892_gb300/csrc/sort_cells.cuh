@@ -151,11 +151,8 @@ __device__ inline void box_body(const SortArgs &a, int tile, int part, int parts
         else atomicOr(a.err, ERR_SORT);   // counts inconsistent with the particles
     };
     auto place_key = [&](int r, int key, int p) {
-        const int dt = key_tile(t, key);
-        if ((unsigned)dt >= (unsigned)t.ntiles) {   // a cell outside the grid (storage never written)
-            atomicOr(a.err, ERR_SORT);
-            return;
-        }
+        // (clamped: the cell may lie outside the grid in storage that was never written)
+        const int dt = (int)min((unsigned)key_tile(t, key), (unsigned)(t.ntiles - 1));
         place(r, ldro(a.tile_start + dt), ldro(a.tile_start + dt + 1), p);
     };
     for (Slot base = t0 + (int)((long long)nt * part / parts); slot_before(base, end);
