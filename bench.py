@@ -456,11 +456,11 @@ FP64_INST_PER_PARTICLE = {3: 186.0, 2: 113.2}
 MIXED_FP32_FLOPS_PER_PARTICLE = {3: 331.8}
 # DRAM bytes (read + written) per particle-step of the 3D push kernel, from one
 # ncu capture of the same kernel and tiling (16x8x4, sort interval 3) on the
-# 64^3 case (profiles/push_mixed_thermal3d_64.md: 1413.5 MB on the step of a sort,
-# whose push moves the particles, and 1051.5 on the two others, for 16,777,216
+# 64^3 case (profiles/push_mixed_thermal3d_64.md: 1612.8 MB on the step of a sort,
+# whose push moves the particles, 1047.9 and 1050.1 on the two others, for 16,777,216
 # particles), scaled to a launch by the particles it processes.  None where no
 # capture exists.
-PUSH_TRAFFIC_B_PER_PARTICLE = {3: (1413.5e6 + 2 * 1051.5e6) / 3 / 16777216}
+PUSH_TRAFFIC_B_PER_PARTICLE = {3: (1612.8e6 + 1047.9e6 + 1050.1e6) / 3 / 16777216}
 PUSH_TRAFFIC_TILING = {3: ([16, 8, 4], 3)}   # (tile, sort interval) of that capture
 
 
