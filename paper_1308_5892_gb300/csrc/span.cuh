@@ -18,7 +18,8 @@ typedef uint32_t Slot;
 PIC_HD Slot slot_at(Slot base, unsigned offset) { return base + offset; }
 PIC_HD bool slot_before(Slot p, int end) { return p < (Slot)end; }
 
-// Rows of 32 that hold n particles.
-PIC_HD int slot_rows(int n) { return (int)(((uint32_t)n + 31u) >> 5); }
+// Rows of 32 that hold n particles; none for a negative n (the difference of two offsets
+// of which a sort that timed out has written one).
+PIC_HD int slot_rows(int n) { return n > 0 ? (int)(((uint32_t)n + 31u) >> 5) : 0; }
 
 }  // namespace pic

@@ -62,3 +62,7 @@ def test_rounds_past_the_end_form_no_position(lib, first, end, step):
 
 def test_rows_at_the_ends_of_the_range(lib):
     assert [lib.rows(n) for n in (0, 1, 32, 33, TOP - 31, TOP)] == [0, 1, 1, 2, 2 ** 26 - 1, 2 ** 26]
+
+
+def test_no_rows_for_offsets_out_of_order(lib):
+    assert [lib.rows(n) for n in (-1, -31, -32, -TOP)] == [0, 0, 0, 0]
